@@ -48,7 +48,7 @@ static DecodePlan make_plan(const Dims& d, int S_cap) {
 
 size_t decode_workspace_bytes(const Dims& d, int dtype, int S_cap, int page_size) {
     // the kernel family is a function of shape, dtype and page size only, so the size is that family's
-    if (decode_fast_supported(d, dtype, page_size) && S_cap > 0) return decode_fast_workspace_bytes(d);
+    if (decode_fast_supported(d, dtype, page_size) && S_cap > 0) return decode_fast_workspace_bytes(d, page_size);
     return make_plan(d, S_cap).total;
 }
 

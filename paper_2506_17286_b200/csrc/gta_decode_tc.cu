@@ -88,9 +88,7 @@ __host__ __device__ inline BtSmem bt_smem_layout(int T, int n_k, int ch) {
     return s;
 }
 
-// kBoxes: a paged pool with pages smaller than a sub-tile.  An instantiation of its own: the same choice at run time
-// cost the other callers 3 - 10 % of their step (32 sequences of 4096 tokens: 59.5 -> 61.5 - 65.2 us).
-template <int T, int NK, int QPK, int CH, bool kBoxes>
+template <int T, int NK, int QPK, int CH>
 __global__ void __launch_bounds__(kBtThreads, 1)
 decode_stream_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_c, Dims d,
                         int S_cap, const __nv_bfloat16* __restrict__ q, const int32_t* __restrict__ seq_lens,
@@ -214,55 +212,27 @@ decode_stream_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         constexpr int n_ops = 2 * NK + 2 * CH;
         int b = b0, k = k0, it = 0;
         bool ok = true;
-        int len_b = kBoxes ? L.len(b0) : 0;
         for (; it < n_sub; ++it, ++k) {
-            while (k >= prefix[b + 1] - prefix[b]) {
-                ++b;
-                k = 0;
-                if (kBoxes) len_b = L.len(b);
-            }
+            while (k >= prefix[b + 1] - prefix[b]) { ++b; k = 0; }
             const int s = it % kBtStages;
             const uint32_t ph = (it / kBtStages) & 1;
-            // Contiguous caches: rows tok0 .. of plane b groups + g.  Paged pool whose pages hold whole sub-tiles: at rows
-            // tok0 % page_size .. of plane page groups + g; the block-table entry is fetched before the wait for the
-            // stage.  An entry outside the pool raises the status word, and the load (of page 0 then) still completes
-            // the stage.  kBoxes (smaller pages): a tile comes in boxes of pm.box rows that each lie inside one page, lane
-            // i looks up the page of box i; boxes past the live length are not loaded (the rows they leave behind are
-            // masked and cleared like every row past the length).
-            int tok0 = k * T, plane = b, live_box = 1;
-            if (kBoxes) {
-                live_box = min(T / pm.box, (len_b - tok0 + pm.box - 1) / pm.box);
-                tok0 += lane * pm.box;
-                if (lane < live_box) {
-                    const int page = page_of(pm, b, tok0, status_word);
-                    plane = page < 0 ? 0 : page;
-                }
-                tok0 %= pm.page_size;
-            } else if (pm.table != nullptr) {
+            // Contiguous caches: rows tok0 .. of plane b groups + g.  Paged pool: the sub-tile lies inside one page
+            // (T divides the page size), at rows tok0 % page_size .. of plane page groups + g; the block-table entry
+            // is fetched before the wait for the stage.  An entry outside the pool raises the status word, and the
+            // load (of page 0 then) still completes the stage.
+            int tok0 = k * T, plane = b;
+            if (pm.table != nullptr) {
                 const int page = page_of(pm, b, tok0, lane == 0 ? status_word : nullptr);
                 plane = page < 0 ? 0 : page;
                 tok0 %= pm.page_size;
             }
             if (lane == 0) {
                 ok = wait(&empty_bar[s], ph ^ 1);
-                if (ok) ptx::mbar_arrive_expect_tx(&full_bar[s], (uint32_t)n_ops * (kBoxes ? live_box * pm.box * 128u : tb));
+                if (ok) ptx::mbar_arrive_expect_tx(&full_bar[s], (uint32_t)n_ops * tb);
             }
             ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
             if (!ok) break;
             uint8_t* stage = ring + s * lay.stage_stride;
-            if (kBoxes) {
-                for (int base = 0; base < n_ops * live_box; base += 32) {
-                    const int i = (base + lane) / n_ops, op = base + lane - i * n_ops;
-                    const int row_i = __shfl_sync(0xffffffffu, tok0, i), plane_i = __shfl_sync(0xffffffffu, plane, i);
-                    uint8_t* dst = stage + op * tb + i * pm.box * 128;
-                    if (i >= live_box) continue;
-                    if (op < 2 * NK)
-                        ptx::tma_load_3d_hint(dst, &tm_k, &full_bar[s], (op / NK) * 64, row_i, plane_i * NK + op % NK, policy);
-                    else
-                        ptx::tma_load_3d_hint(dst, &tm_c, &full_bar[s], (op - 2 * NK) * 64, row_i, plane_i, policy);
-                }
-                continue;
-            }
             for (int op = lane; op < n_ops; op += 32) {
                 if (op < 2 * NK)        // half op / NK of key group op % NK
                     ptx::tma_load_3d_hint(stage + op * tb, &tm_k, &full_bar[s], (op / NK) * 64, tok0, plane * NK + op % NK, policy);
@@ -656,11 +626,11 @@ decode_stream_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     if (tid == 0 && *abort_flag) raise_status(status_word, GTA_ERR_TIMEOUT);
 }
 
-template <int T, int NK, int QPK, int CH, bool kBoxes>
+template <int T, int NK, int QPK, int CH>
 cudaError_t launch_bt(const CUtensorMap& tm_k, const CUtensorMap& tm_c, const Dims& d, int G, int S_cap, const void* q,
                       const int32_t* seq_lens, float* part_o, float* part_ml, int32_t* status_word, cudaStream_t stream,
                       const void* k_new, const void* c_new, void* k_cache, void* c_cache, const PageMap& pm) {
-    auto kern = decode_stream_tc_kernel<T, NK, QPK, CH, kBoxes>;
+    auto kern = decode_stream_tc_kernel<T, NK, QPK, CH>;
     const size_t smem = bt_smem_layout(T, NK, CH).total;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
@@ -692,10 +662,10 @@ cudaError_t launch_bt(const CUtensorMap& tm_k, const CUtensorMap& tm_c, const Di
 
 }  // namespace
 
-// d_h = 128, one latent group, one CTA per SM, one of the instantiated shapes; a paged pool's pages hold whole boxes of 16 rows
+// d_h = 128, one latent group, one CTA per SM, one of the instantiated shapes; a paged pool's pages hold whole sub-tiles
 bool decode_tc_supported(const Dims& d, int T, int occ, int page_size) {
     if (occ != 1 || d.d_h != 128 || d.n_c != 1 || d.B > kBtMaxBatch) return false;
-    if (page_size % 16 != 0) return false;
+    if (page_size % T != 0) return false;
     const int ch = d.d_l / 128, qpk = d.n_k > 0 ? d.n_q / d.n_k : 0;
     if (d.d_l % 128 != 0) return false;
 #define GTA_BT_MATCH(TV, NKV, QPKV, CHV) if (T == TV && d.n_k == NKV && qpk == QPKV && ch == CHV) return true;
@@ -709,7 +679,7 @@ cudaError_t launch_decode_tc_stream(const Dims& d, int G, int T, int S_cap, cons
                                     int32_t* status_word, cudaStream_t stream, const void* k_new, const void* c_new,
                                     const PageMap& pm) {
     CUtensorMap tm_k, tm_c;
-    const uint32_t box[3] = {64, (uint32_t)(pm.table ? pm.box : T), 1};
+    const uint32_t box[3] = {64, (uint32_t)T, 1};
     // planes of rows: one per (sequence, group), S_cap rows each -- or one per (page, group), page_size rows
     const uint64_t rows = pm.table ? (uint64_t)pm.page_size : (uint64_t)S_cap;
     const uint64_t outer = pm.table ? (uint64_t)pm.n_pages : (uint64_t)d.B;
@@ -718,13 +688,11 @@ cudaError_t launch_decode_tc_stream(const Dims& d, int G, int T, int S_cap, cons
     if (!make_bf16_map(&tm_k, k_cache, 3, dk, box) || !make_bf16_map(&tm_c, c_cache, 3, dc, box))
         return cudaErrorInvalidValue;
     const int ch = d.d_l / 128, qpk = d.n_q / d.n_k;
-    const bool boxes = pm.table != nullptr && pm.box < T;
     cudaError_t err = cudaErrorInvalidValue;
 #define GTA_BT_LAUNCH(TV, NKV, QPKV, CHV)                                                                          \
     if (T == TV && d.n_k == NKV && qpk == QPKV && ch == CHV)                                                       \
-        err = (TV > 16 && boxes ? launch_bt<TV, NKV, QPKV, CHV, (TV > 16)> : launch_bt<TV, NKV, QPKV, CHV, false>)( \
-            tm_k, tm_c, d, G, S_cap, q, seq_lens, part_o, part_ml, status_word, stream, k_new, c_new,              \
-            const_cast<void*>(k_cache), const_cast<void*>(c_cache), pm);
+        err = launch_bt<TV, NKV, QPKV, CHV>(tm_k, tm_c, d, G, S_cap, q, seq_lens, part_o, part_ml, status_word,    \
+                                            stream, k_new, c_new, const_cast<void*>(k_cache), const_cast<void*>(c_cache), pm);
     GTA_BT_SHAPES(GTA_BT_LAUNCH)
 #undef GTA_BT_LAUNCH
     if (err != cudaSuccess) return err;

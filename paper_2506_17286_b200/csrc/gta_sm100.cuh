@@ -32,6 +32,9 @@ gta_status_t sm100_attention_debug_wait(unsigned long long limit_ns, int withhol
 gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
                                   void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens = nullptr,
                                   int step_batch = 0, int step_cap = 0, bool release = true);
+// The same for an L in two bf16 planes [2][B, n_q, N, d_l] whose sum it is; the gates are kept in fp32.
+gta_status_t launch_sm100_decoder_fine(const Dims& d, const void* l_planes, const void* x, const void* w_p, const void* w_g,
+                                       void* out, int32_t* status_word, cudaStream_t stream, bool release = true);
 
 // Linear maps of the attention layer around the operator (App. B.1.1), bf16 with fp32 accumulation.
 // True when the tcgen05 kernel covers the layer's projections for this shape.

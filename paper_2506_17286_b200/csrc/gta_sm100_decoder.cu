@@ -22,6 +22,10 @@
 // its time on MMAs over padding.  That case runs the same kernel without pairs (template parameter
 // kPair = false: plain clusters of one, cta_group::1, M = 128) on items of HALF a head (64
 // columns), twice as many CTAs each with half the MMA time.
+//
+// kFine (calls over pages that are not whole tiles, which keep the precision of the plain-ALU kernels): L comes as the sum of
+// two bf16 planes, both contracted with W_P into the same accumulator, and the gates are fp32: in registers without CTA pairs,
+// with pairs (four times the columns per warp) worked out of tensor memory when the item is stored.
 #include "gta_sm100.cuh"
 
 #include <cuda.h>
@@ -61,6 +65,8 @@ __device__ __forceinline__ float sigmoid_tanh(float z) {
     asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * z));
     return fmaf(0.5f, t, 0.5f);
 }
+// to about 2^-19 of its value (an exponential of 2 + 1.2 |z| ulp, a reciprocal of 1): fp32 for what bf16 is to be rounded from
+__device__ __forceinline__ float sigmoid(float z) { return __fdividef(1.f, 1.f + __expf(-z)); }
 
 // Static schedule.  The output columns of a token (n_h d_h of them, head after head) are cut in
 // blocks of 256 -- or 128 where the heads of an attention map do not fill a multiple of 256 -- that
@@ -112,7 +118,7 @@ __device__ __forceinline__ Item item_of(const Schedule& s, int pr, int G, int n)
     return it;
 }
 
-template <bool kPair>
+template <bool kPair, bool kFine>
 __global__ void __launch_bounds__(kDecThreads, 1)
 sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_constant__ CUtensorMap tm_x,
                      const __grid_constant__ CUtensorMap tm_wp, const __grid_constant__ CUtensorMap tm_wg,
@@ -147,7 +153,7 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
     const int G = kPair ? gridDim.x >> 1 : gridDim.x;                   // CTA pairs (or CTAs)
     const int pr = kPair ? blockIdx.x >> 1 : blockIdx.x;                // this pair
     const int n_items = items_of_pair(sch, pr);
-    const int ks_g = d.H / kBlockK, ks_p = d.d_l / kBlockK, ks_total = ks_g + ks_p;
+    const int ks_g = d.H / kBlockK, ks_l = d.d_l / kBlockK, ks_total = ks_g + (kFine ? 2 : 1) * ks_l;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < n_stages; ++s) { ptx::mbar_init(&full_bar[s], kPair ? 2 : 1); ptx::mbar_init(&empty_bar[s], 1); }
@@ -206,7 +212,8 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
                             for (int grp = 0; grp < n_grp; ++grp)
                                 ptx::tma_load_2d(b_s + grp * kBGroupBytes, &tm_wg, bar, fc + grp * 64, ks * kBlockK);
                         } else {
-                            const int kk = ks - ks_g;
+                            const bool lower = kFine && ks - ks_g >= ks_l;      // the second plane of L
+                            const int kk = lower ? ks - ks_g - ks_l : ks - ks_g;
                             if (!l_ready) {
                                 ptx::grid_dependency_wait();
                                 if (release) ptx::grid_launch_dependents();
@@ -217,7 +224,7 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
                                         if (len >= 0 && len < step_cap) step_lens[sb] = len + 1;
                                     }
                             }
-                            ptx::tma_load_3d(a_s, &tm_l, bar, kk * kBlockK, t0, w.b * d.n_q + g);
+                            ptx::tma_load_3d(a_s, &tm_l, bar, kk * kBlockK, t0, (lower ? d.B + w.b : w.b) * d.n_q + g);
                             for (int grp = 0; grp < n_grp; ++grp)
                                 ptx::tma_load_3d(b_s + grp * kBGroupBytes, &tm_wp, bar, wp_col[grp], kk * kBlockK,
                                                  wp_head[grp]);
@@ -231,7 +238,8 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
                         for (int grp = 0; grp < n_grp; ++grp)
                             ptx::tma_load_2d_pair(b_s + grp * kBGroupBytes, &tm_wg, bar, fc + grp * 64, ks * kBlockK);
                     } else {
-                        const int kk = ks - ks_g;
+                        const bool lower = kFine && ks - ks_g >= ks_l;          // the second plane of L
+                        const int kk = lower ? ks - ks_g - ks_l : ks - ks_g;
                         // L comes from the kernel before this one in the stream; this kernel is
                         // launched with programmatic serialisation, so the gate phase above (X, W_G
                         // only) may already have run while that kernel was draining
@@ -245,7 +253,7 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
                                         if (len >= 0 && len < step_cap) step_lens[sb] = len + 1;
                                     }
                             }
-                        ptx::tma_load_3d_pair(a_s, &tm_l, bar, kk * kBlockK, t0, w.b * d.n_q + g);
+                        ptx::tma_load_3d_pair(a_s, &tm_l, bar, kk * kBlockK, t0, (lower ? d.B + w.b : w.b) * d.n_q + g);
                         for (int grp = 0; grp < n_grp; ++grp)
                             ptx::tma_load_3d_pair(b_s + grp * kBGroupBytes, &tm_wp, bar, wp_col[grp], kk * kBlockK,
                                                   wp_head[grp]);
@@ -313,27 +321,35 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
             const int cols = w.nt / 2;               // this warp's columns: 128, 64 or 32
             const int c0 = half * cols;
             const int t = w.t0 + (int)rank * kTileM + row;
-            uint32_t gate[64];                       // sigmoid gates, packed bf16 pairs
+            constexpr bool kLate = kFine && kPair;
+            uint32_t gate[64];                       // sigmoid gates, packed bf16 pairs (kFine: 32 in fp32)
             ok = __all_sync(0xffffffffu, ptx::mbar_wait(accg_full, n & 1, abort_flag));
             if (!ok) break;
             ptx::tc_fence_after_sync();
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
-                if (ch * 32 < cols) {
+                if (!kLate && ch * 32 < cols && (!kFine || ch == 0)) {
                     uint32_t z[32];
                     ptx::tmem_ld32(tmem_g + lane_base + c0 + ch * 32, z);
                     ptx::tmem_wait_ld();
+                    if (kFine) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) gate[e] = __float_as_uint(sigmoid(__uint_as_float(z[e])));
+                        continue;
+                    }
 #pragma unroll
                     for (int e = 0; e < 16; ++e)
                         gate[ch * 16 + e] = pack_bf16x2(sigmoid_tanh(__uint_as_float(z[2 * e])),
                                                         sigmoid_tanh(__uint_as_float(z[2 * e + 1])));
                 }
             }
-            ptx::tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) {
-                if (kPair) ptx::mbar_arrive_cluster(accg_free_leader);
-                else ptx::mbar_arrive(accg_free);
+            if (!kLate) {
+                ptx::tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) {
+                    if (kPair) ptx::mbar_arrive_cluster(accg_free_leader);
+                    else ptx::mbar_arrive(accg_free);
+                }
             }
 
             ok = __all_sync(0xffffffffu, ptx::mbar_wait(accp_full, n & 1, abort_flag));
@@ -344,12 +360,19 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
                 if (ch * 32 < cols) {
-                    uint32_t p[32];
+                    uint32_t p[32], z[32];
                     ptx::tmem_ld32(tmem_p + lane_base + c0 + ch * 32, p);
+                    if (kLate) ptx::tmem_ld32(tmem_g + lane_base + c0 + ch * 32, z);
                     ptx::tmem_wait_ld();
                     uint32_t packed[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
+                        if (kFine) {
+                            const float s0 = kLate ? sigmoid(__uint_as_float(z[2 * e])) : __uint_as_float(gate[2 * e]);
+                            const float s1 = kLate ? sigmoid(__uint_as_float(z[2 * e + 1])) : __uint_as_float(gate[2 * e + 1]);
+                            packed[e] = pack_bf16x2(__uint_as_float(p[2 * e]) * s0, __uint_as_float(p[2 * e + 1]) * s1);
+                            continue;
+                        }
                         const uint32_t gg = gate[ch * 16 + e];
                         const float g0 = __uint_as_float(gg << 16), g1 = __uint_as_float(gg & 0xffff0000u);
                         packed[e] = pack_bf16x2(__uint_as_float(p[2 * e]) * g0, __uint_as_float(p[2 * e + 1]) * g1);
@@ -369,6 +392,7 @@ sm100_decoder_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_cons
             if (lane == 0) {
                 if (kPair) ptx::mbar_arrive_cluster(accp_free_leader);
                 else ptx::mbar_arrive(accp_free);
+                if (kLate) ptx::mbar_arrive_cluster(accg_free_leader);
             }
         }
     }
@@ -398,14 +422,15 @@ int sm_count() {
 
 }  // namespace
 
-gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
-                                  void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens,
-                                  int step_batch, int step_cap, bool release) {
+template <bool kFine>
+static gta_status_t launch_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
+                                   void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens,
+                                   int step_batch, int step_cap, bool release) {
     CUtensorMap tm_l, tm_x, tm_wp, tm_wg;
     const bool solo = d.N <= kTileM;                                    // one row tile: no CTA pairs
     const uint32_t a_rows = solo ? (uint32_t)((d.N + 7) & ~7) : kTileM; // rows of an A tile
     {
-        const uint64_t dims[3] = {(uint64_t)d.d_l, (uint64_t)d.N, (uint64_t)d.B * d.n_q};
+        const uint64_t dims[3] = {(uint64_t)d.d_l, (uint64_t)d.N, (uint64_t)d.B * d.n_q * (kFine ? 2 : 1)};
         const uint32_t box[3] = {kBlockK, a_rows, 1};
         if (!make_bf16_map(&tm_l, l_bf16, 3, dims, box)) return GTA_ERR_CUDA;
     }
@@ -444,7 +469,7 @@ gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void*
         s.RT = 1;
         const long long U = (long long)d.B * s.n_hp;
         if (U > 0x3fffffffLL) return GTA_ERR_UNSUPPORTED;
-        if (cudaFuncSetAttribute(sm100_decoder_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(sm100_decoder_kernel<false, kFine>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem_bytes) != cudaSuccess)
             return GTA_ERR_CUDA;
         const int G = U < sm_count() ? (int)U : sm_count();
@@ -456,7 +481,7 @@ gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void*
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, sm100_decoder_kernel<false>, tm_l, tm_x, tm_wp, tm_wg, d, s, (__nv_bfloat16*)out,
+        if (cudaLaunchKernelEx(&cfg, sm100_decoder_kernel<false, kFine>, tm_l, tm_x, tm_wp, tm_wg, d, s, (__nv_bfloat16*)out,
                                status_word, step_lens, step_batch, step_cap, (int)release) != cudaSuccess)
             return GTA_ERR_CUDA;
         return cudaGetLastError() == cudaSuccess ? GTA_OK : GTA_ERR_CUDA;
@@ -471,7 +496,7 @@ gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void*
     s.RT = (d.N + 2 * kTileM - 1) / (2 * kTileM);
     long long U = (long long)d.B * s.RT * s.n_hp;
     if (U > 0x3fffffffLL) return GTA_ERR_UNSUPPORTED;
-    if (cudaFuncSetAttribute(sm100_decoder_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(sm100_decoder_kernel<true, kFine>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kDecSmemTotal) != cudaSuccess)
         return GTA_ERR_CUDA;
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -490,7 +515,7 @@ gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void*
     if (dev != cached_dev) {
         cfg.gridDim = dim3(2 * (sm_count() / 2));
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, sm100_decoder_kernel<true>, &cfg) != cudaSuccess || n < 1) return GTA_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&n, sm100_decoder_kernel<true, kFine>, &cfg) != cudaSuccess || n < 1) return GTA_ERR_CUDA;
         cached_dev = dev;
         cached_pairs = n;
     }
@@ -506,10 +531,20 @@ gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void*
     s.split_tail = (s.pair && 2 * s.r <= G) ? 1 : 0;
     cfg.gridDim = dim3(2 * G);
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, sm100_decoder_kernel<true>, tm_l, tm_x, tm_wp, tm_wg, d, s, (__nv_bfloat16*)out,
+    if (cudaLaunchKernelEx(&cfg, sm100_decoder_kernel<true, kFine>, tm_l, tm_x, tm_wp, tm_wg, d, s, (__nv_bfloat16*)out,
                            status_word, step_lens, step_batch, step_cap, (int)release) != cudaSuccess)
         return GTA_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? GTA_OK : GTA_ERR_CUDA;
+}
+
+gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
+                                  void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens,
+                                  int step_batch, int step_cap, bool release) {
+    return launch_decoder<false>(d, l_bf16, x, w_p, w_g, out, status_word, stream, step_lens, step_batch, step_cap, release);
+}
+gta_status_t launch_sm100_decoder_fine(const Dims& d, const void* l_planes, const void* x, const void* w_p, const void* w_g,
+                                       void* out, int32_t* status_word, cudaStream_t stream, bool release) {
+    return launch_decoder<true>(d, l_planes, x, w_p, w_g, out, status_word, stream, nullptr, 0, 0, release);
 }
 
 }  // namespace gta

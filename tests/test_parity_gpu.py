@@ -463,7 +463,7 @@ PAGED_DECODE = [
     # 16-token and 64-token sub-tiles of the tensor-memory stream kernel behind a block table
     ("bf16_pages_of_64_eight_key_groups_dl1024", "bf16", 4, 512, 8, 8, 8, 1, 128, 1024, 64, [257, 15, 64, 500]),
     ("bf16_pages_of_128_two_key_groups_dl256", "bf16", 4, 256, 8, 4, 2, 1, 128, 256, 128, [300, 0, 128, 65]),
-    # page sizes the streaming kernel does not take (no multiple of 64), and fp32: the plain-ALU kernels
+    # pages smaller than a sub-tile; fp32: the plain-ALU kernels
     ("bf16_pages_of_16", "bf16", 4, 128, 4, 2, 2, 1, 128, 256, 16, [0, 512, 1, 300]),
     ("bf16_pages_of_48", "bf16", 3, 128, 8, 4, 2, 2, 64, 128, 48, [200, 5, 129]),
     ("f32_pages_of_5", "f32", 3, 96, 6, 6, 3, 1, 32, 64, 5, [100, 7, 260]),
@@ -478,17 +478,20 @@ def test_decode_paged_small_shapes(B, oracle, case):
 
 
 @pytest.mark.parametrize("shape,page_size", [
-    ((20, 5, 1, 1, 64, 128), 16), ((20, 5, 1, 1, 64, 128), 32), ((8, 4, 4, 2, 64, 256), 48),      # warp-level stream kernel
-    ((8, 4, 4, 1, 128, 512), 16), ((8, 4, 2, 1, 128, 256), 16), ((8, 4, 2, 1, 128, 256), 48), ((8, 8, 8, 1, 128, 1024), 16)])
-def test_decode_paged_boxes_within_a_sub_tile_are_bitwise_the_contiguous_decode(B, shape, page_size):
+    ((20, 5, 1, 1, 64, 128), 16), ((20, 5, 1, 1, 64, 128), 32), ((8, 4, 4, 2, 64, 256), 48), ((8, 4, 4, 1, 128, 512), 16),
+    ((8, 4, 2, 1, 128, 256), 16), ((8, 4, 2, 1, 128, 256), 48), ((8, 8, 8, 1, 128, 1024), 16),      # stream kernel
+    ((20, 5, 1, 1, 64, 128), 24)])                                                                  # plain-ALU kernels
+def test_decode_paged_small_pages_round_only_the_output(B, oracle, shape, page_size):
     """Pages smaller than a sub-tile: the same tiles from several boxes, whatever lies behind the live rows; block-table
-    entries behind the live pages are not read."""
+    entries behind the live pages are not read.  Nothing but the output is held in fewer bits than these calls have on the
+    plain-ALU kernels: probabilities to 2^-17, the rest in fp32, so that what is added to the rounding of the output
+    (2^-9 of an element at most, 1.65e-3 over all) is below a hundredth of it; bf16 probabilities alone make it 1.4 times that."""
     n_h, n_q, n_k, n_c, d_h, d_l = shape
     w = I.Workload("small_pages", "decode", "bf16", 8, 0, 256, n_h, n_q, n_k, n_c, d_h, d_l, seed=5)
     lens = [1, 15, 16, 17, 63, 64, 0, 705]
     t = I.paginate(I.decode_inputs(w, device="cuda", s_cap=720, seq_lens=lens), page_size, seed=2)
-    args = (t["q"],), (t["x_t"], t["w_p"], t["w_g"])
-    flat = B.gta_decode(*args[0], t["k_cache"], t["c_cache"], t["seq_lens"], *args[1])
+    want = oracle.decode(oracle_shape(w, seq=0), *(t[n].cpu() for n in ("q", "k_cache", "c_cache")), np.array(lens, np.int32),
+                         t["k_cache"].shape[2], *(t[n].cpu() for n in ("x_t", "w_p", "w_g")))
     owned = torch.zeros(t["n_pages"], dtype=torch.bool)
     for b, n in enumerate(lens):
         used = -(-n // page_size)
@@ -501,10 +504,12 @@ def test_decode_paged_boxes_within_a_sub_tile_are_bitwise_the_contiguous_decode(
     t["k_pool"][~owned.cuda()] = float("nan")
     t["c_pool"][~owned.cuda()] = float("nan")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    paged = B.gta_decode_paged(*args[0], t["k_pool"], t["c_pool"], t["block_table"], t["seq_lens"], *args[1],
-                               status_word=status)
+    out = B.gta_decode_paged(t["q"], t["k_pool"], t["c_pool"], t["block_table"], t["seq_lens"], t["x_t"], t["w_p"], t["w_g"],
+                             status_word=status)
     assert int(status.item()) == 0
-    assert torch.equal(flat.view(torch.int16), paged.view(torch.int16))
+    want = torch.from_numpy(np.asarray(want, np.float64)).reshape(out.shape)
+    rounding = float((want.bfloat16().double() - want).norm())
+    assert float((out.cpu().double() - want).norm()) <= 1.01 * rounding
 
 
 def test_decode_paged_config3_full_size_sampled_sequences(B, oracle):
