@@ -83,9 +83,14 @@ typedef struct {
  *   q   [B, n_q, N, d_h]      k   [B, n_k, N, d_h]      c  [B, n_c, N, d_l]
  *   x   [B, N, H]             w_p [n_h, d_l, d_h]       w_g [H, n_h*d_h]
  *   out [B, N, n_h, d_h]      (written; same dtype as the inputs, round-to-nearest-even)
- *   workspace: at least gta_prefill_workspace_bytes(shape) bytes, 256-byte aligned; holds
- *     the normalised latent attention output L between the two kernels; contents undefined
- *     afterwards.  Calls that share a workspace must be ordered on one stream.
+ *   workspace: gta_prefill_workspace_bytes(shape) bytes, 256-byte aligned; holds the normalised
+ *     latent attention output L between the two kernels and, for calls of few rows on the tensor-core
+ *     path, fp32 partial sums behind it; contents undefined afterwards.  The size never falls as batch
+ *     or seq grow, so a buffer for the largest call serves the smaller ones.  4 B n_q N d_l bytes (at
+ *     least 256, rounded up to 256) are enough: with less room than the query gives, the keys of a call
+ *     are split over fewer parts of the chip, or not at all (same precision, other rounding of the
+ *     probabilities); with less than that, GTA_ERR_WORKSPACE.
+ *     Calls that share a workspace must be ordered on one stream.
  * Arithmetic: fp32 accumulation everywhere.  bf16 fast path (tcgen05 tensor cores) when
  * dtype = bf16, d_h = 64 or 128, d_l a multiple of 128 (at most 1024), H a multiple of 64 and
  * the heads of one attention map fill a multiple of 128 output columns ((n_h / n_q) d_h);

@@ -58,6 +58,12 @@ static gta_status_t prefill_impl(const gta_shape_t* shape, int32_t kv_len, int32
                                  const void* k, const void* c, const void* x, const void* w_p, const void* w_g,
                                  void* out, void* workspace, size_t workspace_bytes, int32_t* status_word,
                                  void* cuda_stream, int32_t stages, const gta::PageMap& pm);
+// What a prefill cannot do without: the normalised latent attention output L[B, n_q, N, d_l], fp32 on the plain-ALU path,
+// bf16 on the tensor-core path; sized for the larger so either path may run.
+static size_t prefill_least_workspace(const gta::Dims& d) {
+    const size_t bytes = (size_t)d.B * d.n_q * d.N * d.d_l * sizeof(float);
+    return bytes < 256 ? 256 : ((bytes + 255) & ~(size_t)255);
+}
 static gta_status_t decode_impl(const gta_shape_t* shape, const void* q, const void* k_cache, const void* c_cache,
                                 const int32_t* seq_lens, int32_t S_cap, const void* x_t, const void* w_p,
                                 const void* w_g, void* out, void* workspace, size_t workspace_bytes,
@@ -127,14 +133,11 @@ int gta_prefill_path(const gta_shape_t* shape) {
 size_t gta_prefill_workspace_bytes(const gta_shape_t* shape) {
     gta::Dims d;
     if (check_shape(shape, true, &d) != GTA_OK) return 0;
-    // normalised latent attention output L[B, n_q, N, d_l]: fp32 on the plain-ALU path, bf16 on
-    // the tensor-core path; sized for the larger so either path may run.
-    size_t bytes = (size_t)d.B * d.n_q * d.N * d.d_l * sizeof(float);
-    if (gta::sm100_prefill_supported(d, shape->dtype)) {      // ... where calls of few rows also split their keys
-        const size_t split = bytes / 2 + 256 + gta::sm100_attention_part_bytes(d);
-        bytes = split > bytes ? split : bytes;
-    }
-    return bytes < 256 ? 256 : ((bytes + 255) & ~(size_t)255);
+    // ... and, on the tensor-core path, room for the partial sums of a call whose keys are split over the chip.  A call is
+    // served with prefill_least_workspace too; it then splits as far as what it was given has room.
+    const size_t least = prefill_least_workspace(d);
+    const size_t split = gta::sm100_prefill_supported(d, shape->dtype) ? gta::sm100_split_workspace_bytes(d) : 0;
+    return split > least ? split : least;
 }
 
 gta_status_t gta_prefill(const gta_shape_t* shape, const void* q, const void* k, const void* c,
@@ -199,7 +202,7 @@ static gta_status_t prefill_impl(const gta_shape_t* shape, int32_t kv_len, int32
     const int path = gta_prefill_path(shape);
     if (path == 0) return GTA_ERR_UNSUPPORTED;
     if (d.B == 0 || d.N == 0) return GTA_OK;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gta_prefill_workspace_bytes(shape))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < prefill_least_workspace(d))
         return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -207,8 +210,8 @@ static gta_status_t prefill_impl(const gta_shape_t* shape, int32_t kv_len, int32
     cudaError_t err;
     // paged pools: the tensor-core attention kernel loads boxes of at least 16 tokens, each inside one page
     if (path == 2 && (pm.table == nullptr || pm.page_size % 16 == 0)) {
-        st = gta::launch_sm100_prefill(d, q, k, c, x, w_p, w_g, out, workspace, status_word, stream, stages, &launches,
-                                       pm);
+        st = gta::launch_sm100_prefill(d, q, k, c, x, w_p, w_g, out, workspace, workspace_bytes, status_word, stream, stages,
+                                       &launches, pm);
         if (st != GTA_OK) return st;
         err = cudaSuccess;
     } else {
@@ -280,13 +283,16 @@ gta_status_t gta_cache_append_paged(const gta_shape_t* shape, void* k_pool, void
 // ---- whole attention layer (App. B.1.1): projections + RoPE + cache write, operator, output projection
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
+// q, the gated heads and the rotation table, in front of the operator's own workspace
+static size_t layer_prefill_own_workspace(const gta::Dims& d, size_t es) {
+    return align256((size_t)d.B * d.n_q * d.N * d.d_h * es) + align256((size_t)d.B * d.N * d.n_h * d.d_h * es) +
+           align256(gta::sm100_rope_table_bytes(d));
+}
+
 extern "C" size_t gta_layer_prefill_workspace_bytes(const gta_shape_t* shape) {
     gta::Dims d;
     if (check_shape(shape, true, &d) != GTA_OK) return 0;
-    const size_t es = elem_size(shape->dtype);
-    const size_t q_bytes = align256((size_t)d.B * d.n_q * d.N * d.d_h * es);
-    const size_t o_bytes = align256((size_t)d.B * d.N * d.n_h * d.d_h * es);
-    return q_bytes + o_bytes + align256(gta::sm100_rope_table_bytes(d)) + gta_prefill_workspace_bytes(shape);
+    return layer_prefill_own_workspace(d, elem_size(shape->dtype)) + gta_prefill_workspace_bytes(shape);
 }
 
 static gta_status_t layer_prefill_impl(const gta_shape_t* shape, int32_t pos0, int32_t S_cap, float rope_base,
@@ -333,7 +339,8 @@ static gta_status_t layer_prefill_impl(const gta_shape_t* shape, int32_t pos0, i
         return GTA_ERR_INVALID_ARG;
     if (!gta::sm100_linear_supported(d, shape->dtype) || gta_prefill_path(shape) == 0) return GTA_ERR_UNSUPPORTED;
     if (d.B == 0 || d.N == 0) return GTA_OK;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gta_layer_prefill_workspace_bytes(shape))
+    if (!workspace || !aligned(workspace, 256) ||
+        workspace_bytes < layer_prefill_own_workspace(d, elem_size(shape->dtype)) + prefill_least_workspace(d))
         return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);

@@ -5,23 +5,23 @@
 
 namespace gta {
 
-// True when the tensor-core kernels cover this shape (bf16, d_h = 128, d_l % 256 == 0, ...).
+// True when the tensor-core kernels cover this shape (bf16, d_h = 64 or 128, d_l % 128 == 0, ...).
 bool sm100_prefill_supported(const Dims& d, int dtype);
 
 // Enqueues the tensor-core prefill (attention kernel + decoder kernel) on `stream`.
 gta_status_t launch_sm100_prefill(const Dims& d, const void* q, const void* k, const void* c, const void* x,
-                                  const void* w_p, const void* w_g, void* out, void* workspace,
+                                  const void* w_p, const void* w_g, void* out, void* workspace, size_t workspace_bytes,
                                   int32_t* status_word, cudaStream_t stream, int stages, int* launches,
                                   const PageMap& pm = PageMap());
 
 // Attention kernel alone: L[B, n_q, N, d_l] (bf16) = Softmax(scale Q K^T) C per attention map; bf16, d_h = 64 or
 // 128, d_l a multiple of 128 or exactly 64.  With a page map, k and c are paged pools (page_size a multiple of 16)
-// and token t of sequence b is looked up through the block table.  part: sm100_attention_part_bytes(d) bytes of scratch,
-// with which the key tiles of a call of few items are split over the chip (and merged by a second kernel); nullptr: no split.
-size_t sm100_attention_part_bytes(const Dims& d);
+// and token t of sequence b is looked up through the block table.  part: scratch with which the key tiles of a call of few
+// items are split over the chip (and merged by a second kernel), into as many units as it holds; nullptr: no split.
+size_t sm100_split_workspace_bytes(const Dims& d);     // L (behind which the scratch begins) and the scratch of any split
 gta_status_t launch_sm100_attention(const Dims& d, const void* q, const void* k, const void* c, void* l_out,
                                     int32_t* status_word, cudaStream_t stream, int* launches, PageMap pm = PageMap(),
-                                    float* part = nullptr);
+                                    float* part = nullptr, size_t part_bytes = 0);
 
 // Test hooks of the attention kernel's bounded waits (see gta_debug_attention_wait in gta.h).
 gta_status_t sm100_attention_debug_wait(unsigned long long limit_ns, int withhold_first_arrive);

@@ -201,6 +201,30 @@ def test_prefill_chunk_against_a_longer_cache(B, oracle, case):
     assert_close(out, want, w.torch_dtype(), name)
 
 
+@pytest.mark.parametrize("units", [0, 7, 8, 31, 74])
+@pytest.mark.parametrize("shape", [(1, 3001, 130, 4, 2, 2, 128, 512), (2, 2000, 300, 4, 2, 1, 64, 128)])
+def test_prefill_chunk_in_any_workspace_from_the_least_on(B, oracle, shape, units):
+    """4 B n_q N d_l bytes are enough for a call that would split its keys; with room for the sums of some units behind
+    L it splits into no more than those, and writes nothing past what it was given."""
+    nb, kv_len, N, n_h, n_q, n_k, d_h, d_l = shape
+    w = I.Workload("least_workspace", "prefill", "bf16", nb, kv_len, 128, n_h, n_q, n_k, 1, d_h, d_l, seed=31)
+    t = I.prefill_inputs(w, device="cuda")
+    first = kv_len - N
+    s = B.make_shape(batch=nb, seq=N, d_model=128, n_heads=n_h, n_q=n_q, n_k=n_k, n_c=1, d_h=d_h, d_l=d_l, dtype=torch.bfloat16)
+    least = -(-4 * nb * n_q * N * d_l // 256) * 256
+    unit = 256 * ((256 if d_l % 256 == 0 else 128) + 2) * 4
+    ws = Guarded((min(max(least, least // 2 + units * unit), B.prefill_workspace_bytes(s)),), torch.uint8)
+    args = [x.contiguous() for x in (t["q"][:, :, first:], t["k"], t["c"], t["x"][:, first:], t["w_p"], t["w_g"])]
+    out = B.gta_prefill_chunk(*args, kv_len, workspace=ws.t)
+    torch.cuda.synchronize()
+    ws.check("least workspace")
+    with pytest.raises(B.GtaError):
+        B.gta_prefill_chunk(*args, kv_len, workspace=torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
+    tc = cpu(t)
+    want = oracle.prefill(oracle_shape(w), tc["q"], tc["k"], tc["c"], tc["x"], tc["w_p"], tc["w_g"], rows=list(range(first, kv_len)))
+    assert_close(out, want, torch.bfloat16, "least workspace")
+
+
 @pytest.mark.parametrize("case", [
     # name, B, kv_len, N, n_h, n_q, n_k, d_h, d_l: several items per CTA pair; a split item; the narrow heads
     ("climb_several_items", 8, 700, 700, 8, 4, 4, 128, 512),
