@@ -18,6 +18,7 @@ gta_status_t launch_sm100_prefill(const Dims& d, const void* q, const void* k, c
 // 128, d_l a multiple of 128 or exactly 64.  With a page map, k and c are paged pools (page_size a multiple of 16)
 // and token t of sequence b is looked up through the block table.  part: scratch with which the key tiles of a call of few
 // items are split over the chip (and merged by a second kernel), into as many units as it holds; nullptr: no split.
+// Over pages that are not whole blocks of 64 tokens, L is two bf16 planes [2][B, n_q, N, d_l] (their sum).
 size_t sm100_split_workspace_bytes(const Dims& d);     // L (behind which the scratch begins) and the scratch of any split
 gta_status_t launch_sm100_attention(const Dims& d, const void* q, const void* k, const void* c, void* l_out,
                                     int32_t* status_word, cudaStream_t stream, int* launches, PageMap pm = PageMap(),

@@ -120,11 +120,68 @@ def test_prefill_chunk_paged_is_bitwise_the_contiguous_chunk_on_the_tensor_core_
     first = kv_len - N
     q, x = t["q"][:, :, first:].contiguous(), t["x"][:, first:].contiguous()
     flat = B.gta_prefill_chunk(q, t["k"], t["c"], x, t["w_p"], t["w_g"], kv_len)
-    for page_size in (16, 32, 48, 64, 128, 256):
+    for page_size in (64, 128, 256):
         k_pool, c_pool, table = _pools(t["k"], t["c"], kv_len, page_size, seed=page_size)
         paged = B.gta_prefill_chunk_paged(q, k_pool, c_pool, table.cuda(), x, t["w_p"], t["w_g"], kv_len)
         torch.cuda.synchronize()
         assert torch.equal(flat, paged), page_size
+
+
+FINE_PAGES = [
+    # B, kv_len, N, page_size, n_h, n_q, n_k, n_c, d_h, d_l
+    (2, 300, 120, 16, 4, 2, 2, 1, 128, 256),          # one 128-row tile: the decoder kernel without CTA pairs
+    (2, 705, 400, 48, 8, 4, 4, 1, 128, 512),          # several items
+    (5, 700, 700, 80, 8, 4, 4, 1, 64, 256),           # several items per CTA pair
+    (1, 2000, 130, 32, 4, 2, 2, 1, 128, 1024),        # keys split over the chip
+    (2, 1999, 33, 48, 4, 2, 1, 1, 64, 128),
+    (1, 3000, 600, 16, 2, 1, 1, 1, 128, 128),         # split items and whole ones
+    (2, 300, 120, 24, 4, 2, 2, 1, 128, 256),          # plain-ALU kernels
+]
+
+
+@pytest.mark.parametrize("case", FINE_PAGES, ids=lambda c: "-".join(map(str, c)))
+def test_prefill_chunk_paged_small_pages_round_only_the_output(B, oracle, case):
+    """Pages that are not whole blocks of 64 tokens: probabilities, L and gates hold what they hold on the plain-ALU kernels
+    (to 2^-17), so what is added to the rounding of the output (2^-9 of an element at most, 1.65e-3 over all) is below a
+    hundredth of it; bf16 probabilities alone make it 1.4 times that."""
+    nb, kv_len, N, page_size, n_h, n_q, n_k, n_c, d_h, d_l = case
+    w = I.Workload("fine_pages", "prefill", "bf16", nb, kv_len, 128, n_h, n_q, n_k, n_c, d_h, d_l, seed=23)
+    t = I.prefill_inputs(w, device="cuda")
+    first = kv_len - N
+    k_pool, c_pool, table = _pools(t["k"], t["c"], kv_len, page_size, seed=4)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = B.gta_prefill_chunk_paged(t["q"][:, :, first:].contiguous(), k_pool, c_pool, table.cuda(), t["x"][:, first:].contiguous(),
+                                    t["w_p"], t["w_g"], kv_len, status_word=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    tc = cpu(t)
+    want = oracle.prefill(oracle_shape(w), tc["q"], tc["k"], tc["c"], tc["x"], tc["w_p"], tc["w_g"], rows=list(range(first, kv_len)))
+    want = torch.from_numpy(np.asarray(want, np.float64)).reshape(out.shape)
+    rounding = float((want.bfloat16().double() - want).norm())
+    assert float((out.cpu().double() - want).norm()) <= 1.01 * rounding
+
+
+@pytest.mark.parametrize("page_size", [16, 48, 64])
+@pytest.mark.parametrize("shape", [(8, 700, 700, 8, 4, 4, 128, 512), (2, 2001, 300, 4, 2, 2, 128, 512), (1, 600, 600, 4, 2, 1, 64, 128)])
+def test_prefill_chunk_paged_scores_that_climb_past_the_first_keys(B, oracle, shape, page_size):
+    """Items that the attention kernel does again (a row sum past 2^60), over pages: several items per CTA pair, split
+    items with a last page of one row, narrow heads."""
+    nb, kv_len, N, n_h, n_q, n_k, d_h, d_l = shape
+    w = I.Workload("climb_paged", "prefill", "bf16", nb, kv_len, 128, n_h, n_q, n_k, 1, d_h, d_l, seed=55)
+    t = I.prefill_inputs(w, device="cuda")
+    s = torch.einsum("nd,td->nt", t["q"][-1, 0].double(), t["k"][-1, 0].double()) / d_h ** 0.5
+    t["k"][-1, 0, 200:] *= float(120 / s[:, 200:].abs().max())       # (at most 120 nats: 1e-3 of fp32 score sums)
+    first = kv_len - N
+    k_pool, c_pool, table = _pools(t["k"], t["c"], kv_len, page_size, seed=6)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = B.gta_prefill_chunk_paged(t["q"][:, :, first:].contiguous(), k_pool, c_pool, table.cuda(), t["x"][:, first:].contiguous(),
+                                    t["w_p"], t["w_g"], kv_len, status_word=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    tc = cpu(t)
+    want = oracle.prefill(oracle_shape(w), tc["q"], tc["k"], tc["c"], tc["x"], tc["w_p"], tc["w_g"], rows=list(range(first, kv_len)))
+    assert_close(out[-1:], want[-1:], w.torch_dtype(), "climb")
+    assert_close(out, want, w.torch_dtype(), "climb")
 
 
 def test_prefill_chunk_paged_full_size_c2_sampled_rows(B, oracle):
