@@ -133,10 +133,13 @@ GTA_API gta_status_t gta_prefill_chunk(const gta_shape_t *shape, int32_t kv_len,
  *            a sequence with length 0 gets an all-zero output row; cache rows at and behind
  *            seq_lens[b] may hold anything (uninitialised memory, NaN bit patterns)
  *   w_p, w_g as in gta_prefill;  out [B, n_h, d_h]
- *   workspace: at least gta_decode_workspace_bytes(shape, S_cap) bytes, 256-byte aligned
- *     (split-KV partial results and gate partial sums).  The size follows the SM count of the
- *     device that is current when the function is asked, so ask with the device the call
- *     will run on (this holds for every *_workspace_bytes function of the decode family).
+ *   workspace: gta_decode_workspace_bytes(shape, S_cap) bytes, 256-byte aligned (split-KV
+ *     partial results).  The size follows the SM count of the device that is current when the
+ *     function is asked, so ask with the device the call will run on (this holds for every
+ *     *_workspace_bytes function of the decode family).  For one kernel family it never falls as
+ *     batch or S_cap grow, so a buffer for the largest batch serves the smaller ones.  On the
+ *     plain-ALU kernels somewhat less is enough for a call (its sequences are then cut into fewer
+ *     chunks); what is too little for it is refused with GTA_ERR_WORKSPACE.
  * Needs d_h and d_l multiples of 8 (bf16) / 4 (fp32) so that rows are 16-byte vectors,
  * d_h <= 256, d_l <= 2048.  bf16 fast path (TMA-streamed caches, tensor-core decoder) when
  * d_h = 64 or 128, d_l = 128, 256, 512 or 1024, n_q <= 8, n_k = 1, 2, 4 or 8, H a
@@ -333,7 +336,7 @@ GTA_API gta_status_t gta_layer_decode_paged(const gta_shape_t *shape, const int3
  * library is used keeps that much memory until the process exits.  The call itself allocates
  * and frees nothing, on the host runtime or the device.
  *
- *   - A problem whose gta_decode_workspace_bytes() exceeds GTA_STATIC_SCRATCH_BYTES is refused
+ *   - A problem that gta_decode would refuse GTA_STATIC_SCRATCH_BYTES of workspace for is refused
  *     with GTA_ERR_STATIC_SCRATCH before anything is launched (for the bf16 kernels the need
  *     grows with batch * n_q * d_l, not with the context length).
  *   - Arguments are checked exactly as gta_decode checks them (same order, same codes; an

@@ -365,12 +365,17 @@ static gta_status_t layer_prefill_impl(const gta_shape_t* shape, int32_t pos0, i
     return GTA_OK;
 }
 
+// q, the gated heads and what the step works out of the lengths, in front of the operator's own workspace
+static size_t layer_decode_own_workspace(const gta::Dims& d, size_t es) {
+    return align256((size_t)d.B * d.n_q * d.d_h * es) + align256((size_t)d.B * d.n_h * d.d_h * es) +
+           align256(gta::sm100_decode_prep_bytes(d));
+}
+
 extern "C" size_t gta_layer_decode_workspace_bytes(const gta_shape_t* shape, int32_t S_cap) {
     gta::Dims d;
     if (check_shape(shape, false, &d) != GTA_OK || S_cap < 0) return 0;
     const size_t es = elem_size(shape->dtype);
-    return align256((size_t)d.B * d.n_q * d.d_h * es) + align256((size_t)d.B * d.n_h * d.d_h * es) +
-           align256(gta::sm100_decode_prep_bytes(d)) + gta::decode_workspace_bytes(d, shape->dtype, S_cap);
+    return layer_decode_own_workspace(d, es) + gta::decode_workspace_bytes(d, shape->dtype, S_cap);
 }
 
 static gta_status_t layer_decode_impl(const gta_shape_t* shape, int32_t S_cap, float rope_base, const void* x_t,
@@ -394,8 +399,7 @@ extern "C" size_t gta_layer_decode_paged_workspace_bytes(const gta_shape_t* shap
         (long long)page_size * max_pages > INT32_MAX)
         return 0;
     const size_t es = elem_size(shape->dtype);
-    return align256((size_t)d.B * d.n_q * d.d_h * es) + align256((size_t)d.B * d.n_h * d.d_h * es) +
-           align256(gta::sm100_decode_prep_bytes(d)) +
+    return layer_decode_own_workspace(d, es) +
            gta::decode_workspace_bytes(d, shape->dtype, page_size * max_pages, page_size);
 }
 
@@ -430,8 +434,8 @@ static gta_status_t layer_decode_impl(const gta_shape_t* shape, int32_t S_cap, f
     if (!gta::sm100_linear_supported(d, shape->dtype) || (size_t)d.d_l * elem_size(shape->dtype) > 4096)
         return GTA_ERR_UNSUPPORTED;
     if (d.B == 0) return GTA_OK;
-    const size_t ws_need = pm.table ? gta_layer_decode_paged_workspace_bytes(shape, pm.page_size, pm.max_pages)
-                                    : gta_layer_decode_workspace_bytes(shape, S_cap);
+    const size_t ws_need = layer_decode_own_workspace(d, elem_size(shape->dtype)) +
+                           gta::decode_least_workspace(d, shape->dtype, S_cap, pm.table ? pm.page_size : 0);
     if (!workspace || !aligned(workspace, 256) || workspace_bytes < ws_need) return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -492,13 +496,13 @@ static gta_status_t decode_impl(const gta_shape_t* shape, const void* q, const v
     if (st != GTA_OK) return st;
     if (empty) return GTA_OK;
     if (!workspace || !aligned(workspace, 256) ||
-        workspace_bytes < gta::decode_workspace_bytes(d, shape->dtype, S_cap, pm.table ? pm.page_size : 0))
+        workspace_bytes < gta::decode_least_workspace(d, shape->dtype, S_cap, pm.table ? pm.page_size : 0))
         return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     int launches = 0;
     cudaError_t err = gta::launch_decode(d, shape->dtype, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g,
-                                         out, workspace, status_word, static_cast<cudaStream_t>(cuda_stream),
-                                         stages, &launches, pm);
+                                         out, workspace, workspace_bytes, status_word,
+                                         static_cast<cudaStream_t>(cuda_stream), stages, &launches, pm);
     if (err != cudaSuccess) return GTA_ERR_CUDA;
     g_last_launches = launches;
     return GTA_OK;
@@ -618,8 +622,8 @@ static gta_status_t fp8_check(const gta_shape_t* shape, gta::Dims* d) {
 }
 
 // enough for either kernel family (which one runs also depends on the alignment of the scale arrays)
-static size_t fp8_workspace(const gta::Dims& d, int dtype, int S_cap) {
-    size_t need = gta::decode_fp8_workspace_bytes(d, S_cap);
+static size_t fp8_workspace(const gta::Dims& d, int dtype, int S_cap, bool least = false) {
+    size_t need = least ? gta::decode_plain_least_workspace(d, S_cap) : gta::decode_plain_workspace_bytes(d, S_cap);
     if (gta::decode_fp8_fast_supported(d, dtype, S_cap)) {
         const size_t fast = gta::decode_fp8_fast_workspace_bytes(d);
         need = fast > need ? fast : need;
@@ -679,7 +683,7 @@ extern "C" gta_status_t gta_decode_fp8(const gta_shape_t* shape, const void* q, 
         !aligned(seq_lens, 4) || !aligned(status_word, 4))
         return GTA_ERR_INVALID_ARG;
     if (d.B == 0) return GTA_OK;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < fp8_workspace(d, shape->dtype, S_cap))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < fp8_workspace(d, shape->dtype, S_cap, true))
         return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     int launches = 0;
@@ -690,7 +694,7 @@ extern "C" gta_status_t gta_decode_fp8(const gta_shape_t* shape, const void* q, 
                                           workspace, status_word, static_cast<cudaStream_t>(cuda_stream), &launches);
     else
         err = gta::launch_decode_fp8(d, shape->dtype, q, k_codes, c_codes, k_scales, c_scales, seq_lens, S_cap,
-                                     x_t, w_p, w_g, out, workspace, status_word,
+                                     x_t, w_p, w_g, out, workspace, workspace_bytes, status_word,
                                      static_cast<cudaStream_t>(cuda_stream), &launches);
     if (err != cudaSuccess) return GTA_ERR_CUDA;
     g_last_launches = launches;
@@ -716,12 +720,13 @@ extern "C" gta_status_t gta_decode_hostcache(const gta_shape_t* shape, const voi
                                              &d, &empty);
     if (st != GTA_OK) return st;
     if (empty) return GTA_OK;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gta::decode_plain_workspace_bytes(d, S_cap))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gta::decode_plain_least_workspace(d, S_cap))
         return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     int launches = 0;
     cudaError_t err = gta::launch_decode_plain(d, shape->dtype, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out,
-                                               workspace, status_word, static_cast<cudaStream_t>(cuda_stream), &launches);
+                                               workspace, workspace_bytes, status_word, static_cast<cudaStream_t>(cuda_stream),
+                                               &launches);
     if (err != cudaSuccess) return GTA_ERR_CUDA;
     g_last_launches = launches;
     return GTA_OK;
@@ -740,7 +745,7 @@ extern "C" gta_status_t gta_decode_append(const gta_shape_t* shape, const void* 
     if (st != GTA_OK) return st;
     if (S_cap <= 0 || !k_new || !c_new || !aligned(k_new, 16) || !aligned(c_new, 16)) return GTA_ERR_INVALID_ARG;
     if (empty) return GTA_OK;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gta::decode_workspace_bytes(d, shape->dtype, S_cap))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < gta::decode_least_workspace(d, shape->dtype, S_cap))
         return GTA_ERR_WORKSPACE;
     if ((st = check_device()) != GTA_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -756,7 +761,7 @@ extern "C" gta_status_t gta_decode_append(const gta_shape_t* shape, const void* 
                                        status_word, stream, &launches);
         if (err == cudaSuccess)
             err = gta::launch_decode(d, shape->dtype, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
-                                     status_word, stream, 7, &launches);
+                                     workspace_bytes, status_word, stream, 7, &launches);
     }
     if (err != cudaSuccess) return GTA_ERR_CUDA;
     g_last_launches = launches;

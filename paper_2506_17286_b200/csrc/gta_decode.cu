@@ -29,27 +29,58 @@ struct DecodePlan {
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-static DecodePlan make_plan(const Dims& d, int S_cap) {
+static DecodePlan plan_of(const Dims& d, long long chunks, int chunk, int S_cap) {
     DecodePlan p;
-    // Aim at >= 8 chunk CTAs per SM over the whole batch, chunks of 64..256 tokens; 32 where 64 would not give every SM
-    // two CTAs (a chunk's time is then latency, not its bytes).
-    const long long tokens = (long long)d.B * (S_cap > 0 ? S_cap : 1), want = tokens / (148 * 8);
-    int chunk = (int)((want + 63) / 64) * 64;
-    if (chunk <= 64) chunk = tokens < 148 * 2 * 64 && tokens * d.n_q * d.d_l <= (1 << 25) ? 32 : 64;   // partials <= 4 MB
-    if (chunk > 256) chunk = 256;
     p.chunk = chunk;
     p.n_chunks = S_cap > 0 ? (S_cap + chunk - 1) / chunk : 1;
-    const size_t part_o = (size_t)d.B * p.n_chunks * d.n_q * d.d_l * sizeof(float);
-    const size_t part_ml = (size_t)d.B * p.n_chunks * d.n_q * 2 * sizeof(float);
-    p.off_ml = align256(part_o);
-    p.total = p.off_ml + align256(part_ml);
+    p.off_ml = align256((size_t)chunks * d.n_q * d.d_l * sizeof(float));
+    p.total = p.off_ml + align256((size_t)chunks * d.n_q * 2 * sizeof(float));
     return p;
 }
+static DecodePlan plan_of(const Dims& d, int chunk, int S_cap) {
+    return plan_of(d, (long long)d.B * (S_cap > 0 ? (S_cap + chunk - 1) / chunk : 1), chunk, S_cap);
+}
+// Aim at >= 8 chunk CTAs per SM over the whole batch, chunks of 64..256 tokens.
+static DecodePlan least_plan(const Dims& d, int S_cap) {
+    const long long want = (long long)d.B * (S_cap > 0 ? S_cap : 1) / (148 * 8);
+    const int chunk = (int)((want + 63) / 64) * 64;
+    return plan_of(d, chunk < 64 ? 64 : chunk > 256 ? 256 : chunk, S_cap);
+}
+// ... and of 32 where 64 would not give every SM two CTAs (a chunk's time is then latency, not its bytes), the partial sums
+// take 4 MB at the most and the workspace has room for them.
+constexpr long long kSmallTokens = 148 * 2 * 64, kSmallPart = 1 << 25;
+static DecodePlan make_plan(const Dims& d, int S_cap, size_t room) {
+    const long long tokens = (long long)d.B * (S_cap > 0 ? S_cap : 1);
+    if (tokens < kSmallTokens && tokens * d.n_q * d.d_l <= kSmallPart) {
+        const DecodePlan p = plan_of(d, 32, S_cap);
+        if (p.total <= room) return p;
+    }
+    return least_plan(d, S_cap);
+}
+// Room for the plan of every smaller batch and capacity too, so that a buffer for the largest call serves the others.  The
+// chunks of a call are at most tokens / chunk + batch: 592 + batch of 32 tokens (fewer where their sums would pass 4 MB),
+// 1203 + batch of 64 (a chunk is 64 up to 65 x 1184 tokens) and of 128 and 192 likewise, and what 256 tokens each make.
+static size_t plan_bound(const Dims& d, int S_cap) {
+    const long long S = S_cap > 0 ? S_cap : 1, small = kSmallPart / 32 / ((long long)d.n_q * d.d_l);
+    const auto least = [](long long a, long long b) { return a < b ? a : b; };
+    const long long n32 = least(d.B * ((S + 31) / 32), least(kSmallTokens / 32, small) + d.B);
+    const long long n64 = least(d.B * ((S + 63) / 64), 1203 + d.B), n256 = d.B * ((S + 255) / 256);
+    const long long most = n32 > n64 ? n32 : n64;
+    return plan_of(d, most > n256 ? most : n256, 64, S_cap).total;
+}
 
+// The kernel family is a function of shape, dtype and page size only, so the sizes are that family's -- but over small pages
+// (which had no other kernels once) the plain-ALU kernels take what the stream kernel's workspace is too much for.
+static bool small_pages(int page_size) { return page_size % 64 != 0; }
 size_t decode_workspace_bytes(const Dims& d, int dtype, int S_cap, int page_size) {
-    // the kernel family is a function of shape, dtype and page size only, so the size is that family's
     if (decode_fast_supported(d, dtype, page_size) && S_cap > 0) return decode_fast_workspace_bytes(d, page_size);
-    return make_plan(d, S_cap).total;
+    return plan_bound(d, S_cap);
+}
+size_t decode_least_workspace(const Dims& d, int dtype, int S_cap, int page_size) {
+    const size_t plain = least_plan(d, S_cap).total;
+    if (!decode_fast_supported(d, dtype, page_size) || S_cap <= 0) return plain;
+    const size_t fast = decode_fast_workspace_bytes(d, page_size);
+    return small_pages(page_size) && plain < fast ? plain : fast;
 }
 
 // ---- 16-byte vector of storage elements, widened to fp32 ----
@@ -557,10 +588,10 @@ static cudaError_t launch_behind(Kern kern, dim3 grid, int threads, size_t smem,
 template <typename T, typename CT>
 static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void* k_cache, const void* c_cache,
                                        const int32_t* seq_lens, int S_cap, const void* x_t, const void* w_p,
-                                       const void* w_g, void* out, void* workspace, int32_t* status_word,
+                                       const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
                                        cudaStream_t stream, int stages, int* launches, const PageMap& pm,
                                        const float* k_scale = nullptr, const float* c_scale = nullptr) {
-    const DecodePlan p = make_plan(d, S_cap);
+    const DecodePlan p = make_plan(d, S_cap, room);
     float* part_o = reinterpret_cast<float*>(workspace);
     float* part_ml = reinterpret_cast<float*>(static_cast<char*>(workspace) + p.off_ml);
     cudaError_t err;
@@ -601,17 +632,15 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
 //      fixes none; its Sec. 5.3 / App. C.2 only observe that decode is bound by the bytes of the cache):
 //      scale = max|row| / 448 (1 for an all-zero row), code = round-to-nearest-even(x / scale), both
 //      divisions in fp32; the operator runs on code * scale.
-size_t decode_fp8_workspace_bytes(const Dims& d, int S_cap) { return make_plan(d, S_cap).total; }
-
 cudaError_t launch_decode_fp8(const Dims& d, int dtype, const void* q, const void* k_codes, const void* c_codes,
                               const float* k_scale, const float* c_scale, const int32_t* seq_lens, int S_cap,
-                              const void* x_t, const void* w_p, const void* w_g, void* out, void* workspace,
+                              const void* x_t, const void* w_p, const void* w_g, void* out, void* workspace, size_t room,
                               int32_t* status_word, cudaStream_t stream, int* launches) {
     if (dtype == GTA_F32)
         return launch_decode_typed<float, Fp8>(d, q, k_codes, c_codes, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
-                                               status_word, stream, 7, launches, PageMap(), k_scale, c_scale);
+                                               room, status_word, stream, 7, launches, PageMap(), k_scale, c_scale);
     return launch_decode_typed<__nv_bfloat16, Fp8>(d, q, k_codes, c_codes, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
-                                                   status_word, stream, 7, launches, PageMap(), k_scale, c_scale);
+                                                   room, status_word, stream, 7, launches, PageMap(), k_scale, c_scale);
 }
 
 // Quantising append.  A new row (token and group) is handled by a group of lanes of one warp, eight elements per lane
@@ -893,33 +922,35 @@ cudaError_t launch_cache_append_fp8(const Dims& d, int dtype, void* k_codes, voi
     return launch_append_fp8_typed<__nv_bfloat16>(a, d.B, seq_lens, status_word, stream, launches);
 }
 
-size_t decode_plain_workspace_bytes(const Dims& d, int S_cap) { return make_plan(d, S_cap).total; }
+size_t decode_plain_workspace_bytes(const Dims& d, int S_cap) { return plan_bound(d, S_cap); }
+size_t decode_plain_least_workspace(const Dims& d, int S_cap) { return least_plan(d, S_cap).total; }
 
 // The plain-ALU kernels whatever the shape: they read the caches with ordinary 16-byte loads, which is what a cache
 // in page-locked host memory (reached over the host link) needs; the TMA path is kept to device memory.
 cudaError_t launch_decode_plain(const Dims& d, int dtype, const void* q, const void* k_cache, const void* c_cache,
                                 const int32_t* seq_lens, int S_cap, const void* x_t, const void* w_p,
-                                const void* w_g, void* out, void* workspace, int32_t* status_word,
+                                const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
                                 cudaStream_t stream, int* launches) {
     if (dtype == GTA_F32)
         return launch_decode_typed<float, float>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out,
-                                                workspace, status_word, stream, 7, launches, PageMap());
+                                                workspace, room, status_word, stream, 7, launches, PageMap());
     return launch_decode_typed<__nv_bfloat16, __nv_bfloat16>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out,
-                                                    workspace, status_word, stream, 7, launches, PageMap());
+                                                    workspace, room, status_word, stream, 7, launches, PageMap());
 }
 
 cudaError_t launch_decode(const Dims& d, int dtype, const void* q, const void* k_cache, const void* c_cache,
                           const int32_t* seq_lens, int S_cap, const void* x_t, const void* w_p,
-                          const void* w_g, void* out, void* workspace, int32_t* status_word,
+                          const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
                           cudaStream_t stream, int stages, int* launches, const PageMap& pm) {
-    if (decode_fast_supported(d, dtype, pm.table ? pm.page_size : 0) && S_cap > 0)
+    const int page_size = pm.table ? pm.page_size : 0;
+    if (decode_fast_supported(d, dtype, page_size) && S_cap > 0 && room >= decode_fast_workspace_bytes(d, page_size))
         return launch_decode_fast(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
                                   status_word, stream, stages, launches, pm);
     if (dtype == GTA_F32)
         return launch_decode_typed<float, float>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out,
-                                          workspace, status_word, stream, stages, launches, pm);
+                                          workspace, room, status_word, stream, stages, launches, pm);
     return launch_decode_typed<__nv_bfloat16, __nv_bfloat16>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out,
-                                              workspace, status_word, stream, stages, launches, pm);
+                                              workspace, room, status_word, stream, stages, launches, pm);
 }
 
 }  // namespace gta

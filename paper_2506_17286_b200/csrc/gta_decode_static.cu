@@ -55,7 +55,7 @@ extern "C" gta_status_t gta_decode_static(const gta_shape_t* shape, const void* 
     if (empty) return GTA_OK;
     // Size check, still on the host: a problem that does not fit the built-in array is refused,
     // never truncated.
-    if (gta_decode_workspace_bytes(shape, S_cap) > (size_t)GTA_STATIC_SCRATCH_BYTES) return GTA_ERR_STATIC_SCRATCH;
+    if (gta::decode_least_workspace(d, shape->dtype, S_cap) > (size_t)GTA_STATIC_SCRATCH_BYTES) return GTA_ERR_STATIC_SCRATCH;
     if ((st = gta::check_current_device()) != GTA_OK) return st;
     // Only a call that will launch looks the array up (the first one on a device loads it).
     void* scratch = nullptr;

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -68,6 +69,53 @@ def test_prefill_workspace_never_falls_as_batch_or_length_grow(B, layer):
             assert r == sorted(r)
         for col in zip(*rows):
             assert list(col) == sorted(col)
+
+
+GTA1B = dict(n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64, d_l=128, d_model=1280)
+
+
+@pytest.mark.parametrize("layer", [dict(GTA1B, dtype=0), dict(), dict(n_heads=6, n_q=6, n_k=3, d_h=40, d_l=200, d_model=96, dtype=0),
+                                   dict(n_heads=32, n_q=8, n_k=8, d_h=128, d_l=1024, d_model=4096, dtype=0)])
+def test_plain_decode_workspace_never_falls_as_batch_or_capacity_grow(B, layer):
+    """A buffer for the largest batch serves what is left of it when sequences finish: contiguous caches, pages that the
+    stream kernels do not take, caches in host memory, 8-bit caches."""
+    caps = [1, 31, 32, 33, 64, 65, 200, 1000, 1024, 2999, 3000, 4096, 6000, 9473, 20000, 32768]
+    fp8 = layer.get("d_h", 32) % 16 == 0 and layer.get("d_l", 64) % 16 == 0
+    for query in (B.decode_workspace_bytes, lambda s, c: B.decode_paged_workspace_bytes(s, 8, -(-c // 8)),
+                  B.decode_hostcache_workspace_bytes) + ((B.decode_fp8_workspace_bytes,) if fp8 else ()):
+        rows = [[query(_shape(B, batch=b, **layer), c) for c in caps] for b in list(range(1, 41)) + [64, 75, 76, 96, 128, 300, 700]]
+        assert all(x > 0 for r in rows for x in r)
+        for r in rows:
+            assert r == sorted(r)
+        for col in zip(*rows):
+            assert list(col) == sorted(col)
+
+
+def test_plain_decode_runs_in_the_workspace_of_64_token_chunks(B):
+    """Partial sums (fp32) and (maximum, sum) pairs of every chunk of 64 tokens, of 128 .. 256 where the batch has more than
+    1184 chunks of fewer: that much, and a buffer for the largest batch, is never refused.  (Without a GPU the call ends at
+    the device check, behind that of the workspace.)"""
+    if torch.cuda.is_available():
+        pytest.skip("the pointers are not device memory")
+    L = B.lib()
+    buf = (ctypes.c_char * 1024)()
+    p = ctypes.c_void_p((ctypes.addressof(buf) + 255) & ~255)
+
+    def status(batch, cap, ws):
+        s = _shape(B, batch=batch, dtype=0, **GTA1B)
+        return L.gta_decode(ctypes.byref(s), p, p, p, p, cap, p, p, p, p, p, ws, None, None)
+
+    def least(batch, cap):
+        chunk = min(256, max(64, -(-(batch * cap // 1184) // 64) * 64))
+        n = batch * -(-cap // chunk) * 5
+        return -(-n * 128 * 4 // 256) * 256 + -(-n * 8 // 256) * 256
+
+    for cap in (1, 100, 3000, 4096, 9000):
+        most = B.decode_workspace_bytes(_shape(B, batch=40, dtype=0, **GTA1B), cap)
+        for batch in range(1, 41):
+            assert status(batch, cap, most) != B.GTA_ERR_WORKSPACE
+            assert status(batch, cap, least(batch, cap)) != B.GTA_ERR_WORKSPACE
+            assert status(batch, cap, least(batch, cap) - 256) == B.GTA_ERR_WORKSPACE
 
 
 def test_bad_arguments_are_rejected_on_the_host(B):

@@ -349,6 +349,46 @@ SMALL_DECODE = [
 ]
 
 
+@pytest.mark.parametrize("room", ["query", "for a batch of 8", "least"])
+@pytest.mark.parametrize("nb", [1, 6])
+def test_decode_with_the_chunks_that_the_workspace_has_room_for(B, oracle, nb, room):
+    """Small batches of fp32 sequences are cut into chunks of 32 tokens, or of 64 where the workspace holds no more."""
+    w = I.Workload("chunks", "decode", "f32", nb, 0, 64, 20, 5, 1, 1, 64, 128, seed=3)
+    lens, cap = [1 + (577 * i + 2990) % 3000 for i in range(nb)], 3000
+    t = I.decode_inputs(w, device="cuda", s_cap=cap, seq_lens=lens)
+
+    def size(b):
+        return B.decode_workspace_bytes(B.make_shape(batch=b, seq=0, d_model=64, n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64,
+                                                     d_l=128, dtype=torch.float32), t["s_cap"])
+
+    chunks = nb * -(-t["s_cap"] // 64) * 5
+    least = -(-chunks * 128 * 4 // 256) * 256 + -(-chunks * 8 // 256) * 256
+    ws = Guarded(({"query": size(nb), "for a batch of 8": size(8), "least": least}[room],), torch.uint8)
+    out = B.gta_decode(t["q"], t["k_cache"], t["c_cache"], t["seq_lens"], t["x_t"], t["w_p"], t["w_g"], workspace=ws.t)
+    torch.cuda.synchronize()
+    ws.check(room)
+    want = oracle.decode(oracle_shape(w, seq=0), *(t[n].cpu() for n in ("q", "k_cache", "c_cache")), np.array(lens, np.int32),
+                         t["s_cap"], *(t[n].cpu() for n in ("x_t", "w_p", "w_g")))
+    assert_close(out, want, torch.float32, room)
+
+
+@pytest.mark.parametrize("page_size", [16, 48])
+def test_decode_paged_small_pages_in_the_plain_kernels_workspace(B, oracle, page_size):
+    """A workspace that the stream kernel's partial sums do not fit in is still enough for the plain-ALU kernels."""
+    w = I.Workload("small_ws", "decode", "bf16", 2, 0, 128, 20, 5, 1, 1, 64, 128, seed=9)
+    lens = [130, 77]
+    t = I.paginate(I.decode_inputs(w, device="cuda", s_cap=192, seq_lens=lens), page_size, seed=2)
+    chunks = 2 * -(-page_size * t["max_pages"] // 64) * 5
+    ws = Guarded((-(-chunks * 128 * 4 // 256) * 256 + -(-chunks * 8 // 256) * 256,), torch.uint8)
+    out = B.gta_decode_paged(t["q"], t["k_pool"], t["c_pool"], t["block_table"], t["seq_lens"], t["x_t"], t["w_p"], t["w_g"],
+                             workspace=ws.t)
+    torch.cuda.synchronize()
+    ws.check("plain workspace")
+    want = oracle.decode(oracle_shape(w, seq=0), *(t[n].cpu() for n in ("q", "k_cache", "c_cache")), np.array(lens, np.int32),
+                         t["k_cache"].shape[2], *(t[n].cpu() for n in ("x_t", "w_p", "w_g")))
+    assert_close(out, want, torch.bfloat16, "plain workspace")
+
+
 @pytest.mark.parametrize("case", SMALL_DECODE, ids=[c[0] for c in SMALL_DECODE])
 def test_decode_small_shapes(B, oracle, case):
     name, dt, nb, H, n_h, n_q, n_k, n_c, d_h, d_l, lens = case
