@@ -91,6 +91,15 @@ void check_tensors(std::initializer_list<const Tensor*> ts) {
         need(t->is_cuda(), "operator tensors must live on a CUDA device");
     }
 }
+// The lengths of B sequences, which the kernels read and advance as they are; None goes on to the library, which refuses it.
+void* lens_ptr(PyObject* o, const Tensor& like, int64_t B) {
+    if (o == Py_None) return nullptr;
+    const Tensor& t = tensor(o);
+    need(t.scalar_type() == at::kInt && t.device() == like.device() && t.is_contiguous(),
+         "seq_lens must be a contiguous int32 tensor on the operator's device");
+    need(is(t, {B}), "seq_lens must hold one length per sequence");
+    return t.data_ptr();
+}
 int32_t dtype_code(const Tensor& t) {
     if (t.scalar_type() == at::kFloat) return GTA_F32;
     if (t.scalar_type() == at::kBFloat16) return GTA_BF16;
@@ -152,7 +161,7 @@ Fp8Caches check_fp8(const Tensor& k, const Tensor& c, const Tensor& ks, const Te
          cs.scalar_type() == at::kFloat && is(c, {f.B, f.n_c, f.cap, f.d_l}) && is(ks, {f.B, f.n_k, f.cap}) &&
          is(cs, {f.B, f.n_c, f.cap}), what);
     for (const Tensor* t : {&k, &c, &ks, &cs})
-        need(t->is_contiguous() && t->is_cuda(), "cache tensors must be contiguous CUDA tensors");
+        need(t->is_contiguous() && t->is_cuda() && t->device() == k.device(), "cache tensors must be contiguous CUDA tensors of one device");
     return f;
 }
 
@@ -176,15 +185,16 @@ PyObject* prefill(PyObject* const* a) {
 PyObject* decode_append(PyObject* const* a) {
     const Tensor &q = tensor(a[0]), &k = tensor(a[1]), &c = tensor(a[2]), &kn = tensor(a[3]), &cn = tensor(a[4]),
                  &x = tensor(a[6]), &wp = tensor(a[7]), &wg = tensor(a[8]);
-    void* lens = ptr_or_null(a[5]);
     check_tensors({&q, &k, &c, &kn, &cn, &x, &wp, &wg});
-    const auto [Bq, n_q, d_hq] = dims<3>(q);
+    const int64_t n_q = dims<3>(q)[1], n_h = dims<3>(wp)[0], H = dims<2>(x)[1];
     const auto [B, n_k, cap, d_h] = dims<4>(k);
-    const auto cd = dims<4>(c);
-    need(x.dim() >= 2 && wp.dim() >= 1, "inconsistent operator tensor shapes");
-    need(kn.numel() == B * n_k * d_h && cn.numel() == B * cd[1] * cd[3], "k_new / c_new hold one row per sequence and group");
-    const gta_shape_t s = shape_of(Bq, 0, x.size(1), wp.size(0), n_q, n_k, cd[1], d_hq, cd[3], dtype_code(q), 1, real(a[9]));
-    Buffers b(a[10], a[11], {Bq, wp.size(0), d_hq}, q,
+    const int64_t n_c = dims<4>(c)[1], d_l = c.size(3);
+    need(is(q, {B, n_q, d_h}) && is(c, {B, n_c, cap, d_l}) && is(x, {B, H}) && is(wp, {n_h, d_l, d_h}) &&
+         is(wg, {H, n_h * d_h}), "inconsistent operator tensor shapes");
+    need(kn.numel() == B * n_k * d_h && cn.numel() == B * n_c * d_l, "k_new / c_new hold one row per sequence and group");
+    void* lens = lens_ptr(a[5], q, B);
+    const gta_shape_t s = shape_of(B, 0, H, n_h, n_q, n_k, n_c, d_h, d_l, dtype_code(q), 1, real(a[9]));
+    Buffers b(a[10], a[11], {B, n_h, d_h}, q,
               a[11] == Py_None ? lib.gta_decode_workspace_bytes(&s, (int32_t)cap) : 0);
     void* status = ptr_or_null(a[12]);
     void* stream = stream_of(a[13]);
@@ -197,9 +207,10 @@ PyObject* decode_append(PyObject* const* a) {
 PyObject* cache_append_fp8(PyObject* const* a) {
     const Tensor &k = tensor(a[0]), &c = tensor(a[1]), &ks = tensor(a[2]), &cs = tensor(a[3]), &kn = tensor(a[4]),
                  &cn = tensor(a[5]);
-    void* lens = ptr_or_null(a[6]);
     const Fp8Caches f = check_fp8(k, c, ks, cs);
     check_tensors({&kn, &cn});
+    need(kn.device() == k.device(), "the new rows and the caches must share one device");
+    void* lens = lens_ptr(a[6], k, f.B);
     need(kn.dim() == 4, "inconsistent new-row shapes");
     const int64_t n_new = kn.size(2);
     need(is(kn, {f.B, f.n_k, n_new, f.d_h}) && is(cn, {f.B, f.n_c, n_new, f.d_l}), "inconsistent new-row shapes");
@@ -221,9 +232,10 @@ PyObject* cache_append_fp8(PyObject* const* a) {
 PyObject* decode_fp8(PyObject* const* a) {
     const Tensor &q = tensor(a[0]), &k = tensor(a[1]), &c = tensor(a[2]), &ks = tensor(a[3]), &cs = tensor(a[4]),
                  &x = tensor(a[6]), &wp = tensor(a[7]), &wg = tensor(a[8]);
-    void* lens = ptr_or_null(a[5]);
     const Fp8Caches f = check_fp8(k, c, ks, cs);
     check_tensors({&q, &x, &wp, &wg});
+    need(q.device() == k.device(), "the operator tensors and the caches must share one device");
+    void* lens = lens_ptr(a[5], q, f.B);
     need(q.dim() >= 2 && wp.dim() >= 1 && x.dim() >= 2, "inconsistent operator tensor shapes");
     const int64_t n_q = q.size(1), n_h = wp.size(0), H = x.size(1);
     need(is(q, {f.B, n_q, f.d_h}) && is(wp, {n_h, f.d_l, f.d_h}) && is(wg, {H, n_h * f.d_h}) && is(x, {f.B, H}),

@@ -740,6 +740,45 @@ def test_a_wait_that_runs_out_unwinds_the_decode_stream_kernel(B, oracle):
 
 
 # --------------------------------------------------------------------------- append + decode in one call
+def test_steps_refuse_tensors_that_do_not_fit_together(B):
+    """gta_decode_append, gta_cache_append_fp8 and gta_decode_fp8 hand addresses on: a tensor of another type, device or size
+    is refused before anything is launched, and nothing is written."""
+    nb, cap, H, n_h, n_q, n_k, n_c, d_h, d_l = 3, 64, 128, 8, 4, 4, 1, 128, 256
+    g = torch.Generator("cuda").manual_seed(1)
+
+    def r(*s):
+        return torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+
+    lens = torch.full((nb,), 7, dtype=torch.int32, device="cuda")
+    bad_lens = [lens.long(), lens.cpu(), lens[:2], torch.zeros(nb + 1, dtype=torch.int32, device="cuda"),
+                torch.zeros(2 * nb, dtype=torch.int32, device="cuda")[::2], lens.float()]
+    step = dict(q=r(nb, n_q, d_h), k=r(nb, n_k, cap, d_h), c=r(nb, n_c, cap, d_l), k_new=r(nb, n_k, 1, d_h), c_new=r(nb, n_c, 1, d_l),
+                lens=lens, x=r(nb, H), w_p=r(n_h, d_l, d_h), w_g=r(H, n_h * d_h))
+    wrong = [("lens", t) for t in bad_lens] + [
+        ("c", r(nb - 1, n_c, cap, d_l)), ("c", r(nb, n_c, cap - 1, d_l)), ("q", r(nb + 1, n_q, d_h)), ("q", r(nb, n_q, d_h // 2)),
+        ("x", r(nb - 1, H)), ("w_p", r(n_h, d_l // 2, d_h)), ("w_p", r(n_h, d_l, d_h // 2)), ("w_g", r(H, n_h * d_h - 8)),
+        ("w_g", r(H // 2, n_h * d_h)), ("k_new", r(nb, n_k - 1, 1, d_h)), ("x", r(nb, H).cpu())]
+    before = step["k"].clone(), step["c"].clone()
+    for name, t in wrong:
+        with pytest.raises(ValueError):
+            B.gta_decode_append(*{**step, name: t}.values())
+    out = B.gta_decode_append(*step.values())
+    assert out.shape == (nb, n_h, d_h) and lens.tolist() == [8] * nb
+    step["k"][:, :, 7], step["c"][:, :, 7] = before[0][:, :, 7], before[1][:, :, 7]
+    assert torch.equal(step["k"], before[0]) and torch.equal(step["c"], before[1])
+
+    codes = [torch.zeros(nb, n_k, cap, d_h, dtype=torch.uint8, device="cuda"), torch.zeros(nb, n_c, cap, d_l, dtype=torch.uint8, device="cuda"),
+             torch.zeros(nb, n_k, cap, device="cuda"), torch.zeros(nb, n_c, cap, device="cuda")]
+    for t in bad_lens:
+        with pytest.raises(ValueError):
+            B.gta_cache_append_fp8(*codes, step["k_new"], step["c_new"], t)
+        with pytest.raises(ValueError):
+            B.gta_decode_fp8(step["q"], *codes, t, step["x"], step["w_p"], step["w_g"])
+    assert not any(bool(t.any()) for t in codes)
+    with pytest.raises(B.GtaError):
+        B.gta_cache_append_fp8(*codes, step["k_new"], step["c_new"], None)
+
+
 STEP_CASES = [
     # name, dtype, H, n_h, n_q, n_k, n_c, d_h, d_l, lens BEFORE the step, S_cap
     ("bf16_around_the_sub_tiles", "bf16", 256, 8, 4, 4, 1, 128, 512, [0, 1, 30, 31, 32, 33, 63, 64, 65, 700], 720),
