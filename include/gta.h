@@ -463,9 +463,11 @@ GTA_API gta_status_t gta_ref_gqa_decode(const gta_shape_t *shape, const void *q,
  * Profiling aids (no counterpart in the paper): the same calls restricted to a subset of their
  * kernels, so that each kernel can be timed or captured alone.  `stages` is a bit mask;
  * gta_prefill_stages: 1 = attention kernel (writes L to the workspace), 2 = decoder + gate
- * kernel (reads L from the workspace); gta_decode_stages: 1 = gate partial sums, 2 = split-KV
- * cache kernel, 4 = merge + decoder.  A mask of all stages equals the plain call.  The
- * workspace must still hold what the skipped stages would have written.
+ * kernel (reads L from the workspace); gta_decode_stages: 2 = split-KV cache kernel, 4 = merge,
+ * decoder and gate (bit 1 has no kernel of its own: the gate is worked out with the decoder).
+ * A mask of all stages equals the plain call.  The workspace, of the same size for all of them,
+ * must still hold what the skipped stages would have written; a stage leaves its own input as it
+ * found it, or in a state that gives the same result again.
  */
 GTA_API gta_status_t gta_prefill_stages(const gta_shape_t *shape, const void *q, const void *k,
                                         const void *c, const void *x, const void *w_p, const void *w_g,

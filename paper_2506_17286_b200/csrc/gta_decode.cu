@@ -9,6 +9,8 @@
 //   decode_finish_kernel  : gate pre-activation x_t W_G, decoder L W_P,i, sigmoid, store, 8 sequences
 //       x 16 columns per CTA; the gate half runs before the kernel's dependency wait.
 // The kernels are chained by programmatic dependent launch.
+#include <float.h>
+
 #include <type_traits>
 
 #include "gta_common.cuh"
@@ -365,23 +367,24 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
 }
 
 // Log-sum-exp merge of the chunk partials of one (map, sequence), in place: the normalised latent L takes the room of the
-// sequence's first chunk.  The threads form groups that cover a
+// sequence's first chunk, whose weight becomes one and that of the others nothing, so that a second merge finds L again
+// (gta_decode_stages).  The threads form groups that cover a
 // pass of the d_l columns, four each; group i takes the chunks i, i + groups, ..., and the groups' results meet in
 // shared memory: a chain of rounds of loads over all chunks would be what the kernel waits for.
 __global__ void __launch_bounds__(kDecodeThreads)
 decode_chunk_merge_kernel(Dims d, int chunk, int n_chunks, int S_cap, const int32_t* __restrict__ seq_lens,
-                          float* part_o, const float* part_ml) {
+                          float* part_o, float* part_ml) {
     __shared__ float4 acc_s[kDecodeThreads];
     __shared__ float2 ml_s[kDecodeThreads];
     ptx::grid_launch_dependents();
     const int g = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
     const int width = min(d.d_l >> 2, kDecodeThreads), groups = kDecodeThreads / width;
     const int grp = tid / width, v = tid - grp * width;
-    int len = seq_lens[b];       // (older than the partial kernel, which was released after its own wait)
+    int len = seq_lens[b];       // (older than the partial kernel, which was released after its own wait; see the launch)
     len = len < 0 ? 0 : (len > S_cap ? S_cap : len);
     const int live = (len + chunk - 1) / chunk;
     ptx::grid_dependency_wait();
-    const float2* ml = reinterpret_cast<const float2*>(part_ml) + (size_t)b * n_chunks * d.n_q + g;
+    float2* ml = reinterpret_cast<float2*>(part_ml) + (size_t)b * n_chunks * d.n_q + g;
     float* po = part_o + ((size_t)b * n_chunks * d.n_q + g) * d.d_l;
     for (int col0 = 0; col0 < d.d_l; col0 += 4 * kDecodeThreads) {
         const int col = col0 + 4 * v;
@@ -439,6 +442,8 @@ decode_chunk_merge_kernel(Dims d, int chunk, int n_chunks, int S_cap, const int3
         }
         __syncthreads();
     }
+    for (int c = tid; c < live; c += kDecodeThreads)
+        ml[(size_t)c * d.n_q] = c == 0 ? make_float2(0.f, 1.f) : make_float2(-FLT_MAX, 0.f);
 }
 
 // Four neighbouring elements as floats.
@@ -566,8 +571,11 @@ decode_finish_kernel(Dims d, int tiles_per_head, const T* __restrict__ x_t, cons
         out[((size_t)(b0 + r) * d.n_h + i) * d.d_h + c] = from_f32<T>(y * (1.f / (1.f + expf(-z))));
 }
 
+// behind: programmatic stream serialisation.  The first kernel of a call is launched so only if it waits before it touches
+// anything; the merge and the finish kernel do not (they rely on the kernel ahead for that), so where a stage mask begins with
+// one of them, it is launched the ordinary way.
 template <typename Kern, typename... Args>
-static cudaError_t launch_behind(Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+static cudaError_t launch_chained(bool behind, Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     if (smem > 48 * 1024) {
         const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err != cudaSuccess) return err;
@@ -581,7 +589,7 @@ static cudaError_t launch_behind(Kern kern, dim3 grid, int threads, size_t smem,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = behind ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
@@ -600,7 +608,7 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
         const int maps = d.n_q / d.n_c;
         const auto go = [&](auto cm) {
             constexpr int CM = decltype(cm)::value;
-            return launch_behind(decode_partial_kernel<T, CT, CM>, dim3(p.n_chunks, d.B), kDecodeThreads,
+            return launch_chained(true, decode_partial_kernel<T, CT, CM>, dim3(p.n_chunks, d.B), kDecodeThreads,
                                  partial_smem(d, p.chunk, CM, LatentVec<CT>::N), stream, d, p.chunk, p.n_chunks, S_cap,
                                  (const T*)q, (const CT*)k_cache, (const CT*)c_cache, seq_lens, part_o, part_ml, pm,
                                  status_word, k_scale, c_scale);
@@ -615,12 +623,12 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
         *launches += 1;
     }
     if (stages & 4) {
-        err = launch_behind(decode_chunk_merge_kernel, dim3(d.n_q, d.B), kDecodeThreads, 0, stream, d, p.chunk, p.n_chunks, S_cap,
-                            seq_lens, part_o, (const float*)part_ml);
+        err = launch_chained((stages & 2) && S_cap > 0, decode_chunk_merge_kernel, dim3(d.n_q, d.B), kDecodeThreads, 0, stream, d,
+                             p.chunk, p.n_chunks, S_cap, seq_lens, part_o, part_ml);
         if (err != cudaSuccess) return err;
         const int tiles = (d.d_h + kFinishCols - 1) / kFinishCols;
         const size_t smem = (2 * kFinishSlab * 4 + 2 * 8 * 128) * sizeof(float);
-        err = launch_behind(decode_finish_kernel<T>, dim3(d.n_h * tiles, (d.B + kFinishSeqs - 1) / kFinishSeqs), kDecodeThreads, smem,
+        err = launch_chained(true, decode_finish_kernel<T>, dim3(d.n_h * tiles, (d.B + kFinishSeqs - 1) / kFinishSeqs), kDecodeThreads, smem,
                             stream, d, tiles, (const T*)x_t, (const float*)part_o, (size_t)p.n_chunks * d.n_q * d.d_l, (const T*)w_p, (const T*)w_g, (T*)out);
         if (err != cudaSuccess) return err;
         *launches += 2;

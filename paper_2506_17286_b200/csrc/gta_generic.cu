@@ -521,9 +521,9 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
 }
 
 // ---------------------------------------------------------------------------------------------
-// Launch with programmatic stream serialisation (the kernel waits for the one before it by itself).
+// Launch with programmatic stream serialisation (the kernel waits for the one before it by itself), or without.
 template <typename Kern, typename... Args>
-static cudaError_t launch_behind(Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+static cudaError_t launch_chained(bool behind, Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -533,7 +533,7 @@ static cudaError_t launch_behind(Kern kern, dim3 grid, int threads, size_t smem,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = behind ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
@@ -546,13 +546,13 @@ static cudaError_t launch_attention(const Dims& d, const T* q, const T* k, const
     auto kern = generic_attention_kernel<T, QW, SW, NC, DH>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    return launch_behind(kern, dim3((d.N + 16 * QW - 1) / (16 * QW), d.n_q * n_slices, d.B), 32 * QW * SW, smem, stream, d, q, k, c, o_lat,
+    return launch_chained(true, kern, dim3((d.N + 16 * QW - 1) / (16 * QW), d.n_q * n_slices, d.B), 32 * QW * SW, smem, stream, d, q, k, c, o_lat,
                          pm, status_word, n_slices);
 }
 
 template <typename T, int RW, int CW, int KW>
 static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x, const T* w_p, const T* w_g, T* out,
-                                  cudaStream_t stream) {
+                                  cudaStream_t stream, bool behind) {
     auto kern = generic_decoder_kernel<T, RW, CW, KW>;
     constexpr size_t smem = dec_smem_bytes(RW, CW, KW);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -560,7 +560,7 @@ static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x,
     const int map_cols = d.n_h / d.n_q * d.d_h;
     const long long M = (long long)d.B * d.N;
     const dim3 grid((unsigned)((M + 16 * RW - 1) / (16 * RW)), d.n_q * ((map_cols + 64 * CW - 1) / (64 * CW)));
-    return launch_behind(kern, grid, 32 * RW * CW * KW, smem, stream, d, o_lat, x, w_p, w_g, out);
+    return launch_chained(behind, kern, grid, 32 * RW * CW * KW, smem, stream, d, o_lat, x, w_p, w_g, out);
 }
 
 template <typename T>
@@ -602,9 +602,10 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
         // columns) 58 / 34 / 30; 640 (2048 rows) 315 / 220 / 200.
         const long long tiles64 = (((long long)d.B * d.N + 63) / 64) * d.n_q * ((d.n_h / d.n_q * d.d_h + 63) / 64);
         const float* l = o_lat_ws;
-        err = tiles64 < 40    ? launch_decoder<T, 1, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream)
-              : tiles64 < 256 ? launch_decoder<T, 1, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream)
-                              : launch_decoder<T, 4, 1, 1>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream);
+        const bool behind = stages & 1;      // X and W_G are read ahead of the wait: they are older than the attention kernel only
+        err = tiles64 < 40    ? launch_decoder<T, 1, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind)
+              : tiles64 < 256 ? launch_decoder<T, 1, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind)
+                              : launch_decoder<T, 4, 1, 1>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind);
         if (err != cudaSuccess) return err;
         *launches += 1;
     }

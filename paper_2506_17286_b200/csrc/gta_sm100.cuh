@@ -29,13 +29,15 @@ gta_status_t sm100_attention_debug_wait(unsigned long long limit_ns, int withhol
 
 // Decoder + gate kernel alone: out = (L W_P) (.) sigmoid(X W_G) with L[B, n_q, N, d_l] in bf16.
 // step_lens (optional; the fused append + decode step): lengths that the kernel advances by one, where there is room
-// below step_cap, once the kernel before it in the stream is complete.
+// below step_cap, once the kernel before it in the stream is complete.  release: the kernel behind this one may be scheduled
+// from then on; behind: this one may overlap the kernel ahead, whose own inputs are then older than its X and W_G.
 gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
                                   void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens = nullptr,
-                                  int step_batch = 0, int step_cap = 0, bool release = true);
+                                  int step_batch = 0, int step_cap = 0, bool release = true, bool behind = true);
 // The same for an L in two bf16 planes [2][B, n_q, N, d_l] whose sum it is; the gates are kept in fp32.
 gta_status_t launch_sm100_decoder_fine(const Dims& d, const void* l_planes, const void* x, const void* w_p, const void* w_g,
-                                       void* out, int32_t* status_word, cudaStream_t stream, bool release = true);
+                                       void* out, int32_t* status_word, cudaStream_t stream, bool release = true,
+                                       bool behind = true);
 
 // Linear maps of the attention layer around the operator (App. B.1.1), bf16 with fp32 accumulation.
 // True when the tcgen05 kernel covers the layer's projections for this shape.

@@ -425,7 +425,7 @@ int sm_count() {
 template <bool kFine>
 static gta_status_t launch_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
                                    void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens,
-                                   int step_batch, int step_cap, bool release) {
+                                   int step_batch, int step_cap, bool release, bool behind) {
     CUtensorMap tm_l, tm_x, tm_wp, tm_wg;
     const bool solo = d.N <= kTileM;                                    // one row tile: no CTA pairs
     const uint32_t a_rows = solo ? (uint32_t)((d.N + 7) & ~7) : kTileM; // rows of an A tile
@@ -480,7 +480,7 @@ static gta_status_t launch_decoder(const Dims& d, const void* l_bf16, const void
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = behind ? 1 : 0;
         if (cudaLaunchKernelEx(&cfg, sm100_decoder_kernel<false, kFine>, tm_l, tm_x, tm_wp, tm_wg, d, s, (__nv_bfloat16*)out,
                                status_word, step_lens, step_batch, step_cap, (int)release) != cudaSuccess)
             return GTA_ERR_CUDA;
@@ -530,7 +530,7 @@ static gta_status_t launch_decoder(const Dims& d, const void* l_bf16, const void
     s.r = (int)(U % G);
     s.split_tail = (s.pair && 2 * s.r <= G) ? 1 : 0;
     cfg.gridDim = dim3(2 * G);
-    cfg.numAttrs = 2;
+    cfg.numAttrs = behind ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, sm100_decoder_kernel<true, kFine>, tm_l, tm_x, tm_wp, tm_wg, d, s, (__nv_bfloat16*)out,
                            status_word, step_lens, step_batch, step_cap, (int)release) != cudaSuccess)
         return GTA_ERR_CUDA;
@@ -539,12 +539,12 @@ static gta_status_t launch_decoder(const Dims& d, const void* l_bf16, const void
 
 gta_status_t launch_sm100_decoder(const Dims& d, const void* l_bf16, const void* x, const void* w_p, const void* w_g,
                                   void* out, int32_t* status_word, cudaStream_t stream, int32_t* step_lens,
-                                  int step_batch, int step_cap, bool release) {
-    return launch_decoder<false>(d, l_bf16, x, w_p, w_g, out, status_word, stream, step_lens, step_batch, step_cap, release);
+                                  int step_batch, int step_cap, bool release, bool behind) {
+    return launch_decoder<false>(d, l_bf16, x, w_p, w_g, out, status_word, stream, step_lens, step_batch, step_cap, release, behind);
 }
 gta_status_t launch_sm100_decoder_fine(const Dims& d, const void* l_planes, const void* x, const void* w_p, const void* w_g,
-                                       void* out, int32_t* status_word, cudaStream_t stream, bool release) {
-    return launch_decoder<true>(d, l_planes, x, w_p, w_g, out, status_word, stream, nullptr, 0, 0, release);
+                                       void* out, int32_t* status_word, cudaStream_t stream, bool release, bool behind) {
+    return launch_decoder<true>(d, l_planes, x, w_p, w_g, out, status_word, stream, nullptr, 0, 0, release, behind);
 }
 
 }  // namespace gta

@@ -349,6 +349,24 @@ SMALL_DECODE = [
 ]
 
 
+@pytest.mark.parametrize("shape", [("f32", 5, 20, 5, 1, 1, 64, 128), ("bf16", 3, 6, 6, 3, 1, 40, 200), ("bf16", 4, 8, 4, 4, 1, 128, 512),
+                                   ("bf16", 2, 3, 3, 1, 1, 24, 2048)])
+def test_decode_stages_one_by_one_and_again(B, shape):
+    """The stages of a decode step give the step's bits, and a stage that runs a second time gives them again."""
+    dt, nb, n_h, n_q, n_k, n_c, d_h, d_l = shape
+    w = I.Workload("stages", "decode", dt, nb, 0, 64, n_h, n_q, n_k, n_c, d_h, d_l, seed=4)
+    t = I.decode_inputs(w, device="cuda", s_cap=700, seq_lens=[0, 33, 700, 64, 501][:nb])
+    args = [t[n] for n in ("q", "k_cache", "c_cache", "seq_lens", "x_t", "w_p", "w_g")]
+    want = B.gta_decode(*args)
+    shape_ = B.decode_shape(t["q"], t["k_cache"], t["c_cache"], t["x_t"], t["w_p"])
+    ws = torch.full((B.decode_workspace_bytes(shape_, t["s_cap"]),), 0xFF, dtype=torch.uint8, device="cuda")
+    for masks in ((2, 4), (4,), (4,), (6,), (4,), (7,), (4,)):
+        for mask in masks:
+            out = torch.full_like(want, float("nan"))
+            B.gta_decode(*args, out=out, workspace=ws, stages=mask)
+        assert torch.equal(out, want), masks
+
+
 @pytest.mark.parametrize("room", ["query", "for a batch of 8", "least"])
 @pytest.mark.parametrize("nb", [1, 6])
 def test_decode_with_the_chunks_that_the_workspace_has_room_for(B, oracle, nb, room):
