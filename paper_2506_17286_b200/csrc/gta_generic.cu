@@ -84,7 +84,7 @@ __host__ __device__ inline AttnSmem attn_smem(int d_h, int rows, int tile_keys, 
 template <typename T, int QW, int SW, int NC, int DH>
 __global__ void __launch_bounds__(32 * QW * SW)
 generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
-                         float* __restrict__ o_lat, const PageMap pm, int32_t* status_word, int n_slices) {
+                         float* __restrict__ o_lat, const PageMap pm, int32_t* status_word, int tiles) {
     constexpr int kWarps = QW * SW, kThreads = 32 * kWarps;
     constexpr int kRows = 16 * QW, kTile = kAttnKeys * SW, kCols = 64 * NC;
     extern __shared__ __align__(16) float smem[];
@@ -102,8 +102,9 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
     float* row_s = reinterpret_cast<float*>(bad_s + kTile) + kWarps * kAttnKeys * kPStride + warp * 32;   // [2][16]
     const int qw = warp % QW, sw = warp / QW;
 
-    const int t0 = (int)(gridDim.x - 1 - blockIdx.x) * kRows;   // the longest rows first
-    const int g = blockIdx.y / n_slices, slice = blockIdx.y % n_slices, b = blockIdx.z;
+    // (row tiles and slices of d_l share x, heads and maps have y to themselves: 65535 of them)
+    const int slice = (int)blockIdx.x / tiles, t0 = (tiles - 1 - ((int)blockIdx.x - slice * tiles)) * kRows;   // the longest rows first
+    const int g = blockIdx.y, b = blockIdx.z;
     const int kg = d.q_to_k(g), cg = d.q_to_c(g);
     const int col0 = slice * kCols, n_cols = min(kCols, d.d_l - col0);
     const int off = d.causal ? d.Nk - d.N : 0;                  // causal: row t attends keys 0 .. t + off
@@ -366,7 +367,7 @@ constexpr size_t dec_smem_bytes(int RW, int CW, int KW) {
 template <typename T, int RW, int CW, int KW>
 __global__ void __launch_bounds__(32 * RW * CW * KW)
 generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restrict__ x, const T* __restrict__ w_p,
-                       const T* __restrict__ w_g, T* __restrict__ out) {
+                       const T* __restrict__ w_g, T* __restrict__ out, int tile0) {
     constexpr int kThreads = 32 * RW * CW * KW, BM = 16 * RW, BN = 64 * CW, BK = dec_bk(KW), KPW = BK / KW;
     constexpr int kLdA = BK + 4, kStage = BM * kLdA + BK * BN;
     extern __shared__ __align__(16) float smem[];
@@ -375,8 +376,8 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
     const int rg = lane >> 3, cg = lane & 7;                 // rows rg + 4 i; columns 4 cg + {0..3}, 32 + 4 cg + {0..3}
 
     const long long M = (long long)d.B * d.N;
-    const int map_cols = d.n_h / d.n_q * d.d_h, tiles_per_map = (map_cols + BN - 1) / BN;
-    const int g = blockIdx.y / tiles_per_map, c0 = (blockIdx.y % tiles_per_map) * BN;     // columns c0 .. of map g
+    const int map_cols = d.n_h / d.n_q * d.d_h;
+    const int g = blockIdx.z, c0 = (tile0 + (int)blockIdx.y) * BN;     // columns c0 .. of map g
     const int n_cols = min(BN, map_cols - c0);
     const long long m0 = (long long)blockIdx.x * BM;
     const int rows = (int)(M - m0 < BM ? M - m0 : BM);
@@ -542,25 +543,30 @@ static cudaError_t launch_attention(const Dims& d, const T* q, const T* k, const
                                     const PageMap& pm, int32_t* status_word) {
     const AttnSmem L = attn_smem(d.d_h, 16 * QW, kAttnKeys * SW, 64 * NC, QW * SW);
     const size_t smem = (size_t)L.total_floats * sizeof(float);
-    const int n_slices = (d.d_l + 64 * NC - 1) / (64 * NC);
+    const int tiles = (d.N + 16 * QW - 1) / (16 * QW), n_slices = (d.d_l + 64 * NC - 1) / (64 * NC);
     auto kern = generic_attention_kernel<T, QW, SW, NC, DH>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    return launch_chained(true, kern, dim3((d.N + 16 * QW - 1) / (16 * QW), d.n_q * n_slices, d.B), 32 * QW * SW, smem, stream, d, q, k, c, o_lat,
-                         pm, status_word, n_slices);
+    return launch_chained(true, kern, dim3(tiles * n_slices, d.n_q, d.B), 32 * QW * SW, smem, stream, d, q, k, c, o_lat, pm, status_word,
+                          tiles);
 }
 
 template <typename T, int RW, int CW, int KW>
 static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x, const T* w_p, const T* w_g, T* out,
-                                  cudaStream_t stream, bool behind) {
+                                  cudaStream_t stream, bool behind, int* launches) {
     auto kern = generic_decoder_kernel<T, RW, CW, KW>;
     constexpr size_t smem = dec_smem_bytes(RW, CW, KW);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int map_cols = d.n_h / d.n_q * d.d_h;
     const long long M = (long long)d.B * d.N;
-    const dim3 grid((unsigned)((M + 16 * RW - 1) / (16 * RW)), d.n_q * ((map_cols + 64 * CW - 1) / (64 * CW)));
-    return launch_chained(behind, kern, grid, 32 * RW * CW * KW, smem, stream, d, o_lat, x, w_p, w_g, out);
+    // a map of more than 65535 column tiles takes several launches (the tiles in x next to the rows' cost 3.5 % of 2 x 1500
+    // tokens of the 1B layer)
+    const int tiles = (map_cols + 64 * CW - 1) / (64 * CW);
+    for (int tile0 = 0; tile0 < tiles && err == cudaSuccess; tile0 += 65535, ++*launches)
+        err = launch_chained(behind, kern, dim3((unsigned)((M + 16 * RW - 1) / (16 * RW)), min(tiles - tile0, 65535), d.n_q),
+                             32 * RW * CW * KW, smem, stream, d, o_lat, x, w_p, w_g, out, tile0);
+    return err;
 }
 
 template <typename T>
@@ -603,11 +609,10 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
         const long long tiles64 = (((long long)d.B * d.N + 63) / 64) * d.n_q * ((d.n_h / d.n_q * d.d_h + 63) / 64);
         const float* l = o_lat_ws;
         const bool behind = stages & 1;      // X and W_G are read ahead of the wait: they are older than the attention kernel only
-        err = tiles64 < 40    ? launch_decoder<T, 1, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind)
-              : tiles64 < 256 ? launch_decoder<T, 1, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind)
-                              : launch_decoder<T, 4, 1, 1>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind);
+        err = tiles64 < 40    ? launch_decoder<T, 1, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
+              : tiles64 < 256 ? launch_decoder<T, 1, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
+                              : launch_decoder<T, 4, 1, 1>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches);
         if (err != cudaSuccess) return err;
-        *launches += 1;
     }
     return cudaSuccess;
 }

@@ -83,6 +83,24 @@ def test_prefill_small_shapes(B, oracle, case):
     _prefill_case(B, oracle, w)
 
 
+@pytest.mark.parametrize("n_h,n_q,d_h,d_l", [(16500, 16500, 8, 512), (32800, 1, 128, 8), (65535, 65535, 8, 8)])
+def test_prefill_more_heads_than_a_grid_has_rows(B, n_h, n_q, d_h, d_l):
+    """Maps x latent slices, columns of a map and heads past 65535, or up to it; every output against fp64 of the same op."""
+    g = torch.Generator("cuda").manual_seed(2)
+    N, H = 3, 8
+    q, k, c, x = (torch.randn(*s, generator=g, device="cuda") for s in
+                  ((1, n_q, N, d_h), (1, 1, N, d_h), (1, 1, N, d_l), (1, N, H)))
+    w_p, w_g = torch.randn(n_h, d_l, d_h, generator=g, device="cuda") * d_l ** -0.5, torch.randn(H, n_h * d_h, generator=g, device="cuda")
+    out = B.gta_prefill(q, k, c, x, w_p, w_g)
+    s = torch.einsum("qnd,td->qnt", q[0].double(), k[0, 0].double()) / d_h ** 0.5
+    p = s.masked_fill(torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1), -float("inf")).softmax(-1)
+    lat = (p @ c[0, 0].double()).repeat_interleave(n_h // n_q, 0)
+    gate = torch.sigmoid(x[0].double() @ w_g.double()).reshape(N, n_h, d_h)
+    want = torch.stack([torch.einsum("nl,nld->nd", lat[:, t], w_p.double()) for t in range(N)]) * gate
+    assert float((out[0].double() - want).norm() / want.norm()) <= 1e-4
+    assert float((out[0].double() - want).abs().max() / want.abs().max()) <= 1e-4
+
+
 @pytest.mark.parametrize("N", [1, 2, 127, 128, 129, 255, 256, 384])
 def test_prefill_tile_boundaries_bf16(B, oracle, N):
     w = I.Workload(f"edge_{N}", "prefill", "bf16", 1, N, 128, 4, 2, 2, 1, 128, 256, seed=77 + N)
