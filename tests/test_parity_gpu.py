@@ -83,6 +83,41 @@ def test_prefill_small_shapes(B, oracle, case):
     _prefill_case(B, oracle, w)
 
 
+@pytest.mark.parametrize("dt,n_q,n_k,d_h,d_l,N,past", [("f32", 2, 2, 64, 128, 200, 0), ("f32", 5, 1, 64, 128, 700, 300), ("f32", 2, 1, 40, 72, 33, 5),
+                                                       ("f32", 8, 8, 128, 64, 1200, 0), ("bf16", 3, 3, 40, 200, 150, 64)])
+@pytest.mark.parametrize("paged", [False, True])
+def test_plain_alu_prefill_keys_after_a_row_do_not_reach_it_whatever_they_hold(B, dt, n_q, n_k, d_h, d_l, N, past, paged):
+    """Causality in the strict form: keys and latents of later positions may be infinite or not a number (a padded prompt), the
+    rows before them keep their bits."""
+    T = torch.float32 if dt == "f32" else torch.bfloat16
+    g = torch.Generator("cuda").manual_seed(N)
+    kv, n_h, H = N + past, n_q, 64
+    q, k, c, x = (torch.randn(*s, generator=g, device="cuda").to(T) for s in ((2, n_q, N, d_h), (2, n_k, kv, d_h), (2, 1, kv, d_l), (2, N, H)))
+    w_p, w_g = (torch.randn(*s, generator=g, device="cuda").to(T) * 0.1 for s in ((n_h, d_l, d_h), (H, n_h * d_h)))
+
+    def run(k, c):
+        if not paged:
+            return B.gta_prefill_chunk(q, k, c, x, w_p, w_g, kv)
+        pages = -(-kv // 8)
+        table = torch.randperm(2 * pages, generator=torch.Generator().manual_seed(1)).reshape(2, pages).int().cuda()
+        pools = []
+        for t in (k, c):
+            pool = torch.zeros(2 * pages, t.shape[1], 8, t.shape[3], device="cuda", dtype=T)
+            padded = torch.nn.functional.pad(t, (0, 0, 0, pages * 8 - kv))
+            pool[table.long().flatten()] = padded.reshape(2, t.shape[1], pages, 8, -1).permute(0, 2, 1, 3, 4).reshape(2 * pages, t.shape[1], 8, -1)
+            pools.append(pool)
+        return B.gta_prefill_chunk_paged(q, *pools, table, x, w_p, w_g, kv)
+
+    want = run(k, c)
+    for first in sorted({1, N // 3, N // 2 + 1, N - 1}):
+        k2, c2 = k.clone(), c.clone()
+        k2[:, :, past + first:], c2[:, :, past + first:] = float("nan"), float("inf")
+        c2[:, :, past + first + 1::2] = float("nan")
+        out = run(k2, c2)
+        assert torch.equal(out[:, :first], want[:, :first])
+        assert torch.isnan(out[:, first:].float()).all()
+
+
 @pytest.mark.parametrize("n_h,n_q,d_h,d_l", [(16500, 16500, 8, 512), (32800, 1, 128, 8), (65535, 65535, 8, 8)])
 def test_prefill_more_heads_than_a_grid_has_rows(B, n_h, n_q, d_h, d_l):
     """Maps x latent slices, columns of a map and heads past 65535, or up to it; every output against fp64 of the same op."""
