@@ -184,6 +184,33 @@ def test_prefill_chunk_paged_scores_that_climb_past_the_first_keys(B, oracle, sh
     assert_close(out, want, w.torch_dtype(), "climb")
 
 
+@pytest.mark.parametrize("page_size", [0, 16, 64])
+@pytest.mark.parametrize("shape", [(4, 700, 700, 8, 4, 4, 128, 512), (2, 2001, 300, 4, 2, 2, 128, 512), (1, 600, 600, 4, 2, 1, 64, 128)])
+def test_prefill_large_latents_behind_scores_that_climb(B, oracle, shape, page_size):
+    """Latents of 1e30 behind scores up to 30 nats above the first keys': the row sums stay in range, the latent sums leave it
+    unless the item is done again with its true maxima.  Whole items and split ones, over pages or not (0)."""
+    nb, kv_len, N, n_h, n_q, n_k, d_h, d_l = shape
+    w = I.Workload("large_latents", "prefill", "bf16", nb, kv_len, 128, n_h, n_q, n_k, 1, d_h, d_l, seed=77)
+    t = I.prefill_inputs(w, device="cuda")
+    s = torch.einsum("nd,td->nt", t["q"][-1, 0].double(), t["k"][-1, 0].double()) / d_h ** 0.5
+    t["k"][-1, 0, 200:] *= float(30 / s[:, 200:].abs().max())
+    t["c"] *= 1e30
+    first = kv_len - N
+    q, x = t["q"][:, :, first:].contiguous(), t["x"][:, first:].contiguous()
+    if page_size:
+        k_pool, c_pool, table = _pools(t["k"], t["c"], kv_len, page_size, seed=6)
+        out = B.gta_prefill_chunk_paged(q, k_pool, c_pool, table.cuda(), x, t["w_p"], t["w_g"], kv_len)
+    else:
+        out = B.gta_prefill_chunk(q, t["k"], t["c"], x, t["w_p"], t["w_g"], kv_len)
+    tc = cpu(t)
+    want = oracle.prefill(oracle_shape(w), tc["q"], tc["k"], tc["c"], tc["x"], tc["w_p"], tc["w_g"], rows=list(range(first, kv_len)))
+    want = torch.from_numpy(np.asarray(want, np.float64)).reshape(out.shape)
+    got = out.cpu().double()
+    assert torch.isfinite(got).all()
+    for b in range(nb):
+        assert float((got[b] - want[b]).norm() / want[b].norm()) <= 1e-2
+
+
 def test_prefill_chunk_paged_full_size_c2_sampled_rows(B, oracle):
     """The benchmark's prefill shape with its keys and latents in 64-token pages."""
     w = I.CONFIGS["c2_prefill_bf16"]
