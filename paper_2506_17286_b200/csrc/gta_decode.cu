@@ -673,7 +673,8 @@ __device__ __forceinline__ uint2 f32_to_e4m3x8(const float (&y)[8]) {
     return make_uint2(f32_to_e4m3x2(y[0], y[1]) | (f32_to_e4m3x2(y[2], y[3]) << 16),
                       f32_to_e4m3x2(y[4], y[5]) | (f32_to_e4m3x2(y[6], y[7]) << 16));
 }
-// Eight elements as they are stored, their largest magnitude, their values, their signs.
+// Eight elements as they are stored, their largest magnitude (not a number if one of them is none; of the numbers among
+// them), their values, their signs.
 template <typename T> struct Piece;
 template <> struct Piece<float> {
     float4 a, b;
@@ -683,6 +684,11 @@ template <> struct Piece<float> {
         b = __ldg(reinterpret_cast<const float4*>(p) + 1);
     }
     __device__ __forceinline__ float amax() const {
+        using ptx::max_nan;
+        return max_nan(max_nan(max_nan(fabsf(a.x), fabsf(a.y)), max_nan(fabsf(a.z), fabsf(a.w))),
+                       max_nan(max_nan(fabsf(b.x), fabsf(b.y)), max_nan(fabsf(b.z), fabsf(b.w))));
+    }
+    __device__ __forceinline__ float amax_of_numbers() const {
         return fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
                      fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
     }
@@ -704,8 +710,15 @@ template <> struct Piece<__nv_bfloat16> {
     __device__ __forceinline__ void load(const __nv_bfloat16* p) { a = __ldg(reinterpret_cast<const uint4*>(p)); }
     __device__ __forceinline__ float amax() const {        // two magnitudes per instruction
         const auto h = [](uint32_t w) { return __habs2(*reinterpret_cast<const __nv_bfloat162*>(&w)); };
-        const __nv_bfloat162 m = __hmax2(__hmax2(h(a.x), h(a.y)), __hmax2(h(a.z), h(a.w)));
-        return fmaxf(__low2float(m), __high2float(m));
+        const __nv_bfloat162 m = __hmax2_nan(__hmax2_nan(h(a.x), h(a.y)), __hmax2_nan(h(a.z), h(a.w)));
+        return ptx::max_nan(__low2float(m), __high2float(m));
+    }
+    __device__ __forceinline__ float amax_of_numbers() const {
+        float v[8], m = 0.f;
+        widen(v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(v[j]));
+        return m;
     }
     __device__ __forceinline__ void widen(float (&v)[8]) const { Vec16<__nv_bfloat16>::widen(a, v); }
     __device__ __forceinline__ uint2 signs() const {
@@ -721,6 +734,16 @@ __device__ __noinline__ uint2 codes_by_division(Piece<T> p, float scale) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = __fdiv_rn(v[j], scale);
     return f32_to_e4m3x8(v);
+}
+
+// The largest magnitude of the numbers of a row.
+template <typename T, int NV>
+__device__ __forceinline__ float largest_number(const Piece<T> (&p)[NV], int lpr) {
+    float amax = p[0].amax_of_numbers();
+#pragma unroll
+    for (int i = 1; i < NV; ++i) amax = fmaxf(amax, p[i].amax_of_numbers());
+    for (int o = lpr >> 1; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    return amax;
 }
 
 // Row of `width` (a multiple of 8, at most 8 lpr NV) elements on `lpr` lanes (a power of two; `sl` is this lane's
@@ -739,11 +762,15 @@ __device__ __forceinline__ void quantise_row(const Piece<T> (&p)[NV], uint8_t* _
                                              float* __restrict__ scale_out, int width, int lpr, int sl, bool live) {
     float amax = p[0].amax();
 #pragma unroll
-    for (int i = 1; i < NV; ++i) amax = fmaxf(amax, p[i].amax());
-    for (int o = lpr >> 1; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    for (int i = 1; i < NV; ++i) amax = ptx::max_nan(amax, p[i].amax());
+    for (int o = lpr >> 1; o > 0; o >>= 1) amax = ptx::max_nan(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    // a row with elements that are no numbers: its scale is that of the others, and it is divided (the code of such an element
+    // has no sign)
+    const bool numbers = amax == amax;
+    if (__any_sync(0xffffffffu, !numbers)) amax = largest_number<T, NV>(p, lpr);
     const float scale = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
     if (!live) return;
-    const bool plain = scale > 8.7e-19f && scale < 1.2e18f;      // 2^-60, 2^60
+    const bool plain = numbers && scale > 8.7e-19f && scale < 1.2e18f;      // 2^-60, 2^60
     const float inv = __frcp_rn(scale);
     const uint64_t inv2 = ptx::f32x2(inv, inv), neg2 = ptx::f32x2(-scale, -scale);
 #pragma unroll

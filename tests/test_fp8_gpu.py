@@ -55,6 +55,37 @@ def test_quantising_append_is_bit_exact(B, oracle, dt, n_new):
             assert np.array_equal(g_, ref), what
 
 
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+@pytest.mark.parametrize("d_l,n_new", [(128, 1), (512, 3), (2048, 70)])
+def test_quantising_append_elements_that_are_no_numbers(B, dt, d_l, n_new):
+    """An element that is not a number gets the code 0x7f whatever its sign bit; the row's scale and its other codes are those of
+    the row without it (with a zero of that sign in its place)."""
+    tdt, idt, qnan = (torch.bfloat16, torch.int16, 0x7FC0) if dt == "bf16" else (torch.float32, torch.int32, 0x7FC00000)
+    g = torch.Generator("cpu").manual_seed(d_l)
+    nb, d_h, cap = 2, 64, n_new + 3
+    rows = [torch.randn(nb, 1, n_new, d, generator=g).to(tdt) for d in (d_h, d_l)]
+    rows[0][0, 0, 0, 1::5] = -0.0
+    holes = [torch.rand(r.shape, generator=g) < 0.1 for r in rows]
+    for h in holes:
+        h[1] = False                                                   # rows that are all numbers
+    holes[1][0, 0, 0] = True                                           # a row without any
+    clean = [torch.where(h, torch.zeros_like(r).copysign(r), r) for r, h in zip(rows, holes)]
+    broken = []
+    for r, h in zip(rows, holes):
+        nan = torch.where(torch.signbit(r), qnan - (1 << (8 * r.element_size() - 1)), qnan).to(idt).view(tdt)
+        broken.append(torch.where(h, nan, r))
+        assert bool((torch.isnan(broken[-1]) == h).all()) and bool((torch.signbit(broken[-1]) == torch.signbit(r)).all())
+    got = []
+    for k_new, c_new in (clean, broken):
+        caches = [t.cuda() for t in (torch.zeros(nb, 1, cap, d_h, dtype=torch.uint8), torch.zeros(nb, 1, cap, d_l, dtype=torch.uint8),
+                                     torch.zeros(nb, 1, cap), torch.zeros(nb, 1, cap))]
+        B.gta_cache_append_fp8(*caches, k_new.cuda(), c_new.cuda(), torch.ones(nb, dtype=torch.int32, device="cuda"))
+        got.append([t[:, :, 1:1 + n_new].cpu() for t in caches])
+    for i, h in enumerate(holes):
+        assert torch.equal(got[0][2 + i], got[1][2 + i])
+        assert torch.equal(torch.where(h, torch.full_like(got[0][i], 0x7F), got[0][i]), got[1][i])
+
+
 @pytest.mark.parametrize("dt,n_k,n_c,d_h,d_l,n_new", [
     ("bf16", 1, 1, 16, 16, 1), ("bf16", 3, 1, 48, 80, 5), ("bf16", 8, 1, 128, 1024, 1), ("bf16", 2, 3, 256, 2048, 33),
     ("f32", 1, 2, 256, 2048, 2), ("f32", 5, 1, 64, 272, 129), ("bf16", 4, 1, 128, 512, 77)])
