@@ -15,9 +15,10 @@ import os
 
 import torch
 
+from .build import native_path
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libgta_b200.so")
-NATIVE_PATH = os.path.join(_HERE, "_gta_binding.so")
 
 GTA_OK, GTA_ERR_INVALID_ARG, GTA_ERR_UNSUPPORTED, GTA_ERR_WORKSPACE = 0, 1, 2, 3
 GTA_ERR_CUDA, GTA_ERR_CACHE_FULL, GTA_ERR_TIMEOUT, GTA_ERR_STATIC_SCRATCH = 4, 5, 6, 7
@@ -152,9 +153,10 @@ def native():
     global _native
     if _native is None:
         L = lib()
-        if not os.path.exists(NATIVE_PATH):
-            raise RuntimeError(f"{NATIVE_PATH} not found: build it with `python -m paper_2506_17286_b200.build`")
-        loader = importlib.machinery.ExtensionFileLoader("_gta_binding", NATIVE_PATH)
+        path = native_path()
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} not found: build it with `python -m paper_2506_17286_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("_gta_binding", path)
         mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_gta_binding", loader))
         loader.exec_module(mod)
         for name in EXPORTS:
@@ -200,16 +202,13 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 # The helpers of the ctypes calls stay with plain integers: addresses and streams go to ctypes as they are, device
 # identity is an index, and the structs are kept by value.
-_raw_stream = torch._C._cuda_getCurrentRawStream
-_current_device = torch._C._cuda_getDevice
-
-
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    return _raw_stream(_current_device()) if stream is None else stream.cuda_stream
+    # (looked up here: a torch without CUDA imports this module too)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def _check_tensors(*ts):

@@ -1,4 +1,4 @@
-"""Build the CUDA library (sm_100a only) and the extension of its binding next to this file: libgta_b200.so, _gta_binding.so.
+"""Build the CUDA library (sm_100a only) and the extension of its binding next to this file: libgta_b200.so, _gta_binding-*.so.
 
 Usage: python -m paper_2506_17286_b200.build [--force] [--verbose]
 nvcc cross-compiles without a GPU; the resulting shared object is loaded by `binding.py`.
@@ -16,7 +16,6 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libgta_b200.so")
 OBJ_DIR = os.path.join(HERE, "_build")
-NATIVE = os.path.join(HERE, "_gta_binding.so")
 NATIVE_SRC = os.path.join(CSRC, "gta_binding.cpp")
 
 NVCC_FLAGS = [
@@ -37,13 +36,22 @@ def _newest(paths) -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
+def native_path() -> str:
+    """The binding's extension for this interpreter and its torch, whose C++ interfaces it is built against: another version of
+    either looks for a file of its own and never loads this one's."""
+    import torch
+    return os.path.join(HERE, f"_gta_binding-torch{torch.__version__}-{sys.implementation.cache_tag}.so")
+
+
 def build_native(force: bool = False) -> str:
     """The binding's extension: plain C++ against the torch of this interpreter."""
-    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < _newest([NATIVE_SRC, os.path.join(INCLUDE, "gta.h")]):
+    native = native_path()
+    sources = [NATIVE_SRC, os.path.join(INCLUDE, "gta.h"), os.path.abspath(__file__)]
+    if force or not os.path.exists(native) or os.path.getmtime(native) < _newest(sources):
         import torch
         t = os.path.dirname(torch.__file__)
         cuda = os.path.dirname(os.path.dirname(_nvcc())) or "/usr/local/cuda"
-        tmp = NATIVE + f".{os.getpid()}.tmp"
+        tmp = native + f".{os.getpid()}.tmp"
         cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
                f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", INCLUDE]
         for inc in (os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
@@ -51,8 +59,8 @@ def build_native(force: bool = False) -> str:
             cmd += ["-isystem", inc]
         cmd += [NATIVE_SRC, "-o", tmp, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
         subprocess.check_call(cmd)
-        os.replace(tmp, NATIVE)
-    return NATIVE
+        os.replace(tmp, native)
+    return native
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

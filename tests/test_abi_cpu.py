@@ -3,6 +3,8 @@ bad arguments on the host before anything could be launched (no GPU is touched).
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -16,6 +18,21 @@ def B():
     build.build()
     binding.lib()
     return binding
+
+
+def test_the_extension_of_another_torch_is_not_loaded(B, monkeypatch):
+    """The extension is built against the C++ interfaces of one torch; after an upgrade it is missing, not stale."""
+    assert B.native() is not None
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    monkeypatch.setattr(B, "_native", None)
+    with pytest.raises(RuntimeError, match="not found"):
+        B.native()
+
+
+def test_the_binding_imports_on_a_torch_without_cuda():
+    code = ("import torch\nfor n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n    delattr(torch._C, n)\n"
+            "import paper_2506_17286_b200.binding")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
 
 
 def _declared_symbols():
