@@ -317,80 +317,60 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
         *reinterpret_cast<float4*>(row_s + 16 + 4 * rg) = make_float4(l[0], l[1], l[2], l[3]);
     }
     float* o_rows = o_lat + (((size_t)b * d.n_q + g) * d.N + t0) * d.d_l + col0;
-    if constexpr (SW == 1) {
-        __syncwarp();
+    // log-sum-exp merge of the SW key splits of every row: the key tiles' memory takes the sums
+    float* o_s = k_s;                                                   // [SW][kRows][kCols]
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = 16 * qw + 8 * rh + i;
-            const float ls = row_s[16 + 8 * rh + i], inv = ls > 0.f ? 1.f / ls : 0.f;
-            if (r >= rows) continue;
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int n = 0; n < NC; ++n) {
-                if (4 * cc + 64 * n < n_cols) {
-                    float4 v;
-                    ptx::f32x2_split(o[i][n][0], v.x, v.y);
-                    ptx::f32x2_split(o[i][n][1], v.z, v.w);
-                    *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * cc + 64 * n) =
-                        make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
-                }
-            }
+        for (int n = 0; n < NC; ++n) {
+            float4 v;
+            ptx::f32x2_split(o[i][n][0], v.x, v.y);
+            ptx::f32x2_split(o[i][n][1], v.z, v.w);
+            *reinterpret_cast<float4*>(o_s + ((size_t)sw * kRows + 16 * qw + 8 * rh + i) * kCols + 4 * cc + 64 * n) = v;
         }
-    } else {
-        // log-sum-exp merge of the SW key splits of every row: the key tiles' memory takes the sums
-        float* o_s = k_s;                                                   // [SW][kRows][kCols]
+    __syncthreads();
+    const float* all_rows = row_s - warp * 32;                          // [warp][2][16]
+    for (int idx = tid; idx < rows * 16 * NC; idx += kThreads) {
+        const int r = idx / (16 * NC), v4 = idx % (16 * NC);
+        if (4 * v4 >= n_cols) continue;
+        float mx = -INFINITY;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int s = 0; s < SW; ++s) mx = fmaxf(mx, all_rows[(s * QW + (r >> 4)) * 32 + (r & 15)]);
+        float ls = 0.f;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int n = 0; n < NC; ++n) {
-                float4 v;
-                ptx::f32x2_split(o[i][n][0], v.x, v.y);
-                ptx::f32x2_split(o[i][n][1], v.z, v.w);
-                *reinterpret_cast<float4*>(o_s + ((size_t)sw * kRows + 16 * qw + 8 * rh + i) * kCols + 4 * cc + 64 * n) = v;
-            }
-        __syncthreads();
-        const float* all_rows = row_s - warp * 32;                          // [warp][2][16]
-        for (int idx = tid; idx < rows * 16 * NC; idx += kThreads) {
-            const int r = idx / (16 * NC), v4 = idx % (16 * NC);
-            if (4 * v4 >= n_cols) continue;
-            float mx = -INFINITY;
-#pragma unroll
-            for (int s = 0; s < SW; ++s) mx = fmaxf(mx, all_rows[(s * QW + (r >> 4)) * 32 + (r & 15)]);
-            float ls = 0.f;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int s = 0; s < SW; ++s) {
-                const float* rs = all_rows + (s * QW + (r >> 4)) * 32 + (r & 15);
-                const float w = rs[0] == -INFINITY ? 0.f : exp2f(rs[0] - mx);
-                ls = fmaf(rs[16], w, ls);
-                const float4 v = *reinterpret_cast<const float4*>(o_s + ((size_t)s * kRows + r) * kCols + 4 * v4);
-                a.x = fmaf(v.x, w, a.x); a.y = fmaf(v.y, w, a.y); a.z = fmaf(v.z, w, a.z); a.w = fmaf(v.w, w, a.w);
-            }
-            const float inv = ls > 0.f ? 1.f / ls : 0.f;
-            *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * v4) = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+        for (int s = 0; s < SW; ++s) {
+            const float* rs = all_rows + (s * QW + (r >> 4)) * 32 + (r & 15);
+            const float w = rs[0] == -INFINITY ? 0.f : exp2f(rs[0] - mx);
+            ls = fmaf(rs[16], w, ls);
+            const float4 v = *reinterpret_cast<const float4*>(o_s + ((size_t)s * kRows + r) * kCols + 4 * v4);
+            a.x = fmaf(v.x, w, a.x); a.y = fmaf(v.y, w, a.y); a.z = fmaf(v.z, w, a.z); a.w = fmaf(v.w, w, a.w);
         }
+        const float inv = ls > 0.f ? 1.f / ls : 0.f;
+        *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * v4) = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Decoder + gate.  CTA tile: 16 RW token rows x 64 CW columns of one attention map's heads; 4 rows x 8 columns per lane
+// Decoder + gate.  CTA tile: 16 RW token rows x 64 columns of one attention map's heads; 4 rows x 8 columns per lane
 // and accumulator (gate pre-activation and decoded value); KW warps share a tile and each contract a KW-th of every
 // k-block (added through shared memory at the end).  The gate's k-blocks (X, W_G) come first: they do not need the
 // attention kernel's result, behind which this kernel is programmatically launched.
 constexpr int kDecStages = 3;
 __host__ __device__ constexpr int dec_bk(int KW) { return KW == 1 ? 32 : 16 * KW; }
-constexpr size_t dec_smem_bytes(int RW, int CW, int KW) {
-    return (size_t)kDecStages * (16 * RW * (dec_bk(KW) + 4) + dec_bk(KW) * 64 * CW) * sizeof(float);
+constexpr size_t dec_smem_bytes(int RW, int KW) {
+    return (size_t)kDecStages * (16 * RW * (dec_bk(KW) + 4) + dec_bk(KW) * 64) * sizeof(float);
 }
 
-template <typename T, int RW, int CW, int KW>
-__global__ void __launch_bounds__(32 * RW * CW * KW)
+template <typename T, int RW, int KW>
+__global__ void __launch_bounds__(32 * RW * KW)
 generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restrict__ x, const T* __restrict__ w_p,
                        const T* __restrict__ w_g, T* __restrict__ out, int tile0) {
-    constexpr int kThreads = 32 * RW * CW * KW, BM = 16 * RW, BN = 64 * CW, BK = dec_bk(KW), KPW = BK / KW;
+    constexpr int kThreads = 32 * RW * KW, BM = 16 * RW, BN = 64, BK = dec_bk(KW), KPW = BK / KW;
     constexpr int kLdA = BK + 4, kStage = BM * kLdA + BK * BN;
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rw = warp % RW, cw = (warp / RW) % CW, kw = warp / (RW * CW);
+    const int rw = warp % RW, kw = warp / RW;
     const int rg = lane >> 3, cg = lane & 7;                 // rows rg + 4 i; columns 4 cg + {0..3}, 32 + 4 cg + {0..3}
 
     const long long M = (long long)d.B * d.N;
@@ -450,7 +430,7 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
 
     auto multiply = [&](int it, uint64_t (&acc)[4][4]) {
         const float* as = smem + (it % kDecStages) * kStage + (16 * rw + rg) * kLdA + kw * KPW;
-        const float* bs = smem + (it % kDecStages) * kStage + BM * kLdA + kw * KPW * BN + 64 * cw + 4 * cg;
+        const float* bs = smem + (it % kDecStages) * kStage + BM * kLdA + kw * KPW * BN + 4 * cg;
 #pragma unroll 2
         for (int k = 0; k < KPW; k += 4) {
             float4 a[4];
@@ -495,8 +475,8 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
         cp_async_wait<0>();
         __syncthreads();
         uint64_t* part = reinterpret_cast<uint64_t*>(smem);
-        static_assert(RW == 1 && CW == 1, "one tile");
-        static_assert((size_t)(KW - 1) * 32 * 32 * 8 <= dec_smem_bytes(1, 1, KW), "the partial sums fit");
+        static_assert(RW == 1, "one tile");
+        static_assert((size_t)(KW - 1) * 32 * 32 * 8 <= dec_smem_bytes(1, KW), "the partial sums fit");
         if (kw > 0) {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -525,7 +505,7 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
         T* o_row = out + (size_t)(m0 + r) * d.n_h * d.d_h + (size_t)g * map_cols + c0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int cc = 64 * cw + 32 * h + 4 * cg;
+            const int cc = 32 * h + 4 * cg;
             if (cc >= n_cols) continue;
             float z[4], y[4];
             ptx::f32x2_split(acc_g[i][2 * h], z[0], z[1]);
@@ -569,21 +549,21 @@ static cudaError_t launch_attention(const Dims& d, const T* q, const T* k, const
                           tiles);
 }
 
-template <typename T, int RW, int CW, int KW>
+template <typename T, int RW, int KW>
 static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x, const T* w_p, const T* w_g, T* out,
                                   cudaStream_t stream, bool behind, int* launches) {
-    auto kern = generic_decoder_kernel<T, RW, CW, KW>;
-    constexpr size_t smem = dec_smem_bytes(RW, CW, KW);
+    auto kern = generic_decoder_kernel<T, RW, KW>;
+    constexpr size_t smem = dec_smem_bytes(RW, KW);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int map_cols = d.n_h / d.n_q * d.d_h;
     const long long M = (long long)d.B * d.N;
     // a map of more than 65535 column tiles takes several launches (the tiles in x next to the rows' cost 3.5 % of 2 x 1500
     // tokens of the 1B layer)
-    const int tiles = (map_cols + 64 * CW - 1) / (64 * CW);
+    const int tiles = (map_cols + 63) / 64;
     for (int tile0 = 0; tile0 < tiles && err == cudaSuccess; tile0 += 65535, ++*launches)
         err = launch_chained(behind, kern, dim3((unsigned)((M + 16 * RW - 1) / (16 * RW)), min(tiles - tile0, 65535), d.n_q),
-                             32 * RW * CW * KW, smem, stream, d, o_lat, x, w_p, w_g, out, tile0);
+                             32 * RW * KW, smem, stream, d, o_lat, x, w_p, w_g, out, tile0);
     return err;
 }
 
@@ -627,9 +607,9 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
         const long long tiles64 = (((long long)d.B * d.N + 63) / 64) * d.n_q * ((d.n_h / d.n_q * d.d_h + 63) / 64);
         const float* l = o_lat_ws;
         const bool behind = stages & 1;      // X and W_G are read ahead of the wait: they are older than the attention kernel only
-        err = tiles64 < 40    ? launch_decoder<T, 1, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
-              : tiles64 < 256 ? launch_decoder<T, 1, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
-                              : launch_decoder<T, 4, 1, 1>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches);
+        err = tiles64 < 40    ? launch_decoder<T, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
+              : tiles64 < 256 ? launch_decoder<T, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
+                              : launch_decoder<T, 4, 1>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches);
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;
