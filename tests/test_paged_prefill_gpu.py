@@ -264,7 +264,8 @@ LAYERS_PAGED = [
     ("two_chunks_p64", 2, 320, 256, 8, 4, 2, 2, 64, 128, [192, 128], 64),
     ("ragged_chunks_last_page_one_row_p128", 1, 257, 256, 4, 2, 2, 1, 128, 256, [5, 251, 1], 128),
     ("c2_shape_small_p64", 1, 384, 512, 8, 4, 4, 1, 128, 512, None, 64),
-    ("plain_alu_page_p16", 2, 130, 256, 8, 4, 2, 2, 64, 128, [100, 30], 16),
+    ("small_pages_p16", 2, 130, 256, 8, 4, 2, 2, 64, 128, [100, 30], 16),
+    ("plain_alu_page_p24", 2, 130, 256, 8, 4, 2, 2, 64, 128, [100, 30], 24),
 ]
 
 

@@ -53,9 +53,13 @@ def test_prefill_paths_repeat_bit_for_bit(B, case):
     q, x = t["q"][:, :, -n_chunk:].contiguous(), t["x"][:, -n_chunk:].contiguous()
     _repeat(lambda: B.gta_prefill_chunk(q, t["k"], t["c"], x, t["w_p"], t["w_g"], N, status_word=status), 30,
             name + " chunk")
-    pg = I.paginate(dict(k_cache=t["k"], c_cache=t["c"]), 64, seed=3)
+    for page_size in (64, 16):
+        pg = I.paginate(dict(k_cache=t["k"], c_cache=t["c"]), page_size, seed=3)
+        _repeat(lambda: B.gta_prefill_chunk_paged(q, pg["k_pool"], pg["c_pool"], pg["block_table"], x, t["w_p"], t["w_g"],
+                                                  N - 37, status_word=status), 30, name + f" paged chunk, pages of {page_size}")
+    q, x = t["q"][:, :, -N // 2:].contiguous(), t["x"][:, -N // 2:].contiguous()      # more items than CTA pairs
     _repeat(lambda: B.gta_prefill_chunk_paged(q, pg["k_pool"], pg["c_pool"], pg["block_table"], x, t["w_p"], t["w_g"],
-                                              N - 37, status_word=status), 30, name + " paged chunk")
+                                              N - 5, status_word=status), 30, name + " long chunk, pages of 16")
     assert int(status.item()) == 0
 
 
@@ -96,9 +100,10 @@ def test_decode_paths_repeat_bit_for_bit(B, case):
         return [out, t["seq_lens"], t["k_cache"], t["c_cache"]]
     _repeat(fused_step, 30, name + " fused step")
     t["k_cache"].copy_(k0); t["c_cache"].copy_(c0); t["seq_lens"].copy_(l0)
-    pg = I.paginate(t, 64, seed=1)
-    _repeat(lambda: B.gta_decode_paged(t["q"], pg["k_pool"], pg["c_pool"], pg["block_table"], t["seq_lens"], *args,
-                                       status_word=status), 30, name + " paged")
+    for page_size in (64, 16):
+        pg = I.paginate(t, page_size, seed=1)
+        _repeat(lambda: B.gta_decode_paged(t["q"], pg["k_pool"], pg["c_pool"], pg["block_table"], t["seq_lens"], *args,
+                                           status_word=status), 30, name + f" paged, pages of {page_size}")
     if d_h == 128:      # the streaming kernel for 8-bit caches
         kq = torch.zeros((nb, n_k, cap, d_h), dtype=torch.uint8, device="cuda")
         cq = torch.zeros((nb, n_c, cap, d_l), dtype=torch.uint8, device="cuda")
@@ -112,6 +117,44 @@ def test_decode_paths_repeat_bit_for_bit(B, case):
                                        z, status_word=status)
         _repeat(lambda: B.gta_decode_fp8(t["q"], kq, cq, ks, cs, l0, *args, status_word=status), 50, name + " 8-bit caches")
     assert int(status.item()) == 0
+
+
+def test_calls_in_flight_behind_one_another(B):
+    """Each kernel may be scheduled while the one ahead of it drains, the first of a call while the last of the call before it
+    does: fused steps, prefills and plain-ALU steps over the same workspaces, queued without waiting, give what each gives
+    alone, and the lengths advance once a step."""
+    w = I.Workload("in_flight", "decode", "bf16", 12, 0, 512, 8, 4, 4, 1, 128, 512, seed=11)
+    lens = [40 + 61 * i for i in range(12)]
+    t = I.decode_inputs(w, device="cuda", s_cap=1024, seq_lens=lens)
+    f = I.decode_inputs(I.Workload("in_flight_f32", "decode", "f32", 3, 0, 256, 4, 2, 2, 1, 64, 128, seed=12), device="cuda", s_cap=256,
+                        seq_lens=[1, 100, 200])
+    p = I.prefill_inputs(I.Workload("in_flight_prefill", "prefill", "bf16", 2, 333, 512, 8, 4, 4, 1, 128, 512, seed=13), device="cuda")
+    ws = torch.empty(1 << 26, dtype=torch.uint8, device="cuda")
+    l0, f0 = t["seq_lens"].clone(), f["seq_lens"].clone()
+
+    def step(d):
+        return B.gta_decode_append(d["q"], d["k_cache"], d["c_cache"], d["k_new"], d["c_new"], d["seq_lens"], d["x_t"], d["w_p"],
+                                   d["w_g"], workspace=ws)
+
+    def calls(wait):
+        outs = []
+        for d, first in ((t, l0), (f, f0)):
+            d["seq_lens"].copy_(first)
+        for _ in range(8):
+            for fn in (lambda: step(t), lambda: B.gta_prefill(p["q"], p["k"], p["c"], p["x"], p["w_p"], p["w_g"], workspace=ws),
+                       lambda: step(t), lambda: step(f), lambda: step(f), lambda: step(t)):
+                outs.append(fn())
+                if wait:
+                    torch.cuda.synchronize()
+        return outs + [t["seq_lens"].clone(), f["seq_lens"].clone()]
+
+    want = calls(True)
+    assert want[-2].tolist() == [n + 24 for n in lens] and want[-1].tolist() == [17, 116, 216]
+    for rep in range(6):
+        got = calls(False)
+        torch.cuda.synchronize()
+        for i, (a, b) in enumerate(zip(got, want)):
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), (rep, i)
 
 
 def test_comparison_operator_repeats_bit_for_bit(B):
