@@ -95,7 +95,9 @@ typedef struct {
  * dtype = bf16, d_h = 64 or 128, d_l a multiple of 128 (at most 1024), H a multiple of 64 and
  * the heads of one attention map fill a multiple of 128 output columns ((n_h / n_q) d_h);
  * other shapes and fp32 run on the plain-ALU kernels of the same library (gta_prefill_path
- * tells which).  N = 0 or B = 0 is a no-op (GTA_OK).
+ * tells which).  On the tensor cores a masked probability is a zero factor, so an infinite or
+ * not-a-number latent can reach rows up to 255 positions before its own; on the plain-ALU kernels a
+ * row is untouched by what it does not attend.  N = 0 or B = 0 is a no-op (GTA_OK).
  */
 GTA_API size_t gta_prefill_workspace_bytes(const gta_shape_t *shape);
 GTA_API gta_status_t gta_prefill(const gta_shape_t *shape, const void *q, const void *k, const void *c,
@@ -195,7 +197,10 @@ GTA_API gta_status_t gta_cache_append(const gta_shape_t *shape, void *k_cache, v
  * page_size, n_pages or max_pages (or page_size * max_pages above INT32_MAX); otherwise as
  * gta_decode / gta_cache_append.  workspace: gta_decode_paged_workspace_bytes(shape, page_size,
  * max_pages).  The bf16 fast path of gta_decode applies when, in addition to its shape rules,
- * page_size is a multiple of 16; other page sizes run on the plain-ALU kernels.
+ * page_size is a multiple of 16; other page sizes run on the plain-ALU kernels.  Where it is not a
+ * multiple of 64, probabilities, latent sums and gates are kept to 2^-17 and better between the kernels
+ * (the plain-ALU kernels' precision), not to bf16, and a workspace that is enough for the plain-ALU
+ * kernels but not for the fast path runs on those.
  */
 GTA_API size_t gta_decode_paged_workspace_bytes(const gta_shape_t *shape, int32_t page_size,
                                                 int32_t max_pages);
@@ -225,7 +230,8 @@ GTA_API gta_status_t gta_cache_append_paged(const gta_shape_t *shape, void *k_po
  * kernels, so that result is unspecified).
  * q, x, weights, out, workspace (gta_prefill_workspace_bytes), arithmetic and errors as for
  * gta_prefill_chunk; the tensor-core path applies when, in addition to gta_prefill's rules, page_size is
- * a multiple of 16, other page sizes run on the plain-ALU kernels.
+ * a multiple of 16 (not of 64: with the precision of the plain-ALU kernels, see gta_decode_paged), other page
+ * sizes run on the plain-ALU kernels.
  */
 GTA_API gta_status_t gta_prefill_chunk_paged(const gta_shape_t *shape, int32_t kv_len, const void *q,
                                              const void *k_pool, const void *c_pool,
