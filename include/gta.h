@@ -85,18 +85,20 @@ typedef struct {
  *   out [B, N, n_h, d_h]      (written; same dtype as the inputs, round-to-nearest-even)
  *   workspace: gta_prefill_workspace_bytes(shape) bytes, 256-byte aligned; holds the normalised
  *     latent attention output L between the two kernels and, for calls of few rows on the tensor-core
- *     path, fp32 partial sums behind it; contents undefined afterwards.  The size never falls as batch
+ *     path, fp32 partial sums behind it, for fp32 calls of d_h = 64 the operands of its attention on the
+ *     tensor cores; contents undefined afterwards.  The size never falls as batch
  *     or seq grow, so a buffer for the largest call serves the smaller ones.  4 B n_q N d_l bytes (at
  *     least 256, rounded up to 256) are enough: with less room than the query gives, the keys of a call
- *     are split over fewer parts of the chip, or not at all (same precision, other rounding of the
- *     probabilities); with less than that, GTA_ERR_WORKSPACE.
+ *     are split over fewer parts of the chip, or not at all, and fp32 attention runs on the plain-ALU
+ *     kernel (same precision, other rounding); with less than that, GTA_ERR_WORKSPACE.
  *     Calls that share a workspace must be ordered on one stream.
  * Arithmetic: fp32 accumulation everywhere.  bf16 fast path (tcgen05 tensor cores) when
  * dtype = bf16, d_h = 64 or 128, d_l a multiple of 128 (at most 1024), H a multiple of 64 and
  * the heads of one attention map fill a multiple of 128 output columns ((n_h / n_q) d_h);
- * other shapes and fp32 run on the plain-ALU kernels of the same library (gta_prefill_path
- * tells which).  On the tensor cores a masked probability is a zero factor, so an infinite or
- * not-a-number latent can reach rows up to 255 positions before its own; on the plain-ALU kernels a
+ * other shapes and fp32 run with fp32 precision on the plain-ALU kernels of the same library or, where
+ * d_h is a multiple of 64, on the tensor cores in three bf16 pieces per operand (gta_prefill_path is 1
+ * for both).  On the bf16 path a masked probability is a zero factor, so an infinite or
+ * not-a-number latent can reach rows up to 255 positions before its own; on the other a
  * row is untouched by what it does not attend.  N = 0 or B = 0 is a no-op (GTA_OK).
  */
 GTA_API size_t gta_prefill_workspace_bytes(const gta_shape_t *shape);

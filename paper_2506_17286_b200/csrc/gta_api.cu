@@ -137,7 +137,9 @@ size_t gta_prefill_workspace_bytes(const gta_shape_t* shape) {
     // served with prefill_least_workspace too; it then splits as far as what it was given has room.
     const size_t least = prefill_least_workspace(d);
     const size_t split = gta::sm100_prefill_supported(d, shape->dtype) ? gta::sm100_split_workspace_bytes(d) : 0;
-    return split > least ? split : least;
+    // fp32: the pieces of K and C behind L
+    const size_t pieces = shape->dtype == GTA_F32 && gta::sm100_attention_f32_supported(d) ? least + gta::sm100_attention_f32_scratch(d) : 0;
+    return split > least ? split : pieces > least ? pieces : least;
 }
 
 gta_status_t gta_prefill(const gta_shape_t* shape, const void* q, const void* k, const void* c,
@@ -216,7 +218,7 @@ static gta_status_t prefill_impl(const gta_shape_t* shape, int32_t kv_len, int32
         err = cudaSuccess;
     } else {
         err = gta::launch_generic_prefill(d, shape->dtype, q, k, c, x, w_p, w_g, out,
-                                          static_cast<float*>(workspace), stream, stages, &launches, pm, status_word);
+                                          static_cast<float*>(workspace), workspace_bytes, stream, stages, &launches, pm, status_word);
     }
     if (err != cudaSuccess) return GTA_ERR_CUDA;
     g_last_launches = launches;

@@ -1,8 +1,8 @@
 // Plain-ALU (fp32 FMA) prefill kernels: any supported shape, fp32 or bf16 storage.
-// They carry the fp32 workload (tensor-core tf32 would not meet its 1e-4 bound) and every
-// shape the tcgen05 kernels do not cover.  Two kernels:
+// They carry small fp32 calls (larger ones run on the tensor cores in bf16 pieces, f32_plan below) and every shape
+// the tcgen05 kernels do not cover.  Two kernels:
 //   generic_attention_kernel : shared attention map per query group, online softmax, latent
-//                              P·C  ->  normalised L[B, n_q, N, d_l] (fp32, workspace)
+//                              P·C  ->  normalised L[n_q, B, N, d_l] (fp32, workspace)
 //   generic_decoder_kernel   : out_i = (L_{q(i)} W_P,i) (.) sigmoid(X W_G,i)
 // (Sec. 3.3 reformulated equation; causal sum of App. B.1.1.)
 //
@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "gta_common.cuh"
+#include "gta_sm100.cuh"
 #include "sm100_ptx.cuh"
 
 namespace gta {
@@ -316,7 +317,7 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
         *reinterpret_cast<float4*>(row_s + 4 * rg) = make_float4(m[0], m[1], m[2], m[3]);
         *reinterpret_cast<float4*>(row_s + 16 + 4 * rg) = make_float4(l[0], l[1], l[2], l[3]);
     }
-    float* o_rows = o_lat + (((size_t)b * d.n_q + g) * d.N + t0) * d.d_l + col0;
+    float* o_rows = o_lat + (((size_t)g * d.B + b) * d.N + t0) * d.d_l + col0;
     // log-sum-exp merge of the SW key splits of every row: the key tiles' memory takes the sums
     float* o_s = k_s;                                                   // [SW][kRows][kCols]
 #pragma unroll
@@ -408,8 +409,7 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
             if (gate) {
                 stage4(dst, x + (size_t)m * d.H + (live ? kk : 0), live);
             } else {
-                const int b = (int)(m / d.N), t = (int)(m - (long long)b * d.N);
-                stage4(dst, o_lat + (((size_t)b * d.n_q + g) * d.N + t) * d.d_l + (live ? kk : 0), live);
+                stage4(dst, o_lat + ((size_t)g * M + m) * d.d_l + (live ? kk : 0), live);
             }
         }
         const T* w = gate ? wg_col : wp_col;
@@ -567,13 +567,62 @@ static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x,
     return err;
 }
 
+// Which kernels serve an fp32 call.  Measured, us, plain-ALU / tensor cores.  Attention: 1B layer, 64 tokens 18.5 / 21.2, 128
+// 29.6 / 32.4, 2 x 100 47.4 / 32.3, 200 47.4 / 32.7; tiny layer, 4 x 128 17.3 / 20.1, 8 x 128 23.0 / 20.8, 333 28.5 / 23.3, 8 x 2048
+// 527 / 160: from 192 keys, or more than 64 plain CTAs of 16 rows, on.  Decoder: 1B 200 tokens (80 tiles of 64 x 64) 32.7 / 42.7, 333
+// (120) 54.4 / 42.6; tiny 700 (44) 28.4 / 30.3, 2048 (128) 45.3 / 38.7: from 100 tiles on; in blocks of 128 columns while those of
+// 256 are few (1B, 1000 tokens, 20 blocks of 256: 54.3 / 47.1 with 128; 1500, 30: 66.2 / 73.6).
+//
+// CTAs that share the keys of a row tile: a key tile takes 1.25 us, a CTA 6 us more and 1 for every one that it merges with, a stage
+// of the decoder 0.9 or 1.05 us.  The decoder's gates run beside the attention kernel where both fit the chip at once (1B, 1000
+// tokens: 47.1 with one, 54.6 with two; tiny, 2048: 75.5 / 48.8 / 38.7 with one / two / four); a plain decoder wants the SMs that a
+// split takes (1B, 200 tokens: 32.7 / 43.3; tiny, 333: 26.0 / 23.3).
+struct F32Plan { int split = 0, cols = 0; };       // 0: the plain-ALU kernel
+static size_t l_bytes(const Dims& d) { return ((size_t)d.B * d.n_q * d.N * d.d_l * sizeof(float) + 255) & ~(size_t)255; }
+static F32Plan f32_plan(const Dims& d, const PageMap& pm, size_t room) {
+    F32Plan plan;
+    const long long M = (long long)d.B * d.N;
+    const int map_cols = d.n_h / d.n_q * d.d_h;
+    if (M > (1 << 30) || (long long)d.n_h * d.d_h > (1 << 30)) return plan;       // (the kernels count rows and columns in 32 bits)
+    const long long tiles64 = ((M + 63) / 64) * d.n_q * ((map_cols + 63) / 64);
+    if (d.d_h % 64 == 0 && tiles64 >= 100) plan.cols = map_cols > 128 && sm100_decoder_f32_units(d, 256) > 28 ? 256 : 128;
+    const long long plain = (long long)d.B * d.n_q * ((d.N + 15) / 16);
+    if (pm.table != nullptr || !sm100_attention_f32_supported(d) || (d.Nk < 192 && plain <= 64) ||
+        room < l_bytes(d) + sm100_attention_f32_scratch(d))
+        return plan;
+    const long long items = (long long)((d.N + 127) / 128) * (d.d_l / 128) * d.n_q * d.B;
+    const long long dec_ctas = plan.cols ? 2 * sm100_decoder_f32_units(d, plan.cols) : 0;
+    const float stage = plan.cols == 256 ? 1.05f : 0.9f, dec_waves = (float)((dec_ctas + 147) / 148);
+    const float gates = dec_waves * stage * ((d.H + 31) / 32), values = dec_waves * stage * ((d.d_l + 31) / 32);
+    const float most = (float)((d.Nk + 63) / 64), mean = d.causal ? most - 0.5f * d.N / 64.f + 0.5f : most;       // key tiles of an item
+    float best = 0.f;
+    for (int split = 1; split <= 4; split *= 2) {
+        const float fixed = 6.f + split;
+        const float waves = (float)((items * split + 147) / 148);
+        const float att = fmaxf(1.25f * most / split + fixed, waves * (1.25f * mean / split + fixed));
+        const float total = plan.cols == 0                        ? att + (split > 1 ? 2.f : 0.f)
+                            : items * split + dec_ctas <= 148 ? fmaxf(att, gates) + values
+                                                              : att + gates + values;
+        if (plan.split == 0 || total < best) { best = total; plan.split = split; }
+    }
+    return plan;
+}
+
 template <typename T>
 static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, const void* c, const void* x,
-                                const void* w_p, const void* w_g, void* out, float* o_lat_ws,
+                                const void* w_p, const void* w_g, void* out, float* o_lat_ws, size_t room,
                                 cudaStream_t stream, int stages, int* launches, const PageMap& pm,
                                 int32_t* status_word) {
     cudaError_t err;
-    if (stages & 1) {
+    const F32Plan plan = std::is_same_v<T, float> ? f32_plan(d, pm, room) : F32Plan{};
+    if constexpr (std::is_same_v<T, float>) {
+        if ((stages & 1) && plan.split) {
+            err = launch_sm100_attention_f32(d, (const float*)q, (const float*)k, (const float*)c, o_lat_ws,
+                                             reinterpret_cast<uint8_t*>(o_lat_ws) + l_bytes(d), status_word, stream, plan.split, launches);
+            if (err != cudaSuccess) return err;
+        }
+    }
+    if ((stages & 1) && !plan.split) {
         // Which split: the CTAs of 64 rows that the call would have.  Measured (us; (1,4) / (2,4) / (2,2) warps over rows and
         // keys; four warps on 64 rows were never the best): 20 (1B layer, 256 tokens) 16 / 20 / 24; 56 (tiny layer, 1767)
         // 86 / 112 / 162; 80 (1B, 1000) 84 / 67 / 101; 128 (tiny, 8 x 512) 72 / 59 / 72; 160 (1B, 2048) 268 / 209 / 269;
@@ -606,6 +655,15 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
         // columns) 58 / 34 / 30; 640 (2048 rows) 315 / 220 / 200.
         const long long tiles64 = (((long long)d.B * d.N + 63) / 64) * d.n_q * ((d.n_h / d.n_q * d.d_h + 63) / 64);
         const float* l = o_lat_ws;
+        if constexpr (std::is_same_v<T, float>) {
+            if (plan.cols) {
+                err = launch_sm100_decoder_f32(d, l, (const float*)x, (const float*)w_p, (const float*)w_g, (float*)out, status_word,
+                                               stream, stages & 1, plan.cols);
+                if (err != cudaSuccess) return err;
+                *launches += 1;
+                return cudaSuccess;
+            }
+        }
         const bool behind = stages & 1;      // X and W_G are read ahead of the wait: they are older than the attention kernel only
         err = tiles64 < 40    ? launch_decoder<T, 1, 8>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
               : tiles64 < 256 ? launch_decoder<T, 1, 4>(d, l, (const T*)x, (const T*)w_p, (const T*)w_g, (T*)out, stream, behind, launches)
@@ -617,11 +675,11 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
 
 cudaError_t launch_generic_prefill(const Dims& d, int dtype, const void* q, const void* k, const void* c,
                                    const void* x, const void* w_p, const void* w_g, void* out,
-                                   float* o_lat_ws, cudaStream_t stream, int stages, int* launches,
+                                   float* o_lat_ws, size_t room, cudaStream_t stream, int stages, int* launches,
                                    const PageMap& pm, int32_t* status_word) {
     if (dtype == GTA_F32)
-        return launch_typed<float>(d, q, k, c, x, w_p, w_g, out, o_lat_ws, stream, stages, launches, pm, status_word);
-    return launch_typed<__nv_bfloat16>(d, q, k, c, x, w_p, w_g, out, o_lat_ws, stream, stages, launches, pm,
+        return launch_typed<float>(d, q, k, c, x, w_p, w_g, out, o_lat_ws, room, stream, stages, launches, pm, status_word);
+    return launch_typed<__nv_bfloat16>(d, q, k, c, x, w_p, w_g, out, o_lat_ws, room, stream, stages, launches, pm,
                                        status_word);
 }
 

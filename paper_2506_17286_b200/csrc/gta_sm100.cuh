@@ -39,6 +39,20 @@ gta_status_t launch_sm100_decoder_fine(const Dims& d, const void* l_planes, cons
                                        void* out, int32_t* status_word, cudaStream_t stream, bool release = true,
                                        bool behind = true);
 
+// Attention of an fp32 call on the tensor cores (gta_sm100_f32_attention.cu): d_h = 64, d_l a multiple of 128, contiguous K and
+// C; L fp32 [n_q, B, N, d_l]; scratch of the given size (256-byte aligned) for the pieces of K and C; split: CTAs (1, 2 or
+// 4) that share the keys of a row tile.
+bool sm100_attention_f32_supported(const Dims& d);
+size_t sm100_attention_f32_scratch(const Dims& d);
+cudaError_t launch_sm100_attention_f32(const Dims& d, const float* q, const float* k, const float* c, float* o_lat, void* scratch,
+                                       int32_t* status_word, cudaStream_t stream, int split, int* launches);
+
+// Decoder + gate of an fp32 call on the tensor cores (gta_sm100_f32_decoder.cu): L fp32 [n_q, B, N, d_l]; d_h a multiple of 64;
+// nt: columns of an item (256 or 128), whose number is the other function's result.
+long long sm100_decoder_f32_units(const Dims& d, int nt);
+cudaError_t launch_sm100_decoder_f32(const Dims& d, const float* o_lat, const float* x, const float* w_p, const float* w_g,
+                                     float* out, int32_t* status_word, cudaStream_t stream, bool behind, int nt);
+
 // Linear maps of the attention layer around the operator (App. B.1.1), bf16 with fp32 accumulation.
 // True when the tcgen05 kernel covers the layer's projections for this shape.
 bool sm100_linear_supported(const Dims& d, int dtype);

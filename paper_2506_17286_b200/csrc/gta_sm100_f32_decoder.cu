@@ -1,0 +1,465 @@
+// fp32 decoder + gate on the tensor cores:
+//     out_i = (L_{q(i)} W_P,i) (.) Sigmoid(X W_G,i)          (Sec. 3.3, reformulated equation)
+//
+// Every fp32 operand is the sum of three bf16 pieces, exactly (8 significant bits each, rounded to nearest, the rest handed
+// on); six of the nine products of pieces are taken (what is left out is below 2^-25 of a product), each exact in the
+// tensor core, which adds them in fp32 but cuts where fp32 arithmetic rounds.  So a sum stays in tensor memory for 32
+// elements of the contraction only, small products first, and is added up in registers (rounded) from there: against 64
+// bits the result is closer than the FMA chain of the plain-ALU kernel.
+//
+// CTA pairs, one item of 256 token rows x NT output columns of one attention map per pair.
+//   warp 0       (leader CTA) issues the MMAs: twelve per stage, two accumulators in tensor memory in turn.
+//   warp 1       brings the fp32 operands in by TMA, two or three blocks of 32 k ahead of the
+//   warps 4-11   that split them and store the pieces into a ring of swizzled stages.
+//   warps 12-19  add finished accumulators to their registers: a lane is a token row, a warp has half of the item's columns.
+// The gates come first (they need nothing of the attention kernel, behind which this kernel is launched) and then wait in one
+// of the two accumulators, while the decoded values take the other.
+//
+// What bounds it: a stage of 256 x 256 x 32 takes 1536 cycles of MMAs and 208 KB of shared-memory traffic (raw blocks in and
+// out, pieces in, operands read once per product: 1664 cycles); measured 1800.
+//
+// An element that is infinite, not a number or rounds to infinity in bf16 makes its row or column of the item not a number
+// (0 x infinity); the splitting threads see it, and those rows and columns are done again with plain FMAs.
+#include "gta_sm100.cuh"
+
+#include <cuda.h>
+
+#include "sm100_ptx.cuh"
+#include "tma_host.cuh"
+
+namespace gta {
+
+namespace {
+
+constexpr int kSplitWarp0 = 4, kSplitThreads = 256, kAddWarp0 = 12, kAddWarps = 8, kThreads = 640;
+constexpr int kBoth = kSplitThreads + 32 * kAddWarps;
+// registers: 640 threads start with 96 each (61440), which the warpgroups share out anew: 128 x 48 + 256 x 64 + 256 x 152
+constexpr int kIssueRegs = 48, kSplitRegs = 64, kAddRegs = 152;
+constexpr int kTileM = 128, kBlockK = 32;      // token rows of a CTA; elements of the contraction per stage
+constexpr uint32_t kRawBlock = kBlockK * 64 * 4;         // 64 columns of a block of the weights, in fp32
+constexpr uint32_t kAPlane = kTileM * kBlockK * 2;      // one piece of the A tile: rows of 64 bytes
+
+template <int NT> struct Cfg {
+    static constexpr int kCols = NT / 2;                         // columns that a CTA stages
+    static constexpr uint32_t kBPlane = kBlockK * kCols * 2;     // blocks of 64 columns, [k][128 bytes]
+    static constexpr uint32_t kStageBytes = 3 * (kAPlane + kBPlane);
+    // 16-byte pieces of a block, per splitting thread: rows of the A tile, then k-rows of the weight tile
+    static constexpr int kAPieces = kTileM * kBlockK / 4 / kSplitThreads, kBPieces = kBlockK * kCols / 4 / kSplitThreads;
+    static constexpr uint32_t kRawBytes = (kAPieces + kBPieces) * kSplitThreads * 16;
+    static constexpr int kStages = NT == 256 ? 3 : 4, kRaw = NT == 256 ? 2 : 3;
+    static constexpr uint32_t kBarOffset = kStages * kStageBytes + kRaw * kRawBytes;
+    static constexpr uint32_t kSmem = kBarOffset + 1024 /* barriers, flags */ + 1024 /* alignment */;
+    static_assert(kSmem <= 227 * 1024, "shared memory of a CTA");
+};
+
+// Sigmoid to an ulp or two: an exponential, a reciprocal of 1 ulp and a Newton step (a denominator near the end of the range
+// stays without it: 1 - d r would not be a number).
+__device__ __forceinline__ float sigmoid(float z) {
+    const float den = 1.f + expf(-z), r = ptx::rcp_approx(den);
+    return den < 1e37f ? fmaf(r, fmaf(-den, r, 1.f), r) : r;
+}
+
+// What a CTA works on
+struct Block {
+    int g, n0, n_cols, map_cols, rows;     // map, first column inside it, columns, columns of the map, token rows
+    long long m0;                          // first token row
+};
+template <int NT> __device__ __forceinline__ Block block_of(const Dims& d, int row_tiles, int col_tiles, uint32_t block) {
+    // items of one column block and map follow one another: their CTAs read the same weights
+    const int pr = block >> 1, rt = pr % row_tiles, ct = pr / row_tiles % col_tiles;
+    const long long M = (long long)d.B * d.N;
+    Block w;
+    w.g = pr / (row_tiles * col_tiles);
+    w.map_cols = d.n_h / d.n_q * d.d_h;
+    w.m0 = (long long)rt * 2 * kTileM + (block & 1) * kTileM;
+    w.rows = (int)(M - w.m0 < 0 ? 0 : M - w.m0 < kTileM ? M - w.m0 : kTileM);
+    w.n0 = ct * NT;
+    w.n_cols = min(NT, w.map_cols - w.n0);
+    return w;
+}
+
+// The rows and columns that hold an element which the pieces cannot: plain FMAs, by the adding warps.
+template <int NT>
+__device__ __forceinline__ void redo(const Dims& d, const float* o_lat, const float* x, const float* w_p, const float* w_g, float* out,
+                                     int row_tiles, int col_tiles, uint32_t block, const uint8_t* row_bad, const uint8_t* col_bad) {
+    const Block w = block_of<NT>(d, row_tiles, col_tiles, block);
+    const size_t ldw = (size_t)d.n_h * d.d_h;
+    const int tid = threadIdx.x - 32 * kAddWarp0;
+    auto again = [&](int r, int c) {
+        const long long m = w.m0 + r;
+        const int f = w.n0 + c, head = w.g * (d.n_h / d.n_q) + f / d.d_h, elem = f % d.d_h;
+        const float* xr = x + m * d.H;
+        const float* wg = w_g + (size_t)head * d.d_h + elem;
+        float z = 0.f, y = 0.f;
+        for (int k = 0; k < d.H; ++k) z = fmaf(xr[k], wg[k * ldw], z);
+        const float* lr = o_lat + ((size_t)w.g * d.B * d.N + m) * d.d_l;
+        const float* wp = w_p + (size_t)head * d.d_l * d.d_h + elem;
+        for (int k = 0; k < d.d_l; ++k) y = fmaf(lr[k], wp[(size_t)k * d.d_h], y);
+        out[m * ldw + (size_t)w.g * w.map_cols + f] = y * (1.f / (1.f + expf(-z)));
+    };
+    for (int r = 0; r < w.rows; ++r)
+        if (row_bad[r])
+            for (int c = tid; c < w.n_cols; c += 32 * kAddWarps) again(r, c);
+    for (int c4 = 0; 4 * c4 < w.n_cols; ++c4)
+        if (col_bad[c4])
+            for (int i = tid; i < 4 * w.rows; i += 32 * kAddWarps) again(i >> 2, 4 * c4 + (i & 3));
+}
+
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 1)
+sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_constant__ CUtensorMap tm_x,
+                         const __grid_constant__ CUtensorMap tm_wp, const __grid_constant__ CUtensorMap tm_wg,
+                         const __grid_constant__ CUtensorMap tm_out, Dims d, const float* __restrict__ o_lat,
+                         const float* __restrict__ x, const float* __restrict__ w_p, const float* __restrict__ w_g, float* out,
+                         int row_tiles, int col_tiles, int32_t* status_word) {
+    using C = Cfg<NT>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* raw = smem + C::kStages * C::kStageBytes;
+    uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + C::kBarOffset);     // leader CTA: 16 warps arrive
+    uint64_t* empty_bar = full_bar + C::kStages;                                 // both CTAs
+    uint64_t* raw_full = empty_bar + C::kStages;                                 // own CTA
+    uint64_t* raw_empty = raw_full + C::kRaw;                                    // own CTA: 8 warps arrive
+    uint64_t* acc_full = raw_empty + C::kRaw;                                    // both CTAs, [2]
+    uint64_t* acc_free = acc_full + 2;                                           // leader CTA, [2]: 16 warps arrive
+    uint64_t* drain_bar = acc_free + 2;                                          // leader CTA: an unwinding issuer's
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* drain_flag = abort_flag + 1;
+    uint32_t* any_bad = tmem_slot + 3;
+    uint8_t* row_bad = smem + C::kBarOffset + 256;                               // [128]
+    uint8_t* col_bad = row_bad + kTileM;                                         // [NT / 4]: four columns each
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = ptx::cluster_ctarank();
+    const int n_g = (d.H + kBlockK - 1) / kBlockK, n_it = n_g + (d.d_l + kBlockK - 1) / kBlockK;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < C::kStages; ++s) { ptx::mbar_init(&full_bar[s], 2 * kSplitThreads / 32); ptx::mbar_init(&empty_bar[s], 1); }
+        for (int r = 0; r < C::kRaw; ++r) { ptx::mbar_init(&raw_full[r], 1); ptx::mbar_init(&raw_empty[r], kSplitThreads / 32); }
+        for (int s = 0; s < 2; ++s) { ptx::mbar_init(&acc_full[s], 1); ptx::mbar_init(&acc_free[s], 2 * kAddWarps); }
+        ptx::mbar_init(drain_bar, 1);
+        *abort_flag = 0;
+        *drain_flag = 0;
+        *any_bad = 0;
+        ptx::fence_mbar_init();
+    }
+    if (threadIdx.x < (kTileM + NT / 4) / 4) reinterpret_cast<uint32_t*>(row_bad)[threadIdx.x] = 0;
+    if (warp == 0) ptx::tmem_alloc_pair(tmem_slot, 2 * NT);
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::cluster_arrive();         // the peer's barriers exist before anything is signalled to them
+    ptx::cluster_wait();
+    ptx::tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
+    // Accumulators take turns up to the gates' last; it keeps the gates, and the decoded values have the other to themselves.
+    const auto buf_of = [&](int it) { return (it < n_g ? it : n_g) & 1; };
+    const auto use_of = [&](int it) { return it < n_g ? it >> 1 : (n_g >> 1) + (it - n_g); };      // how often it was used before
+
+    if (warp < kSplitWarp0) {
+        ptx::set_max_regs_dec<kIssueRegs>();
+        if (warp == 0 && rank == 0 && ptx::elect_one()) {
+            const uint32_t idesc = ptx::make_idesc_bf16(2 * kTileM, NT, 0, 1);   // A K-major, B MN-major
+            const uint64_t a_desc = ptx::make_smem_desc_sw64(ptx::smem_addr(smem), 512);
+            const uint64_t b_desc = ptx::make_smem_desc(ptx::smem_addr(smem) + 3 * kAPlane, kBlockK * 128, 1024);
+            const uint32_t a_lo0 = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32), b_lo0 = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
+            bool ok = true;
+            int s = 0;
+            uint32_t ph = 0;
+            for (int it = 0; it < n_it; ++it, s = (s + 1 == C::kStages) ? 0 : s + 1, ph ^= (s == 0)) {
+                const int buf = buf_of(it);
+                ok = ptx::mbar_wait(&acc_free[buf], (use_of(it) & 1) ^ 1, abort_flag) && ptx::mbar_wait(&full_bar[s], ph, abort_flag);
+                if (!ok) break;
+                ptx::mbar_try_wait_acquire_cluster(&full_bar[s], ph);    // (both CTAs' pieces, written by ordinary stores)
+                ptx::tc_fence_after_sync();
+                const uint32_t a_lo = a_lo0 + s * (C::kStageBytes >> 4), b_lo = b_lo0 + s * (C::kStageBytes >> 4);
+                const uint32_t d_tmem = tmem_base + buf * NT;
+                constexpr int kPa[6] = {2, 1, 0, 1, 0, 0}, kPb[6] = {0, 1, 2, 0, 1, 0};       // pieces, the smallest products first
+#pragma unroll
+                for (int u = 0; u < 6; ++u)
+#pragma unroll
+                    for (int k2 = 0; k2 < kBlockK / 16; ++k2)
+                        ptx::mma_ss_pair(d_tmem, ptx::desc_of(a_lo + ((kPa[u] * kAPlane + k2 * 32) >> 4), a_hi),
+                                         ptx::desc_of(b_lo + ((kPb[u] * C::kBPlane + k2 * 16 * 128) >> 4), b_hi), idesc, (u | k2) ? 1u : 0u);
+                ptx::tc_commit_pair(&empty_bar[s], 3);
+                ptx::tc_commit_pair(&acc_full[buf], 3);
+            }
+            if (!ok) {      // tensor memory is freed below: nothing may be on its way there
+                ptx::tc_commit_pair(drain_bar, 1);
+                ptx::mbar_wait_drain(drain_bar, 0, drain_flag);
+            }
+        }
+        if (warp == 1 && ptx::elect_one()) {
+            const Block w = block_of<NT>(d, row_tiles, col_tiles, blockIdx.x);
+            ptx::prefetch_tensormap(&tm_x); ptx::prefetch_tensormap(&tm_wg);
+            ptx::prefetch_tensormap(&tm_l); ptx::prefetch_tensormap(&tm_wp);
+            const int col = w.g * w.map_cols + w.n0 + (int)rank * C::kCols;      // this CTA's first output column (of n_h d_h)
+            const int m0 = (int)w.m0;
+            int r = 0;
+            uint32_t ph = 1;
+            bool ok = true;
+            int it = 0;
+            for (; it < n_it; ++it) {
+                ok = ptx::mbar_wait(&raw_empty[r], ph, abort_flag);
+                if (!ok) break;
+                const bool gate = it < n_g;
+                const int k0 = (gate ? it : it - n_g) * kBlockK;
+                uint8_t* dst = raw + r * C::kRawBytes;
+                uint8_t* dst_w = dst + kTileM * kBlockK * 4;
+                if (it == n_g) {                // L is the attention kernel's; X and the weights are older
+                    ptx::grid_dependency_wait();
+                    ptx::grid_launch_dependents();
+                }
+                ptx::mbar_arrive_expect_tx(&raw_full[r], C::kRawBytes);
+                if (gate) {
+                    ptx::tma_load_2d(dst, &tm_x, &raw_full[r], k0, m0);
+                    for (int u = 0; u < C::kCols / 64; ++u) ptx::tma_load_2d(dst_w + u * kRawBlock, &tm_wg, &raw_full[r], col + 64 * u, k0);
+                } else {
+                    ptx::tma_load_3d(dst, &tm_l, &raw_full[r], k0, m0, w.g);
+                    for (int u = 0; u < C::kCols / 64; ++u)
+                        ptx::tma_load_3d(dst_w + u * kRawBlock, &tm_wp, &raw_full[r], (col + 64 * u) % d.d_h, k0, (col + 64 * u) / d.d_h);
+                }
+                r = r + 1 == C::kRaw ? 0 : r + 1;
+                ph ^= r == 0;
+            }
+            if (!ok)                             // every armed block either lands or the wait gives up
+                for (int back = 1; back <= C::kRaw && it - back >= 0; ++back)
+                    ptx::mbar_wait_drain(&raw_full[(it - back) % C::kRaw], ((it - back) / C::kRaw) & 1, drain_flag);
+        }
+    } else if (warp < kAddWarp0) {
+        ptx::set_max_regs_dec<kSplitRegs>();
+        const int tid = threadIdx.x - 32 * kSplitWarp0;
+        // this thread's pieces: A row 32 i + tid / 8, elements 4 (tid % 8) of the block; of the i-th 16 k of the weights (64 columns
+        // after 64 columns) k = tid / 16, columns 4 (tid % 16) of the 64
+        const int a_row = tid >> 3, b_k = tid >> 4, b_vec = tid & 15;
+        // four floats -> 8 bytes of each piece.  0 x (what is left) tells a number from an odd one.
+        uint64_t odd = 0ull;
+        auto split = [&](const ulonglong2 v, uint8_t* dst, uint32_t plane) {
+            uint64_t r0 = v.x, r1 = v.y;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                float a, b, e, f;
+                ptx::f32x2_split(r0, a, b);
+                ptx::f32x2_split(r1, e, f);
+                const uint32_t h0 = ptx::cvt_bf16x2(a, b), h1 = ptx::cvt_bf16x2(e, f);
+                *reinterpret_cast<uint2*>(dst + p * plane) = make_uint2(h0, h1);
+                if (p < 2) {
+                    r0 = ptx::sub2(r0, ptx::f32x2(__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xffff0000u)));
+                    r1 = ptx::sub2(r1, ptx::f32x2(__uint_as_float(h1 << 16), __uint_as_float(h1 & 0xffff0000u)));
+                }
+            }
+            odd = ptx::fma2(r0, 0ull, odd);
+            odd = ptx::fma2(r1, 0ull, odd);
+        };
+        auto note_odd = [&](const uint8_t* src) {
+            auto is_odd = [](float v) { return !(fabsf(v) < 3.38e38f); };       // (3.3895e38 is bf16's largest)
+            auto any_odd = [&](const float4 v) { return is_odd(v.x) || is_odd(v.y) || is_odd(v.z) || is_odd(v.w); };
+            for (int i = 0; i < C::kAPieces; ++i)
+                if (any_odd(*reinterpret_cast<const float4*>(src + i * kSplitThreads * 16))) { row_bad[a_row + 32 * i] = 1; *any_bad = 1; }
+            for (int i = 0; i < C::kBPieces; ++i)
+                if (any_odd(*reinterpret_cast<const float4*>(src + (C::kAPieces + i) * kSplitThreads * 16)))
+                    for (uint32_t r = 0; r < 2; ++r) {       // both CTAs have these columns
+                        ptx::st_cluster_u8(ptx::map_to_cta(ptx::smem_addr(col_bad + rank * (C::kCols / 4) + (i >> 1) * 16 + b_vec), r), 1);
+                        ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_addr(any_bad), r), 1);
+                    }
+        };
+        // where the pieces go: A rows of 64 bytes (64-byte swizzle), weights [64 columns][k][128 bytes] (128-byte swizzle); rows 32 i
+        // and k 16 i apart have the same swizzle
+        const uint32_t a_dst = a_row * 64 + ((((tid & 7) >> 1) ^ ((a_row >> 1) & 3)) << 4) + 8 * (tid & 1);
+        const uint32_t b_dst = 3 * kAPlane + b_k * 128 + (((b_vec >> 1) ^ (b_k & 7)) << 4) + 8 * (b_vec & 1);
+        const uint32_t full_leader = ptx::map_to_cta(ptx::smem_addr(full_bar), 0);
+        // (a wait that has given up makes every later one return at once: the loops run to their end on meaningless data)
+        int s = 0, r = 0;
+        uint32_t ph = 1, raw_ph = 0;
+        for (int it = 0; it < n_it; ++it) {
+            ptx::mbar_wait(&raw_full[r], raw_ph, abort_flag);
+            ptx::mbar_wait(&empty_bar[s], ph, abort_flag);
+            __syncwarp();
+            const uint8_t* src = raw + r * C::kRawBytes + tid * 16;
+            uint8_t* st = smem + s * C::kStageBytes;
+            // (four loads ahead of the stores, which the compiler cannot move them across)
+            ulonglong2 v[4];
+            constexpr int kPieces = C::kAPieces + C::kBPieces;
+#pragma unroll
+            for (int i0 = 0; i0 < kPieces; i0 += 4) {
+#pragma unroll
+                for (int i = i0; i < i0 + 4 && i < kPieces; ++i) v[i & 3] = *reinterpret_cast<const ulonglong2*>(src + i * kSplitThreads * 16);
+#pragma unroll
+                for (int i = i0; i < i0 + 4 && i < kPieces; ++i)
+                    if (i < C::kAPieces) split(v[i & 3], st + a_dst + i * 32 * 64, kAPlane);
+                    else split(v[i & 3], st + b_dst + (i - C::kAPieces) * 16 * 128, C::kBPlane);
+            }
+            if (!(odd == 0ull || odd == 0x8000000000000000ull || odd == 0x80000000ull || odd == 0x8000000080000000ull)) {
+                note_odd(src);
+                odd = 0ull;
+            }
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                ptx::mbar_arrive_cluster(full_leader + 8 * s);
+                ptx::mbar_arrive(&raw_empty[r]);
+            }
+            s = s + 1 == C::kStages ? 0 : s + 1;
+            ph ^= s == 0;
+            r = r + 1 == C::kRaw ? 0 : r + 1;
+            raw_ph ^= r == 0;
+        }
+        // the gates, in place, while the last decoded values are summed up (the adding warps, with their registers full, would take
+        // 5 us more for a pair's 65536)
+        ptx::named_sync(1, kBoth);
+        ptx::tc_fence_after_sync();
+        const uint32_t z_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + ((n_g - 1) & 1) * NT + ((warp - kSplitWarp0) >> 2) * C::kCols;
+#pragma unroll 1
+        for (int ch = 0; ch < C::kCols / 16; ++ch) {
+            uint32_t z[16];
+            ptx::tmem_ld16(z_tmem + ch * 16, z);
+            ptx::tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) z[e] = __float_as_uint(sigmoid(__uint_as_float(z[e])));
+            ptx::tmem_st16(z_tmem + ch * 16, z);
+        }
+        ptx::tmem_wait_st();
+        ptx::tc_fence_before_sync();
+        ptx::named_arrive(2, kBoth);
+    } else {
+        ptx::set_max_regs_inc<kAddRegs>();
+        const Block w = block_of<NT>(d, row_tiles, col_tiles, blockIdx.x);
+        const int quarter = warp & 3, half = (warp - kAddWarp0) >> 2;    // TMEM lanes, columns
+        const uint32_t d_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * C::kCols;
+        const uint32_t free_leader = ptx::map_to_cta(ptx::smem_addr(acc_free), 0);
+        uint64_t acc[C::kCols / 2];
+#pragma unroll
+        for (int e = 0; e < C::kCols / 2; ++e) acc[e] = 0ull;
+        for (int it = 0; it < n_it; ++it) {
+            const int buf = buf_of(it);
+            ptx::mbar_wait(&acc_full[buf], use_of(it) & 1, abort_flag);
+            __syncwarp();
+            ptx::tc_fence_after_sync();
+#pragma unroll
+            for (int ch = 0; ch < C::kCols / 16; ++ch) {
+                uint32_t v[16];
+                ptx::tmem_ld16(d_tmem + buf * NT + ch * 16, v);
+                ptx::tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    acc[ch * 8 + e] = ptx::add2(acc[ch * 8 + e], ptx::f32x2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])));
+            }
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_cluster(free_leader + 8 * buf);
+            if (it == n_g - 1) {                // the gates' sums are complete: the splitting warps make gates of them
+#pragma unroll
+                for (int ch = 0; ch < C::kCols / 16; ++ch) {
+                    uint32_t v[16];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        float z0, z1;
+                        ptx::f32x2_split(acc[ch * 8 + e], z0, z1);
+                        acc[ch * 8 + e] = 0ull;
+                        v[2 * e] = __float_as_uint(z0);
+                        v[2 * e + 1] = __float_as_uint(z1);
+                    }
+                    ptx::tmem_st16(d_tmem + buf * NT + ch * 16, v);
+                }
+                ptx::tmem_wait_st();
+                ptx::tc_fence_before_sync();
+                ptx::named_arrive(1, kBoth);
+            }
+        }
+        ptx::named_sync(2, kBoth);               // the gates are there
+        ptx::tc_fence_after_sync();
+        // out = decoded value x gate: 32 rows x 32 columns at a time through the ring's memory, which nothing uses any more (rows
+        // of 128 bytes, 128-byte swizzle), and out by TMA: whole lines, and rows past the last are not written
+        const int g_buf = (n_g - 1) & 1;
+        uint8_t* stage = smem + (warp - kAddWarp0) * (C::kCols * 32 * 4);
+#pragma unroll
+        for (int ch = 0; ch < C::kCols / 16; ++ch) {
+            uint32_t z[16];
+            ptx::tmem_ld16(d_tmem + g_buf * NT + ch * 16, z);
+            ptx::tmem_wait_ld();
+            uint8_t* box = stage + (ch >> 1) * 4096 + lane * 128;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                float y[4];
+                ptx::f32x2_split(acc[ch * 8 + 2 * h], y[0], y[1]);
+                ptx::f32x2_split(acc[ch * 8 + 2 * h + 1], y[2], y[3]);
+                *reinterpret_cast<float4*>(box + (((4 * (ch & 1) + h) ^ (lane & 7)) << 4)) =
+                    make_float4(y[0] * __uint_as_float(z[4 * h]), y[1] * __uint_as_float(z[4 * h + 1]),
+                                y[2] * __uint_as_float(z[4 * h + 2]), y[3] * __uint_as_float(z[4 * h + 3]));
+            }
+            if (ch & 1) {
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                const int c = half * C::kCols + 16 * (ch - 1);         // (a map's columns are a multiple of 64)
+                if (lane == 0 && c < w.n_cols && quarter * 32 < w.rows) {
+                    ptx::tma_store_2d(&tm_out, stage + (ch >> 1) * 4096, w.g * w.map_cols + w.n0 + c, (int)w.m0 + quarter * 32);
+                    ptx::bulk_commit_group();
+                }
+            }
+        }
+        ptx::bulk_wait_group_all();        // (rows done again below come after this; and the memory may go)
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::cluster_arrive();         // neither CTA leaves (or frees tensor memory) while the other may still signal it
+    ptx::cluster_wait();
+    if (warp == 0) ptx::tmem_dealloc_pair(tmem_base, 2 * NT);
+    if (warp >= kAddWarp0 && *any_bad) {
+        uint32_t block;             // (worked out anew: nothing of this is kept in registers until here)
+        asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
+        redo<NT>(d, o_lat, x, w_p, w_g, out, row_tiles, col_tiles, block, row_bad, col_bad);
+    }
+    if (threadIdx.x == 0 && *abort_flag) raise_status(status_word, GTA_ERR_TIMEOUT);
+}
+
+template <int NT>
+cudaError_t launch_tile(const Dims& d, const float* o_lat, const float* x, const float* w_p, const float* w_g, float* out,
+                        int32_t* status_word, cudaStream_t stream, bool behind) {
+    auto kern = sm100_decoder_f32_kernel<NT>;
+    const uint64_t M = (uint64_t)d.B * d.N, n_out = (uint64_t)d.n_h * d.d_h;
+    CUtensorMap tm_l, tm_x, tm_wp, tm_wg, tm_out;
+    {
+        const uint64_t dl[3] = {(uint64_t)d.d_l, M, (uint64_t)d.n_q}, dx[2] = {(uint64_t)d.H, M};
+        const uint64_t dp[3] = {(uint64_t)d.d_h, (uint64_t)d.d_l, (uint64_t)d.n_h}, dg[2] = {n_out, (uint64_t)d.H};
+        const uint64_t dout[2] = {n_out, M};
+        const uint32_t rows[3] = {kBlockK, kTileM, 1}, cols[3] = {64, kBlockK, 1}, box[2] = {32, 32};
+        if (!make_f32_map(&tm_l, o_lat, 3, dl, rows) || !make_f32_map(&tm_x, x, 2, dx, rows) ||
+            !make_f32_map(&tm_wp, w_p, 3, dp, cols) || !make_f32_map(&tm_wg, w_g, 2, dg, cols) ||
+            !make_f32_map(&tm_out, out, 2, dout, box, true))
+            return cudaErrorInvalidValue;
+    }
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<NT>::kSmem);
+    if (err != cudaSuccess) return err;
+    const int row_tiles = (int)((M + 2 * kTileM - 1) / (2 * kTileM));
+    const int col_tiles = (d.n_h / d.n_q * d.d_h + NT - 1) / NT;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2u * row_tiles * col_tiles * d.n_q);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Cfg<NT>::kSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = behind ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, tm_l, tm_x, tm_wp, tm_wg, tm_out, d, o_lat, x, w_p, w_g, out, row_tiles, col_tiles,
+                              status_word);
+}
+
+}  // namespace
+
+long long sm100_decoder_f32_units(const Dims& d, int nt) {
+    return (((long long)d.B * d.N + 2 * kTileM - 1) / (2 * kTileM)) * ((d.n_h / d.n_q * d.d_h + nt - 1) / nt) * d.n_q;
+}
+
+cudaError_t launch_sm100_decoder_f32(const Dims& d, const float* o_lat, const float* x, const float* w_p, const float* w_g,
+                                     float* out, int32_t* status_word, cudaStream_t stream, bool behind, int nt) {
+    if (nt == 256) return launch_tile<256>(d, o_lat, x, w_p, w_g, out, status_word, stream, behind);
+    return launch_tile<128>(d, o_lat, x, w_p, w_g, out, status_word, stream, behind);
+}
+
+}  // namespace gta

@@ -1,0 +1,119 @@
+"""fp32 prefill on the tensor cores (three bf16 pieces per operand): tile edges, remainders and splits against torch in 64 bits,
+the plain-ALU attention (a smallest workspace selects it) on elements that the pieces cannot hold, guard bands."""
+import numpy as np
+import pytest
+import torch
+
+from tests.parity_utils import Guarded
+
+pytestmark = pytest.mark.gpu
+
+# Pieces are exact and the products left out below 2^-25 of a product; a sum of 64 products is cut at 2^-23 of its value up to
+# eight times, sums are rounded to 2^-24 from there, an exponential is good to 2 ulp: 2.1e-7 measured (3.9e-7 the FMA chain).
+REL, MAX = 8e-7, 4e-5
+
+
+@pytest.fixture(scope="module")
+def G():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2506_17286_b200 import build, binding
+    build.build()
+    binding.lib()
+    return binding
+
+
+def _inputs(B, N, cap, H, n_h, n_q, n_k, n_c, d_h, d_l, seed=0):
+    gen = torch.Generator("cuda").manual_seed(seed)
+
+    def r(*s, std=1.0):
+        return torch.randn(s, generator=gen, device="cuda") * std
+    return dict(q=r(B, n_q, N, d_h), k=r(B, n_k, cap, d_h), c=r(B, n_c, cap, d_l), x=r(B, N, H),
+                w_p=r(n_h, d_l, d_h, std=d_l ** -0.5), w_g=r(H, n_h * d_h, std=H ** -0.5))
+
+
+def _exact(t, kv, causal):
+    q, k, c, x, w_p, w_g = (t[n].double() for n in ("q", "k", "c", "x", "w_p", "w_g"))
+    B, n_q, N, d_h = q.shape
+    k, c, n_h = k[:, :, :kv], c[:, :, :kv], w_p.shape[0]
+    s = torch.einsum("bgtd,bgsd->bgts", q, k.repeat_interleave(n_q // k.shape[1], 1)) * d_h ** -0.5
+    if causal:
+        s = s.masked_fill(torch.ones(N, kv, device="cuda", dtype=torch.bool).triu(kv - N + 1), -float("inf"))
+    lat = torch.einsum("bgts,bgsl->bgtl", s.softmax(-1), c.repeat_interleave(n_q // c.shape[1], 1))
+    y = torch.einsum("bhtl,hld->bthd", lat.repeat_interleave(n_h // n_q, 1), w_p)
+    return y * torch.sigmoid(x @ w_g).reshape(B, N, n_h, -1)
+
+
+def _run(G, t, kv, causal, least=False):
+    B, n_q, N, d_h = t["q"].shape
+    n_h, d_l = t["w_p"].shape[:2]
+    shape = G.make_shape(batch=B, seq=N, d_model=t["x"].shape[2], n_heads=n_h, n_q=n_q, n_k=t["k"].shape[1],
+                         n_c=t["c"].shape[1], d_h=d_h, d_l=d_l, dtype=torch.float32)
+    plain = (4 * B * n_q * N * d_l + 255) // 256 * 256
+    # (behind longer keys the pieces need more than the query of the chunk's shape says)
+    room = plain if least else max(G.prefill_workspace_bytes(shape), plain + 12 * B * kv * (n_q * d_h + n_q * d_l) + 65536)
+    ws, out = Guarded((room,), torch.uint8), Guarded((B, N, n_h, d_h), torch.float32)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    G.gta_prefill_chunk(t["q"], t["k"], t["c"], t["x"], t["w_p"], t["w_g"], kv, causal=causal, workspace=ws.t, out=out.t,
+                        status_word=status)
+    torch.cuda.synchronize()
+    ws.check("workspace"); out.check("out")
+    assert int(status.item()) == 0
+    return out.t
+
+
+CASES = [  # B, N, kv, cap, H, n_h, n_q, n_k, n_c, d_h, d_l, causal
+    (1, 192, 192, 192, 1280, 20, 5, 1, 1, 64, 128, True),       # plain decoder behind the tensor-core attention
+    (2, 257, 257, 257, 200, 20, 5, 1, 1, 64, 128, True),        # a row past two row tiles; H not a multiple of 32; four CTAs a tile
+    (1, 1000, 1000, 1000, 64, 16, 4, 2, 2, 64, 256, True),      # two latent groups, two slices; one key tile of 40 rows at the end
+    (3, 1025, 1025, 1025, 96, 10, 5, 1, 1, 64, 128, True),      # a row past a pair's tile; 128 columns a map; 256 | 3075 does not hold
+    (2, 1500, 1500, 1500, 1280, 20, 5, 1, 1, 64, 128, True),    # 256-column blocks, two CTAs a row tile
+    (2, 700, 700, 700, 72, 18, 6, 3, 1, 64, 128, True),         # 192 columns a map: the second block is half empty
+    (1, 300, 300, 320, 256, 20, 5, 1, 1, 64, 384, False),       # not causal, three slices, rows behind the keys in the cache
+    (2, 130, 777, 800, 256, 20, 5, 1, 1, 64, 128, True),        # a chunk behind a longer cache
+    (1, 5, 300, 300, 64, 2, 2, 1, 1, 64, 128, True),            # fewer rows than a warp
+    (5, 333, 333, 333, 64, 8, 4, 4, 1, 128, 72, True),          # plain attention in front of the tensor-core decoder; d_l = 72
+    (9, 1024, 1024, 1024, 32, 4, 2, 2, 1, 64, 128, True),       # more than one wave, one CTA a row tile
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=[f"B{c[0]}_N{c[1]}_kv{c[2]}_H{c[4]}_dh{c[9]}_dl{c[10]}" for c in CASES])
+def test_against_64_bits(G, case):
+    B, N, kv, cap, H, n_h, n_q, n_k, n_c, d_h, d_l, causal = case
+    t = _inputs(B, N, cap, H, n_h, n_q, n_k, n_c, d_h, d_l)
+    t["k"][:, :, kv:], t["c"][:, :, kv:] = float("nan"), float("inf")
+    got, want = _run(G, t, kv, causal).double(), _exact(t, kv, causal)
+    err = got - want
+    rms = want.pow(2).mean().sqrt()
+    assert torch.isfinite(got).all()
+    assert float(err.norm() / want.norm()) <= REL and float((err.abs() / torch.maximum(want.abs(), rms)).max()) <= MAX
+
+
+@pytest.mark.parametrize("size", [1e-30, 1e15])
+def test_range_of_the_pieces(G, size):
+    """Latents and decoder weights near both ends of the range: the pieces have fp32's exponents."""
+    t = _inputs(1, 300, 300, 64, 20, 5, 1, 1, 64, 128)
+    t["c"] *= size
+    t["w_p"] *= size if size > 1 else 1e3
+    got, want = _run(G, t, 300, True).double(), _exact(t, 300, True)
+    assert float((got - want).norm() / want.norm()) <= REL
+
+
+BAD = [("q", (0, 1, 40, 3), float("nan")), ("q", (0, 0, 299, 0), float("inf")), ("k", (0, 0, 130, 5), float("inf")),
+       ("k", (0, 0, 299, 63), float("nan")), ("c", (0, 0, 70, 127), float("nan")), ("c", (0, 0, 290, 1), -float("inf")),
+       ("c", (0, 0, 5, 1), 3.4e38), ("x", (0, 17, 9), float("inf")), ("x", (0, 299, 63), float("nan")),
+       ("w_g", (3, 700), -float("inf")), ("w_p", (7, 11, 2), float("nan")), ("x", (0, 30, 0), 3.4e38)]
+
+
+@pytest.mark.parametrize("what,where,value", BAD, ids=[f"{w}_{v}_{p[-2]}" for w, p, v in BAD])
+def test_elements_that_the_pieces_cannot_hold(G, what, where, value):
+    """They reach the rows and columns that see them, and no others."""
+    t = _inputs(1, 300, 300, 64, 20, 5, 1, 1, 64, 128)
+    t[what][where] = value
+    got, plain, want = _run(G, t, 300, True), _run(G, t, 300, True, least=True), _exact(t, 300, True)
+    if what in ("q", "k", "c"):         # the plain-ALU attention, whose masked rows do not see the element
+        assert torch.equal(torch.isnan(got), torch.isnan(plain)) and torch.equal(torch.isinf(got), torch.isinf(plain))
+        ok = torch.isfinite(got)
+        assert float((got - plain)[ok].double().norm() / plain[ok].double().norm()) <= 2 * REL
+    else:
+        torch.testing.assert_close(got, want.float(), rtol=1e-4, atol=1e-5, equal_nan=True)
