@@ -759,11 +759,8 @@ extern "C" gta_status_t gta_decode_append(const gta_shape_t* shape, const void* 
         err = gta::launch_decode_fast(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace, status_word,
                                       stream, 7, &launches, gta::PageMap(), k_new, c_new);
     } else {
-        err = gta::launch_cache_append(d, (int)elem_size(shape->dtype), k_cache, c_cache, S_cap, k_new, c_new, 1, seq_lens,
-                                       status_word, stream, &launches);
-        if (err == cudaSuccess)
-            err = gta::launch_decode(d, shape->dtype, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
-                                     workspace_bytes, status_word, stream, 7, &launches);
+        err = gta::launch_decode_plain_append(d, shape->dtype, q, k_cache, c_cache, k_new, c_new, seq_lens, S_cap, x_t, w_p, w_g,
+                                              out, workspace, workspace_bytes, status_word, stream, &launches);
     }
     if (err != cudaSuccess) return GTA_ERR_CUDA;
     g_last_launches = launches;

@@ -21,7 +21,6 @@ namespace gta {
 constexpr int kDecodeThreads = 256;
 constexpr int kFinishSeqs = 8;      // sequences per finish CTA
 constexpr int kFinishCols = 16;     // output columns per finish CTA
-constexpr int kFinishSlab = 2048;   // elements of the contraction staged in shared memory at a time
 
 struct DecodePlan {
     int chunk;       // tokens per partial CTA
@@ -156,6 +155,12 @@ static size_t partial_smem(const Dims& d, int chunk, int cm, int vec) {
     return ((size_t)d.n_q * d.d_h + (size_t)((chunk * d.n_q + 3) & ~3) + (size_t)cm * R * d.d_l) * sizeof(float);
 }
 
+// Tokens of a sequence that a step attends over: those of the cache, and the new one where the step appends it and it fits.
+__device__ __forceinline__ int step_len(int len, int S_cap, bool append) {
+    if (append && len >= 0 && len < S_cap) return len + 1;
+    return len < 0 ? 0 : (len > S_cap ? S_cap : len);
+}
+
 // CT: storage type of the caches (T, or Fp8 with one fp32 scale per cached row in k_scale / c_scale).  CM: maps of a
 // latent group that a pass over its rows serves (the last pass may have fewer).
 // Every key row is loaded once, whatever the number of maps of its group, and a latent row once per CM maps: the caches
@@ -170,18 +175,21 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
                       const CT* __restrict__ k_cache, const CT* __restrict__ c_cache,
                       const int32_t* __restrict__ seq_lens, float* __restrict__ part_o,
                       float* __restrict__ part_ml, PageMap pm, int32_t* status_word,
-                      const float* __restrict__ k_scale, const float* __restrict__ c_scale) {
+                      const float* __restrict__ k_scale, const float* __restrict__ c_scale,
+                      const CT* __restrict__ k_new, const CT* __restrict__ c_new) {
     constexpr int VEC = Vec16<CT>::N, CV = LatentVec<CT>::N;
     constexpr bool kScaled = !std::is_same<CT, T>::value;
     using Raw = typename LatentVec<CT>::Raw;
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     const int b = blockIdx.y, ck = blockIdx.x;
-    int len = seq_lens[b];
-    len = len < 0 ? 0 : (len > S_cap ? S_cap : len);
+    const int old = seq_lens[b], len = step_len(old, S_cap, k_new != nullptr);
     const int j_begin = ck * chunk;
+    if (k_new != nullptr && ck == 0 && threadIdx.x == 0 && (old < 0 || old >= S_cap)) raise_status(status_word, GTA_ERR_CACHE_FULL);
     if (j_begin >= len) return;
     const int n_tok = min(chunk, len - j_begin);
+    // the new token of a fused step: attended from where the caller has it, put into the caches by the CTA of its chunk
+    const int j_new = k_new != nullptr && len == old + 1 ? old - j_begin : -1;
 
     extern __shared__ __align__(16) float smem[];
     float* q_s = smem;
@@ -197,6 +205,13 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
         return (size_t)(i < 0 ? 0 : i);
     };
 
+    auto key_row = [&](int kg, int j) {
+        return j == j_new ? k_new + ((size_t)b * d.n_k + kg) * d.d_h : k_cache + row_of(d.n_k, kg, j) * d.d_h;
+    };
+    auto latent_row = [&](int cg, int j) {
+        return j == j_new ? c_new + ((size_t)b * d.n_c + cg) * d.d_l : c_cache + row_of(d.n_c, cg, j) * d.d_l;
+    };
+
     // ---- latent rows: tpr threads per row, R rows of the CTA at once, U of them per thread in flight
     constexpr int U = 8;
     const int tpr = d.d_l / CV, R = kDecodeThreads / tpr;
@@ -209,9 +224,8 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
         for (int u = 0; u < U; ++u) {
             const int j = j0 + r + u * R;
             if (active && j < n_tok) {
-                const size_t idx = row_of(d.n_c, cg, j);
-                raw[u] = __ldg(reinterpret_cast<const Raw*>(c_cache + idx * d.d_l + v * CV));
-                cs[u] = kScaled ? c_scale[idx] : 1.f;
+                raw[u] = __ldg(reinterpret_cast<const Raw*>(latent_row(cg, j) + v * CV));
+                cs[u] = kScaled ? c_scale[row_of(d.n_c, cg, j)] : 1.f;
             }
         }
     };
@@ -242,12 +256,12 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
 #pragma unroll
                     for (int s = 0; s < kSlots; ++s) kraw[u][s] = make_uint4(0u, 0u, 0u, 0u);
                     if (j < n_tok) {
-                        const size_t idx = row_of(d.n_k, kg, j);
-                        if (kScaled) row_scale[u] *= k_scale[idx];
+                        const CT* row = key_row(kg, j);
+                        if (kScaled) row_scale[u] *= k_scale[row_of(d.n_k, kg, j)];
 #pragma unroll
                         for (int s = 0; s < kSlots; ++s)
                             if (sl + s * lpr < vecs_per_row)
-                                kraw[u][s] = __ldg(reinterpret_cast<const uint4*>(k_cache + idx * d.d_h + (sl + s * lpr) * VEC));
+                                kraw[u][s] = __ldg(reinterpret_cast<const uint4*>(row + (sl + s * lpr) * VEC));
                     }
                 }
 #pragma unroll 1
@@ -364,6 +378,18 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
             }
         }
     }
+    if (j_new >= 0 && j_new < n_tok) {
+        const auto put = [&](const CT* src, CT* cache, int groups, int width) {
+            const int vecs = width / VEC;
+            for (int i = tid; i < groups * vecs; i += kDecodeThreads) {
+                const int grp = i / vecs, e = (i - grp * vecs) * VEC;
+                *reinterpret_cast<uint4*>(cache + row_of(groups, grp, j_new) * width + e) =
+                    __ldg(reinterpret_cast<const uint4*>(src + ((size_t)b * groups + grp) * width + e));
+            }
+        };
+        put(k_new, const_cast<CT*>(k_cache), d.n_k, d.d_h);
+        put(c_new, const_cast<CT*>(c_cache), d.n_c, d.d_l);
+    }
 }
 
 // Log-sum-exp merge of the chunk partials of one (map, sequence), in place: the normalised latent L takes the room of the
@@ -373,15 +399,14 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
 // shared memory: a chain of rounds of loads over all chunks would be what the kernel waits for.
 __global__ void __launch_bounds__(kDecodeThreads)
 decode_chunk_merge_kernel(Dims d, int chunk, int n_chunks, int S_cap, const int32_t* __restrict__ seq_lens,
-                          float* part_o, float* part_ml) {
+                          float* part_o, float* part_ml, bool append) {
     __shared__ float4 acc_s[kDecodeThreads];
     __shared__ float2 ml_s[kDecodeThreads];
     ptx::grid_launch_dependents();
     const int g = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
     const int width = min(d.d_l >> 2, kDecodeThreads), groups = kDecodeThreads / width;
     const int grp = tid / width, v = tid - grp * width;
-    int len = seq_lens[b];       // (older than the partial kernel, which was released after its own wait; see the launch)
-    len = len < 0 ? 0 : (len > S_cap ? S_cap : len);
+    const int len = step_len(seq_lens[b], S_cap, append);  // (older than the partial kernel, which was released after its own wait)
     const int live = (len + chunk - 1) / chunk;
     ptx::grid_dependency_wait();
     float2* ml = reinterpret_cast<float2*>(part_ml) + (size_t)b * n_chunks * d.n_q + g;
@@ -448,67 +473,51 @@ decode_chunk_merge_kernel(Dims d, int chunk, int n_chunks, int S_cap, const int3
 
 // Four neighbouring elements as floats.
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float4 ldg4(const __nv_bfloat16* p) {
-    const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+__device__ __forceinline__ float4 widen4(const uint2 r) {
     return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
                        __uint_as_float(r.y & 0xffff0000u));
 }
+__device__ __forceinline__ float4 ldg4(const __nv_bfloat16* p) { return widen4(__ldg(reinterpret_cast<const uint2*>(p))); }
 
-// acc[row][column] += sum over this thread's k of src[row][k] w[k][4 columns], k = tid / 4 + 64 i.  The rows of a slab lie
-// in shared memory four by four ([2][slab][4]), so that the eight k of a warp are 128 contiguous bytes.
-// kBehind: src is the kernel ahead's result; the first weights are fetched before the dependency wait.
-template <bool kBehind, typename TA, typename TW>
-__device__ __forceinline__ void finish_contract(const TA* src, size_t stride, int rows, int K, const TW* __restrict__ w,
-                                                size_t ldw, bool live, float* xs, float (&acc)[8][4]) {
-    const int tid = threadIdx.x, ks = tid >> 2;
-    constexpr int U = 8;
-    for (int k0 = 0; k0 < K; k0 += kFinishSlab) {
-        const int n = min(kFinishSlab, K - k0);
-        float4 wv[U], wn[U];
-        auto fetch = [&](float4 (&dst)[U], int kb) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int k = kb + ks + 64 * u;
-                dst[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (live && k < n) dst[u] = ldg4(w + (size_t)(k0 + k) * ldw);
-            }
-        };
-        fetch(wv, 0);
-        if (kBehind) ptx::grid_dependency_wait();
-        __syncthreads();                                     // the slab before has been read
-        for (int idx = tid; idx < 2 * n; idx += kDecodeThreads) {
-            const int r = idx & 7, k = (idx >> 3) * 4;
-            if (r < rows) {
-                float4 x;
-                if constexpr (kBehind) x = *reinterpret_cast<const float4*>(src + (size_t)r * stride + k0 + k);
-                else x = ldg4(src + (size_t)r * stride + k0 + k);
-                float* dst = xs + ((r >> 2) * kFinishSlab + k) * 4 + (r & 3);
-                dst[0] = x.x; dst[4] = x.y; dst[8] = x.z; dst[12] = x.w;
-            }
-        }
-        __syncthreads();
-        for (int kb = 0; kb < n; kb += 64 * U) {
-            if (kb + 64 * U < n) fetch(wn, kb + 64 * U);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int k = kb + ks + 64 * u;
-                if (k < n) {
-                    const float4 a = *reinterpret_cast<const float4*>(xs + k * 4);
-                    const float4 c = *reinterpret_cast<const float4*>(xs + (kFinishSlab + k) * 4);
-                    const float xr[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        acc[i][0] = fmaf(xr[i], wv[u].x, acc[i][0]);
-                        acc[i][1] = fmaf(xr[i], wv[u].y, acc[i][1]);
-                        acc[i][2] = fmaf(xr[i], wv[u].z, acc[i][2]);
-                        acc[i][3] = fmaf(xr[i], wv[u].w, acc[i][3]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) wv[u] = wn[u];
-        }
+// Four neighbouring weights as they are stored, on their way to shared memory by cp.async and from there.
+template <typename T> struct Weights4;
+template <> struct Weights4<float> {
+    using Raw = float4;
+    static __device__ __forceinline__ void copy(Raw* dst, const float* src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ptx::smem_addr(dst)), "l"(src) : "memory");
     }
+    static __device__ __forceinline__ float4 widen(const Raw& r) { return r; }
+};
+template <> struct Weights4<__nv_bfloat16> {
+    using Raw = uint2;
+    static __device__ __forceinline__ void copy(Raw* dst, const __nv_bfloat16* src) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ptx::smem_addr(dst)), "l"(src) : "memory");
+    }
+    static __device__ __forceinline__ float4 widen(const Raw& r) { return widen4(r); }
+};
+
+// The finish kernel's contractions in slabs of at most `size` elements: those of X W_G, then those of L W_P.  The weights
+// of a slab and of the one behind it are on their way at once: buffers of even and odd slabs in turn, every thread the
+// pieces that it uses itself.  1280 elements where every CTA has an SM to itself, 640, which leaves room for two, otherwise
+// (the whole fp32 step of the 1B layer, us, 1280 / 640: four sequences of about 1100 tokens 17.0 / 18.4, 32 of 256 35.3 / 30.3).
+struct FinishSlabs {
+    int size;                      // a multiple of 64
+    int gate, all;                 // slabs of the gate; of both
+    int even_pieces, odd_pieces;   // of a thread, in the two buffers
+};
+static FinishSlabs finish_slabs(const Dims& d, long long ctas) {
+    FinishSlabs f;
+    f.size = ctas <= 148 ? 1280 : 640;
+    f.gate = (d.H + f.size - 1) / f.size;
+    f.all = f.gate + (d.d_l + f.size - 1) / f.size;
+    f.even_pieces = f.odd_pieces = 0;
+    for (int i = 0; i < f.all; ++i) {
+        const int left = i < f.gate ? d.H - i * f.size : d.d_l - (i - f.gate) * f.size;
+        const int pieces = ((left < f.size ? left : f.size) + 63) / 64;
+        int& most = i & 1 ? f.odd_pieces : f.even_pieces;
+        if (pieces > most) most = pieces;
+    }
+    return f;
 }
 // Adds acc up over the 64 k-slices of the CTA; the sum of (row, column) ends in thread row 16 + column (tid < 128).
 __device__ __forceinline__ float finish_reduce(float (&acc)[8][4], float* red) {
@@ -541,31 +550,102 @@ __device__ __forceinline__ float finish_reduce(float (&acc)[8][4], float* red) {
 // Gate, decoder and store of 8 sequences x 16 columns of one head.  The gate's half needs only x_t and W_G and runs
 // before the dependency wait, under the kernels ahead; after it come one pass over W_P's columns and the store.
 // Narrow tiles, because at small batches the weights' way through few SMs sets the time (1280 columns: 80 CTAs; the
-// former pair of kernels, a head and a 128-column block per CTA, took 18.6 + 19.6 us for four fp32 sequences; 9.9 now, most of it under the kernels ahead).
-// Dynamic shared memory (floats): xs [2][kFinishSlab][4] | red [2][8 warps][8][16]
+// former pair of kernels, a head and a 128-column block per CTA, took 18.6 + 19.6 us for four fp32 sequences), and all of a
+// CTA's weights asked for at once (four fp32 sequences of about 1100 tokens, the whole step: 17.0 us; with eight
+// pieces a thread in registers 20.5).
+// Dynamic shared memory: weights [even pieces][256], [odd pieces][256] | xs [2][slab][4] | red [2][8 warps][8][16]
 template <typename T>
 __global__ void __launch_bounds__(kDecodeThreads)
-decode_finish_kernel(Dims d, int tiles_per_head, const T* __restrict__ x_t, const float* l_in, size_t seq_stride,
-                     const T* __restrict__ w_p, const T* __restrict__ w_g, T* __restrict__ out) {
+decode_finish_kernel(Dims d, int tiles_per_head, FinishSlabs slabs, const T* __restrict__ x_t, const float* l_in, size_t seq_stride,
+                     const T* __restrict__ w_p, const T* __restrict__ w_g, T* __restrict__ out, int32_t* step_lens, int S_cap) {
+    using W = Weights4<T>;
     extern __shared__ __align__(16) float smem[];
-    float* xs = smem;
-    float* red = xs + 2 * kFinishSlab * 4;
+    typename W::Raw* w_s = reinterpret_cast<typename W::Raw*>(smem);
+    float* xs = reinterpret_cast<float*>(w_s + (slabs.even_pieces + slabs.odd_pieces) * kDecodeThreads);
+    float* red = xs + 2 * slabs.size * 4;
     ptx::grid_launch_dependents();
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, ks = tid >> 2;
     const int i = blockIdx.x / tiles_per_head, e0 = (blockIdx.x % tiles_per_head) * kFinishCols, b0 = blockIdx.y * kFinishSeqs;
     const int nb = min(kFinishSeqs, d.B - b0), col = e0 + 4 * (tid & 3);
     const bool live = col < d.d_h;                          // (d_h is a multiple of 8)
-    float acc[8][4];
+    const T* wg_col = w_g + (size_t)i * d.d_h + col;
+    const T* wp_col = w_p + (size_t)i * d.d_l * d.d_h + col;
+    const size_t ldw_g = (size_t)d.n_h * d.d_h;
+
+    // this thread's weights of a slab: k = ks + 64 u
+    const auto fetch = [&](int s) {
+        if (s < slabs.all && live) {
+            const bool gate = s < slabs.gate;
+            const int k0 = (gate ? s : s - slabs.gate) * slabs.size, n = min(slabs.size, (gate ? d.H : d.d_l) - k0);
+            const T* src = (gate ? wg_col : wp_col) + (size_t)(k0 + ks) * (gate ? ldw_g : (size_t)d.d_h);
+            typename W::Raw* dst = w_s + (s & 1 ? slabs.even_pieces * kDecodeThreads : 0) + tid;
+            for (int k = ks; k < n; k += 64, src += 64 * (gate ? ldw_g : (size_t)d.d_h), dst += kDecodeThreads) W::copy(dst, src);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(0);
+    fetch(1);
+
+    float acc[8][4], z = 0.f;
 #pragma unroll
     for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
-    finish_contract<false, T, T>(x_t + (size_t)b0 * d.H, d.H, nb, d.H, w_g + (size_t)i * d.d_h + col, (size_t)d.n_h * d.d_h,
-                                 live, xs, acc);
-    const float z = finish_reduce(acc, red);
+    for (int s = 0; s < slabs.all; ++s) {
+        const bool gate = s < slabs.gate;
+        if (s == slabs.gate) {
+            z = finish_reduce(acc, red);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
-    finish_contract<true, float, T>(l_in + (size_t)b0 * seq_stride + (size_t)d.head_to_q(i) * d.d_l, seq_stride, nb, d.d_l,
-                                    w_p + (size_t)i * d.d_l * d.d_h + col, d.d_h, live, xs, acc);
+            for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
+            ptx::grid_dependency_wait();
+        }
+        const int k0 = (gate ? s : s - slabs.gate) * slabs.size, n = min(slabs.size, (gate ? d.H : d.d_l) - k0);
+        if (s > 0) __syncthreads();                          // the slab before has been read
+        // its rows lie in shared memory four by four ([2][slab][4]), so that the eight k of a warp are 128 contiguous bytes
+        for (int idx = tid; idx < 2 * n; idx += kDecodeThreads) {
+            const int r = idx & 7, k = (idx >> 3) * 4;
+            if (r < nb) {
+                float4 x;
+                if (gate) x = ldg4(x_t + (size_t)(b0 + r) * d.H + k0 + k);
+                else x = *reinterpret_cast<const float4*>(l_in + (size_t)(b0 + r) * seq_stride + (size_t)d.head_to_q(i) * d.d_l + k0 + k);
+                float* dst = xs + ((r >> 2) * slabs.size + k) * 4 + (r & 3);
+                dst[0] = x.x; dst[4] = x.y; dst[8] = x.z; dst[12] = x.w;
+            }
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        if (live) {
+            const typename W::Raw* wv = w_s + (s & 1 ? slabs.even_pieces * kDecodeThreads : 0) + tid;
+            const auto rows = [&](int k, const float4 w, int h) {
+                const float4 a = *reinterpret_cast<const float4*>(xs + (h * slabs.size + k) * 4);
+                const float xr[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    acc[4 * h + r][0] = fmaf(xr[r], w.x, acc[4 * h + r][0]);
+                    acc[4 * h + r][1] = fmaf(xr[r], w.y, acc[4 * h + r][1]);
+                    acc[4 * h + r][2] = fmaf(xr[r], w.z, acc[4 * h + r][2]);
+                    acc[4 * h + r][3] = fmaf(xr[r], w.w, acc[4 * h + r][3]);
+                }
+            };
+            if (nb > 4) {
+#pragma unroll 4
+                for (int k = ks; k < n; k += 64, wv += kDecodeThreads) {
+                    const float4 w = W::widen(*wv);
+                    rows(k, w, 0);
+                    rows(k, w, 1);
+                }
+            } else {
+#pragma unroll 4
+                for (int k = ks; k < n; k += 64, wv += kDecodeThreads) rows(k, W::widen(*wv), 0);
+            }
+        }
+        fetch(s + 2);                                        // into the pieces that this thread has just used
+    }
     const float y = finish_reduce(acc, red + 8 * 128);
+    // a fused step: the kernels that read the lengths are complete
+    if (step_lens != nullptr && blockIdx.x == 0 && blockIdx.y == 0)
+        for (int b = tid; b < d.B; b += kDecodeThreads) {
+            const int len = step_lens[b];
+            if (len >= 0 && len < S_cap) step_lens[b] = len + 1;
+        }
     const int r = tid >> 4, c = e0 + (tid & 15);
     if (tid < 128 && r < nb && c < d.d_h)
         out[((size_t)(b0 + r) * d.n_h + i) * d.d_h + c] = from_f32<T>(y * (1.f / (1.f + expf(-z))));
@@ -598,7 +678,8 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
                                        const int32_t* seq_lens, int S_cap, const void* x_t, const void* w_p,
                                        const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
                                        cudaStream_t stream, int stages, int* launches, const PageMap& pm,
-                                       const float* k_scale = nullptr, const float* c_scale = nullptr) {
+                                       const float* k_scale = nullptr, const float* c_scale = nullptr,
+                                       const void* k_new = nullptr, const void* c_new = nullptr) {
     const DecodePlan p = make_plan(d, S_cap, room);
     float* part_o = reinterpret_cast<float*>(workspace);
     float* part_ml = reinterpret_cast<float*>(static_cast<char*>(workspace) + p.off_ml);
@@ -611,7 +692,7 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
             return launch_chained(true, decode_partial_kernel<T, CT, CM>, dim3(p.n_chunks, d.B), kDecodeThreads,
                                  partial_smem(d, p.chunk, CM, LatentVec<CT>::N), stream, d, p.chunk, p.n_chunks, S_cap,
                                  (const T*)q, (const CT*)k_cache, (const CT*)c_cache, seq_lens, part_o, part_ml, pm,
-                                 status_word, k_scale, c_scale);
+                                 status_word, k_scale, c_scale, (const CT*)k_new, (const CT*)c_new);
         };
         // as few passes over the latent rows as the accumulators allow (and as shared memory does, with very many maps)
         const auto fits = [&](int cm) { return partial_smem(d, p.chunk, cm, LatentVec<CT>::N) <= 227 * 1024; };
@@ -624,12 +705,16 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
     }
     if (stages & 4) {
         err = launch_chained((stages & 2) && S_cap > 0, decode_chunk_merge_kernel, dim3(d.n_q, d.B), kDecodeThreads, 0, stream, d,
-                             p.chunk, p.n_chunks, S_cap, seq_lens, part_o, part_ml);
+                             p.chunk, p.n_chunks, S_cap, seq_lens, part_o, part_ml, k_new != nullptr);
         if (err != cudaSuccess) return err;
         const int tiles = (d.d_h + kFinishCols - 1) / kFinishCols;
-        const size_t smem = (2 * kFinishSlab * 4 + 2 * 8 * 128) * sizeof(float);
-        err = launch_chained(true, decode_finish_kernel<T>, dim3(d.n_h * tiles, (d.B + kFinishSeqs - 1) / kFinishSeqs), kDecodeThreads, smem,
-                            stream, d, tiles, (const T*)x_t, (const float*)part_o, (size_t)p.n_chunks * d.n_q * d.d_l, (const T*)w_p, (const T*)w_g, (T*)out);
+        const dim3 grid(d.n_h * tiles, (d.B + kFinishSeqs - 1) / kFinishSeqs);
+        const FinishSlabs slabs = finish_slabs(d, (long long)grid.x * grid.y);
+        const size_t smem = (size_t)(slabs.even_pieces + slabs.odd_pieces) * kDecodeThreads * sizeof(typename Weights4<T>::Raw) +
+                            (2 * slabs.size * 4 + 2 * 8 * 128) * sizeof(float);
+        err = launch_chained(true, decode_finish_kernel<T>, grid, kDecodeThreads, smem,
+                            stream, d, tiles, slabs, (const T*)x_t, (const float*)part_o, (size_t)p.n_chunks * d.n_q * d.d_l, (const T*)w_p,
+                            (const T*)w_g, (T*)out, k_new != nullptr ? const_cast<int32_t*>(seq_lens) : nullptr, S_cap);
         if (err != cudaSuccess) return err;
         *launches += 2;
     }
@@ -986,6 +1071,19 @@ cudaError_t launch_decode(const Dims& d, int dtype, const void* q, const void* k
                                           workspace, room, status_word, stream, stages, launches, pm);
     return launch_decode_typed<__nv_bfloat16, __nv_bfloat16>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out,
                                               workspace, room, status_word, stream, stages, launches, pm);
+}
+
+// The step with the append of its token folded in (contiguous caches): no kernel of its own in front.
+cudaError_t launch_decode_plain_append(const Dims& d, int dtype, const void* q, void* k_cache, void* c_cache, const void* k_new,
+                                       const void* c_new, int32_t* seq_lens, int S_cap, const void* x_t, const void* w_p,
+                                       const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
+                                       cudaStream_t stream, int* launches) {
+    if (dtype == GTA_F32)
+        return launch_decode_typed<float, float>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace, room,
+                                                 status_word, stream, 7, launches, PageMap(), nullptr, nullptr, k_new, c_new);
+    return launch_decode_typed<__nv_bfloat16, __nv_bfloat16>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
+                                                             room, status_word, stream, 7, launches, PageMap(), nullptr, nullptr,
+                                                             k_new, c_new);
 }
 
 }  // namespace gta
