@@ -81,14 +81,14 @@ __host__ __device__ inline AttnSmem attn_smem(int d_h, int rows, int tile_keys, 
     return s;
 }
 
-// DH: the head width where it is a compile-time constant, 0 otherwise.
-template <typename T, int QW, int SW, int NC, int DH>
-__global__ void __launch_bounds__(32 * QW * SW)
-generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
-                         float* __restrict__ o_lat, const PageMap pm, int32_t* status_word, int tiles) {
+// DH: the head width where it is a compile-time constant, 0 otherwise.  Rows t0 .. of map g of sequence b, latent columns col0 ..;
+// `tid` of the 32 QW SW threads, which `sync` brings together; put(row, float4 column, v) takes the normalised sums.
+template <typename T, int QW, int SW, int NC, int DH, typename Sync, typename Put>
+__device__ __forceinline__ void attention_tile(const Dims& d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
+                                               const PageMap& pm, int32_t* status_word, float* smem, int tid, int t0, int col0, int g,
+                                               int b, Sync sync, Put put) {
     constexpr int kWarps = QW * SW, kThreads = 32 * kWarps;
     constexpr int kRows = 16 * QW, kTile = kAttnKeys * SW, kCols = 64 * NC;
-    extern __shared__ __align__(16) float smem[];
     const int d_h = DH > 0 ? DH : d.d_h;
     const AttnSmem L = attn_smem(d_h, kRows, kTile, kCols, kWarps);
     const int ld = d_h + 4;
@@ -96,18 +96,13 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
     float* k_s = q_s + kRows * ld;                              // [kTile][ld]
     float* c_s = k_s + L.k_floats;                              // [kTile][kCols]
     int* bad_s = reinterpret_cast<int*>(c_s + L.c_floats);      // [kTile]: key on a page outside the pool
-    ptx::grid_dependency_wait();
-    ptx::grid_launch_dependents();       // (the decoder kernel's gate phase may start as SMs free up)
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int warp = tid >> 5, lane = tid & 31;
     float* p_s = reinterpret_cast<float*>(bad_s + kTile) + warp * kAttnKeys * kPStride;   // [32][kPStride]
     float* row_s = reinterpret_cast<float*>(bad_s + kTile) + kWarps * kAttnKeys * kPStride + warp * 32;   // [2][16]
     const int qw = warp % QW, sw = warp / QW;
 
-    // (row tiles and slices of d_l share x, heads and maps have y to themselves: 65535 of them)
-    const int slice = (int)blockIdx.x / tiles, t0 = (tiles - 1 - ((int)blockIdx.x - slice * tiles)) * kRows;   // the longest rows first
-    const int g = blockIdx.y, b = blockIdx.z;
     const int kg = d.q_to_k(g), cg = d.q_to_c(g);
-    const int col0 = slice * kCols, n_cols = min(kCols, d.d_l - col0);
+    const int n_cols = min(kCols, d.d_l - col0);
     const int off = d.causal ? d.Nk - d.N : 0;                  // causal: row t attends keys 0 .. t + off
     const int rows = min(kRows, d.N - t0);
     const int n_keys = d.causal ? min(t0 + rows + off, d.Nk) : d.Nk;
@@ -183,7 +178,7 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
 
     for (int it = 0; it < n_iter; ++it) {
         cp_async_wait<0>();
-        __syncthreads();                 // the key tile is there, the latent tile before has been used
+        sync();                 // the key tile is there, the latent tile before has been used
         load_latents(it);
         cp_async_commit();
         const int j0 = it * kTile + sw * kAttnKeys;
@@ -261,7 +256,7 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
             }
         }
         cp_async_wait<0>();
-        __syncthreads();                 // the latent tile is there, the key tile has been used
+        sync();                 // the latent tile is there, the key tile has been used
         if (it + 1 < n_iter) load_keys(it + 1);
         cp_async_commit();
         if (mine) {
@@ -306,7 +301,7 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
             __syncwarp();
         }
     }
-    __syncthreads();                     // (the tiles' memory is used again below)
+    sync();                     // (the tiles' memory is used again below)
 
     // ---- row sums over the lanes of a row, then (maximum, row sum) in the lanes that hold the row's sums
 #pragma unroll
@@ -317,7 +312,6 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
         *reinterpret_cast<float4*>(row_s + 4 * rg) = make_float4(m[0], m[1], m[2], m[3]);
         *reinterpret_cast<float4*>(row_s + 16 + 4 * rg) = make_float4(l[0], l[1], l[2], l[3]);
     }
-    float* o_rows = o_lat + (((size_t)g * d.B + b) * d.N + t0) * d.d_l + col0;
     // log-sum-exp merge of the SW key splits of every row: the key tiles' memory takes the sums
     float* o_s = k_s;                                                   // [SW][kRows][kCols]
 #pragma unroll
@@ -329,7 +323,7 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
             ptx::f32x2_split(o[i][n][1], v.z, v.w);
             *reinterpret_cast<float4*>(o_s + ((size_t)sw * kRows + 16 * qw + 8 * rh + i) * kCols + 4 * cc + 64 * n) = v;
         }
-    __syncthreads();
+    sync();
     const float* all_rows = row_s - warp * 32;                          // [warp][2][16]
     for (int idx = tid; idx < rows * 16 * NC; idx += kThreads) {
         const int r = idx / (16 * NC), v4 = idx % (16 * NC);
@@ -348,8 +342,24 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
             a.x = fmaf(v.x, w, a.x); a.y = fmaf(v.y, w, a.y); a.z = fmaf(v.z, w, a.z); a.w = fmaf(v.w, w, a.w);
         }
         const float inv = ls > 0.f ? 1.f / ls : 0.f;
-        *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * v4) = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+        put(r, v4, make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv));
     }
+}
+
+template <typename T, int QW, int SW, int NC, int DH>
+__global__ void __launch_bounds__(32 * QW * SW)
+generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
+                         float* __restrict__ o_lat, const PageMap pm, int32_t* status_word, int tiles) {
+    extern __shared__ __align__(16) float smem[];
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();       // (the decoder kernel's gate phase may start as SMs free up)
+    // (row tiles and slices of d_l share x, heads and maps have y to themselves: 65535 of them)
+    const int slice = (int)blockIdx.x / tiles, t0 = (tiles - 1 - ((int)blockIdx.x - slice * tiles)) * 16 * QW;   // the longest rows first
+    const int g = blockIdx.y, b = blockIdx.z, col0 = slice * 64 * NC;
+    float* o_rows = o_lat + (((size_t)g * d.B + b) * d.N + t0) * d.d_l + col0;
+    attention_tile<T, QW, SW, NC, DH>(
+        d, q, k, c, pm, status_word, smem, threadIdx.x, t0, col0, g, b, [] { __syncthreads(); },
+        [&](int r, int v4, const float4 v) { *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * v4) = v; });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -520,6 +530,147 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
 }
 
 // ---------------------------------------------------------------------------------------------
+// A short fp32 prompt in one kernel (d_h = 64, d_l = 128): 16 rows x 64 output columns of one map per CTA.  Warps 0-3 do the rows'
+// attention (once more for every column block: it is latency, not work), warps 4-7 the gates meanwhile, with the first weights and
+// W_P on their way from the start; then all eight contract L, which never leaves shared memory, with W_P.
+// What bounds it is one chain of latencies; two kernels have two, and a result through L2 between them (128 tokens of the tiny
+// layer 16.9 us, 11.7 in one; 100 tokens of the 1B layer 31.2, 18.3).
+constexpr int kShortBk = 64, kShortStages = 3, kShortLdA = kShortBk + 4, kShortLdL = 132;
+constexpr int kShortStage = 16 * kShortLdA + kShortBk * 64;
+__host__ __device__ inline int short_attn_floats() { return attn_smem(64, 16, 4 * kAttnKeys, 128, 4).total_floats; }
+static size_t short_smem_bytes() {
+    return (size_t)(short_attn_floats() + kShortStages * kShortStage + 128 * 64 + 16 * kShortLdL) * sizeof(float);
+}
+
+__global__ void __launch_bounds__(256)
+short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ c,
+                         const float* __restrict__ x, const float* __restrict__ w_p, const float* __restrict__ w_g,
+                         float* __restrict__ out, int tiles) {
+    extern __shared__ __align__(16) float smem[];
+    float* ring = smem + short_attn_floats();
+    float* wp_s = ring + kShortStages * kShortStage;             // [128][64]
+    float* l_s = wp_s + 128 * 64;                                // [16][kShortLdL]
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ct = (int)blockIdx.x / tiles, t0 = (tiles - 1 - ((int)blockIdx.x - ct * tiles)) * 16;
+    const int g = blockIdx.y, b = blockIdx.z, rows = min(16, d.N - t0);
+    const int map_cols = d.n_h / d.n_q * d.d_h, c0 = ct * 64;    // (a multiple of 64)
+    const int rg = lane >> 3, cg = lane & 7;                     // rows rg + 4 i; columns 4 cg + {0..3}, 32 + 4 cg + {0..3}
+    const int head = g * (d.n_h / d.n_q) + ct;                   // (64 columns are a head)
+
+    // 16 rows x 64 columns: a (rows apart by lda) times w [k][64], k = 0 .. 15
+    const auto multiply16 = [&](const float* a_s, int lda, const float* w_s, uint64_t (&acc)[4][4]) {
+        const float* as = a_s + rg * lda;
+        const float* bs = w_s + 4 * cg;
+#pragma unroll
+        for (int kk = 0; kk < 16; kk += 4) {
+            float4 a[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(as + 4 * i * lda + kk);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const Pair2 b0 = lds_pair2(bs + (kk + u) * 64), b1 = lds_pair2(bs + (kk + u) * 64 + 32);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float av = u == 0 ? a[i].x : u == 1 ? a[i].y : u == 2 ? a[i].z : a[i].w;
+                    const uint64_t aa = ptx::f32x2(av, av);
+                    acc[i][0] = ptx::fma2(aa, b0.lo, acc[i][0]);
+                    acc[i][1] = ptx::fma2(aa, b0.hi, acc[i][1]);
+                    acc[i][2] = ptx::fma2(aa, b1.lo, acc[i][2]);
+                    acc[i][3] = ptx::fma2(aa, b1.hi, acc[i][3]);
+                }
+            }
+        }
+    };
+    uint64_t acc_g[4][4], acc_p[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc_g[i][j] = acc_p[i][j] = 0ull;
+
+    if (warp < 4) {
+        attention_tile<float, 1, 4, 2, 64>(
+            d, q, k, c, PageMap(), nullptr, smem, tid, t0, 0, g, b, [] { ptx::named_sync(1, 128); },
+            [&](int r, int v4, const float4 v) { *reinterpret_cast<float4*>(l_s + r * kShortLdL + 4 * v4) = v; });
+        // (rows past the last meet W_P too; their results go nowhere)
+        for (int idx = tid; idx < (16 - rows) * 32; idx += 128)
+            *reinterpret_cast<float4*>(l_s + (rows + idx / 32) * kShortLdL + 4 * (idx % 32)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+        const int tg = tid - 128, n_blocks = (d.H + kShortBk - 1) / kShortBk;
+        const float* x_rows = x + ((size_t)b * d.N + t0) * d.H;
+        const float* wg = w_g + (size_t)head * d.d_h;
+        const size_t ldw = (size_t)d.n_h * d.d_h;
+        const auto load = [&](int it) {
+            if (it < n_blocks) {
+                float* as = ring + it % kShortStages * kShortStage;
+                float* ws = as + 16 * kShortLdA;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int r = (tg >> 4) + 8 * i, kk = it * kShortBk + 4 * (tg & 15);
+                    const bool live = r < rows && kk < d.H;
+                    cp_async_16(as + r * kShortLdA + 4 * (tg & 15), x_rows + (live ? (size_t)r * d.H + kk : 0), live);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int kl = (tg >> 4) + 8 * i, kk = it * kShortBk + kl;
+                    cp_async_16(ws + kl * 64 + 4 * (tg & 15), wg + (kk < d.H ? kk * ldw : 0) + 4 * (tg & 15), kk < d.H);
+                }
+            }
+        };
+        load(0);
+        cp_async_commit();
+        load(1);
+        for (int i = 0; i < 16; ++i)
+            cp_async_16(wp_s + ((tg >> 4) + 8 * i) * 64 + 4 * (tg & 15), w_p + ((size_t)head * 128 + (tg >> 4) + 8 * i) * 64 + 4 * (tg & 15), true);
+        cp_async_commit();
+        for (int it = 0; it < n_blocks; ++it) {
+            cp_async_wait<kShortStages - 2>();
+            ptx::named_sync(2, 128);
+            load(it + kShortStages - 1);         // into the stage that everybody has left
+            cp_async_commit();
+            const float* as = ring + it % kShortStages * kShortStage;
+            multiply16(as + 16 * (warp - 4), kShortLdA, as + 16 * kShortLdA + 16 * (warp - 4) * 64, acc_g);
+        }
+        cp_async_wait<0>();
+    }
+    __syncthreads();
+    multiply16(l_s + 16 * warp, kShortLdL, wp_s + 16 * warp * 64, acc_p);
+    // the warps' partial sums meet where the latents were: [warp][pair of accumulators][lane], values, then gates
+    uint64_t* part = reinterpret_cast<uint64_t*>(smem);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            part[(warp * 16 + 4 * i + j) * 32 + lane] = acc_p[i][j];
+            if (warp >= 4) part[((warp + 4) * 16 + 4 * i + j) * 32 + lane] = acc_g[i][j];
+        }
+    __syncthreads();
+    const int i = warp >> 1, j = 2 * (warp & 1), r = rg + 4 * i;     // this thread's four outputs
+    float y[4], z[4];
+    uint64_t s0 = 0ull, s1 = 0ull;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        s0 = ptx::add2(s0, part[(w * 16 + 4 * i + j) * 32 + lane]);
+        s1 = ptx::add2(s1, part[(w * 16 + 4 * i + j + 1) * 32 + lane]);
+    }
+    ptx::f32x2_split(s0, y[0], y[1]);
+    ptx::f32x2_split(s1, y[2], y[3]);
+    s0 = s1 = 0ull;
+#pragma unroll
+    for (int w = 8; w < 12; ++w) {
+        s0 = ptx::add2(s0, part[(w * 16 + 4 * i + j) * 32 + lane]);
+        s1 = ptx::add2(s1, part[(w * 16 + 4 * i + j + 1) * 32 + lane]);
+    }
+    ptx::f32x2_split(s0, z[0], z[1]);
+    ptx::f32x2_split(s1, z[2], z[3]);
+    if (r >= rows) return;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) y[u] *= 1.f / (1.f + expf(-z[u]));
+    store4(out + ((size_t)b * d.N + t0 + r) * d.n_h * d.d_h + (size_t)g * map_cols + c0 + 16 * j + 4 * cg, y);
+}
+
+// ---------------------------------------------------------------------------------------------
 // Launch with programmatic stream serialisation (the kernel waits for the one before it by itself), or without.
 template <typename Kern, typename... Args>
 static cudaError_t launch_chained(bool behind, Kern kern, dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
@@ -577,7 +728,10 @@ static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x,
 // of the decoder 0.9 or 1.05 us.  The decoder's gates run beside the attention kernel where both fit the chip at once (1B, 1000
 // tokens: 47.1 with one, 54.6 with two; tiny, 2048: 75.5 / 48.8 / 38.7 with one / two / four); a plain decoder wants the SMs that a
 // split takes (1B, 200 tokens: 32.7 / 43.3; tiny, 333: 26.0 / 23.3).
-struct F32Plan { int split = 0, cols = 0; };       // 0: the plain-ALU kernel
+//
+// Below both lines, d_h = 64 and d_l = 128 run in one kernel while its CTAs are one wave (tiny, 4 x 128, 128 CTAs: 17.8 us in two, 12.8;
+// a second wave would bring every column block's attention once more).
+struct F32Plan { int split = 0, cols = 0; bool one = false; };       // 0: the plain-ALU kernel; one: both in one kernel
 static size_t l_bytes(const Dims& d) { return ((size_t)d.B * d.n_q * d.N * d.d_l * sizeof(float) + 255) & ~(size_t)255; }
 static F32Plan f32_plan(const Dims& d, const PageMap& pm, size_t room) {
     F32Plan plan;
@@ -588,8 +742,11 @@ static F32Plan f32_plan(const Dims& d, const PageMap& pm, size_t room) {
     if (d.d_h % 64 == 0 && tiles64 >= 100) plan.cols = map_cols > 128 && sm100_decoder_f32_units(d, 256) > 28 ? 256 : 128;
     const long long plain = (long long)d.B * d.n_q * ((d.N + 15) / 16);
     if (pm.table != nullptr || !sm100_attention_f32_supported(d) || (d.Nk < 192 && plain <= 64) ||
-        room < l_bytes(d) + sm100_attention_f32_scratch(d))
+        room < l_bytes(d) + sm100_attention_f32_scratch(d)) {
+        plan.one = pm.table == nullptr && plan.cols == 0 && d.d_h == 64 && d.d_l == 128 && d.Nk < 192 &&
+                   plain * (d.n_h / d.n_q) <= 148;
         return plan;
+    }
     const long long items = (long long)((d.N + 127) / 128) * (d.d_l / 128) * d.n_q * d.B;
     const long long dec_ctas = plan.cols ? 2 * sm100_decoder_f32_units(d, plan.cols) : 0;
     const float stage = plan.cols == 256 ? 1.05f : 0.9f, dec_waves = (float)((dec_ctas + 147) / 148);
@@ -615,6 +772,17 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
                                 int32_t* status_word) {
     cudaError_t err;
     const F32Plan plan = std::is_same_v<T, float> ? f32_plan(d, pm, room) : F32Plan{};
+    if constexpr (std::is_same_v<T, float>) {
+        if (plan.one && (stages & 3) == 3) {
+            const size_t smem = short_smem_bytes();
+            const int tiles = (d.N + 15) / 16;
+            err = cudaFuncSetAttribute(short_prefill_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (err != cudaSuccess) return err;
+            *launches += 1;
+            return launch_chained(true, short_prefill_f32_kernel, dim3(tiles * (d.n_h / d.n_q), d.n_q, d.B), 256, smem, stream, d, (const float*)q,
+                                  (const float*)k, (const float*)c, (const float*)x, (const float*)w_p, (const float*)w_g, (float*)out, tiles);
+        }
+    }
     if constexpr (std::is_same_v<T, float>) {
         if ((stages & 1) && plan.split) {
             err = launch_sm100_attention_f32(d, (const float*)q, (const float*)k, (const float*)c, o_lat_ws,

@@ -89,6 +89,26 @@ def test_against_64_bits(G, case):
     assert float(err.norm() / want.norm()) <= REL and float((err.abs() / torch.maximum(want.abs(), rms)).max()) <= MAX
 
 
+SHORT = [  # both stages in one plain-ALU kernel: row and key tile edges, k-blocks of the gate, a chunk, heads of a map
+    (1, 1, 1, 1, 8, 2, 2, 1, 1, 64, 128, True), (2, 16, 16, 16, 72, 3, 1, 1, 1, 64, 128, True),
+    (1, 17, 17, 17, 1280, 20, 5, 1, 1, 64, 128, True), (2, 128, 128, 128, 256, 4, 2, 2, 2, 64, 128, True),
+    (1, 129, 129, 140, 256, 4, 2, 2, 1, 64, 128, False), (1, 191, 191, 191, 200, 4, 2, 1, 1, 64, 128, True),
+    (3, 33, 190, 200, 136, 6, 2, 1, 1, 64, 128, True),
+]
+
+
+@pytest.mark.parametrize("case", SHORT, ids=[f"B{c[0]}_N{c[1]}_kv{c[2]}_H{c[4]}" for c in SHORT])
+def test_short_prompts_against_64_bits(G, case):
+    test_against_64_bits(G, case)
+
+
+def test_short_prompt_rows_before_an_odd_element_keep_their_bits(G):
+    t = _inputs(1, 100, 100, 256, 4, 2, 2, 1, 64, 128)
+    want = _run(G, t, 100, True).clone()
+    t["k"][:, :, 41:], t["c"][:, :, 41:] = float("nan"), float("inf")
+    assert torch.equal(_run(G, t, 100, True)[:, :41], want[:, :41])
+
+
 @pytest.mark.parametrize("size", [1e-30, 1e15])
 def test_range_of_the_pieces(G, size):
     """Latents and decoder weights near both ends of the range: the pieces have fp32's exponents."""
