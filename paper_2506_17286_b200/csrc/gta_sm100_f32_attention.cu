@@ -8,10 +8,12 @@
 //   sm100_attention_f32_kernel  a CTA (or a cluster of two or four that take the key tiles in turn and merge at the end through
 //                            distributed shared memory) owns 128 query rows x 128 latent columns of a map:
 //     warp 0       brings the pieces of key tiles in by TMA (64 keys x (64 + 128) columns x 3 = 72 KB a stage, 3 stages).
-//     warp 1       issues the MMAs: S = Q K^T (pieces of Q in tensor memory), then O = P C (pieces of P in tensor memory).
+//     warp 1       issues the MMAs: S = Q K^T (pieces of Q in tensor memory), two tiles ahead of O = P C (pieces of P in tensor
+//                  memory, the first two where the scores were), 64 latent columns after 64.
 //     warps 4-11   softmax, two warpgroups on alternating tiles with a running maximum and row sum each: a thread is a row.
 //     warps 12-19  add the O of a tile to their registers, in the scale of the largest maximum so far.
-// Per key tile: 24 MMAs of N = 64 (768 cycles) and 24 of N = 128 (1536): the tensor pipe is the bound; the rest hides under it.
+// Per key tile: 72 MMAs of N = 64, 2304 cycles of the tensor pipe, which the rest is to hide under: measured 2850.  (With one
+// buffer of P, written between two products, and O in one piece: 3060.)
 //
 // An element that is infinite, not a number or rounds to infinity in bf16 has no pieces.  In K and C zeros stand in for it, so
 // that rows which do not see it keep their bits (0 x infinity); the rows that do, and the rows of Q that hold one, are done
@@ -34,13 +36,13 @@ constexpr int kStages = 3;
 constexpr uint32_t kKPlane = kKeys * kDh * 2, kCPlane = kKeys * kCols * 2, kCBlock = kKeys * 128;
 constexpr uint32_t kStageBytes = 3 * (kKPlane + kCPlane);            // 72 KB
 constexpr uint32_t kBarOffset = kStages * kStageBytes;
-constexpr uint32_t kSmem = kBarOffset + 512 + 6 * kRows * 4 + 1024;  // barriers; maxima and sums of rows; alignment
+constexpr uint32_t kSmem = kBarOffset + 512 + 8 * kRows * 4 + 1024;  // barriers; maxima and sums of rows; alignment
 static_assert(kSmem <= 227 * 1024, "shared memory of a CTA");
 constexpr int kSoftWarp0 = 4, kAddWarp0 = 12, kThreads = 640;
 // registers: 640 threads start with 96 each (61440): 128 x 48 + 256 x 104 + 256 x 112
 constexpr int kIssueRegs = 48, kSoftRegs = 104, kAddRegs = 112;
 // tensor memory columns
-constexpr uint32_t kTmS = 0, kTmP = 128, kTmQ = 224, kTmO = 320;
+constexpr uint32_t kTmS = 0, kTmSP = 96, kTmQ = 192, kTmO = 320;      // [2] 64 columns of scores or 96 of P; Q 96; O 128
 
 // ---------------------------------------------------------------------------------------------
 // Pieces of four floats; not-a-number in `rest` where they do not add up to them.
@@ -138,21 +140,22 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* k_full = reinterpret_cast<uint64_t*>(smem + kBarOffset);
     uint64_t* c_full = k_full + kStages;
-    uint64_t* empty_bar = c_full + kStages;
-    uint64_t* s_full = empty_bar + kStages;      // [2]
-    uint64_t* s_free = s_full + 2;               // [2]: 4 warps
-    uint64_t* p_full = s_free + 2;               // 4 warps
-    uint64_t* o_full = p_full + 1;               // P read, O written
-    uint64_t* o_free = o_full + 1;               // 8 warps
-    uint64_t* q_full = o_free + 1;               // 8 warps
+    uint64_t* k_empty = c_full + kStages;        // 4 warps: the softmax warpgroup that has seen the scores complete ...
+    uint64_t* c_empty = k_empty + kStages;       // ... and the adding one that has seen the last sums complete (a commit more
+                                                 // by the issuing thread takes it some 200 cycles)
+    uint64_t* s_full = c_empty + kStages;        // [2]
+    uint64_t* p_full = s_full + 2;               // [2]: 4 warps
+    uint64_t* o_full = p_full + 2;               // [2] halves of the columns
+    uint64_t* o_free = o_full + 2;               // [2]: 4 warps
+    uint64_t* q_full = o_free + 2;               // 8 warps
     uint64_t* drain_bar = q_full + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* drain_flag = abort_flag + 1;
     int* odd_key = reinterpret_cast<int*>(tmem_slot + 3);                     // first key of the item without pieces
     uint32_t* odd_rows = tmem_slot + 4;                                       // [4]: query rows, a bit each
-    float* ref_s = reinterpret_cast<float*>(smem + kBarOffset + 512);        // [2][128]: the scale of a tile's P
-    float* fin_m = ref_s + 2 * kRows;                                         // [2][128]
+    float* ref_s = reinterpret_cast<float*>(smem + kBarOffset + 512);        // [4][128]: the scale of a tile's P
+    float* fin_m = ref_s + 4 * kRows;                                         // [2][128]
     float* fin_l = fin_m + 2 * kRows;                                         // [2][128]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -169,11 +172,8 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     const int n_my = n_tiles > rank ? (n_tiles - rank + SW - 1) / SW : 0;     // tiles rank, rank + SW, ...
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) { ptx::mbar_init(&k_full[s], 1); ptx::mbar_init(&c_full[s], 1); ptx::mbar_init(&empty_bar[s], 1); }
-        for (int s = 0; s < 2; ++s) { ptx::mbar_init(&s_full[s], 1); ptx::mbar_init(&s_free[s], 4); }
-        ptx::mbar_init(p_full, 4);
-        ptx::mbar_init(o_full, 1);
-        ptx::mbar_init(o_free, 8);
+        for (int s = 0; s < kStages; ++s) { ptx::mbar_init(&k_full[s], 1); ptx::mbar_init(&c_full[s], 1); ptx::mbar_init(&k_empty[s], 4); ptx::mbar_init(&c_empty[s], 4); }
+        for (int s = 0; s < 2; ++s) { ptx::mbar_init(&s_full[s], 1); ptx::mbar_init(&p_full[s], 4); ptx::mbar_init(&o_full[s], 1); ptx::mbar_init(&o_free[s], 4); }
         ptx::mbar_init(q_full, 8);
         ptx::mbar_init(drain_bar, 1);
         *abort_flag = 0;
@@ -195,16 +195,18 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             ptx::prefetch_tensormap(&tm_k); ptx::prefetch_tensormap(&tm_c); ptx::prefetch_tensormap(&tm_l);
             ptx::grid_dependency_wait();
             const int k_plane = b * d.n_k + kg, c_plane = b * d.n_c + cg;
-            bool ok = true;
+            bool ok = true, c_last = true;       // (whether the last tile's latents were asked for too)
             int i = 0, s = 0;
             uint32_t ph = 1;
             for (; i < n_my; ++i) {
-                ok = ptx::mbar_wait(&empty_bar[s], ph, abort_flag);
+                ok = ptx::mbar_wait(&k_empty[s], ph, abort_flag);
                 if (!ok) break;
                 const int j0 = (rank + SW * i) * kKeys;
                 uint8_t* st = smem + s * kStageBytes;
                 ptx::mbar_arrive_expect_tx(&k_full[s], 3 * kKPlane);
                 for (int p = 0; p < 3; ++p) ptx::tma_load_3d(st + p * kKPlane, &tm_k, &k_full[s], 0, j0, p * d.B * d.n_k + k_plane);
+                ok = ptx::mbar_wait(&c_empty[s], ph, abort_flag);
+                if (!ok) { ++i; c_last = false; break; }
                 ptx::mbar_arrive_expect_tx(&c_full[s], 3 * kCPlane);
                 for (int p = 0; p < 3; ++p)
                     for (int v = 0; v < kCols / 64; ++v)
@@ -216,19 +218,20 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             if (!ok)                     // every armed tile either lands or the wait gives up
                 for (int back = 1; back <= kStages && i - back >= 0; ++back) {
                     ptx::mbar_wait_drain(&k_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
-                    ptx::mbar_wait_drain(&c_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
+                    if (back > 1 || c_last) ptx::mbar_wait_drain(&c_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
                 }
         } else if (warp == 1 && ptx::elect_one()) {
-            const uint32_t idesc_s = ptx::make_idesc_bf16(kRows, kKeys, 0, 0), idesc_o = ptx::make_idesc_bf16(kRows, kCols, 0, 1);
+            const uint32_t idesc_s = ptx::make_idesc_bf16(kRows, kKeys, 0, 0), idesc_o = ptx::make_idesc_bf16(kRows, 64, 0, 1);
             const uint64_t k_desc = ptx::make_smem_desc(ptx::smem_addr(smem), 16, 1024);
             const uint64_t c_desc = ptx::make_smem_desc(ptx::smem_addr(smem) + 3 * kKPlane, kCBlock, 1024);
             const uint32_t k_lo0 = (uint32_t)k_desc, k_hi = (uint32_t)(k_desc >> 32), c_lo0 = (uint32_t)c_desc, c_hi = (uint32_t)(c_desc >> 32);
             constexpr int kPa[6] = {2, 1, 0, 1, 0, 0}, kPb[6] = {0, 1, 2, 0, 1, 0};       // products of pieces, the smallest first
             bool ok = true;
             int ss = 0, so = 0;          // stages of the next scores and sums
-            uint32_t phs = 0, pho = 0;
+            uint32_t phs = 0;
+            // (the scores of i - 2 have been read and their P used: both by MMAs and waits before)
             auto scores = [&](int i) {
-                ok = ptx::mbar_wait(&k_full[ss], phs, abort_flag) && ptx::mbar_wait(&s_free[i & 1], ((i >> 1) & 1) ^ 1, abort_flag);
+                ok = ptx::mbar_wait(&k_full[ss], phs, abort_flag);
                 if (!ok) return;
                 ptx::tc_fence_after_sync();
                 const uint32_t lo = k_lo0 + ss * (kStageBytes >> 4);
@@ -236,7 +239,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 for (int v = 0; v < 6; ++v)
 #pragma unroll
                     for (int k4 = 0; k4 < kDh / 16; ++k4)
-                        ptx::mma_ts(tmem + kTmS + (i & 1) * kKeys, tmem + kTmQ + kPa[v] * 32 + k4 * 8,
+                        ptx::mma_ts(tmem + kTmS + (i & 1) * kTmSP, tmem + kTmQ + kPa[v] * 32 + k4 * 8,
                                     ptx::desc_of(lo + ((kPb[v] * kKPlane + k4 * 32) >> 4), k_hi), idesc_s, (v | k4) ? 1u : 0u);
                 ptx::tc_commit(&s_full[i & 1]);
                 ss = ss + 1 == kStages ? 0 : ss + 1;
@@ -245,25 +248,29 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             if (n_my > 0) {
                 ok = ptx::mbar_wait(q_full, 0, abort_flag);
                 if (ok) scores(0);
+                if (ok && n_my > 1) scores(1);
             }
             for (int i = 0; i < n_my && ok; ++i) {
-                if (i + 1 < n_my) scores(i + 1);
+                ok = ptx::mbar_wait(&p_full[i & 1], (i >> 1) & 1, abort_flag);      // (and the latents are there)
                 if (!ok) break;
-                ok = ptx::mbar_wait(&c_full[so], pho, abort_flag) && ptx::mbar_wait(p_full, i & 1, abort_flag) &&
-                     ptx::mbar_wait(o_free, (i & 1) ^ 1, abort_flag);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
                 const uint32_t lo = c_lo0 + so * (kStageBytes >> 4);
 #pragma unroll
-                for (int v = 0; v < 6; ++v)
+                for (int h = 0; h < 2; ++h) {
+                    ok = ptx::mbar_wait(&o_free[h], (i & 1) ^ 1, abort_flag);
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
 #pragma unroll
-                    for (int k4 = 0; k4 < kKeys / 16; ++k4)
-                        ptx::mma_ts(tmem + kTmO, tmem + kTmP + kPa[v] * 32 + k4 * 8,
-                                    ptx::desc_of(lo + ((kPb[v] * kCPlane + k4 * 16 * 128) >> 4), c_hi), idesc_o, (v | k4) ? 1u : 0u);
-                ptx::tc_commit(&empty_bar[so]);
-                ptx::tc_commit(o_full);
+                    for (int v = 0; v < 6; ++v)
+#pragma unroll
+                        for (int k4 = 0; k4 < kKeys / 16; ++k4)
+                            ptx::mma_ts(tmem + kTmO + 64 * h, tmem + kTmS + (i & 1) * kTmSP + kPa[v] * 32 + k4 * 8,
+                                        ptx::desc_of(lo + ((kPb[v] * kCPlane + h * kCBlock + k4 * 16 * 128) >> 4), c_hi), idesc_o,
+                                        (v | k4) ? 1u : 0u);
+                    ptx::tc_commit(&o_full[h]);
+                }
+                if (!ok) break;
                 so = so + 1 == kStages ? 0 : so + 1;
-                pho ^= so == 0;
+                if (i + 2 < n_my) scores(i + 2);
             }
             if (!ok) {                   // tensor memory is freed below: nothing may be on its way there
                 ptx::tc_commit(drain_bar);
@@ -319,13 +326,13 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             ptx::mbar_wait(&s_full[w], (i >> 1) & 1, abort_flag);
             __syncwarp();
             ptx::tc_fence_after_sync();
+            const int st = i % kStages;
+            const uint32_t st_ph = (i / kStages) & 1;
+            if (lane == 0) ptx::mbar_arrive(&k_empty[st]);
             uint32_t sv[2][32];
-            ptx::tmem_ld32(tmem + kTmS + lane_base + w * kKeys, sv[0]);
-            ptx::tmem_ld32(tmem + kTmS + lane_base + w * kKeys + 32, sv[1]);
+            ptx::tmem_ld32(tmem + kTmS + lane_base + w * kTmSP, sv[0]);
+            ptx::tmem_ld32(tmem + kTmS + lane_base + w * kTmSP + 32, sv[1]);
             ptx::tmem_wait_ld();
-            ptx::tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&s_free[w]);
             if (__any_sync(0xffffffffu, j0 + kKeys > live)) {
 #pragma unroll
                 for (int e = 0; e < kKeys; ++e)
@@ -349,10 +356,8 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 sum[e & 3] += p;
             }
             l = fmaf(l, alpha, (sum[0] + sum[1]) + (sum[2] + sum[3]));
-            if (i > 0) ptx::mbar_wait(o_full, (i - 1) & 1, abort_flag);      // the P before has been read
-            __syncwarp();
-            ptx::tc_fence_after_sync();
-            ref_s[w * kRows + row] = m_new;
+            // (P of i - 2 was read before the scores of i came; the adding warps are through with the scale of i - 4)
+            ref_s[(i & 3) * kRows + row] = m_new;
 #pragma unroll
             for (int p = 0; p < 3; ++p) {
 #pragma unroll
@@ -369,13 +374,14 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                             sv[h][2 * e + 1] = __float_as_uint(y);
                         }
                     }
-                    ptx::tmem_st16(tmem + kTmP + lane_base + p * 32 + h * 16, pc);
+                    ptx::tmem_st16(tmem + kTmS + lane_base + w * kTmSP + p * 32 + h * 16, pc);
                 }
             }
             ptx::tmem_wait_st();
             ptx::tc_fence_before_sync();
+            ptx::mbar_wait(&c_full[st], st_ph, abort_flag);
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(p_full);
+            if (lane == 0) ptx::mbar_arrive(&p_full[w]);
         }
         fin_m[w * kRows + row] = m;
         fin_l[w * kRows + row] = l;
@@ -393,10 +399,11 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 #pragma unroll
         for (int e = 0; e < kCols / 4; ++e) acc[e] = 0ull;
         for (int i = 0; i < n_my; ++i) {
-            ptx::mbar_wait(o_full, i & 1, abort_flag);
+            ptx::mbar_wait(&o_full[half], i & 1, abort_flag);
             __syncwarp();
+            if (half == 1 && lane == 0) ptx::mbar_arrive(&c_empty[i % kStages]);
             ptx::tc_fence_after_sync();
-            const float r = ref_s[(i & 1) * kRows + row];
+            const float r = ref_s[(i & 3) * kRows + row];
             const float R_new = fmaxf(R, r);
             const float fa = R == R_new || R == -INFINITY ? 1.f : exp2f(R - R_new);
             const float fb = r == R_new ? 1.f : r == -INFINITY ? 0.f : exp2f(r - R_new);
@@ -418,7 +425,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(o_free);
+            if (lane == 0) ptx::mbar_arrive(&o_free[half]);
         }
         ptx::named_sync(1, 512);         // maxima and row sums are there
         {
