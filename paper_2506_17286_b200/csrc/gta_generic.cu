@@ -83,8 +83,10 @@ __host__ __device__ inline AttnSmem attn_smem(int d_h, int rows, int tile_keys, 
 
 // DH: the head width where it is a compile-time constant, 0 otherwise.  Rows t0 .. of map g of sequence b, latent columns col0 ..;
 // `tid` of the 32 QW SW threads, which `sync` brings together; put(row, float4 column, v) takes the normalised sums.
+// bulk != nullptr (fp32, contiguous caches, d_l = 64 NC): a latent tile is one bulk copy, counted on the barrier there.
+struct BulkLatents { uint64_t* bar; volatile int* abort_flag; };
 template <typename T, int QW, int SW, int NC, int DH, typename Sync, typename Put>
-__device__ __forceinline__ void attention_tile(const Dims& d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
+__device__ __forceinline__ void attention_tile(const BulkLatents* bulk, const Dims& d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
                                                const PageMap& pm, int32_t* status_word, float* smem, int tid, int t0, int col0, int g,
                                                int b, Sync sync, Put put) {
     constexpr int kWarps = QW * SW, kThreads = 32 * kWarps;
@@ -138,6 +140,17 @@ __device__ __forceinline__ void attention_tile(const Dims& d, const T* __restric
     };
     auto load_latents = [&](int it) {       // (a row that does not exist meets zero probabilities: it is cleared)
         const int j0 = it * kTile;
+        if (bulk != nullptr) {
+            const int n = min(kTile, n_keys - j0);
+            if (tid == 0) {
+                ptx::fence_proxy_async_smem();           // (the memory has been read by ordinary loads)
+                ptx::mbar_arrive_expect_tx(bulk->bar, (uint32_t)(n * kCols * 4));
+                ptx::bulk_load_1d(c_s, c_plane + (size_t)j0 * kCols, (uint32_t)(n * kCols * 4), bulk->bar);
+            }
+            for (int i = tid; i < (kTile - n) * kCols / 4; i += kThreads)
+                reinterpret_cast<float4*>(c_s + n * kCols)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            return;
+        }
         if (pm.table == nullptr) {
             const T* src = c_plane + (size_t)(j0 + c_row) * d.d_l;
             for (int r = c_row; r < kTile; r += c_step, src += (size_t)c_step * d.d_l) {
@@ -153,6 +166,7 @@ __device__ __forceinline__ void attention_tile(const Dims& d, const T* __restric
         }
     };
 
+    if (bulk != nullptr && n_iter > 0) load_latents(0);
     {
         const T* q_rows = q + (((size_t)b * d.n_q + g) * d.N + t0) * d_h;
         for (int r = h_row; r < kRows; r += h_step)
@@ -179,7 +193,7 @@ __device__ __forceinline__ void attention_tile(const Dims& d, const T* __restric
     for (int it = 0; it < n_iter; ++it) {
         cp_async_wait<0>();
         sync();                 // the key tile is there, the latent tile before has been used
-        load_latents(it);
+        if (bulk == nullptr || it > 0) load_latents(it);
         cp_async_commit();
         const int j0 = it * kTile + sw * kAttnKeys;
         const bool mine = j0 < warp_keys;
@@ -255,6 +269,7 @@ __device__ __forceinline__ void attention_tile(const Dims& d, const T* __restric
                 }
             }
         }
+        if (bulk != nullptr) ptx::mbar_wait(bulk->bar, it & 1, bulk->abort_flag);
         cp_async_wait<0>();
         sync();                 // the latent tile is there, the key tile has been used
         if (it + 1 < n_iter) load_keys(it + 1);
@@ -358,7 +373,7 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
     const int g = blockIdx.y, b = blockIdx.z, col0 = slice * 64 * NC;
     float* o_rows = o_lat + (((size_t)g * d.B + b) * d.N + t0) * d.d_l + col0;
     attention_tile<T, QW, SW, NC, DH>(
-        d, q, k, c, pm, status_word, smem, threadIdx.x, t0, col0, g, b, [] { __syncthreads(); },
+        nullptr, d, q, k, c, pm, status_word, smem, threadIdx.x, t0, col0, g, b, [] { __syncthreads(); },
         [&](int r, int v4, const float4 v) { *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * v4) = v; });
 }
 
@@ -533,8 +548,10 @@ generic_decoder_kernel(Dims d, const float* __restrict__ o_lat, const T* __restr
 // A short fp32 prompt in one kernel (d_h = 64, d_l = 128): 16 rows x 64 output columns of one map per CTA.  Warps 0-3 do the rows'
 // attention (once more for every column block: it is latency, not work), warps 4-7 the gates meanwhile, with the first weights and
 // W_P on their way from the start; then all eight contract L, which never leaves shared memory, with W_P.
-// What bounds it is one chain of latencies; two kernels have two, and a result through L2 between them (128 tokens of the tiny
-// layer 16.9 us, 11.7 in one; 100 tokens of the 1B layer 31.2, 18.3).
+// What bounds it is one chain of latencies and the way of 210 KB into an SM; two kernels have two chains, and a result through L2
+// between them (128 tokens of the tiny layer 16.9 us, 11.7 in one; 100 tokens of the 1B layer 31.2, 18.3).  The latents and W_P, one
+// piece each, travel by bulk copies beside the others' cp.async: 9.9 us.  (Keys and W_G by TMA too: 11.3; rows of 256 bytes by
+// bulk copies: 15.5.)
 constexpr int kShortBk = 64, kShortStages = 3, kShortLdA = kShortBk + 4, kShortLdL = 132;
 constexpr int kShortStage = 16 * kShortLdA + kShortBk * 64;
 __host__ __device__ inline int short_attn_floats() { return attn_smem(64, 16, 4 * kAttnKeys, 128, 4).total_floats; }
@@ -545,11 +562,21 @@ static size_t short_smem_bytes() {
 __global__ void __launch_bounds__(256)
 short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ c,
                          const float* __restrict__ x, const float* __restrict__ w_p, const float* __restrict__ w_g,
-                         float* __restrict__ out, int tiles) {
+                         float* __restrict__ out, int tiles, int32_t* status_word) {
     extern __shared__ __align__(16) float smem[];
+    __shared__ uint64_t latent_bar, wp_bar;
+    __shared__ int abort_word;
+    volatile int* abort_flag = &abort_word;
     float* ring = smem + short_attn_floats();
     float* wp_s = ring + kShortStages * kShortStage;             // [128][64]
     float* l_s = wp_s + 128 * 64;                                // [16][kShortLdL]
+    if (threadIdx.x == 0) {
+        ptx::mbar_init(&latent_bar, 1);
+        ptx::mbar_init(&wp_bar, 1);
+        *abort_flag = 0;
+        ptx::fence_mbar_init();
+    }
+    __syncthreads();
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -590,8 +617,9 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
         for (int j = 0; j < 4; ++j) acc_g[i][j] = acc_p[i][j] = 0ull;
 
     if (warp < 4) {
+        const BulkLatents bars{&latent_bar, abort_flag};
         attention_tile<float, 1, 4, 2, 64>(
-            d, q, k, c, PageMap(), nullptr, smem, tid, t0, 0, g, b, [] { ptx::named_sync(1, 128); },
+            &bars, d, q, k, c, PageMap(), nullptr, smem, tid, t0, 0, g, b, [] { ptx::named_sync(1, 128); },
             [&](int r, int v4, const float4 v) { *reinterpret_cast<float4*>(l_s + r * kShortLdL + 4 * v4) = v; });
         // (rows past the last meet W_P too; their results go nowhere)
         for (int idx = tid; idx < (16 - rows) * 32; idx += 128)
@@ -601,6 +629,10 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
         const float* x_rows = x + ((size_t)b * d.N + t0) * d.H;
         const float* wg = w_g + (size_t)head * d.d_h;
         const size_t ldw = (size_t)d.n_h * d.d_h;
+        if (tg == 0) {
+            ptx::mbar_arrive_expect_tx(&wp_bar, 128 * 64 * 4);
+            ptx::bulk_load_1d(wp_s, w_p + (size_t)head * 128 * 64, 128 * 64 * 4, &wp_bar);
+        }
         const auto load = [&](int it) {
             if (it < n_blocks) {
                 float* as = ring + it % kShortStages * kShortStage;
@@ -618,12 +650,11 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
                 }
             }
         };
-        load(0);
-        cp_async_commit();
-        load(1);
-        for (int i = 0; i < 16; ++i)
-            cp_async_16(wp_s + ((tg >> 4) + 8 * i) * 64 + 4 * (tg & 15), w_p + ((size_t)head * 128 + (tg >> 4) + 8 * i) * 64 + 4 * (tg & 15), true);
-        cp_async_commit();
+#pragma unroll
+        for (int it = 0; it < kShortStages - 1; ++it) {
+            load(it);
+            cp_async_commit();
+        }
         for (int it = 0; it < n_blocks; ++it) {
             cp_async_wait<kShortStages - 2>();
             ptx::named_sync(2, 128);
@@ -633,6 +664,7 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
             multiply16(as + 16 * (warp - 4), kShortLdA, as + 16 * kShortLdA + 16 * (warp - 4) * 64, acc_g);
         }
         cp_async_wait<0>();
+        ptx::mbar_wait(&wp_bar, 0, abort_flag);
     }
     __syncthreads();
     multiply16(l_s + 16 * warp, kShortLdL, wp_s + 16 * warp * 64, acc_p);
@@ -664,6 +696,13 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
     }
     ptx::f32x2_split(s0, z[0], z[1]);
     ptx::f32x2_split(s1, z[2], z[3]);
+    if (tid == 0 && *abort_flag) {           // a wait gave up: whatever is still on its way lands before the CTA leaves
+        int gave_up = 0;
+        const int n_iter = ((d.causal ? min(t0 + rows + d.Nk - d.N, d.Nk) : d.Nk) + 4 * kAttnKeys - 1) / (4 * kAttnKeys);
+        ptx::mbar_wait_drain(&latent_bar, (n_iter - 1) & 1, &gave_up);
+        ptx::mbar_wait_drain(&wp_bar, 0, &gave_up);
+        raise_status(status_word, GTA_ERR_TIMEOUT);
+    }
     if (r >= rows) return;
 #pragma unroll
     for (int u = 0; u < 4; ++u) y[u] *= 1.f / (1.f + expf(-z[u]));
@@ -780,7 +819,7 @@ static cudaError_t launch_typed(const Dims& d, const void* q, const void* k, con
             if (err != cudaSuccess) return err;
             *launches += 1;
             return launch_chained(true, short_prefill_f32_kernel, dim3(tiles * (d.n_h / d.n_q), d.n_q, d.B), 256, smem, stream, d, (const float*)q,
-                                  (const float*)k, (const float*)c, (const float*)x, (const float*)w_p, (const float*)w_g, (float*)out, tiles);
+                                  (const float*)k, (const float*)c, (const float*)x, (const float*)w_p, (const float*)w_g, (float*)out, tiles, status_word);
         }
     }
     if constexpr (std::is_same_v<T, float>) {
