@@ -745,10 +745,10 @@ cudaError_t launch_decode_fp8(const Dims& d, int dtype, const void* q, const voi
 // processor", 1990: q' = fl(q + fl(x - q s) r) is the correctly rounded quotient when q is within one unit in the last
 // place of it and r = fl(1 / s); the first correction brings fl(x r), which is within 1.5 units, there), two elements
 // per instruction.  Rows whose scale is far from 1, where a residual could leave the normal numbers, divide.
-// What bounds the kernel: latency (one wave of CTAs, each waiting for the length and then for its rows) and about 110
-// instructions per piece; 4 prompts of 2048 tokens (25 MB): 9.5 us.  With a division per element it was bound by issue
-// slots (390 instructions per two pieces, 13.3 us); one CTA per sequence with 2-byte loads, the form before that, left
-// the chip idle (1318 us).
+// What bounds the kernel: issue slots (about 175 instructions per piece where a lane has one of a row, fewer with four), and the
+// latency of a CTA's length and rows; 4 prompts of 2048 tokens (25 MB): 9.1 us.  (One or two pieces per lane 11.1, a division per
+// element 13.3; one CTA per sequence with 2-byte loads, the first form, left the chip idle: 1318 us.  CTAs that stay, behind a ring
+// of bulk copies: 14.7.)
 __device__ __forceinline__ uint32_t f32_to_e4m3x2(float lo, float hi) {
     uint16_t r;   // the low byte of the pair is the second source operand
     asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
@@ -957,7 +957,7 @@ __device__ __forceinline__ void append_fp8_plane(const T* __restrict__ src, uint
 // Many new rows (a prompt): grid (n_k k_parts + n_c c_parts, B) quantises, the lengths advance in the launch behind it.
 // A warp takes two key rows (times 32 / lpr) or one latent row at once: with more in flight the registers cost CTAs.
 __host__ __device__ constexpr int append_fp8_rows_at_once(int nv) { return nv < 2 ? 2 : 1; }
-template <typename T, int NV>
+template <typename T, int NK, int NV>
 __global__ void __launch_bounds__(256)
 append_fp8_bulk_kernel(AppendFp8Args a, const int32_t* __restrict__ seq_lens, int k_parts, int c_parts) {
     ptx::grid_dependency_wait();
@@ -967,10 +967,10 @@ append_fp8_bulk_kernel(AppendFp8Args a, const int32_t* __restrict__ seq_lens, in
     if (len < 0 || (long long)len + a.n_new > a.S_cap) return;
     const int k_blocks = a.n_k * k_parts;
     if ((int)blockIdx.x < k_blocks) {
-        constexpr int U = append_fp8_rows_at_once(1);
+        constexpr int U = append_fp8_rows_at_once(NK);
         const int g = blockIdx.x / k_parts, part = blockIdx.x - g * k_parts;
         const size_t plane = (size_t)b * a.n_k + g, row = plane * a.S_cap + len;
-        append_fp8_plane<T, 1, U>(static_cast<const T*>(a.k_new) + plane * a.n_new * a.d_h, a.k_codes + row * a.d_h,
+        append_fp8_plane<T, NK, U>(static_cast<const T*>(a.k_new) + plane * a.n_new * a.d_h, a.k_codes + row * a.d_h,
                                   a.k_scale + row, a.n_new, a.d_h, a.k_lpr, (part * 8 + warp) * U * (32 / a.k_lpr));
     } else {
         constexpr int U = append_fp8_rows_at_once(NV);
@@ -981,7 +981,7 @@ append_fp8_bulk_kernel(AppendFp8Args a, const int32_t* __restrict__ seq_lens, in
     }
 }
 
-template <typename T, int NV>
+template <typename T, int NK, int NV>
 static cudaError_t launch_append_fp8(const AppendFp8Args& a, int B, int32_t* seq_lens, int32_t* status_word,
                                      cudaStream_t stream, int* launches) {
     const int k_per = 32 / a.k_lpr, c_per = 32 / a.c_lpr;
@@ -996,7 +996,7 @@ static cudaError_t launch_append_fp8(const AppendFp8Args& a, int B, int32_t* seq
     cfg.numAttrs = 1;
     // one CTA per sequence up to four units per warp (its 2 - 3 us are launch and latency); beyond that the second
     // launch, about 2 us, is the smaller part
-    if (units <= 32) {
+    if (NK == 1 && units <= 32) {
         cfg.gridDim = dim3(B);
         *launches += 1;
         return cudaLaunchKernelEx(&cfg, append_fp8_small_kernel<T, NV>, a, seq_lens, status_word);
@@ -1005,22 +1005,39 @@ static cudaError_t launch_append_fp8(const AppendFp8Args& a, int B, int32_t* seq
         const int rows = 8 * per * append_fp8_rows_at_once(nv);
         return (a.n_new + rows - 1) / rows;
     };
-    const int k_parts = parts(k_per, 1), c_parts = parts(c_per, NV);
+    const int k_parts = parts(k_per, NK), c_parts = parts(c_per, NV);
     cfg.gridDim = dim3(a.n_k * k_parts + a.n_c * c_parts, B);
-    cudaError_t err = cudaLaunchKernelEx(&cfg, append_fp8_bulk_kernel<T, NV>, a, (const int32_t*)seq_lens, k_parts, c_parts);
+    cudaError_t err = cudaLaunchKernelEx(&cfg, append_fp8_bulk_kernel<T, NK, NV>, a, (const int32_t*)seq_lens, k_parts, c_parts);
     if (err != cudaSuccess) return err;
     *launches += 2;
     return launch_append_advance(B, a.S_cap, a.n_new, seq_lens, status_word, stream);
 }
 
+// Lanes of a row of `width` elements with up to `pieces` pieces each (d_h <= 256; latent rows up to 8 pieces a lane).
+static int append_fp8_lanes(int width, int pieces) {
+    int n = 1;
+    while (n < 32 && n * 8 * pieces < width) n *= 2;
+    return n;
+}
+
 template <typename T>
-static cudaError_t launch_append_fp8_typed(const AppendFp8Args& a, int B, int32_t* seq_lens, int32_t* status_word,
+static cudaError_t launch_append_fp8_typed(AppendFp8Args a, int B, int32_t* seq_lens, int32_t* status_word,
                                            cudaStream_t stream, int* launches) {
+    // Long prompts: four pieces per lane, so that what a row costs whatever its width -- its largest element among the lanes, its
+    // scale, the reciprocal, addresses -- is spent on fewer lanes of more elements (us, one piece of a key row and up to four of a
+    // latent row per lane / four of both: 25 MB 11.1 / 9.1, 101 MB 33.0 / 24.4, 202 MB with rows of 1024 53.5 / 43.9, 10 MB of the 1B
+    // layer 6.7 / 5.5; 6 MB 5.3 / 5.3, 2 MB 4.6 / 4.8).
+    const long long elements = (long long)B * a.n_new * (a.n_k * a.d_h + a.n_c * a.d_l);
+    if (elements >= 3 << 20 && a.d_l <= 1024) {
+        a.k_lpr = append_fp8_lanes(a.d_h, 4);
+        a.c_lpr = append_fp8_lanes(a.d_l, 4);
+        return launch_append_fp8<T, 4, 4>(a, B, seq_lens, status_word, stream, launches);
+    }
     const int nv = (a.d_l / 8 + a.c_lpr - 1) / a.c_lpr;     // 8-element pieces per lane of a latent row
-    if (nv <= 1) return launch_append_fp8<T, 1>(a, B, seq_lens, status_word, stream, launches);
-    if (nv <= 2) return launch_append_fp8<T, 2>(a, B, seq_lens, status_word, stream, launches);
-    if (nv <= 4) return launch_append_fp8<T, 4>(a, B, seq_lens, status_word, stream, launches);
-    return launch_append_fp8<T, 8>(a, B, seq_lens, status_word, stream, launches);
+    if (nv <= 1) return launch_append_fp8<T, 1, 1>(a, B, seq_lens, status_word, stream, launches);
+    if (nv <= 2) return launch_append_fp8<T, 1, 2>(a, B, seq_lens, status_word, stream, launches);
+    if (nv <= 4) return launch_append_fp8<T, 1, 4>(a, B, seq_lens, status_word, stream, launches);
+    return launch_append_fp8<T, 1, 8>(a, B, seq_lens, status_word, stream, launches);
 }
 
 cudaError_t launch_cache_append_fp8(const Dims& d, int dtype, void* k_codes, void* c_codes, float* k_scale,
@@ -1031,13 +1048,8 @@ cudaError_t launch_cache_append_fp8(const Dims& d, int dtype, void* k_codes, voi
     a.k_scale = k_scale; a.c_scale = c_scale;
     a.k_new = k_new; a.c_new = c_new;
     a.n_k = d.n_k; a.n_c = d.n_c; a.d_h = d.d_h; a.d_l = d.d_l; a.S_cap = S_cap; a.n_new = n_new;
-    const auto lanes = [](int width) {       // d_h <= 256: one piece per lane; latent rows up to 8 pieces
-        int n = 1;
-        while (n < 32 && n * 8 < width) n *= 2;
-        return n;
-    };
-    a.k_lpr = lanes(d.d_h);
-    a.c_lpr = lanes(d.d_l);
+    a.k_lpr = append_fp8_lanes(d.d_h, 1);
+    a.c_lpr = append_fp8_lanes(d.d_l, 1);
     if (dtype == GTA_F32) return launch_append_fp8_typed<float>(a, d.B, seq_lens, status_word, stream, launches);
     return launch_append_fp8_typed<__nv_bfloat16>(a, d.B, seq_lens, status_word, stream, launches);
 }
