@@ -39,6 +39,11 @@ gta_status_t launch_sm100_decoder_fine(const Dims& d, const void* l_planes, cons
                                        void* out, int32_t* status_word, cudaStream_t stream, bool release = true,
                                        bool behind = true);
 
+// The fp32 kernels below take an operand as three bf16 pieces.  bf16 ends at 2^-133, so an element below 2^-110 loses what it has
+// below that: at most 2^-133.  Where the largest element of its row (or column of the weights) is no smaller than this, that is
+// 2^-43 of it and less than the sums over the row round; rows and columns of smaller ones are done again with FMAs.
+constexpr float kPiecesFloor = 0x1p-90f;
+
 // Attention of an fp32 call on the tensor cores (gta_sm100_f32_attention.cu): d_h = 64, d_l a multiple of 128, contiguous K and
 // C; L fp32 [n_q, B, N, d_l]; scratch of the given size (256-byte aligned) for the pieces of K and C; split: CTAs (1, 2 or
 // 4) that share the keys of a row tile.

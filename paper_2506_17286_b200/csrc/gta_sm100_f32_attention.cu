@@ -1,7 +1,7 @@
 // fp32 attention on the tensor cores (head width 64): L = Softmax(scale Q K^T) C per attention map.
 //
-// Operands are sums of three bf16 pieces, exactly, and six of the nine products of pieces are taken (what is left out is below
-// 2^-25 of a product); see gta_sm100_f32_decoder.cu.  A sum stays in tensor memory for 64 elements of its contraction
+// Operands are sums of three bf16 pieces, exactly from 2^-110 on, and six of the nine products of pieces are taken (what is left
+// out is below 2^-24 of a product, 2^-26.5 rms); see gta_sm100_f32_decoder.cu.  A sum stays in tensor memory for 64 elements of its contraction
 // (the head width; the keys of a tile), small products first, and is added up in registers (rounded) from there.
 //   split_rows_kernel        writes the pieces of K and C once ([piece][row], bf16, workspace), and per tile of 64
 //                            rows the first that holds an element without pieces: every map and row tile reads them.
@@ -17,7 +17,8 @@
 //
 // An element that is infinite, not a number or rounds to infinity in bf16 has no pieces.  In K and C zeros stand in for it, so
 // that rows which do not see it keep their bits (0 x infinity); the rows that do, and the rows of Q that hold one, are done
-// again with plain FMAs.
+// again with plain FMAs.  So are those that see, or are, a row of elements too small for pieces (kPiecesFloor).  A probability
+// is taken against the largest of its row so far: one below 2^-110 of it loses at most 2^-134 of it.
 #include "gta_sm100.cuh"
 
 #include <cuda.h>
@@ -45,28 +46,34 @@ constexpr int kIssueRegs = 48, kSoftRegs = 104, kAddRegs = 112;
 constexpr uint32_t kTmS = 0, kTmSP = 96, kTmQ = 192, kTmO = 320;      // [2] 64 columns of scores or 96 of P; Q 96; O 128
 
 // ---------------------------------------------------------------------------------------------
-// Pieces of four floats; not-a-number in `rest` where they do not add up to them.
-struct Pieces { uint2 p[3]; uint64_t rest; };
+// Pieces of four floats.  What two pieces leave of a number has eight bits, which are the upper half of its word; the lower half
+// of `rest` (an OR over the four) is not zero where one leaves more: it ends below bf16's range, or has no pieces.
+struct Pieces { uint2 p[3]; uint32_t rest; };
 __device__ __forceinline__ Pieces split4(uint64_t r0, uint64_t r1) {
     Pieces o;
+    float a, b, e, f;
 #pragma unroll
-    for (int p = 0; p < 3; ++p) {
-        float a, b, e, f;
+    for (int p = 0; p < 2; ++p) {
         ptx::f32x2_split(r0, a, b);
         ptx::f32x2_split(r1, e, f);
         o.p[p] = make_uint2(ptx::cvt_bf16x2(a, b), ptx::cvt_bf16x2(e, f));
-        if (p < 2) {
-            r0 = ptx::sub2(r0, ptx::f32x2(__uint_as_float(o.p[p].x << 16), __uint_as_float(o.p[p].x & 0xffff0000u)));
-            r1 = ptx::sub2(r1, ptx::f32x2(__uint_as_float(o.p[p].y << 16), __uint_as_float(o.p[p].y & 0xffff0000u)));
-        }
+        r0 = ptx::sub2(r0, ptx::f32x2(__uint_as_float(o.p[p].x << 16), __uint_as_float(o.p[p].x & 0xffff0000u)));
+        r1 = ptx::sub2(r1, ptx::f32x2(__uint_as_float(o.p[p].y << 16), __uint_as_float(o.p[p].y & 0xffff0000u)));
     }
-    o.rest = ptx::add2(r0, r1);
+    ptx::f32x2_split(r0, a, b);
+    ptx::f32x2_split(r1, e, f);
+    o.p[2] = make_uint2(ptx::upper_halves(__float_as_uint(a), __float_as_uint(b)), ptx::upper_halves(__float_as_uint(e), __float_as_uint(f)));
+    o.rest = __float_as_uint(a) | __float_as_uint(b) | __float_as_uint(e) | __float_as_uint(f);
     return o;
 }
-__device__ __forceinline__ bool is_nan2(uint64_t v) {
-    float a, b;
-    ptx::f32x2_split(v, a, b);
-    return a != a || b != b;
+// Does what its pieces do not add up to matter to a row: has it an element without pieces, or small ones alone?
+__device__ __noinline__ bool is_odd_row(const float* row, int width) {
+    float mx = 0.f;
+    for (int e = 0; e < width; ++e) {
+        if (!(fabsf(row[e]) < 3.3895e38f)) return true;
+        mx = fmaxf(mx, fabsf(row[e]));
+    }
+    return mx < kPiecesFloor;
 }
 
 // The pair with zeros for what has no pieces (3.3895e38 is bf16's largest).
@@ -93,16 +100,24 @@ split_rows_kernel(Dims d, const float* __restrict__ k, const float* __restrict__
     __shared__ int first;
     if (threadIdx.x == 0) first = INT32_MAX;
     __syncthreads();
-#pragma unroll 4
-    for (int i = threadIdx.x; i < live; i += 256) {
-        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(src) + i);
-        Pieces s = split4(v.x, v.y);
-        if (is_nan2(s.rest)) {
-            atomicMin(&first, tile * kKeys + i / vecs);
-            s = split4(whole2(v.x), whole2(v.y));
-        }
+    // (four loads ahead of the stores, which the compiler cannot move them across)
+    for (int i0 = threadIdx.x; i0 < live; i0 += 4 * 256) {
+        ulonglong2 v[4];
 #pragma unroll
-        for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(dst + (size_t)p * n_rows * width * 2 + (size_t)i * 8) = s.p[p];
+        for (int u = 0; u < 4; ++u)
+            if (i0 + 256 * u < live) v[u] = __ldg(reinterpret_cast<const ulonglong2*>(src) + i0 + 256 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 256 * u;
+            if (i >= live) break;
+            Pieces s = split4(v[u].x, v[u].y);
+            if ((s.rest & 0xffffu) != 0u) {
+                if (is_odd_row(src + (size_t)(i / vecs) * width, width)) atomicMin(&first, tile * kKeys + i / vecs);
+                s = split4(whole2(v[u].x), whole2(v[u].y));
+            }
+#pragma unroll
+            for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(dst + (size_t)p * n_rows * width * 2 + (size_t)i * 8) = s.p[p];
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) first_odd[(size_t)blockIdx.y * tiles + tile] = first;
@@ -152,7 +167,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* drain_flag = abort_flag + 1;
-    int* odd_key = reinterpret_cast<int*>(tmem_slot + 3);                     // first key of the item without pieces
+    int* odd_key = reinterpret_cast<int*>(tmem_slot + 3);                     // first key of the item that is done again
     uint32_t* odd_rows = tmem_slot + 4;                                       // [4]: query rows, a bit each
     float* ref_s = reinterpret_cast<float*>(smem + kBarOffset + 512);        // [4][128]: the scale of a tile's P
     float* fin_m = ref_s + 4 * kRows;                                         // [2][128]
@@ -290,20 +305,20 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         {   // pieces of Q: this warpgroup's 32 elements of the row
             const ulonglong2* src = reinterpret_cast<const ulonglong2*>(q + (((size_t)b * d.n_q + g) * d.N + t0 + (row < rows ? row : 0)) * kDh + 32 * w);
             uint32_t pc[3][16];
-            bool odd = false;
+            uint32_t rest = 0u;
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
                 ulonglong2 e = __ldg(src + v);
                 if (row >= rows) e = make_ulonglong2(0ull, 0ull);
                 const Pieces s = split4(e.x, e.y);
-                odd |= is_nan2(s.rest);
+                rest |= s.rest;
 #pragma unroll
                 for (int p = 0; p < 3; ++p) { pc[p][2 * v] = s.p[p].x; pc[p][2 * v + 1] = s.p[p].y; }
             }
 #pragma unroll
             for (int p = 0; p < 3; ++p) ptx::tmem_st16(tmem + kTmQ + lane_base + p * 32 + 16 * w, pc[p]);
             ptx::tmem_wait_st();
-            if (odd) atomicOr(&odd_rows[quarter], 1u << lane);
+            if ((rest & 0xffffu) != 0u && is_odd_row(reinterpret_cast<const float*>(src) - 32 * w, kDh)) atomicOr(&odd_rows[quarter], 1u << lane);
             ptx::tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(q_full);

@@ -1,10 +1,10 @@
 // fp32 decoder + gate on the tensor cores:
 //     out_i = (L_{q(i)} W_P,i) (.) Sigmoid(X W_G,i)          (Sec. 3.3, reformulated equation)
 //
-// Every fp32 operand is the sum of three bf16 pieces, exactly (8 significant bits each, rounded to nearest, the rest handed
-// on); six of the nine products of pieces are taken (what is left out is below 2^-25 of a product), each exact in the
-// tensor core, which adds them in fp32 but cuts where fp32 arithmetic rounds.  So a sum stays in tensor memory for 32
-// elements of the contraction only, small products first, and is added up in registers (rounded) from there: against 64
+// Every fp32 operand is the sum of three bf16 pieces, exactly from 2^-110 on (8 significant bits each, rounded to nearest, the
+// rest handed on); six of the nine products of pieces are taken (what is left out, of which two can reach 2^-25 of a product
+// each, is below 2^-24 of it, 2^-26.5 rms), each exact in the tensor core, which adds them in fp32 but cuts where fp32
+// arithmetic rounds.  So a sum stays in tensor memory for 32 elements of the contraction only, small products first, and is added up in registers (rounded) from there: against 64
 // bits the result is closer than the FMA chain of the plain-ALU kernel.
 //
 // CTA pairs, one item of 256 token rows x NT output columns of one attention map per pair.
@@ -19,7 +19,8 @@
 // out, pieces in, operands read once per product: 1664 cycles); measured 1800.
 //
 // An element that is infinite, not a number or rounds to infinity in bf16 makes its row or column of the item not a number
-// (0 x infinity); the splitting threads see it, and those rows and columns are done again with plain FMAs.
+// (0 x infinity); the splitting threads see it, and those rows and columns are done again with plain FMAs.  So are rows and
+// columns whose elements are all too small for pieces (kPiecesFloor).
 #include "gta_sm100.cuh"
 
 #include <cuda.h>
@@ -78,13 +79,45 @@ template <int NT> __device__ __forceinline__ Block block_of(const Dims& d, int r
     return w;
 }
 
+// What the splitting threads found: rows and groups of four columns to be done again (`bad`), and those that hold an element which
+// its pieces do not add up to (`small`).
+template <int NT> struct Marks {
+    uint8_t row_bad[kTileM], col_bad[NT / 4], row_small[kTileM], col_small[NT / 4];
+};
+
 // The rows and columns that hold an element which the pieces cannot: plain FMAs, by the adding warps.
 template <int NT>
 __device__ __forceinline__ void redo(const Dims& d, const float* o_lat, const float* x, const float* w_p, const float* w_g, float* out,
-                                     int row_tiles, int col_tiles, uint32_t block, const uint8_t* row_bad, const uint8_t* col_bad) {
+                                     int row_tiles, int col_tiles, uint32_t block, Marks<NT>* marks) {
     const Block w = block_of<NT>(d, row_tiles, col_tiles, block);
     const size_t ldw = (size_t)d.n_h * d.d_h;
-    const int tid = threadIdx.x - 32 * kAddWarp0;
+    const int tid = threadIdx.x - 32 * kAddWarp0, warp = tid >> 5, lane = tid & 31;
+    uint8_t *row_bad = marks->row_bad, *col_bad = marks->col_bad;
+    for (int r = warp; r < w.rows; r += kAddWarps)
+        if (marks->row_small[r] && !row_bad[r]) {
+            const float* xr = x + (w.m0 + r) * d.H;
+            const float* lr = o_lat + ((size_t)w.g * d.B * d.N + w.m0 + r) * d.d_l;
+            float mx = 0.f, ml = 0.f;
+            for (int k = lane; k < d.H; k += 32) mx = fmaxf(mx, fabsf(xr[k]));
+            for (int k = lane; k < d.d_l; k += 32) ml = fmaxf(ml, fabsf(lr[k]));
+            if (fminf(warp_max(mx), warp_max(ml)) < kPiecesFloor) row_bad[r] = 1;
+        }
+    for (int c4 = warp; 4 * c4 < w.n_cols; c4 += kAddWarps)
+        if (marks->col_small[c4] && !col_bad[c4]) {
+            const int f = w.n0 + 4 * c4, head = w.g * (d.n_h / d.n_q) + f / d.d_h;       // (four columns of one head)
+            const float* wg = w_g + (size_t)w.g * w.map_cols + f;
+            const float* wp = w_p + (size_t)head * d.d_l * d.d_h + f % d.d_h;
+            float4 mg = make_float4(0.f, 0.f, 0.f, 0.f), mp = mg;
+            const auto larger = [](float4& m, const float4 v) {
+                m.x = fmaxf(m.x, fabsf(v.x)); m.y = fmaxf(m.y, fabsf(v.y)); m.z = fmaxf(m.z, fabsf(v.z)); m.w = fmaxf(m.w, fabsf(v.w));
+            };
+            for (int k = lane; k < d.H; k += 32) larger(mg, *reinterpret_cast<const float4*>(wg + k * ldw));
+            for (int k = lane; k < d.d_l; k += 32) larger(mp, *reinterpret_cast<const float4*>(wp + (size_t)k * d.d_h));
+            const float least = fminf(fminf(fminf(warp_max(mg.x), warp_max(mg.y)), fminf(warp_max(mg.z), warp_max(mg.w))),
+                                      fminf(fminf(warp_max(mp.x), warp_max(mp.y)), fminf(warp_max(mp.z), warp_max(mp.w))));
+            if (least < kPiecesFloor) col_bad[c4] = 1;
+        }
+    ptx::named_sync(3, 32 * kAddWarps);
     auto again = [&](int r, int c) {
         const long long m = w.m0 + r;
         const int f = w.n0 + c, head = w.g * (d.n_h / d.n_q) + f / d.d_h, elem = f % d.d_h;
@@ -127,8 +160,8 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* drain_flag = abort_flag + 1;
     uint32_t* any_bad = tmem_slot + 3;
-    uint8_t* row_bad = smem + C::kBarOffset + 256;                               // [128]
-    uint8_t* col_bad = row_bad + kTileM;                                         // [NT / 4]: four columns each
+    Marks<NT>* marks = reinterpret_cast<Marks<NT>*>(smem + C::kBarOffset + 256);
+    static_assert(256 + sizeof(Marks<NT>) <= 1024 && sizeof(Marks<NT>) % 4 == 0, "room behind the barriers");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();
@@ -144,7 +177,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
         *any_bad = 0;
         ptx::fence_mbar_init();
     }
-    if (threadIdx.x < (kTileM + NT / 4) / 4) reinterpret_cast<uint32_t*>(row_bad)[threadIdx.x] = 0;
+    if (threadIdx.x < sizeof(Marks<NT>) / 4) reinterpret_cast<uint32_t*>(marks)[threadIdx.x] = 0;
     if (warp == 0) ptx::tmem_alloc_pair(tmem_slot, 2 * NT);
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -232,36 +265,48 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
         // this thread's pieces: A row 32 i + tid / 8, elements 4 (tid % 8) of the block; of the i-th 16 k of the weights (64 columns
         // after 64 columns) k = tid / 16, columns 4 (tid % 16) of the 64
         const int a_row = tid >> 3, b_k = tid >> 4, b_vec = tid & 15;
-        // four floats -> 8 bytes of each piece.  0 x (what is left) tells a number from an odd one.
-        uint64_t odd = 0ull;
+        // four floats -> 8 bytes of each piece.  What two pieces leave of a number has eight bits, which are the upper half of its
+        // word; the lower half of `odd` is not zero where one leaves more: it ends below bf16's range, or has no pieces
+        uint32_t odd = 0u;
         auto split = [&](const ulonglong2 v, uint8_t* dst, uint32_t plane) {
             uint64_t r0 = v.x, r1 = v.y;
+            float a, b, e, f;
 #pragma unroll
-            for (int p = 0; p < 3; ++p) {
-                float a, b, e, f;
+            for (int p = 0; p < 2; ++p) {
                 ptx::f32x2_split(r0, a, b);
                 ptx::f32x2_split(r1, e, f);
                 const uint32_t h0 = ptx::cvt_bf16x2(a, b), h1 = ptx::cvt_bf16x2(e, f);
                 *reinterpret_cast<uint2*>(dst + p * plane) = make_uint2(h0, h1);
-                if (p < 2) {
-                    r0 = ptx::sub2(r0, ptx::f32x2(__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xffff0000u)));
-                    r1 = ptx::sub2(r1, ptx::f32x2(__uint_as_float(h1 << 16), __uint_as_float(h1 & 0xffff0000u)));
-                }
+                r0 = ptx::sub2(r0, ptx::f32x2(__uint_as_float(h0 << 16), __uint_as_float(h0 & 0xffff0000u)));
+                r1 = ptx::sub2(r1, ptx::f32x2(__uint_as_float(h1 << 16), __uint_as_float(h1 & 0xffff0000u)));
             }
-            odd = ptx::fma2(r0, 0ull, odd);
-            odd = ptx::fma2(r1, 0ull, odd);
+            ptx::f32x2_split(r0, a, b);
+            ptx::f32x2_split(r1, e, f);
+            const uint32_t wa = __float_as_uint(a), wb = __float_as_uint(b), we = __float_as_uint(e), wf = __float_as_uint(f);
+            *reinterpret_cast<uint2*>(dst + 2 * plane) = make_uint2(ptx::upper_halves(wa, wb), ptx::upper_halves(we, wf));
+            odd |= wa | wb;
+            odd |= we | wf;
         };
         auto note_odd = [&](const uint8_t* src) {
             auto is_odd = [](float v) { return !(fabsf(v) < 3.38e38f); };       // (3.3895e38 is bf16's largest)
             auto any_odd = [&](const float4 v) { return is_odd(v.x) || is_odd(v.y) || is_odd(v.z) || is_odd(v.w); };
-            for (int i = 0; i < C::kAPieces; ++i)
-                if (any_odd(*reinterpret_cast<const float4*>(src + i * kSplitThreads * 16))) { row_bad[a_row + 32 * i] = 1; *any_bad = 1; }
-            for (int i = 0; i < C::kBPieces; ++i)
-                if (any_odd(*reinterpret_cast<const float4*>(src + (C::kAPieces + i) * kSplitThreads * 16)))
+            auto is_small = [](float v) { return v != 0.f && fabsf(v) < 0x1p-109f; };
+            auto any_small = [&](const float4 v) { return is_small(v.x) || is_small(v.y) || is_small(v.z) || is_small(v.w); };
+            for (int i = 0; i < C::kAPieces; ++i) {
+                const float4 v = *reinterpret_cast<const float4*>(src + i * kSplitThreads * 16);
+                if (any_odd(v)) { marks->row_bad[a_row + 32 * i] = 1; *any_bad = 1; }
+                else if (any_small(v)) { marks->row_small[a_row + 32 * i] = 1; *any_bad = 1; }
+            }
+            for (int i = 0; i < C::kBPieces; ++i) {
+                const float4 v = *reinterpret_cast<const float4*>(src + (C::kAPieces + i) * kSplitThreads * 16);
+                const bool bad = any_odd(v);
+                if (bad || any_small(v))
                     for (uint32_t r = 0; r < 2; ++r) {       // both CTAs have these columns
-                        ptx::st_cluster_u8(ptx::map_to_cta(ptx::smem_addr(col_bad + rank * (C::kCols / 4) + (i >> 1) * 16 + b_vec), r), 1);
+                        uint8_t* mark = (bad ? marks->col_bad : marks->col_small) + rank * (C::kCols / 4) + (i >> 1) * 16 + b_vec;
+                        ptx::st_cluster_u8(ptx::map_to_cta(ptx::smem_addr(mark), r), 1);
                         ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_addr(any_bad), r), 1);
                     }
+            }
         };
         // where the pieces go: A rows of 64 bytes (64-byte swizzle), weights [64 columns][k][128 bytes] (128-byte swizzle); rows 32 i
         // and k 16 i apart have the same swizzle
@@ -289,9 +334,9 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
                     if (i < C::kAPieces) split(v[i & 3], st + a_dst + i * 32 * 64, kAPlane);
                     else split(v[i & 3], st + b_dst + (i - C::kAPieces) * 16 * 128, C::kBPlane);
             }
-            if (!(odd == 0ull || odd == 0x8000000000000000ull || odd == 0x80000000ull || odd == 0x8000000080000000ull)) {
+            if ((odd & 0xffffu) != 0u) {
                 note_odd(src);
-                odd = 0ull;
+                odd = 0u;
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();
@@ -407,7 +452,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
     if (warp >= kAddWarp0 && *any_bad) {
         uint32_t block;             // (worked out anew: nothing of this is kept in registers until here)
         asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
-        redo<NT>(d, o_lat, x, w_p, w_g, out, row_tiles, col_tiles, block, row_bad, col_bad);
+        redo<NT>(d, o_lat, x, w_p, w_g, out, row_tiles, col_tiles, block, marks);
     }
     if (threadIdx.x == 0 && *abort_flag) raise_status(status_word, GTA_ERR_TIMEOUT);
 }

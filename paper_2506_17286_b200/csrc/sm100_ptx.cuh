@@ -305,6 +305,12 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+// The upper halves of two words (of two fp32 values: bf16, cut): lo's in bits 0-15.
+__device__ __forceinline__ uint32_t upper_halves(uint32_t lo, uint32_t hi) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(d) : "r"(lo), "r"(hi));
+    return d;
+}
 __device__ __forceinline__ float rcp_approx(float v) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));

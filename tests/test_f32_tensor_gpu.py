@@ -8,7 +8,7 @@ from tests.parity_utils import Guarded
 
 pytestmark = pytest.mark.gpu
 
-# Pieces are exact and the products left out below 2^-25 of a product; a sum of 64 products is cut at 2^-23 of its value up to
+# Pieces are exact (from 2^-110 on) and the products left out below 2^-24 of a product, 2^-26.5 rms; a sum of 64 products is cut at 2^-23 of its value up to
 # eight times, sums are rounded to 2^-24 from there, an exponential is good to 2 ulp: 2.1e-7 measured (3.9e-7 the FMA chain).
 REL, MAX = 8e-7, 4e-5
 
@@ -111,12 +111,39 @@ def test_short_prompt_rows_before_an_odd_element_keep_their_bits(G):
 
 @pytest.mark.parametrize("size", [1e-30, 1e15])
 def test_range_of_the_pieces(G, size):
-    """Latents and decoder weights near both ends of the range: the pieces have fp32's exponents."""
+    """Latents and decoder weights far from one: the pieces have fp32's exponents."""
     t = _inputs(1, 300, 300, 64, 20, 5, 1, 1, 64, 128)
     t["c"] *= size
     t["w_p"] *= size if size > 1 else 1e3
     got, want = _run(G, t, 300, True).double(), _exact(t, 300, True)
     assert float((got - want).norm() / want.norm()) <= REL
+
+
+@pytest.mark.parametrize("small,large", [("c", "w_p"), ("w_p", "c"), ("x", "w_g"), ("w_g", "x"), ("q", "k"), ("k", "q")])
+def test_operands_too_small_for_pieces(G, small, large):
+    """At 1e-36 three pieces hold 15 bits of an element, and the other operand makes ordinary numbers of it: done again with FMAs, in
+    one chain of up to 300 (2^-24 of the sum at each step, at random: 6e-8 x 17)."""
+    t = _inputs(1, 300, 300, 64, 20, 5, 1, 1, 64, 128)
+    t[small] *= 1e-36
+    t[large] *= 1e36
+    got, want = _run(G, t, 300, True).double(), _exact(t, 300, True)
+    assert float((got - want).norm() / want.norm()) <= 2 * REL
+
+
+def test_few_small_elements_and_rows(G):
+    """Rows of the result that are made of small elements alone keep their precision; a few of them in ordinary rows and columns
+    cost none."""
+    t = _inputs(1, 300, 300, 64, 20, 5, 1, 1, 64, 128)
+    t["c"][:, :, :3] *= 1e-36
+    t["w_p"][3, :, 40:44] *= 1e-35              # (results of 1e-36: below 1.2e-38 a result, and every sum on the way, ends at 2^-149)
+    t["x"][:, 50] *= 1e-36
+    for n in ("q", "k", "c", "x", "w_p", "w_g"):
+        t[n].view(-1)[::1009] *= 1e-37
+    got, want = _run(G, t, 300, True).double(), _exact(t, 300, True)
+    err = (got - want).norm(dim=-1) / want.norm(dim=-1)           # of each token and head
+    tail = slice(3, None)                       # (1e-36 x 1e-35 is nothing)
+    err[:, tail, 3] = (got - want)[:, tail, 3, 40:44].norm(dim=-1) / want[:, tail, 3, 40:44].norm(dim=-1)
+    assert float(err.max()) <= 8 * REL          # (a head's 64 outputs, or four of them, against a row's latents)
 
 
 BAD = [("q", (0, 1, 40, 3), float("nan")), ("q", (0, 0, 299, 0), float("inf")), ("k", (0, 0, 130, 5), float("inf")),
