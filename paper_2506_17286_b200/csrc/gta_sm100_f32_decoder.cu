@@ -341,7 +341,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
             ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-                ptx::mbar_arrive_cluster(full_leader + 8 * s);
+                ptx::mbar_arrive_release_smem_cluster(full_leader + 8 * s);      // (the leader's issuing thread acquires the pieces)
                 ptx::mbar_arrive(&raw_empty[r]);
             }
             s = s + 1 == C::kStages ? 0 : s + 1;
@@ -391,7 +391,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster(free_leader + 8 * buf);
+            if (lane == 0) ptx::mbar_arrive_release_smem_cluster(free_leader + 8 * buf);
             if (it == n_g - 1) {                // the gates' sums are complete: the splitting warps make gates of them
 #pragma unroll
                 for (int ch = 0; ch < C::kCols / 16; ++ch) {

@@ -500,6 +500,12 @@ __device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t cluster_addr, ui
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// The same for shared memory alone: the fence is about this CTA's shared memory and does not wait for stores to global memory,
+// which the release above does (the fp32 decoder of 2 x 1500 tokens of the 1B layer: 52 us with this, 71 with that).
+__device__ __forceinline__ void mbar_arrive_release_smem_cluster(uint32_t cluster_addr) {
+    asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
 __device__ __forceinline__ void st_cluster_u8(uint32_t cluster_addr, uint32_t v) {
     asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
