@@ -508,10 +508,11 @@ GTA_API int gta_last_launch_count(void);
  * that waits longer than a time limit gives up, tells the other threads of its CTA and of its
  * cluster, the kernel unwinds (outstanding copies and MMAs are waited for, tensor memory is
  * freed), raises GTA_ERR_TIMEOUT in the status word and returns; the context stays usable.
- * This call lets a test exercise that path of the tensor-core attention kernel on a healthy
- * GPU: limit_ns replaces the limit of its waits (0 = the built-in two seconds), and with
- * withhold_first_arrive != 0 one softmax warp of every CTA pair keeps its first arrival to
- * itself, so that the first sum of every pair is never released and the limit runs out.
+ * This call lets a test exercise that path of the prefill kernels on a healthy GPU: limit_ns
+ * replaces the limit of their waits (0 = the built-in two seconds), and with
+ * withhold_first_arrive != 0 the limit runs out: one softmax warp of every CTA pair of the
+ * tensor-core attention kernel keeps its first arrival to itself, so that the first sum of every
+ * pair is never released, and the kernel of short fp32 prompts does not ask for its first latents.
  * The settings live in device memory of the current device and hold for later launches on it
  * until they are changed back; the call synchronises the device.  Not for production use.
  */

@@ -182,7 +182,7 @@ def debug_decode_wait(limit_ns: int = 0, withhold_first_arrive: bool = False) ->
 
 def debug_attention_wait(limit_ns: int = 0, withhold_first_arrive: bool = False) -> None:
     """Test hook: time limit of the attention kernel's bounded waits (0 = built-in) and the switch that
-    makes the first sum of every CTA pair wait in vain (see gta_debug_attention_wait in include/gta.h)."""
+    makes the first hand-over of the prefill kernels wait in vain (see gta_debug_attention_wait in include/gta.h)."""
     st = lib().gta_debug_attention_wait(int(limit_ns), int(bool(withhold_first_arrive)))
     if st != GTA_OK:
         raise GtaError(st, "gta_debug_attention_wait")

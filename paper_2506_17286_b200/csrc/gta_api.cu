@@ -111,7 +111,9 @@ int gta_last_launch_count(void) { return g_last_launches; }
 gta_status_t gta_debug_attention_wait(uint64_t limit_ns, int32_t withhold_first_arrive) {
     gta_status_t st = check_device();
     if (st != GTA_OK) return st;
-    return gta::sm100_attention_debug_wait(limit_ns, withhold_first_arrive);
+    st = gta::sm100_attention_debug_wait(limit_ns, withhold_first_arrive);
+    if (st != GTA_OK) return st;
+    return gta::short_prefill_debug_wait(limit_ns, withhold_first_arrive);
 }
 
 gta_status_t gta_debug_decode_wait(uint64_t limit_ns, int32_t withhold_first_arrive) {

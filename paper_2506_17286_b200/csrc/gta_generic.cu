@@ -83,10 +83,15 @@ __host__ __device__ inline AttnSmem attn_smem(int d_h, int rows, int tile_keys, 
 
 // DH: the head width where it is a compile-time constant, 0 otherwise.  Rows t0 .. of map g of sequence b, latent columns col0 ..;
 // `tid` of the 32 QW SW threads, which `sync` brings together; put(row, float4 column, v) takes the normalised sums.
-// bulk != nullptr (fp32, contiguous caches, d_l = 64 NC): a latent tile is one bulk copy, counted on the barrier there.
-struct BulkLatents { uint64_t* bar; volatile int* abort_flag; };
+// bulk != nullptr (fp32, contiguous caches, d_l = 64 NC): a latent tile is one bulk copy, counted on the barrier there.  `armed`: how
+// many copies thread 0 has asked for; none once a wait has given up, behind which the copy before may still be on its way.
+struct BulkLatents { uint64_t* bar; volatile int* abort_flag; int armed; };
+// Test hook of the bounded waits of short_prefill_f32_kernel (gta_debug_attention_wait): their time limit, and a switch that keeps
+// the first latents back.
+struct ShortWait { unsigned long long limit_ns; int withhold; };
+static __constant__ ShortWait c_short_wait = {ptx::kWaitLimitNs, 0};
 template <typename T, int QW, int SW, int NC, int DH, typename Sync, typename Put>
-__device__ __forceinline__ void attention_tile(const BulkLatents* bulk, const Dims& d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
+__device__ __forceinline__ void attention_tile(BulkLatents* bulk, const Dims& d, const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ c,
                                                const PageMap& pm, int32_t* status_word, float* smem, int tid, int t0, int col0, int g,
                                                int b, Sync sync, Put put) {
     constexpr int kWarps = QW * SW, kThreads = 32 * kWarps;
@@ -142,7 +147,8 @@ __device__ __forceinline__ void attention_tile(const BulkLatents* bulk, const Di
         const int j0 = it * kTile;
         if (bulk != nullptr) {
             const int n = min(kTile, n_keys - j0);
-            if (tid == 0) {
+            if (tid == 0 && *bulk->abort_flag == 0 && !(it == 0 && c_short_wait.withhold != 0)) {
+                ++bulk->armed;
                 ptx::fence_proxy_async_smem();           // (the memory has been read by ordinary loads)
                 ptx::mbar_arrive_expect_tx(bulk->bar, (uint32_t)(n * kCols * 4));
                 ptx::bulk_load_1d(c_s, c_plane + (size_t)j0 * kCols, (uint32_t)(n * kCols * 4), bulk->bar);
@@ -269,7 +275,7 @@ __device__ __forceinline__ void attention_tile(const BulkLatents* bulk, const Di
                 }
             }
         }
-        if (bulk != nullptr) ptx::mbar_wait(bulk->bar, it & 1, bulk->abort_flag);
+        if (bulk != nullptr) ptx::mbar_wait_sleep(bulk->bar, it & 1, bulk->abort_flag, 0, c_short_wait.limit_ns);
         cp_async_wait<0>();
         sync();                 // the latent tile is there, the key tile has been used
         if (it + 1 < n_iter) load_keys(it + 1);
@@ -616,8 +622,8 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc_g[i][j] = acc_p[i][j] = 0ull;
 
+    BulkLatents bars{&latent_bar, abort_flag, 0};
     if (warp < 4) {
-        const BulkLatents bars{&latent_bar, abort_flag};
         attention_tile<float, 1, 4, 2, 64>(
             &bars, d, q, k, c, PageMap(), nullptr, smem, tid, t0, 0, g, b, [] { ptx::named_sync(1, 128); },
             [&](int r, int v4, const float4 v) { *reinterpret_cast<float4*>(l_s + r * kShortLdL + 4 * v4) = v; });
@@ -664,7 +670,7 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
             multiply16(as + 16 * (warp - 4), kShortLdA, as + 16 * kShortLdA + 16 * (warp - 4) * 64, acc_g);
         }
         cp_async_wait<0>();
-        ptx::mbar_wait(&wp_bar, 0, abort_flag);
+        ptx::mbar_wait_sleep(&wp_bar, 0, abort_flag, 0, c_short_wait.limit_ns);
     }
     __syncthreads();
     multiply16(l_s + 16 * warp, kShortLdL, wp_s + 16 * warp * 64, acc_p);
@@ -698,8 +704,7 @@ short_prefill_f32_kernel(Dims d, const float* __restrict__ q, const float* __res
     ptx::f32x2_split(s1, z[2], z[3]);
     if (tid == 0 && *abort_flag) {           // a wait gave up: whatever is still on its way lands before the CTA leaves
         int gave_up = 0;
-        const int n_iter = ((d.causal ? min(t0 + rows + d.Nk - d.N, d.Nk) : d.Nk) + 4 * kAttnKeys - 1) / (4 * kAttnKeys);
-        ptx::mbar_wait_drain(&latent_bar, (n_iter - 1) & 1, &gave_up);
+        if (bars.armed > 0) ptx::mbar_wait_drain(&latent_bar, (bars.armed - 1) & 1, &gave_up);
         ptx::mbar_wait_drain(&wp_bar, 0, &gave_up);
         raise_status(status_word, GTA_ERR_TIMEOUT);
     }
@@ -802,6 +807,13 @@ static F32Plan f32_plan(const Dims& d, const PageMap& pm, size_t room) {
         if (plan.split == 0 || total < best) { best = total; plan.split = split; }
     }
     return plan;
+}
+
+gta_status_t short_prefill_debug_wait(unsigned long long limit_ns, int withhold_first_arrive) {
+    const ShortWait w = {limit_ns ? limit_ns : ptx::kWaitLimitNs, withhold_first_arrive ? 1 : 0};
+    if (cudaMemcpyToSymbol(c_short_wait, &w, sizeof(w)) == cudaSuccess) return GTA_OK;
+    cudaGetLastError();
+    return GTA_ERR_CUDA;
 }
 
 template <typename T>

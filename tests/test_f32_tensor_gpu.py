@@ -109,6 +109,26 @@ def test_short_prompt_rows_before_an_odd_element_keep_their_bits(G):
     assert torch.equal(_run(G, t, 100, True)[:, :41], want[:, :41])
 
 
+def _times_out(G, t, N):
+    """With the first hand-over withheld and a limit of 2 ms the call comes back with GTA_ERR_TIMEOUT, and the next ordinary call gives
+    bit for bit what the call before gave."""
+    want = _run(G, t, N, True).clone()
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    G.debug_attention_wait(limit_ns=2_000_000, withhold_first_arrive=True)
+    try:
+        G.gta_prefill(t["q"], t["k"], t["c"], t["x"], t["w_p"], t["w_g"], status_word=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == G.GTA_ERR_TIMEOUT
+    finally:
+        G.debug_attention_wait()
+    assert torch.equal(_run(G, t, N, True).view(torch.int32), want.view(torch.int32))
+
+
+@pytest.mark.parametrize("N", [100, 170])       # one key tile; two, the second of which must not be asked for any more
+def test_a_wait_that_runs_out_unwinds_the_short_prompt_kernel(G, N):
+    _times_out(G, _inputs(1, N, N, 256, 4, 2, 2, 1, 64, 128), N)
+
+
 @pytest.mark.parametrize("size", [1e-30, 1e15])
 def test_range_of_the_pieces(G, size):
     """Latents and decoder weights far from one: the pieces have fp32's exponents."""
