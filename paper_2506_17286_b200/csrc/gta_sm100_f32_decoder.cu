@@ -201,6 +201,8 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
             uint32_t ph = 0;
             for (int it = 0; it < n_it; ++it, s = (s + 1 == C::kStages) ? 0 : s + 1, ph ^= (s == 0)) {
                 const int buf = buf_of(it);
+                if (it == n_g) ptx::grid_dependency_wait();      // (every waiting role: how long the attention kernel takes is not bounded
+                                                                 // by the waits' limit, and the CTA does not end before it)
                 ok = ptx::mbar_wait(&acc_free[buf], (use_of(it) & 1) ^ 1, abort_flag) && ptx::mbar_wait(&full_bar[s], ph, abort_flag);
                 if (!ok) break;
                 ptx::mbar_try_wait_acquire_cluster(&full_bar[s], ph);    // (both CTAs' pieces, written by ordinary stores)
@@ -317,6 +319,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
         int s = 0, r = 0;
         uint32_t ph = 1, raw_ph = 0;
         for (int it = 0; it < n_it; ++it) {
+            if (it == n_g) ptx::grid_dependency_wait();
             ptx::mbar_wait(&raw_full[r], raw_ph, abort_flag);
             ptx::mbar_wait(&empty_bar[s], ph, abort_flag);
             __syncwarp();
@@ -377,6 +380,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
         for (int e = 0; e < C::kCols / 2; ++e) acc[e] = 0ull;
         for (int it = 0; it < n_it; ++it) {
             const int buf = buf_of(it);
+            if (it == n_g) ptx::grid_dependency_wait();
             ptx::mbar_wait(&acc_full[buf], use_of(it) & 1, abort_flag);
             __syncwarp();
             ptx::tc_fence_after_sync();
