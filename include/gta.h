@@ -512,7 +512,9 @@ GTA_API int gta_last_launch_count(void);
  * replaces the limit of their waits (0 = the built-in two seconds), and with
  * withhold_first_arrive != 0 the limit runs out: one softmax warp of every CTA pair of the
  * tensor-core attention kernel keeps its first arrival to itself, so that the first sum of every
- * pair is never released, and the kernel of short fp32 prompts does not ask for its first latents.
+ * pair is never released, a softmax warp of the fp32 one does the same, the fp32 decoder kernel
+ * keeps its first sums' completion to itself, and the kernel of short fp32 prompts does not ask for
+ * its first latents.
  * The settings live in device memory of the current device and hold for later launches on it
  * until they are changed back; the call synchronises the device.  Not for production use.
  */

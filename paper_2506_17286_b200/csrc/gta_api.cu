@@ -113,7 +113,11 @@ gta_status_t gta_debug_attention_wait(uint64_t limit_ns, int32_t withhold_first_
     if (st != GTA_OK) return st;
     st = gta::sm100_attention_debug_wait(limit_ns, withhold_first_arrive);
     if (st != GTA_OK) return st;
-    return gta::short_prefill_debug_wait(limit_ns, withhold_first_arrive);
+    st = gta::short_prefill_debug_wait(limit_ns, withhold_first_arrive);
+    if (st != GTA_OK) return st;
+    st = gta::sm100_attention_f32_debug_wait(limit_ns, withhold_first_arrive);
+    if (st != GTA_OK) return st;
+    return gta::sm100_decoder_f32_debug_wait(limit_ns, withhold_first_arrive);
 }
 
 gta_status_t gta_debug_decode_wait(uint64_t limit_ns, int32_t withhold_first_arrive) {

@@ -27,6 +27,8 @@ gta_status_t launch_sm100_attention(const Dims& d, const void* q, const void* k,
 // Test hooks of the attention kernels' bounded waits (see gta_debug_attention_wait in gta.h).
 gta_status_t sm100_attention_debug_wait(unsigned long long limit_ns, int withhold_first_arrive);
 gta_status_t short_prefill_debug_wait(unsigned long long limit_ns, int withhold_first_arrive);
+gta_status_t sm100_attention_f32_debug_wait(unsigned long long limit_ns, int withhold_first_arrive);
+gta_status_t sm100_decoder_f32_debug_wait(unsigned long long limit_ns, int withhold_first_arrive);
 
 // Decoder + gate kernel alone: out = (L W_P) (.) sigmoid(X W_G) with L[B, n_q, N, d_l] in bf16.
 // step_lens (optional; the fused append + decode step): lengths that the kernel advances by one, where there is room

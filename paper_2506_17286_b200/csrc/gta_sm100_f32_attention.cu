@@ -145,6 +145,11 @@ __device__ __forceinline__ void plain_row(const Dims& d, const float* __restrict
     reinterpret_cast<float4*>(out)[lane] = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
 }
 
+// Test hook of the bounded waits (gta_debug_attention_wait): their time limit, and a switch that makes one softmax warp keep its first
+// arrival to itself.
+struct WaitHook { unsigned long long limit_ns; int withhold; };
+static __constant__ WaitHook c_wait = {ptx::kWaitLimitNs, 0};
+
 template <int SW>
 __global__ void __launch_bounds__(kThreads, 1)
 sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_c,
@@ -204,6 +209,8 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
     const uint32_t tmem = *tmem_slot;
     ptx::grid_launch_dependents();       // (the decoder kernel's gates may start as SMs free up)
 
+    const auto wait = [&](uint64_t* bar, uint32_t parity) { return ptx::mbar_wait_sleep(bar, parity, abort_flag, 0, c_wait.limit_ns); };
+
     if (warp < kSoftWarp0) {
         ptx::set_max_regs_dec<kIssueRegs>();
         if (warp == 0 && ptx::elect_one()) {
@@ -214,13 +221,13 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             int i = 0, s = 0;
             uint32_t ph = 1;
             for (; i < n_my; ++i) {
-                ok = ptx::mbar_wait(&k_empty[s], ph, abort_flag);
+                ok = wait(&k_empty[s], ph);
                 if (!ok) break;
                 const int j0 = (rank + SW * i) * kKeys;
                 uint8_t* st = smem + s * kStageBytes;
                 ptx::mbar_arrive_expect_tx(&k_full[s], 3 * kKPlane);
                 for (int p = 0; p < 3; ++p) ptx::tma_load_3d(st + p * kKPlane, &tm_k, &k_full[s], 0, j0, p * d.B * d.n_k + k_plane);
-                ok = ptx::mbar_wait(&c_empty[s], ph, abort_flag);
+                ok = wait(&c_empty[s], ph);
                 if (!ok) { ++i; c_last = false; break; }
                 ptx::mbar_arrive_expect_tx(&c_full[s], 3 * kCPlane);
                 for (int p = 0; p < 3; ++p)
@@ -230,11 +237,11 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 s = s + 1 == kStages ? 0 : s + 1;
                 ph ^= s == 0;
             }
-            if (!ok)                     // every armed tile either lands or the wait gives up
-                for (int back = 1; back <= kStages && i - back >= 0; ++back) {
-                    ptx::mbar_wait_drain(&k_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
-                    if (back > 1 || c_last) ptx::mbar_wait_drain(&c_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
-                }
+            // every armed tile lands (or the wait gives up) before this thread is done: others may give up behind its last wait
+            for (int back = 1; back <= kStages && i - back >= 0; ++back) {
+                ptx::mbar_wait_drain(&k_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
+                if (back > 1 || c_last) ptx::mbar_wait_drain(&c_full[(i - back) % kStages], ((i - back) / kStages) & 1, drain_flag);
+            }
         } else if (warp == 1 && ptx::elect_one()) {
             const uint32_t idesc_s = ptx::make_idesc_bf16(kRows, kKeys, 0, 0), idesc_o = ptx::make_idesc_bf16(kRows, 64, 0, 1);
             const uint64_t k_desc = ptx::make_smem_desc(ptx::smem_addr(smem), 16, 1024);
@@ -246,7 +253,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             uint32_t phs = 0;
             // (the scores of i - 2 have been read and their P used: both by MMAs and waits before)
             auto scores = [&](int i) {
-                ok = ptx::mbar_wait(&k_full[ss], phs, abort_flag);
+                ok = wait(&k_full[ss], phs);
                 if (!ok) return;
                 ptx::tc_fence_after_sync();
                 const uint32_t lo = k_lo0 + ss * (kStageBytes >> 4);
@@ -261,17 +268,17 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 phs ^= ss == 0;
             };
             if (n_my > 0) {
-                ok = ptx::mbar_wait(q_full, 0, abort_flag);
+                ok = wait(q_full, 0);
                 if (ok) scores(0);
                 if (ok && n_my > 1) scores(1);
             }
             for (int i = 0; i < n_my && ok; ++i) {
-                ok = ptx::mbar_wait(&p_full[i & 1], (i >> 1) & 1, abort_flag);      // (and the latents are there)
+                ok = wait(&p_full[i & 1], (i >> 1) & 1);      // (and the latents are there)
                 if (!ok) break;
                 const uint32_t lo = c_lo0 + so * (kStageBytes >> 4);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    ok = ptx::mbar_wait(&o_free[h], (i & 1) ^ 1, abort_flag);
+                    ok = wait(&o_free[h], (i & 1) ^ 1);
                     if (!ok) break;
                     ptx::tc_fence_after_sync();
 #pragma unroll
@@ -287,10 +294,9 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
                 so = so + 1 == kStages ? 0 : so + 1;
                 if (i + 2 < n_my) scores(i + 2);
             }
-            if (!ok) {                   // tensor memory is freed below: nothing may be on its way there
-                ptx::tc_commit(drain_bar);
-                ptx::mbar_wait_drain(drain_bar, 0, drain_flag);
-            }
+            // tensor memory is freed below: nothing may be on its way there, also where others give up behind this thread's last wait
+            ptx::tc_commit(drain_bar);
+            ptx::mbar_wait_drain(drain_bar, 0, drain_flag);
         }
         __syncwarp();
         if constexpr (SW > 1) {
@@ -338,7 +344,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
         // (a wait that has given up makes every later one return at once: the loops run to their end on meaningless data)
         for (int i = w; i < n_my; i += 2) {
             const int j0 = (rank + SW * i) * kKeys;
-            ptx::mbar_wait(&s_full[w], (i >> 1) & 1, abort_flag);
+            wait(&s_full[w], (i >> 1) & 1);
             __syncwarp();
             ptx::tc_fence_after_sync();
             const int st = i % kStages;
@@ -394,9 +400,9 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             }
             ptx::tmem_wait_st();
             ptx::tc_fence_before_sync();
-            ptx::mbar_wait(&c_full[st], st_ph, abort_flag);
+            wait(&c_full[st], st_ph);
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&p_full[w]);
+            if (lane == 0 && !(i == 0 && quarter == 0 && rank == 0 && c_wait.withhold != 0)) ptx::mbar_arrive(&p_full[w]);
         }
         fin_m[w * kRows + row] = m;
         fin_l[w * kRows + row] = l;
@@ -414,7 +420,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 #pragma unroll
         for (int e = 0; e < kCols / 4; ++e) acc[e] = 0ull;
         for (int i = 0; i < n_my; ++i) {
-            ptx::mbar_wait(&o_full[half], i & 1, abort_flag);
+            wait(&o_full[half], i & 1);
             __syncwarp();
             if (half == 1 && lane == 0) ptx::mbar_arrive(&c_empty[i % kStages]);
             ptx::tc_fence_after_sync();
@@ -535,6 +541,13 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 }  // namespace
+
+gta_status_t sm100_attention_f32_debug_wait(unsigned long long limit_ns, int withhold_first_arrive) {
+    const WaitHook w = {limit_ns ? limit_ns : ptx::kWaitLimitNs, withhold_first_arrive ? 1 : 0};
+    if (cudaMemcpyToSymbol(c_wait, &w, sizeof(w)) == cudaSuccess) return GTA_OK;
+    cudaGetLastError();
+    return GTA_ERR_CUDA;
+}
 
 bool sm100_attention_f32_supported(const Dims& d) {
     const long long ctas = 4ll * ((d.N + kRows - 1) / kRows) * (d.d_l / kCols) * d.n_q * d.B;

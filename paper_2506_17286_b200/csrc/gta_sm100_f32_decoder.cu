@@ -138,6 +138,11 @@ __device__ __forceinline__ void redo(const Dims& d, const float* o_lat, const fl
             for (int i = tid; i < 4 * w.rows; i += 32 * kAddWarps) again(i >> 2, 4 * c4 + (i & 3));
 }
 
+// Test hook of the bounded waits (gta_debug_attention_wait): their time limit, and a switch that keeps the first accumulator's
+// completion from the adding warps.
+struct WaitHook { unsigned long long limit_ns; int withhold; };
+static __constant__ WaitHook c_wait = {ptx::kWaitLimitNs, 0};
+
 template <int NT>
 __global__ void __launch_bounds__(kThreads, 1)
 sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_constant__ CUtensorMap tm_x,
@@ -160,6 +165,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* drain_flag = abort_flag + 1;
     uint32_t* any_bad = tmem_slot + 3;
+    int* armed = reinterpret_cast<int*>(tmem_slot + 4);                          // blocks that were asked for
     Marks<NT>* marks = reinterpret_cast<Marks<NT>*>(smem + C::kBarOffset + 256);
     static_assert(256 + sizeof(Marks<NT>) <= 1024 && sizeof(Marks<NT>) % 4 == 0, "room behind the barriers");
 
@@ -189,6 +195,8 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
     const auto buf_of = [&](int it) { return (it < n_g ? it : n_g) & 1; };
     const auto use_of = [&](int it) { return it < n_g ? it >> 1 : (n_g >> 1) + (it - n_g); };      // how often it was used before
 
+    const auto wait = [&](uint64_t* bar, uint32_t parity) { return ptx::mbar_wait_sleep(bar, parity, abort_flag, 0, c_wait.limit_ns); };
+
     if (warp < kSplitWarp0) {
         ptx::set_max_regs_dec<kIssueRegs>();
         if (warp == 0 && rank == 0 && ptx::elect_one()) {
@@ -203,7 +211,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
                 const int buf = buf_of(it);
                 if (it == n_g) ptx::grid_dependency_wait();      // (every waiting role: how long the attention kernel takes is not bounded
                                                                  // by the waits' limit, and the CTA does not end before it)
-                ok = ptx::mbar_wait(&acc_free[buf], (use_of(it) & 1) ^ 1, abort_flag) && ptx::mbar_wait(&full_bar[s], ph, abort_flag);
+                ok = wait(&acc_free[buf], (use_of(it) & 1) ^ 1) && wait(&full_bar[s], ph);
                 if (!ok) break;
                 ptx::mbar_try_wait_acquire_cluster(&full_bar[s], ph);    // (both CTAs' pieces, written by ordinary stores)
                 ptx::tc_fence_after_sync();
@@ -217,11 +225,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
                         ptx::mma_ss_pair(d_tmem, ptx::desc_of(a_lo + ((kPa[u] * kAPlane + k2 * 32) >> 4), a_hi),
                                          ptx::desc_of(b_lo + ((kPb[u] * C::kBPlane + k2 * 16 * 128) >> 4), b_hi), idesc, (u | k2) ? 1u : 0u);
                 ptx::tc_commit_pair(&empty_bar[s], 3);
-                ptx::tc_commit_pair(&acc_full[buf], 3);
-            }
-            if (!ok) {      // tensor memory is freed below: nothing may be on its way there
-                ptx::tc_commit_pair(drain_bar, 1);
-                ptx::mbar_wait_drain(drain_bar, 0, drain_flag);
+                if (it != 0 || c_wait.withhold == 0) ptx::tc_commit_pair(&acc_full[buf], 3);
             }
         }
         if (warp == 1 && ptx::elect_one()) {
@@ -235,7 +239,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
             bool ok = true;
             int it = 0;
             for (; it < n_it; ++it) {
-                ok = ptx::mbar_wait(&raw_empty[r], ph, abort_flag);
+                ok = wait(&raw_empty[r], ph);
                 if (!ok) break;
                 const bool gate = it < n_g;
                 const int k0 = (gate ? it : it - n_g) * kBlockK;
@@ -257,9 +261,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
                 r = r + 1 == C::kRaw ? 0 : r + 1;
                 ph ^= r == 0;
             }
-            if (!ok)                             // every armed block either lands or the wait gives up
-                for (int back = 1; back <= C::kRaw && it - back >= 0; ++back)
-                    ptx::mbar_wait_drain(&raw_full[(it - back) % C::kRaw], ((it - back) / C::kRaw) & 1, drain_flag);
+            *armed = it;
         }
     } else if (warp < kAddWarp0) {
         ptx::set_max_regs_dec<kSplitRegs>();
@@ -320,8 +322,8 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
         uint32_t ph = 1, raw_ph = 0;
         for (int it = 0; it < n_it; ++it) {
             if (it == n_g) ptx::grid_dependency_wait();
-            ptx::mbar_wait(&raw_full[r], raw_ph, abort_flag);
-            ptx::mbar_wait(&empty_bar[s], ph, abort_flag);
+            wait(&raw_full[r], raw_ph);
+            wait(&empty_bar[s], ph);
             __syncwarp();
             const uint8_t* src = raw + r * C::kRawBytes + tid * 16;
             uint8_t* st = smem + s * C::kStageBytes;
@@ -381,7 +383,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
         for (int it = 0; it < n_it; ++it) {
             const int buf = buf_of(it);
             if (it == n_g) ptx::grid_dependency_wait();
-            ptx::mbar_wait(&acc_full[buf], use_of(it) & 1, abort_flag);
+            wait(&acc_full[buf], use_of(it) & 1);
             __syncwarp();
             ptx::tc_fence_after_sync();
 #pragma unroll
@@ -450,6 +452,16 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
+    if (*abort_flag) {             // a wait gave up, maybe behind the last one of the threads that issue: what is on its way comes to its end
+        if (warp == 0 && rank == 0 && ptx::elect_one()) {        // (the thread that issued the MMAs: the election is the same each time)
+            ptx::tc_commit_pair(drain_bar, 1);
+            ptx::mbar_wait_drain(drain_bar, 0, drain_flag);
+        }
+        if (warp == 1 && ptx::elect_one())
+            for (int n = *armed, back = 1; back <= C::kRaw && n - back >= 0; ++back)
+                ptx::mbar_wait_drain(&raw_full[(n - back) % C::kRaw], ((n - back) / C::kRaw) & 1, drain_flag);
+        __syncwarp();
+    }
     ptx::cluster_arrive();         // neither CTA leaves (or frees tensor memory) while the other may still signal it
     ptx::cluster_wait();
     if (warp == 0) ptx::tmem_dealloc_pair(tmem_base, 2 * NT);
@@ -500,6 +512,13 @@ cudaError_t launch_tile(const Dims& d, const float* o_lat, const float* x, const
 }
 
 }  // namespace
+
+gta_status_t sm100_decoder_f32_debug_wait(unsigned long long limit_ns, int withhold_first_arrive) {
+    const WaitHook w = {limit_ns ? limit_ns : ptx::kWaitLimitNs, withhold_first_arrive ? 1 : 0};
+    if (cudaMemcpyToSymbol(c_wait, &w, sizeof(w)) == cudaSuccess) return GTA_OK;
+    cudaGetLastError();
+    return GTA_ERR_CUDA;
+}
 
 long long sm100_decoder_f32_units(const Dims& d, int nt) {
     return (((long long)d.B * d.N + 2 * kTileM - 1) / (2 * kTileM)) * ((d.n_h / d.n_q * d.d_h + nt - 1) / nt) * d.n_q;

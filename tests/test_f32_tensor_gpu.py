@@ -129,6 +129,27 @@ def test_a_wait_that_runs_out_unwinds_the_short_prompt_kernel(G, N):
     _times_out(G, _inputs(1, N, N, 256, 4, 2, 2, 1, 64, 128), N)
 
 
+# one CTA a row tile and four, tiles in flight when the wait runs out; the tensor-core decoder behind plain attention (d_l = 72)
+@pytest.mark.parametrize("case", [(9, 1024, 32, 4, 2, 2, 1, 64, 128), (1, 333, 64, 20, 5, 1, 1, 64, 128), (1, 192, 64, 4, 2, 2, 1, 64, 128),
+                                  (5, 333, 64, 8, 4, 4, 1, 128, 72)])
+def test_a_wait_that_runs_out_unwinds_the_tensor_core_kernels(G, case):
+    B, N, H, n_h, n_q, n_k, n_c, d_h, d_l = case
+    _times_out(G, _inputs(B, N, N, H, n_h, n_q, n_k, n_c, d_h, d_l), N)
+
+
+def test_a_long_attention_kernel_does_not_run_out_the_decoders_waits(G):
+    """700 rows behind 40000 keys take some 200 us, four CTAs a row tile; the decoder kernel starts beside them, and its waits may
+    take 50 us here."""
+    t = _inputs(1, 700, 40000, 64, 20, 5, 1, 1, 64, 128)
+    want = _run(G, t, 40000, True).clone()
+    G.debug_attention_wait(limit_ns=50_000)
+    try:
+        got = _run(G, t, 40000, True)
+    finally:
+        G.debug_attention_wait()
+    assert torch.equal(got, want)
+
+
 @pytest.mark.parametrize("size", [1e-30, 1e15])
 def test_range_of_the_pieces(G, size):
     """Latents and decoder weights far from one: the pieces have fp32's exponents."""
