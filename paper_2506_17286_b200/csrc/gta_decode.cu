@@ -981,11 +981,17 @@ append_fp8_bulk_kernel(AppendFp8Args a, const int32_t* __restrict__ seq_lens, in
     }
 }
 
+// Turns of a warp over the new rows of a sequence, with the lanes that `a` gives a row.  One CTA per sequence takes up to four turns
+// per warp (its 2 - 3 us are launch and latency); beyond that the launch behind, about 2 us, is the smaller part.
+static bool append_fp8_one_cta(const AppendFp8Args& a) {
+    const int k_per = 32 / a.k_lpr, c_per = 32 / a.c_lpr;
+    return ((long long)a.n_k * a.n_new + k_per - 1) / k_per + ((long long)a.n_c * a.n_new + c_per - 1) / c_per <= 32;
+}
+
 template <typename T, int NK, int NV>
 static cudaError_t launch_append_fp8(const AppendFp8Args& a, int B, int32_t* seq_lens, int32_t* status_word,
                                      cudaStream_t stream, int* launches) {
     const int k_per = 32 / a.k_lpr, c_per = 32 / a.c_lpr;
-    const long long units = ((long long)a.n_k * a.n_new + k_per - 1) / k_per + ((long long)a.n_c * a.n_new + c_per - 1) / c_per;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(256);
     cfg.stream = stream;
@@ -994,9 +1000,7 @@ static cudaError_t launch_append_fp8(const AppendFp8Args& a, int B, int32_t* seq
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // one CTA per sequence up to four units per warp (its 2 - 3 us are launch and latency); beyond that the second
-    // launch, about 2 us, is the smaller part
-    if (NK == 1 && units <= 32) {
+    if (NK == 1 && append_fp8_one_cta(a)) {
         cfg.gridDim = dim3(B);
         *launches += 1;
         return cudaLaunchKernelEx(&cfg, append_fp8_small_kernel<T, NV>, a, seq_lens, status_word);
@@ -1026,9 +1030,11 @@ static cudaError_t launch_append_fp8_typed(AppendFp8Args a, int B, int32_t* seq_
     // Long prompts: four pieces per lane, so that what a row costs whatever its width -- its largest element among the lanes, its
     // scale, the reciprocal, addresses -- is spent on fewer lanes of more elements (us, one piece of a key row and up to four of a
     // latent row per lane / four of both: 25 MB 11.1 / 9.1, 101 MB 33.0 / 24.4, 202 MB with rows of 1024 53.5 / 43.9, 10 MB of the 1B
-    // layer 6.7 / 5.5; 6 MB 5.3 / 5.3, 2 MB 4.6 / 4.8).
+    // layer 6.7 / 5.5; 6 MB 5.3 / 5.3, 2 MB 4.6 / 4.8).  Few rows of many sequences leave such lanes idle: they stay as they are (1000
+    // sequences, 10 rows of 2048 elements: 28.3 / 30.4), or with one CTA each where that takes them (4096 sequences, a token of
+    // 2048 elements: 18.0 / 103.5).
     const long long elements = (long long)B * a.n_new * (a.n_k * a.d_h + a.n_c * a.d_l);
-    if (elements >= 3 << 20 && a.d_l <= 1024) {
+    if (elements >= 3 << 20 && a.d_l <= 1024 && a.n_new >= 16 && !append_fp8_one_cta(a)) {
         a.k_lpr = append_fp8_lanes(a.d_h, 4);
         a.c_lpr = append_fp8_lanes(a.d_l, 4);
         return launch_append_fp8<T, 4, 4>(a, B, seq_lens, status_word, stream, launches);

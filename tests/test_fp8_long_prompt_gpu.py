@@ -50,3 +50,25 @@ def test_a_long_prompt_is_its_pieces(B, case):
     torch.cuda.synchronize()
     for a, b in zip(whole, pieces):
         assert torch.equal(a.view(torch.int32) if a.dtype == torch.float32 else a, b.view(torch.int32) if b.dtype == torch.float32 else b)
+
+
+@pytest.mark.parametrize("case", [("bf16", 4, 1, 128, 512, 4096, 1), ("f32", 1, 1, 64, 128, 20000, 1), ("bf16", 8, 1, 128, 1024, 900, 2)],
+                         ids=lambda c: f"{c[0]}_dl{c[4]}_B{c[5]}_n{c[6]}")
+def test_few_rows_of_many_sequences_are_one_launch(B, case):
+    """As many elements as a long prompt, a row or two of each sequence: one launch, and what parts of the batch give."""
+    dt, n_k, n_c, d_h, d_l, nb, n = case
+    assert nb * n * (n_k * d_h + n_c * d_l) >= 3 << 20
+    T = torch.bfloat16 if dt == "bf16" else torch.float32
+    g = torch.Generator("cuda").manual_seed(nb)
+    k, c = torch.randn(nb, n_k, n, d_h, generator=g, device="cuda").to(T), torch.randn(nb, n_c, n, d_l, generator=g, device="cuda").to(T)
+    whole = [torch.zeros(nb, n_k, 5, d_h, dtype=torch.uint8, device="cuda"), torch.zeros(nb, n_c, 5, d_l, dtype=torch.uint8, device="cuda"),
+             torch.zeros(nb, n_k, 5, device="cuda"), torch.zeros(nb, n_c, 5, device="cuda"),
+             torch.arange(nb, dtype=torch.int32, device="cuda") % 4]
+    parts = [t.clone() for t in whole]
+    B.gta_cache_append_fp8(*whole[:4], k, c, whole[4])
+    assert B.last_launch_count() == 1
+    for i in range(0, nb, 100):
+        B.gta_cache_append_fp8(*(t[i:i + 100] for t in parts[:4]), k[i:i + 100], c[i:i + 100], parts[4][i:i + 100])
+    torch.cuda.synchronize()
+    for a, b in zip(whole, parts):
+        assert torch.equal(a, b)
