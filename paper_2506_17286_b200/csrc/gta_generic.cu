@@ -377,10 +377,12 @@ generic_attention_kernel(Dims d, const T* __restrict__ q, const T* __restrict__ 
     // (row tiles and slices of d_l share x, heads and maps have y to themselves: 65535 of them)
     const int slice = (int)blockIdx.x / tiles, t0 = (tiles - 1 - ((int)blockIdx.x - slice * tiles)) * 16 * QW;   // the longest rows first
     const int g = blockIdx.y, b = blockIdx.z, col0 = slice * 64 * NC;
-    float* o_rows = o_lat + (((size_t)g * d.B + b) * d.N + t0) * d.d_l + col0;
     attention_tile<T, QW, SW, NC, DH>(
         nullptr, d, q, k, c, pm, status_word, smem, threadIdx.x, t0, col0, g, b, [] { __syncthreads(); },
-        [&](int r, int v4, const float4 v) { *reinterpret_cast<float4*>(o_rows + (size_t)r * d.d_l + 4 * v4) = v; });
+        // (the address is made here: held in registers from the start it costs some of these kernels a CTA of an SM)
+        [&](int r, int v4, const float4 v) {
+            *reinterpret_cast<float4*>(o_lat + (((size_t)blockIdx.y * d.B + blockIdx.z) * d.N + t0 + r) * d.d_l + col0 + 4 * v4) = v;
+        });
 }
 
 // ---------------------------------------------------------------------------------------------
