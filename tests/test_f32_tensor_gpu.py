@@ -102,6 +102,14 @@ def test_short_prompts_against_64_bits(G, case):
     test_against_64_bits(G, case)
 
 
+# (sequences, rows, keys) of a layer with four maps: which side of the rule, one launch fewer on the plain one (no pieces of K and C)
+@pytest.mark.parametrize("case", [(256, 1, 1, 2), (40, 95, 95, 2), (40, 96, 96, 3), (100, 3, 300, 2), (100, 3, 640, 3), (40, 3, 300, 3), (100, 64, 300, 3)])
+def test_few_rows_of_many_sequences_stay_on_the_plain_kernel(G, case):
+    B, N, kv, launches = case
+    test_against_64_bits(G, (B, N, kv, kv, 64, 4, 4, 1, 1, 64, 128, True))
+    assert G.last_launch_count() == launches
+
+
 def test_short_prompt_rows_before_an_odd_element_keep_their_bits(G):
     t = _inputs(1, 100, 100, 256, 4, 2, 2, 1, 64, 128)
     want = _run(G, t, 100, True).clone()
