@@ -161,6 +161,12 @@ __device__ __forceinline__ int step_len(int len, int S_cap, bool append) {
     return len < 0 ? 0 : (len > S_cap ? S_cap : len);
 }
 
+// A piece of a cached row; kAppend: of a row that this CTA may have written.
+template <bool kAppend, typename V> __device__ __forceinline__ V cache_load(const V* p) {
+    if constexpr (kAppend) return *p;
+    else return __ldg(p);
+}
+
 // CT: storage type of the caches (T, or Fp8 with one fp32 scale per cached row in k_scale / c_scale).  CM: maps of a
 // latent group that a pass over its rows serves (the last pass may have fewer).
 // Every key row is loaded once, whatever the number of maps of its group, and a latent row once per CM maps: the caches
@@ -169,10 +175,13 @@ __device__ __forceinline__ int step_len(int len, int S_cap, bool append) {
 // rows, scores, CTA barriers, sums -- and the length of a warp's instruction stream, on host memory the link.  (Four fp32
 // sequences of about 1100 tokens, five maps, under the profiler: 16.8 us with the loops over maps unrolled and predicated,
 // 9.4 us now; a pass over the latent rows and a pair of barriers per map took about the former.)
-template <typename T, typename CT, int CM>
+// kAppend: a fused step, whose new rows the CTA of their chunk puts into the caches and then reads like the others, with loads that see
+// what the CTA has written.  (Rows told apart at every load cost the long contexts more than the launch that is saved: 16 sequences
+// of 8000 tokens, eight maps, 285 -> 305 us; a body of its own for that CTA 2 us of code that is fetched late.)
+template <typename T, typename CT, int CM, bool kAppend>
 __global__ void __launch_bounds__(kDecodeThreads)
 decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __restrict__ q,
-                      const CT* __restrict__ k_cache, const CT* __restrict__ c_cache,
+                      std::conditional_t<kAppend, CT*, const CT*> k_cache, std::conditional_t<kAppend, CT*, const CT*> c_cache,
                       const int32_t* __restrict__ seq_lens, float* __restrict__ part_o,
                       float* __restrict__ part_ml, PageMap pm, int32_t* status_word,
                       const float* __restrict__ k_scale, const float* __restrict__ c_scale,
@@ -183,13 +192,32 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     const int b = blockIdx.y, ck = blockIdx.x;
-    const int old = seq_lens[b], len = step_len(old, S_cap, k_new != nullptr);
+    const int old = seq_lens[b];
+    // (a thread's first piece of the new rows is asked for beside the length)
+    uint4 piece = make_uint4(0u, 0u, 0u, 0u);
+    const int k_vecs = d.n_k * d.d_h / VEC, new_vecs = kAppend ? k_vecs + d.n_c * d.d_l / VEC : 0;
+    const auto new_piece = [&](int i) {
+        return __ldg(i < k_vecs ? reinterpret_cast<const uint4*>(k_new) + (size_t)b * k_vecs + i
+                                : reinterpret_cast<const uint4*>(c_new) + (size_t)b * (new_vecs - k_vecs) + i - k_vecs);
+    };
+    if (kAppend && (int)threadIdx.x < new_vecs) piece = new_piece(threadIdx.x);
+    const int len = step_len(old, S_cap, kAppend);
     const int j_begin = ck * chunk;
-    if (k_new != nullptr && ck == 0 && threadIdx.x == 0 && (old < 0 || old >= S_cap)) raise_status(status_word, GTA_ERR_CACHE_FULL);
+    if (kAppend && ck == 0 && threadIdx.x == 0 && (old < 0 || old >= S_cap)) raise_status(status_word, GTA_ERR_CACHE_FULL);
     if (j_begin >= len) return;
     const int n_tok = min(chunk, len - j_begin);
-    // the new token of a fused step: attended from where the caller has it, put into the caches by the CTA of its chunk
-    const int j_new = k_new != nullptr && len == old + 1 ? old - j_begin : -1;
+    if constexpr (kAppend) {
+        if (len == old + 1 && j_begin + n_tok == len) {
+            for (int i = threadIdx.x; i < new_vecs; i += kDecodeThreads) {
+                const bool key = i < k_vecs;
+                const int e = (key ? i : i - k_vecs) * VEC, width = key ? d.d_h : d.d_l, grp = e / width;
+                CT* plane = key ? k_cache + (size_t)b * d.n_k * S_cap * d.d_h : c_cache + (size_t)b * d.n_c * S_cap * d.d_l;
+                *reinterpret_cast<uint4*>(plane + ((size_t)grp * S_cap + old) * width + (e - grp * width)) = piece;
+                if (i + kDecodeThreads < new_vecs) piece = new_piece(i + kDecodeThreads);
+            }
+            __syncthreads();
+        }
+    }
 
     extern __shared__ __align__(16) float smem[];
     float* q_s = smem;
@@ -205,13 +233,6 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
         return (size_t)(i < 0 ? 0 : i);
     };
 
-    auto key_row = [&](int kg, int j) {
-        return j == j_new ? k_new + ((size_t)b * d.n_k + kg) * d.d_h : k_cache + row_of(d.n_k, kg, j) * d.d_h;
-    };
-    auto latent_row = [&](int cg, int j) {
-        return j == j_new ? c_new + ((size_t)b * d.n_c + cg) * d.d_l : c_cache + row_of(d.n_c, cg, j) * d.d_l;
-    };
-
     // ---- latent rows: tpr threads per row, R rows of the CTA at once, U of them per thread in flight
     constexpr int U = 8;
     const int tpr = d.d_l / CV, R = kDecodeThreads / tpr;
@@ -224,8 +245,9 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
         for (int u = 0; u < U; ++u) {
             const int j = j0 + r + u * R;
             if (active && j < n_tok) {
-                raw[u] = __ldg(reinterpret_cast<const Raw*>(latent_row(cg, j) + v * CV));
-                cs[u] = kScaled ? c_scale[row_of(d.n_c, cg, j)] : 1.f;
+                const size_t idx = row_of(d.n_c, cg, j);
+                raw[u] = cache_load<kAppend>(reinterpret_cast<const Raw*>(c_cache + idx * d.d_l + v * CV));
+                cs[u] = kScaled ? c_scale[idx] : 1.f;
             }
         }
     };
@@ -256,12 +278,12 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
 #pragma unroll
                     for (int s = 0; s < kSlots; ++s) kraw[u][s] = make_uint4(0u, 0u, 0u, 0u);
                     if (j < n_tok) {
-                        const CT* row = key_row(kg, j);
-                        if (kScaled) row_scale[u] *= k_scale[row_of(d.n_k, kg, j)];
+                        const size_t idx = row_of(d.n_k, kg, j);
+                        if (kScaled) row_scale[u] *= k_scale[idx];
 #pragma unroll
                         for (int s = 0; s < kSlots; ++s)
                             if (sl + s * lpr < vecs_per_row)
-                                kraw[u][s] = __ldg(reinterpret_cast<const uint4*>(row + (sl + s * lpr) * VEC));
+                                kraw[u][s] = cache_load<kAppend>(reinterpret_cast<const uint4*>(k_cache + idx * d.d_h + (sl + s * lpr) * VEC));
                     }
                 }
 #pragma unroll 1
@@ -378,19 +400,14 @@ decode_partial_kernel(Dims d, int chunk, int n_chunks, int S_cap, const T* __res
             }
         }
     }
-    if (j_new >= 0 && j_new < n_tok) {
-        const auto put = [&](const CT* src, CT* cache, int groups, int width) {
-            const int vecs = width / VEC;
-            for (int i = tid; i < groups * vecs; i += kDecodeThreads) {
-                const int grp = i / vecs, e = (i - grp * vecs) * VEC;
-                *reinterpret_cast<uint4*>(cache + row_of(groups, grp, j_new) * width + e) =
-                    __ldg(reinterpret_cast<const uint4*>(src + ((size_t)b * groups + grp) * width + e));
-            }
-        };
-        put(k_new, const_cast<CT*>(k_cache), d.n_k, d.d_h);
-        put(c_new, const_cast<CT*>(c_cache), d.n_c, d.d_l);
-    }
 }
+
+// What a fused step appends, and where: rows [B, groups, width], the caches they go to, the lengths that advance.
+struct StepAppend {
+    const void *k_new, *c_new;
+    void *k_cache, *c_cache;
+    int32_t* seq_lens;
+};
 
 // Log-sum-exp merge of the chunk partials of one (map, sequence), in place: the normalised latent L takes the room of the
 // sequence's first chunk, whose weight becomes one and that of the others nothing, so that a second merge finds L again
@@ -679,7 +696,7 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
                                        const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
                                        cudaStream_t stream, int stages, int* launches, const PageMap& pm,
                                        const float* k_scale = nullptr, const float* c_scale = nullptr,
-                                       const void* k_new = nullptr, const void* c_new = nullptr) {
+                                       const StepAppend* append = nullptr) {
     const DecodePlan p = make_plan(d, S_cap, room);
     float* part_o = reinterpret_cast<float*>(workspace);
     float* part_ml = reinterpret_cast<float*>(static_cast<char*>(workspace) + p.off_ml);
@@ -689,10 +706,17 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
         const int maps = d.n_q / d.n_c;
         const auto go = [&](auto cm) {
             constexpr int CM = decltype(cm)::value;
-            return launch_chained(true, decode_partial_kernel<T, CT, CM>, dim3(p.n_chunks, d.B), kDecodeThreads,
-                                 partial_smem(d, p.chunk, CM, LatentVec<CT>::N), stream, d, p.chunk, p.n_chunks, S_cap,
-                                 (const T*)q, (const CT*)k_cache, (const CT*)c_cache, seq_lens, part_o, part_ml, pm,
-                                 status_word, k_scale, c_scale, (const CT*)k_new, (const CT*)c_new);
+            const size_t smem = partial_smem(d, p.chunk, CM, LatentVec<CT>::N);
+            if constexpr (std::is_same<CT, T>::value) {
+                if (append != nullptr)
+                    return launch_chained(true, decode_partial_kernel<T, CT, CM, true>, dim3(p.n_chunks, d.B), kDecodeThreads, smem, stream, d,
+                                         p.chunk, p.n_chunks, S_cap, (const T*)q, (CT*)append->k_cache, (CT*)append->c_cache, seq_lens,
+                                         part_o, part_ml, pm, status_word, k_scale, c_scale, (const CT*)append->k_new,
+                                         (const CT*)append->c_new);
+            }
+            return launch_chained(true, decode_partial_kernel<T, CT, CM, false>, dim3(p.n_chunks, d.B), kDecodeThreads, smem, stream, d, p.chunk,
+                                 p.n_chunks, S_cap, (const T*)q, (const CT*)k_cache, (const CT*)c_cache, seq_lens, part_o, part_ml, pm,
+                                 status_word, k_scale, c_scale, (const CT*)nullptr, (const CT*)nullptr);
         };
         // as few passes over the latent rows as the accumulators allow (and as shared memory does, with very many maps)
         const auto fits = [&](int cm) { return partial_smem(d, p.chunk, cm, LatentVec<CT>::N) <= 227 * 1024; };
@@ -705,7 +729,7 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
     }
     if (stages & 4) {
         err = launch_chained((stages & 2) && S_cap > 0, decode_chunk_merge_kernel, dim3(d.n_q, d.B), kDecodeThreads, 0, stream, d,
-                             p.chunk, p.n_chunks, S_cap, seq_lens, part_o, part_ml, k_new != nullptr);
+                             p.chunk, p.n_chunks, S_cap, seq_lens, part_o, part_ml, append != nullptr);
         if (err != cudaSuccess) return err;
         const int tiles = (d.d_h + kFinishCols - 1) / kFinishCols;
         const dim3 grid(d.n_h * tiles, (d.B + kFinishSeqs - 1) / kFinishSeqs);
@@ -714,7 +738,7 @@ static cudaError_t launch_decode_typed(const Dims& d, const void* q, const void*
                             (2 * slabs.size * 4 + 2 * 8 * 128) * sizeof(float);
         err = launch_chained(true, decode_finish_kernel<T>, grid, kDecodeThreads, smem,
                             stream, d, tiles, slabs, (const T*)x_t, (const float*)part_o, (size_t)p.n_chunks * d.n_q * d.d_l, (const T*)w_p,
-                            (const T*)w_g, (T*)out, k_new != nullptr ? const_cast<int32_t*>(seq_lens) : nullptr, S_cap);
+                            (const T*)w_g, (T*)out, append != nullptr ? append->seq_lens : nullptr, S_cap);
         if (err != cudaSuccess) return err;
         *launches += 2;
     }
@@ -1096,12 +1120,13 @@ cudaError_t launch_decode_plain_append(const Dims& d, int dtype, const void* q, 
                                        const void* c_new, int32_t* seq_lens, int S_cap, const void* x_t, const void* w_p,
                                        const void* w_g, void* out, void* workspace, size_t room, int32_t* status_word,
                                        cudaStream_t stream, int* launches) {
+    const StepAppend append = {k_new, c_new, k_cache, c_cache, seq_lens};
     if (dtype == GTA_F32)
         return launch_decode_typed<float, float>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace, room,
-                                                 status_word, stream, 7, launches, PageMap(), nullptr, nullptr, k_new, c_new);
+                                                 status_word, stream, 7, launches, PageMap(), nullptr, nullptr, &append);
     return launch_decode_typed<__nv_bfloat16, __nv_bfloat16>(d, q, k_cache, c_cache, seq_lens, S_cap, x_t, w_p, w_g, out, workspace,
                                                              room, status_word, stream, 7, launches, PageMap(), nullptr, nullptr,
-                                                             k_new, c_new);
+                                                             &append);
 }
 
 }  // namespace gta
