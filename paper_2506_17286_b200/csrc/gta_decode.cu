@@ -515,8 +515,10 @@ template <> struct Weights4<__nv_bfloat16> {
 
 // The finish kernel's contractions in slabs of at most `size` elements: those of X W_G, then those of L W_P.  The weights
 // of a slab and of the one behind it are on their way at once: buffers of even and odd slabs in turn, every thread the
-// pieces that it uses itself.  1280 elements where every CTA has an SM to itself, 640, which leaves room for two, otherwise
-// (the whole fp32 step of the 1B layer, us, 1280 / 640: four sequences of about 1100 tokens 17.0 / 18.4, 32 of 256 35.3 / 30.3).
+// pieces that it uses itself.  1280 elements where every CTA has an SM to itself and the gate's weights are one such slab, 640
+// otherwise: a CTA then leaves room for another, and for the partial kernel's CTAs, beside which it fetches its weights (the whole
+// fp32 step, us, 1280 / 640: 1B layer, four sequences of about 1100 tokens 16.4 / 17.9, 8 of 500 15.9 / 19.0, 16 of 500 23.1 / 20.0;
+// 2048 wide, 16 heads of 128: 4 of 100 22.7 / 19.0, 8 of 100 26.7 / 21.5, 4 of 2000 24.8 / 28.2).
 struct FinishSlabs {
     int size;                      // a multiple of 64
     int gate, all;                 // slabs of the gate; of both
@@ -524,7 +526,7 @@ struct FinishSlabs {
 };
 static FinishSlabs finish_slabs(const Dims& d, long long ctas) {
     FinishSlabs f;
-    f.size = ctas <= 148 ? 1280 : 640;
+    f.size = ctas <= 148 && d.H <= 1280 ? 1280 : 640;
     f.gate = (d.H + f.size - 1) / f.size;
     f.all = f.gate + (d.d_l + f.size - 1) / f.size;
     f.even_pieces = f.odd_pieces = 0;
@@ -568,7 +570,7 @@ __device__ __forceinline__ float finish_reduce(float (&acc)[8][4], float* red) {
 // before the dependency wait, under the kernels ahead; after it come one pass over W_P's columns and the store.
 // Narrow tiles, because at small batches the weights' way through few SMs sets the time (1280 columns: 80 CTAs; the
 // former pair of kernels, a head and a 128-column block per CTA, took 18.6 + 19.6 us for four fp32 sequences), and all of a
-// CTA's weights asked for at once (four fp32 sequences of about 1100 tokens, the whole step: 17.0 us; with eight
+// CTA's weights asked for at once (four fp32 sequences of about 1100 tokens, the whole step: 16.4 us; with eight
 // pieces a thread in registers 20.5).
 // Dynamic shared memory: weights [even pieces][256], [odd pieces][256] | xs [2][slab][4] | red [2][8 warps][8][16]
 template <typename T>
