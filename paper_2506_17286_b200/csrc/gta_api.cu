@@ -58,8 +58,8 @@ static gta_status_t prefill_impl(const gta_shape_t* shape, int32_t kv_len, int32
                                  const void* k, const void* c, const void* x, const void* w_p, const void* w_g,
                                  void* out, void* workspace, size_t workspace_bytes, int32_t* status_word,
                                  void* cuda_stream, int32_t stages, const gta::PageMap& pm);
-// What a prefill cannot do without: the normalised latent attention output L[B, n_q, N, d_l], fp32 on the plain-ALU path,
-// bf16 on the tensor-core path; sized for the larger so either path may run.
+// What a prefill cannot do without: the normalised latent attention output L, [n_q, B, N, d_l] in fp32 on the plain-ALU and
+// fp32 paths, bf16 on the tensor-core path; sized for the larger so either path may run.
 static size_t prefill_least_workspace(const gta::Dims& d) {
     const size_t bytes = (size_t)d.B * d.n_q * d.N * d.d_l * sizeof(float);
     return bytes < 256 ? 256 : ((bytes + 255) & ~(size_t)255);
@@ -143,8 +143,8 @@ size_t gta_prefill_workspace_bytes(const gta_shape_t* shape) {
     // served with prefill_least_workspace too; it then splits as far as what it was given has room.
     const size_t least = prefill_least_workspace(d);
     const size_t split = gta::sm100_prefill_supported(d, shape->dtype) ? gta::sm100_split_workspace_bytes(d) : 0;
-    // fp32: the pieces of K and C behind L
-    const size_t pieces = shape->dtype == GTA_F32 && gta::sm100_attention_f32_supported(d) ? least + gta::sm100_attention_f32_scratch(d) : 0;
+    // fp32: the pieces of K and C behind L (by the layer alone: the size does not fall where a call is too large for a grid)
+    const size_t pieces = shape->dtype == GTA_F32 && gta::sm100_attention_f32_shape(d) ? least + gta::sm100_attention_f32_scratch(d) : 0;
     return split > least ? split : pieces > least ? pieces : least;
 }
 

@@ -50,6 +50,7 @@ constexpr float kPiecesFloor = 0x1p-90f;
 // Attention of an fp32 call on the tensor cores (gta_sm100_f32_attention.cu): d_h = 64, d_l a multiple of 128, contiguous K and
 // C; L fp32 [n_q, B, N, d_l]; scratch of the given size (256-byte aligned) for the pieces of K and C; split: CTAs (1, 2 or
 // 4) that share the keys of a row tile.
+bool sm100_attention_f32_shape(const Dims& d);           // whatever the batch and the lengths
 bool sm100_attention_f32_supported(const Dims& d);
 size_t sm100_attention_f32_scratch(const Dims& d);
 cudaError_t launch_sm100_attention_f32(const Dims& d, const float* q, const float* k, const float* c, float* o_lat, void* scratch,

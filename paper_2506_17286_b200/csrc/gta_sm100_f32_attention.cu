@@ -83,15 +83,15 @@ __device__ __forceinline__ uint64_t whole2(uint64_t v) {
     return ptx::f32x2(fabsf(a) < 3.3895e38f ? a : 0.f, fabsf(b) < 3.3895e38f ? b : 0.f);
 }
 
-// One CTA per tile of 64 rows of one (sequence, group) of K (blockIdx.y < B n_k) or C.
+// One CTA per tile of 64 rows of one (sequence, group) of K (the first B n_k of them) or C, tiles of a group next to one another.
 __global__ void __launch_bounds__(256)
 split_rows_kernel(Dims d, const float* __restrict__ k, const float* __restrict__ c, uint8_t* __restrict__ k_planes,
                   uint8_t* __restrict__ c_planes, int32_t* __restrict__ first_odd, int tiles) {
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
-    const int tile = blockIdx.x, n_kp = d.B * d.n_k;
-    const bool latent = (int)blockIdx.y >= n_kp;
-    const int plane = latent ? blockIdx.y - n_kp : blockIdx.y;
+    const int n_kp = d.B * d.n_k, tile = (int)blockIdx.x % tiles, which = (int)blockIdx.x / tiles;
+    const bool latent = which >= n_kp;
+    const int plane = latent ? which - n_kp : which;
     const int width = latent ? d.d_l : kDh, vecs = width / 4;
     const float* src = (latent ? c : k) + ((size_t)plane * d.S + (size_t)tile * kKeys) * width;
     const size_t n_rows = (size_t)d.B * (latent ? d.n_c : d.n_k) * d.Nk;
@@ -120,7 +120,7 @@ split_rows_kernel(Dims d, const float* __restrict__ k, const float* __restrict__
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) first_odd[(size_t)blockIdx.y * tiles + tile] = first;
+    if (threadIdx.x == 0) first_odd[blockIdx.x] = first;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -551,8 +551,12 @@ gta_status_t sm100_attention_f32_debug_wait(unsigned long long limit_ns, int wit
 
 bool sm100_attention_f32_supported(const Dims& d) {
     const long long ctas = 4ll * ((d.N + kRows - 1) / kRows) * (d.d_l / kCols) * d.n_q * d.B;
-    return d.d_h == kDh && d.d_l % kCols == 0 && (long long)d.B * (d.n_k + d.n_c) <= 65535 && ctas <= INT32_MAX;
+    const long long tiles = (long long)((d.Nk + kKeys - 1) / kKeys) * d.B * (d.n_k + d.n_c);
+    return sm100_attention_f32_shape(d) && ctas <= INT32_MAX && tiles <= INT32_MAX;
 }
+
+bool sm100_attention_f32_shape(const Dims& d) { return d.d_h == kDh && d.d_l % kCols == 0; }
+
 
 size_t sm100_attention_f32_scratch(const Dims& d) {
     const size_t rows = (size_t)d.B * d.Nk, tiles = ((size_t)d.Nk + kKeys - 1) / kKeys;
@@ -578,7 +582,7 @@ cudaError_t launch_sm100_attention_f32(const Dims& d, const float* q, const floa
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(key_tiles, d.B * (d.n_k + d.n_c));
+    cfg.gridDim = dim3((unsigned)key_tiles * d.B * (d.n_k + d.n_c));
     cfg.blockDim = dim3(256);
     cfg.stream = stream;
     cfg.attrs = attr;

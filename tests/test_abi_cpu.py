@@ -75,12 +75,14 @@ def test_workspace_sizes(B):
 
 @pytest.mark.parametrize("layer", [
     dict(n_heads=16, n_q=4, n_k=4, n_c=1, d_h=128, d_l=512, d_model=2048), dict(n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64, d_l=128, d_model=1280),
-    dict(n_heads=4, n_q=2, n_k=2, n_c=1, d_h=128, d_l=256, d_model=64), dict()], ids=["h2048", "gta1b", "small", "plain_alu"])
+    dict(n_heads=4, n_q=2, n_k=2, n_c=1, d_h=128, d_l=256, d_model=64), dict(),
+    dict(n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64, d_l=128, d_model=1280, dtype=0),
+    dict(n_heads=4, n_q=2, n_k=2, n_c=1, d_h=64, d_l=128, d_model=256, dtype=0)], ids=["h2048", "gta1b", "small", "plain_alu", "gta1b_f32", "tiny_f32"])
 def test_prefill_workspace_never_falls_as_batch_or_length_grow(B, layer):
     """A buffer for the longest prompt of the largest batch serves every shorter one and every chunk."""
     sizes = [1, 2, 64, 128, 129, 255, 256, 257, 1000, 2048, 2304, 2305, 2560, 3500, 4096, 4097, 9000, 16384]
     for query in (B.prefill_workspace_bytes, B.layer_prefill_workspace_bytes):
-        rows = [[query(_shape(B, batch=b, seq=n, **layer)) for n in sizes] for b in (1, 2, 3, 4, 7, 8, 32)]
+        rows = [[query(_shape(B, batch=b, seq=n, **layer)) for n in sizes] for b in (1, 2, 3, 4, 7, 8, 32, 21845, 21846, 32767, 32768, 65535)]
         assert all(x > 0 for r in rows for x in r)
         for r in rows:
             assert r == sorted(r)

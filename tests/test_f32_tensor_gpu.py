@@ -110,6 +110,18 @@ def test_few_rows_of_many_sequences_stay_on_the_plain_kernel(G, case):
     assert G.last_launch_count() == launches
 
 
+def test_more_key_and_latent_groups_than_a_grid_dimension(G):
+    """520 sequences x (128 key groups + 1): more than 65535 of them are cut into pieces, the last like the first."""
+    t = _inputs(520, 96, 96, 8, 128, 128, 128, 1, 64, 128)
+    for n in ("q", "k", "c", "x"):
+        t[n][519] = t[n][0]
+    got = _run(G, t, 96, True)
+    assert G.last_launch_count() == 3 and torch.equal(got[519], got[0])
+    few = {n: v[518:].contiguous() if n in ("q", "k", "c", "x") else v for n, v in t.items()}
+    want = _exact(few, 96, True)
+    assert float((got[518:].double() - want).norm() / want.norm()) <= REL
+
+
 def test_short_prompt_rows_before_an_odd_element_keep_their_bits(G):
     t = _inputs(1, 100, 100, 256, 4, 2, 2, 1, 64, 128)
     want = _run(G, t, 100, True).clone()
