@@ -118,8 +118,14 @@ GTA_API gta_status_t gta_prefill(const gta_shape_t *shape, const void *q, const 
  *   k   [B, n_k, kv_cap, d_h]     c   [B, n_c, kv_cap, d_l]    rows 0 .. kv_len-1 are read; the rows
  *   behind them may hold anything (uninitialised memory, NaN bit patterns): nothing of them reaches out
  *   N <= kv_len <= kv_cap (else GTA_ERR_INVALID_ARG); kv_len = kv_cap = N is gta_prefill.
- * Workspace, weights, arithmetic, paths and errors as for gta_prefill.
+ * Weights, arithmetic, paths and errors as for gta_prefill, and the workspace too: what
+ * gta_prefill_workspace_bytes gives for the chunk's shape is enough.  With it, an fp32 call of
+ * d_h = 64 whose kv_len is longer than N runs its attention on the plain-ALU kernel; with
+ * gta_prefill_chunk_workspace_bytes(shape, kv_len) (0 where kv_len < N), which has room for the
+ * operands of all kv_len positions, on the tensor cores where that is faster.  That size never
+ * falls as batch, seq or kv_len grow; for other shapes it is the smaller one.
  */
+GTA_API size_t gta_prefill_chunk_workspace_bytes(const gta_shape_t *shape, int32_t kv_len);
 GTA_API gta_status_t gta_prefill_chunk(const gta_shape_t *shape, int32_t kv_len, int32_t kv_cap,
                                        const void *q, const void *k, const void *c, const void *x,
                                        const void *w_p, const void *w_g, void *out, void *workspace,

@@ -29,7 +29,7 @@ GTA_F32, GTA_BF16 = 0, 1
 EXPORTS = (
     "gta_prefill_workspace_bytes", "gta_prefill", "gta_decode_workspace_bytes", "gta_decode",
     "gta_cache_append", "gta_status_string", "gta_version", "gta_prefill_path", "gta_last_launch_count",
-    "gta_prefill_stages", "gta_decode_stages", "gta_decode_static", "gta_prefill_chunk",
+    "gta_prefill_stages", "gta_decode_stages", "gta_decode_static", "gta_prefill_chunk", "gta_prefill_chunk_workspace_bytes",
     "gta_decode_paged_workspace_bytes", "gta_decode_paged", "gta_cache_append_paged",
     "gta_layer_prefill_workspace_bytes", "gta_layer_prefill", "gta_layer_decode_workspace_bytes", "gta_layer_decode",
     "gta_layer_decode_paged_workspace_bytes", "gta_layer_decode_paged", "gta_debug_attention_wait",
@@ -74,6 +74,8 @@ def lib():
         sp = ctypes.POINTER(GtaShape)
         L.gta_prefill_workspace_bytes.argtypes = [sp]
         L.gta_prefill_workspace_bytes.restype = sz
+        L.gta_prefill_chunk_workspace_bytes.argtypes = [sp, i32]
+        L.gta_prefill_chunk_workspace_bytes.restype = sz
         L.gta_prefill.argtypes = [sp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp, vp]
         L.gta_prefill.restype = i32
         L.gta_prefill_stages.argtypes = [sp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp, vp, i32]
@@ -239,6 +241,10 @@ def prefill_workspace_bytes(shape: GtaShape) -> int:
     return int(lib().gta_prefill_workspace_bytes(ctypes.byref(shape)))
 
 
+def prefill_chunk_workspace_bytes(shape: GtaShape, kv_len: int) -> int:
+    return int(lib().gta_prefill_chunk_workspace_bytes(ctypes.byref(shape), int(kv_len)))
+
+
 def decode_workspace_bytes(shape: GtaShape, s_cap: int) -> int:
     return int(lib().gta_decode_workspace_bytes(ctypes.byref(shape), int(s_cap)))
 
@@ -295,7 +301,7 @@ def gta_prefill_chunk(q, k, c, x, w_p, w_g, kv_len, *, causal=True, softmax_scal
     if out is None:
         out = q.new_empty((B, N, n_h, d_h))
     if workspace is None:
-        workspace = _workspace(prefill_workspace_bytes(shape), q.device)
+        workspace = _workspace(prefill_chunk_workspace_bytes(shape, kv_len), q.device)
     st = lib().gta_prefill_chunk(ctypes.byref(shape), int(kv_len), int(kv_cap), _ptr(q), _ptr(k), _ptr(c), _ptr(x),
                                  _ptr(w_p), _ptr(w_g), _ptr(out), _ptr(workspace),
                                  workspace.nbytes, _ptr(status_word), _stream(stream))

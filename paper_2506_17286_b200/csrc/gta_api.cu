@@ -136,9 +136,10 @@ int gta_prefill_path(const gta_shape_t* shape) {
     return 1;
 }
 
-size_t gta_prefill_workspace_bytes(const gta_shape_t* shape) {
+static size_t prefill_workspace(const gta_shape_t* shape, int32_t kv_len) {
     gta::Dims d;
-    if (check_shape(shape, true, &d) != GTA_OK) return 0;
+    if (check_shape(shape, true, &d) != GTA_OK || kv_len < d.N) return 0;
+    d.Nk = kv_len;
     // ... and, on the tensor-core path, room for the partial sums of a call whose keys are split over the chip.  A call is
     // served with prefill_least_workspace too; it then splits as far as what it was given has room.
     const size_t least = prefill_least_workspace(d);
@@ -147,6 +148,10 @@ size_t gta_prefill_workspace_bytes(const gta_shape_t* shape) {
     const size_t pieces = shape->dtype == GTA_F32 && gta::sm100_attention_f32_shape(d) ? least + gta::sm100_attention_f32_scratch(d) : 0;
     return split > least ? split : pieces > least ? pieces : least;
 }
+
+size_t gta_prefill_workspace_bytes(const gta_shape_t* shape) { return shape ? prefill_workspace(shape, shape->seq) : 0; }
+
+size_t gta_prefill_chunk_workspace_bytes(const gta_shape_t* shape, int32_t kv_len) { return prefill_workspace(shape, kv_len); }
 
 gta_status_t gta_prefill(const gta_shape_t* shape, const void* q, const void* k, const void* c,
                          const void* x, const void* w_p, const void* w_g, void* out, void* workspace,

@@ -769,7 +769,8 @@ static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x,
 // 527 / 160: from 192 keys, or more than 64 plain CTAs of 16 rows, on; but a tile of 128 rows that is half empty loses (64 tokens of 64
 // sequences, w512 (16 heads, 8 maps, latents of 512) 222 / 236, 1B 131 / 128; 16 of 256 270 / 549, 135 / 176; 96 of 64 369 / 308,
 // 150 / 137), and so do few rows behind short caches once there is more than a wave of them (64 sequences, a row behind 300 keys:
-// w512 192 / 235, tiny 28 / 28; behind 1000 550 / 532, 63 / 62): both stay on the FMA pipe.  Decoder: 1B 200 tokens (80 tiles of 64 x 64) 32.7 / 42.7, 333
+// w512 192 / 235, tiny 28 / 28; behind 1000 503 / 533, 69 / 62), the longer the more elements a token has, whose pieces are made for so
+// few rows: all of these stay on the FMA pipe.  Decoder: 1B 200 tokens (80 tiles of 64 x 64) 32.7 / 42.7, 333
 // (120) 54.4 / 42.6; tiny 700 (44) 28.4 / 30.3, 2048 (128) 45.3 / 38.7: from 100 tiles on; in blocks of 128 columns while those of
 // 256 are few (1B, 1000 tokens, 20 blocks of 256: 54.3 / 47.1 with 128; 1500, 30: 66.2 / 73.6).
 //
@@ -791,7 +792,8 @@ static F32Plan f32_plan(const Dims& d, const PageMap& pm, size_t room) {
     if (d.d_h % 64 == 0 && tiles64 >= 100) plan.cols = map_cols > 128 && sm100_decoder_f32_units(d, 256) > 28 ? 256 : 128;
     const long long plain = (long long)d.B * d.n_q * ((d.N + 15) / 16);
     const long long items = (long long)((d.N + 127) / 128) * (d.d_l / 128) * d.n_q * d.B;
-    const bool few_rows = d.Nk < 192 ? plain <= 64 || d.N < 96 : d.N < 64 && d.Nk < 640 && items > 296;
+    const int token = d.n_k * d.d_h + d.n_c * d.d_l;             // cached elements of a token
+    const bool few_rows = d.Nk < 192 ? plain <= 64 || d.N < 96 : d.N < 64 && (token < 512 ? items > 296 && d.Nk < 640 : items > 148 && d.Nk < 1536);
     if (pm.table != nullptr || !sm100_attention_f32_supported(d) || few_rows ||
         room < l_bytes(d) + sm100_attention_f32_scratch(d)) {
         plan.one = pm.table == nullptr && plan.cols == 0 && d.d_h == 64 && d.d_l == 128 && d.Nk < 192 &&

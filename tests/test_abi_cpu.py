@@ -90,6 +90,20 @@ def test_prefill_workspace_never_falls_as_batch_or_length_grow(B, layer):
             assert list(col) == sorted(col)
 
 
+def test_prefill_chunk_workspace(B):
+    """Room for the fp32 attention's operands behind a longer cache; the plain query's size where there are none."""
+    f32 = dict(n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64, d_l=128, d_model=1280, dtype=0)
+    for layer in (f32, dict(f32, dtype=1), dict(), dict(f32, d_l=72)):
+        pieces = layer == f32
+        for b in (1, 8, 40000):
+            s = _shape(B, batch=b, seq=100, **layer)
+            sizes = [B.prefill_chunk_workspace_bytes(s, kv) for kv in (100, 101, 128, 129, 1000, 100000)]
+            assert sizes[0] == B.prefill_workspace_bytes(s) and sizes == sorted(sizes) and (sizes[-1] > sizes[0]) == pieces
+            assert B.prefill_chunk_workspace_bytes(s, 99) == 0
+            assert [B.prefill_chunk_workspace_bytes(_shape(B, batch=b, seq=n, **layer), 1000) for n in (1, 2, 100, 1000)] == \
+                sorted(B.prefill_chunk_workspace_bytes(_shape(B, batch=b, seq=n, **layer), 1000) for n in (1, 2, 100, 1000))
+
+
 GTA1B = dict(n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64, d_l=128, d_model=1280)
 
 

@@ -50,8 +50,7 @@ def _run(G, t, kv, causal, least=False):
     shape = G.make_shape(batch=B, seq=N, d_model=t["x"].shape[2], n_heads=n_h, n_q=n_q, n_k=t["k"].shape[1],
                          n_c=t["c"].shape[1], d_h=d_h, d_l=d_l, dtype=torch.float32)
     plain = (4 * B * n_q * N * d_l + 255) // 256 * 256
-    # (behind longer keys the pieces need more than the query of the chunk's shape says)
-    room = plain if least else max(G.prefill_workspace_bytes(shape), plain + 12 * B * kv * (n_q * d_h + n_q * d_l) + 65536)
+    room = plain if least else G.prefill_chunk_workspace_bytes(shape, kv)
     ws, out = Guarded((room,), torch.uint8), Guarded((B, N, n_h, d_h), torch.float32)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     G.gta_prefill_chunk(t["q"], t["k"], t["c"], t["x"], t["w_p"], t["w_g"], kv, causal=causal, workspace=ws.t, out=out.t,
@@ -205,6 +204,22 @@ def test_few_small_elements_and_rows(G):
     tail = slice(3, None)                       # (1e-36 x 1e-35 is nothing)
     err[:, tail, 3] = (got - want)[:, tail, 3, 40:44].norm(dim=-1) / want[:, tail, 3, 40:44].norm(dim=-1)
     assert float(err.max()) <= 8 * REL          # (a head's 64 outputs, or four of them, against a row's latents)
+
+
+def test_workspace_of_a_chunk_behind_a_longer_cache(G):
+    """With the size that its query gives, or without a workspace, the chunk takes the tensor cores; a byte less and it takes the plain
+    kernel, in place."""
+    B, N, kv = 2, 130, 777
+    t = _inputs(B, N, 800, 256, 20, 5, 1, 1, 64, 128)
+    shape = G.make_shape(batch=B, seq=N, d_model=256, n_heads=20, n_q=5, n_k=1, n_c=1, d_h=64, d_l=128, dtype=torch.float32)
+    args = (t["q"], t["k"], t["c"], t["x"], t["w_p"], t["w_g"], kv)
+    want, plain = _run(G, t, kv, True).clone(), _run(G, t, kv, True, least=True).clone()
+    assert G.last_launch_count() == 2 and not torch.equal(want, plain)
+    assert torch.equal(G.gta_prefill_chunk(*args), want) and G.last_launch_count() == 3
+    for room in (G.prefill_chunk_workspace_bytes(shape, kv) - 1, G.prefill_workspace_bytes(shape)):
+        ws = Guarded((room,), torch.uint8)
+        assert torch.equal(G.gta_prefill_chunk(*args, workspace=ws.t), plain) and G.last_launch_count() == 2
+        ws.check("workspace")
 
 
 BAD = [("q", (0, 1, 40, 3), float("nan")), ("q", (0, 0, 299, 0), float("inf")), ("k", (0, 0, 130, 5), float("inf")),
