@@ -124,25 +124,110 @@ split_rows_kernel(Dims d, const float* __restrict__ k, const float* __restrict__
 }
 
 // ---------------------------------------------------------------------------------------------
-// One query row with plain FMAs by a warp: lanes share the head width and the columns (four each).
-__device__ __forceinline__ void plain_row(const Dims& d, const float* __restrict__ q_row, const float* __restrict__ k_rows,
-                                          const float* __restrict__ c_rows, float* __restrict__ out, int live, int lane) {
+// 32 neighbouring query rows with plain FMAs by eight warps (`tid` of 256, barrier 2), four rows each, 32 keys at a time: a lane has a
+// key's scores, then four columns of the sums.  Row r has live0 + r live_step keys, live_max at most, and none of the others is
+// looked at (0 x infinity).  odd(r): is the row to be stored?
+// (A warp per row and a key at a time, the lanes sharing the head width, took 12 ms where an infinity in the first key or latent made
+// all rows of 2 x 1500 tokens of the 1B layer odd; four rows a warp with keys from L1 1.4 ms, 0.65 now; the plain-ALU kernel takes 0.21 for all.)
+constexpr int kOddRows = 32, kOddLd = kDh + 4;
+constexpr uint32_t kOddSmem = (32 * kOddLd + 32 * kCols + kOddRows * kDh + kOddRows * 32) * 4;
+static_assert(kOddSmem <= kBarOffset, "in the ring's memory");
+template <typename Odd>
+__device__ __forceinline__ void plain_rows(const Dims& d, const float* __restrict__ q_rows, const float* __restrict__ k_rows,
+                                           const float* __restrict__ c_rows, float* __restrict__ out, int live0, int live_step, int live_max,
+                                           int n_rows, float* smem, int tid, Odd odd) {
     const float scale2 = d.scale * 1.4426950408889634f;
-    const float2 q = reinterpret_cast<const float2*>(q_row)[lane];
-    float m = -INFINITY, l = 0.f;
-    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j = 0; j < live; ++j) {
-        const float2 kv = reinterpret_cast<const float2*>(k_rows + (size_t)j * kDh)[lane];
-        const float s = warp_sum(fmaf(q.x, kv.x, q.y * kv.y)) * scale2;
-        const float4 cv = reinterpret_cast<const float4*>(c_rows + (size_t)j * d.d_l)[lane];
-        const float m_new = fmaxf(m, s), ref = m_new == -INFINITY ? 0.f : m_new;
-        const float al = m_new == m ? 1.f : exp2f(m - ref), p = exp2f(s - ref);
-        m = m_new;
-        l = fmaf(l, al, p);
-        o.x = fmaf(o.x, al, p * cv.x); o.y = fmaf(o.y, al, p * cv.y); o.z = fmaf(o.z, al, p * cv.z); o.w = fmaf(o.w, al, p * cv.w);
+    float* k_s = smem;                                         // [32][kOddLd]
+    float* c_s = k_s + 32 * kOddLd;                            // [32][kCols]
+    float* q_s = c_s + 32 * kCols;                             // [row][kDh]
+    float* p_s = q_s + kOddRows * kDh;                         // [row][32]
+    const int warp = tid >> 5, lane = tid & 31, r0 = 4 * warp;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = tid; i < kOddRows * kDh / 4; i += 256)
+        reinterpret_cast<float4*>(q_s)[i] = i < n_rows * kDh / 4 ? reinterpret_cast<const float4*>(q_rows)[i] : zero;
+    float m[4], l[4];
+    float4 o[4];
+    int live[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        m[r] = -INFINITY;
+        l[r] = 0.f;
+        o[r] = zero;
+        live[r] = r0 + r < n_rows ? min(live0 + (r0 + r) * live_step, live_max) : 0;
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    reinterpret_cast<float4*>(out)[lane] = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
+    const int most = min(live0 + (n_rows - 1) * live_step, live_max);
+#pragma unroll 1
+    for (int j0 = 0; j0 < most; j0 += 32) {
+        const int n = min(32, most - j0);
+        // (what a thread stages is asked for at once)
+        float4 kv[2], cv[4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            kv[u] = reinterpret_cast<const float4*>(k_rows + (size_t)(j0 + min((tid >> 4) + 16 * u, n - 1)) * kDh)[tid & 15];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            cv[u] = reinterpret_cast<const float4*>(c_rows + (size_t)(j0 + min((tid >> 5) + 8 * u, n - 1)) * d.d_l)[tid & 31];
+        ptx::named_sync(2, 256);                               // (the keys before have been used; q is there)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) *reinterpret_cast<float4*>(k_s + ((tid >> 4) + 16 * u) * kOddLd + 4 * (tid & 15)) = kv[u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) reinterpret_cast<float4*>(c_s)[tid + 256 * u] = cv[u];
+        ptx::named_sync(2, 256);
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int e = 0; e < kDh; e += 4) {
+            const float4 kv = *reinterpret_cast<const float4*>(k_s + lane * kOddLd + e);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 qv = *reinterpret_cast<const float4*>(q_s + (r0 + r) * kDh + e);
+                s[r] = fmaf(qv.x, kv.x, fmaf(qv.y, kv.y, fmaf(qv.z, kv.z, fmaf(qv.w, kv.w, s[r]))));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float v = j0 + lane < live[r] ? s[r] * scale2 : -INFINITY;
+            const float m_new = fmaxf(m[r], warp_max(v)), ref = m_new == -INFINITY ? 0.f : m_new;
+            const float al = m_new == m[r] ? 1.f : exp2f(m[r] - ref), pr = exp2f(v - ref);
+            m[r] = m_new;
+            l[r] = fmaf(l[r], al, pr);
+            o[r].x *= al; o[r].y *= al; o[r].z *= al; o[r].w *= al;
+            p_s[(r0 + r) * 32 + lane] = pr;
+        }
+        __syncwarp();
+#pragma unroll 4
+        for (int jj = 0; jj < n; ++jj) {
+            const float4 cv = *reinterpret_cast<const float4*>(c_s + jj * kCols + 4 * lane);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (j0 + jj < live[r]) {
+                    const float pr = p_s[(r0 + r) * 32 + jj];
+                    o[r].x = fmaf(pr, cv.x, o[r].x); o[r].y = fmaf(pr, cv.y, o[r].y);
+                    o[r].z = fmaf(pr, cv.z, o[r].z); o[r].w = fmaf(pr, cv.w, o[r].w);
+                }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float sum = warp_sum(l[r]), inv = sum > 0.f ? 1.f / sum : 0.f;
+        if (r0 + r < n_rows && odd(r0 + r))
+            reinterpret_cast<float4*>(out + (size_t)(r0 + r) * d.d_l)[lane] = make_float4(o[r].x * inv, o[r].y * inv, o[r].z * inv, o[r].w * inv);
+    }
+    ptx::named_sync(2, 256);
+}
+
+// The rows of an item that see, or are, odd elements (see the top), by the adding warps.
+__device__ __forceinline__ void redo_rows(const Dims& d, const float* q, const float* k, const float* c, float* o_lat, int t0, int slice, int g, int b,
+                                       int first, const uint32_t* odd_rows, float* smem, int tid) {
+    const int off = d.causal ? d.Nk - d.N : 0, rows = min(kRows, d.N - t0);
+    for (int r = 0; r < rows; r += kOddRows) {
+        const int n = min(kOddRows, rows - r), live0 = d.causal ? t0 + r + off + 1 : d.Nk, step = d.causal ? 1 : 0;
+        const uint32_t bits = odd_rows[r >> 5];
+        if (bits == 0 && min(live0 + (n - 1) * step, d.Nk) <= first) continue;
+        plain_rows(d, q + (((size_t)b * d.n_q + g) * d.N + t0 + r) * kDh, k + ((size_t)b * d.n_k + d.q_to_k(g)) * d.S * kDh,
+                   c + ((size_t)b * d.n_c + d.q_to_c(g)) * d.S * d.d_l + slice * kCols,
+                   o_lat + (((size_t)g * d.B + b) * d.N + t0 + r) * d.d_l + slice * kCols, live0, step, d.Nk, n, smem, tid,
+                   [&](int i) { return (bits >> i & 1) != 0 || min(live0 + i * step, d.Nk) > first; });
+    }
 }
 
 // Test hook of the bounded waits (gta_debug_attention_wait): their time limit, and a switch that makes one softmax warp keep its first
@@ -522,13 +607,7 @@ sm100_attention_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __gri
             if (first < n_keys || (odd_rows[0] | odd_rows[1] | odd_rows[2] | odd_rows[3]) != 0) {
                 ptx::bulk_wait_group_all();
                 ptx::named_sync(2, 256);
-                for (int r = warp - kAddWarp0; r < rows; r += 8) {
-                    const int live = d.causal ? min(t0 + r + off + 1, d.Nk) : d.Nk;
-                    if (live > first || (odd_rows[r >> 5] >> (r & 31) & 1) != 0)
-                        plain_row(d, q + (((size_t)b * d.n_q + g) * d.N + t0 + r) * kDh, k + ((size_t)b * d.n_k + kg) * d.S * kDh,
-                                  c + ((size_t)b * d.n_c + cg) * d.S * d.d_l + slice * kCols,
-                                  o_lat + (((size_t)g * d.B + b) * d.N + t0 + r) * d.d_l + slice * kCols, live, lane);
-                }
+                redo_rows(d, q, k, c, o_lat, t0, slice, g, b, first, odd_rows, reinterpret_cast<float*>(smem), threadIdx.x - 32 * kAddWarp0);
             }
         }
     }

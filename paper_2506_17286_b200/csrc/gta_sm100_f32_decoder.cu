@@ -19,7 +19,8 @@
 // out, pieces in, operands read once per product: 1664 cycles); measured 1800.
 //
 // An element that is infinite, not a number or rounds to infinity in bf16 makes its row or column of the item not a number
-// (0 x infinity); the splitting threads see it, and those rows and columns are done again with plain FMAs.  So are rows and
+// (0 x infinity); the splitting threads see it, and where it is an infinity or a large number those rows and columns are done again
+// with plain FMAs.  So are rows and
 // columns whose elements are all too small for pieces (kPiecesFloor).
 #include "gta_sm100.cuh"
 
@@ -88,7 +89,7 @@ template <int NT> struct Marks {
 // The rows and columns that hold an element which the pieces cannot: plain FMAs, by the adding warps.
 template <int NT>
 __device__ __forceinline__ void redo(const Dims& d, const float* o_lat, const float* x, const float* w_p, const float* w_g, float* out,
-                                     int row_tiles, int col_tiles, uint32_t block, Marks<NT>* marks) {
+                                     int row_tiles, int col_tiles, uint32_t block, Marks<NT>* marks, float* smem) {
     const Block w = block_of<NT>(d, row_tiles, col_tiles, block);
     const size_t ldw = (size_t)d.n_h * d.d_h;
     const int tid = threadIdx.x - 32 * kAddWarp0, warp = tid >> 5, lane = tid & 31;
@@ -118,24 +119,99 @@ __device__ __forceinline__ void redo(const Dims& d, const float* o_lat, const fl
             if (least < kPiecesFloor) col_bad[c4] = 1;
         }
     ptx::named_sync(3, 32 * kAddWarps);
-    auto again = [&](int r, int c) {
+    // kPass rows after kPass rows, where one of them or one of the columns is to be done again: 32 elements of the contraction at a time
+    // through the ring's memory, two slabs in turn, four rows x four columns to a thread.  (Few registers: all roles come here, so the
+    // compiler has the 48 of the smallest.  A row and a column at a time, with strided loads, an infinity in all rows of X took 9.5 ms
+    // for 2 x 1500 tokens of the 1B layer, 0.9 now, 0.42 where the plain-ALU kernels take the whole call; eight rows a thread, mostly in
+    // local memory, 2.1.)
+    constexpr int kThr = 32 * kAddWarps, kGroups = kThr / (NT / 4), kPass = 4 * kGroups, kSlab = 32, kLd = kSlab + 4;
+    constexpr int kSlabFloats = kSlab * NT + kPass * kLd;
+    float* z_s = smem + 2 * kSlabFloats;        // [kPass][NT]; slabs: weights [kSlab][NT], rows [kPass][kLd]
+    static_assert((2 * kSlabFloats + kPass * NT) * 4 <= Cfg<NT>::kBarOffset, "in the ring's memory");
+    int n_col = 0;
+    for (int c4 = 0; 4 * c4 < w.n_cols; ++c4) n_col += col_bad[c4];
+    const bool any_col = n_col > 4;             // (fewer columns one by one, below)
+    const int cg = tid % (NT / 4), rg = tid / (NT / 4), f = w.n0 + min(4 * cg, w.n_cols - 4), head = w.g * (d.n_h / d.n_q) + f / d.d_h;
+    const auto copy16 = [](float* dst, const float* src, bool there) {      // zeros where there is nothing
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_addr(dst)), "l"(src), "r"(there ? 16 : 0) : "memory");
+    };
+    for (int r0 = 0; r0 < w.rows; r0 += kPass) {
+        bool any = any_col;
+        for (int r = r0; r < min(r0 + kPass, w.rows); ++r) any |= row_bad[r] != 0;
+        if (!any) continue;
+        float acc[4][4];
+        // col: this thread's four columns
+        const auto contract = [&](const float* rows, int K, const float* col, size_t ld) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+            const auto fetch = [&](int k0) {
+                float* w_s = smem + (k0 / kSlab & 1) * kSlabFloats;
+                for (int k = rg; k < kSlab; k += kGroups) copy16(w_s + k * NT + 4 * cg, col + (k0 + k < K ? (size_t)(k0 + k) * ld : 0), k0 + k < K);
+                for (int i = tid; i < kPass * (kSlab / 4); i += kThr) {
+                    const int r = i / (kSlab / 4), e = k0 + 4 * (i % (kSlab / 4));
+                    copy16(w_s + kSlab * NT + r * kLd + e - k0, rows + (size_t)min(r0 + r, w.rows - 1) * K + (e < K ? e : 0), e < K);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            ptx::named_sync(3, kThr);                               // (the slabs before have been used)
+            fetch(0);
+            for (int k0 = 0; k0 < K; k0 += kSlab) {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                ptx::named_sync(3, kThr);
+                if (k0 + kSlab < K) fetch(k0 + kSlab);
+                const float* w_s = smem + (k0 / kSlab & 1) * kSlabFloats + 4 * cg;
+                const float* a_s = smem + (k0 / kSlab & 1) * kSlabFloats + kSlab * NT + 4 * rg * kLd;
+#pragma unroll 1
+                for (int k = 0; k < kSlab; k += 2) {
+                    float2 x2[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) x2[i] = *reinterpret_cast<const float2*>(a_s + i * kLd + k);
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const float4 v = *reinterpret_cast<const float4*>(w_s + (k + u) * NT);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float xi = u == 0 ? x2[i].x : x2[i].y;
+                            acc[i][0] = fmaf(xi, v.x, acc[i][0]);
+                            acc[i][1] = fmaf(xi, v.y, acc[i][1]);
+                            acc[i][2] = fmaf(xi, v.z, acc[i][2]);
+                            acc[i][3] = fmaf(xi, v.w, acc[i][3]);
+                        }
+                    }
+                }
+            }
+        };
+        contract(x + w.m0 * d.H, d.H, w_g + (size_t)w.g * w.map_cols + f, ldw);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(z_s + (4 * rg + i) * NT + 4 * cg) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        contract(o_lat + ((size_t)w.g * d.B * d.N + w.m0) * d.d_l, d.d_l, w_p + (size_t)head * d.d_l * d.d_h + f % d.d_h, d.d_h);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + 4 * rg + i;
+            if (r < w.rows && 4 * cg < w.n_cols && (row_bad[r] | col_bad[cg]) != 0) {
+                const float4 z = *reinterpret_cast<const float4*>(z_s + (4 * rg + i) * NT + 4 * cg);
+                *reinterpret_cast<float4*>(out + (w.m0 + r) * ldw + (size_t)w.g * w.map_cols + w.n0 + 4 * cg) =
+                    make_float4(acc[i][0] * (1.f / (1.f + expf(-z.x))), acc[i][1] * (1.f / (1.f + expf(-z.y))),
+                                acc[i][2] * (1.f / (1.f + expf(-z.z))), acc[i][3] * (1.f / (1.f + expf(-z.w))));
+            }
+        }
+    }
+    if (any_col || n_col == 0) return;
+    const auto again = [&](int r, int c) {
         const long long m = w.m0 + r;
-        const int f = w.n0 + c, head = w.g * (d.n_h / d.n_q) + f / d.d_h, elem = f % d.d_h;
+        const int fc = w.n0 + c, hd = w.g * (d.n_h / d.n_q) + fc / d.d_h;
         const float* xr = x + m * d.H;
-        const float* wg = w_g + (size_t)head * d.d_h + elem;
+        const float* wg = w_g + (size_t)w.g * w.map_cols + fc;
         float z = 0.f, y = 0.f;
         for (int k = 0; k < d.H; ++k) z = fmaf(xr[k], wg[k * ldw], z);
         const float* lr = o_lat + ((size_t)w.g * d.B * d.N + m) * d.d_l;
-        const float* wp = w_p + (size_t)head * d.d_l * d.d_h + elem;
+        const float* wp = w_p + (size_t)hd * d.d_l * d.d_h + fc % d.d_h;
         for (int k = 0; k < d.d_l; ++k) y = fmaf(lr[k], wp[(size_t)k * d.d_h], y);
-        out[m * ldw + (size_t)w.g * w.map_cols + f] = y * (1.f / (1.f + expf(-z)));
+        out[m * ldw + (size_t)w.g * w.map_cols + fc] = y * (1.f / (1.f + expf(-z)));
     };
-    for (int r = 0; r < w.rows; ++r)
-        if (row_bad[r])
-            for (int c = tid; c < w.n_cols; c += 32 * kAddWarps) again(r, c);
     for (int c4 = 0; 4 * c4 < w.n_cols; ++c4)
         if (col_bad[c4])
-            for (int i = tid; i < 4 * w.rows; i += 32 * kAddWarps) again(i >> 2, 4 * c4 + (i & 3));
+            for (int e = tid; e < 4 * w.rows; e += kThr) again(e >> 2, 4 * c4 + (e & 3));
 }
 
 // Test hook of the bounded waits (gta_debug_attention_wait): their time limit, and a switch that keeps the first accumulator's
@@ -292,7 +368,8 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
             odd |= we | wf;
         };
         auto note_odd = [&](const uint8_t* src) {
-            auto is_odd = [](float v) { return !(fabsf(v) < 3.38e38f); };       // (3.3895e38 is bf16's largest)
+            auto is_odd = [](float v) { return fabsf(v) >= 3.38e38f; };         // (3.3895e38 is bf16's largest; what is not a number
+                                                                               // makes the row or column none by itself)
             auto any_odd = [&](const float4 v) { return is_odd(v.x) || is_odd(v.y) || is_odd(v.z) || is_odd(v.w); };
             auto is_small = [](float v) { return v != 0.f && fabsf(v) < 0x1p-109f; };
             auto any_small = [&](const float4 v) { return is_small(v.x) || is_small(v.y) || is_small(v.z) || is_small(v.w); };
@@ -468,7 +545,7 @@ sm100_decoder_f32_kernel(const __grid_constant__ CUtensorMap tm_l, const __grid_
     if (warp >= kAddWarp0 && *any_bad) {
         uint32_t block;             // (worked out anew: nothing of this is kept in registers until here)
         asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
-        redo<NT>(d, o_lat, x, w_p, w_g, out, row_tiles, col_tiles, block, marks);
+        redo<NT>(d, o_lat, x, w_p, w_g, out, row_tiles, col_tiles, block, marks, reinterpret_cast<float*>(smem));
     }
     if (threadIdx.x == 0 && *abort_flag) raise_status(status_word, GTA_ERR_TIMEOUT);
 }

@@ -222,6 +222,25 @@ def test_workspace_of_a_chunk_behind_a_longer_cache(G):
         ws.check("workspace")
 
 
+@pytest.mark.parametrize("case", [(2, 500, 500, 64, 20, 5, 1, 1, True), (1, 300, 600, 64, 4, 2, 2, 1, False), (3, 1025, 1025, 96, 10, 5, 1, 1, True)])
+@pytest.mark.parametrize("what,where,value", [("c", (slice(None), slice(None), 0, 1), float("inf")), ("k", (slice(None), slice(None), 2, 5), -float("inf")),
+                                              ("x", (slice(None), slice(None), 3), float("inf")), ("w_g", (3, slice(None)), float("inf")),
+                                              ("w_p", (1, slice(None), 7), float("inf"))], ids=["c", "k", "x", "w_g", "w_p"])
+def test_infinities_that_every_row_or_column_sees(G, case, what, where, value):
+    """All rows of all tiles are done again, in blocks of rows with remainders: against the plain-ALU attention, and torch for the rest."""
+    B, N, kv, H, n_h, n_q, n_k, n_c, causal = case
+    t = _inputs(B, N, kv, H, n_h, n_q, n_k, n_c, 64, 128)
+    t[what][where] = value
+    got = _run(G, t, kv, causal)
+    if what in ("c", "k"):
+        want = _run(G, t, kv, causal, least=True)
+        assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(torch.isinf(got), torch.isinf(want))
+        ok = torch.isfinite(want)
+        assert not ok.any() or float((got - want)[ok].double().norm() / want[ok].double().norm()) <= 2 * REL
+    else:
+        torch.testing.assert_close(got, _exact(t, kv, causal).float(), rtol=1e-4, atol=1e-5, equal_nan=True)
+
+
 BAD = [("q", (0, 1, 40, 3), float("nan")), ("q", (0, 0, 299, 0), float("inf")), ("k", (0, 0, 130, 5), float("inf")),
        ("k", (0, 0, 299, 63), float("nan")), ("c", (0, 0, 70, 127), float("nan")), ("c", (0, 0, 290, 1), -float("inf")),
        ("c", (0, 0, 5, 1), 3.4e38), ("x", (0, 17, 9), float("inf")), ("x", (0, 299, 63), float("nan")),
