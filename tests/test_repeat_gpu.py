@@ -63,6 +63,68 @@ def test_prefill_paths_repeat_bit_for_bit(B, case):
     assert int(status.item()) == 0
 
 
+PREFILL_F32 = [
+    # name, B, N, kv, H, n_h, n_q, n_k, n_c, d_h, d_l
+    ("four_ctas_a_row_tile", 1, 333, 333, 256, 20, 5, 1, 1, 64, 128),
+    ("two_ctas_blocks_of_256", 2, 1500, 1500, 1280, 20, 5, 1, 1, 64, 128),
+    ("more_items_than_sms", 9, 1024, 1024, 64, 4, 2, 2, 1, 64, 128),
+    ("two_slices_a_chunk", 2, 200, 700, 128, 16, 4, 2, 2, 64, 256),
+    ("plain_attention_in_front", 5, 333, 333, 64, 8, 4, 4, 1, 128, 72),
+    ("one_kernel", 2, 128, 128, 256, 4, 2, 2, 1, 64, 128),
+]
+
+
+@pytest.mark.parametrize("case", PREFILL_F32, ids=[c[0] for c in PREFILL_F32])
+def test_fp32_prefill_paths_repeat_bit_for_bit(B, case):
+    name, nb, N, kv, H, n_h, n_q, n_k, n_c, d_h, d_l = case
+    t = I.prefill_inputs(I.Workload(name, "prefill", "f32", nb, kv, H, n_h, n_q, n_k, n_c, d_h, d_l, seed=15), device="cuda")
+    q, x = t["q"][:, :, -N:].contiguous(), t["x"][:, -N:].contiguous()
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    _repeat(lambda: B.gta_prefill_chunk(q, t["k"], t["c"], x, t["w_p"], t["w_g"], kv, status_word=status), 60, name)
+    assert int(status.item()) == 0
+
+
+def test_fp32_prefills_and_layers_in_flight_behind_one_another(B):
+    """fp32 prefills of three kernels, of two and of one over one workspace, and whole layers whose input is the output of the layer
+    before (their projections read it ahead of the kernel in front's end), queued without waiting: what each gives alone."""
+    def prefill(nb, N, H, n_h, n_q, n_k, seed):
+        w = I.Workload(f"flight{seed}", "prefill", "f32", nb, N, H, n_h, n_q, n_k, 1, 64, 128, seed=seed)
+        return I.prefill_inputs(w, device="cuda")
+    ps = [prefill(1, 333, 256, 20, 5, 1, 21), prefill(2, 120, 256, 4, 2, 2, 22), prefill(4, 500, 64, 4, 2, 2, 23), prefill(1, 700, 1280, 20, 5, 1, 24)]
+    t = I.layer_inputs(I.Workload("flight_layer", "prefill", "bf16", 2, 200, 512, 8, 4, 4, 1, 128, 512, seed=25), device="cuda")
+    ws, lws = torch.empty(1 << 26, dtype=torch.uint8, device="cuda"), torch.empty(1 << 26, dtype=torch.uint8, device="cuda")
+    k, c = torch.zeros(2, 4, 256, 128, dtype=torch.bfloat16, device="cuda"), torch.zeros(2, 1, 256, 512, dtype=torch.bfloat16, device="cuda")
+    lens0 = torch.tensor([200, 3], dtype=torch.int32, device="cuda")
+
+    def calls(wait):
+        outs, x, lens = [], t["x"], lens0.clone()
+        x_t = t["x"][:, 0].contiguous()
+
+        def keep(o):
+            outs.append(o)
+            if wait:
+                torch.cuda.synchronize()
+            return o
+        for rep in range(6):
+            for p in ps:
+                keep(B.gta_prefill(p["q"], p["k"], p["c"], p["x"], p["w_p"], p["w_g"], workspace=ws))
+            for _ in range(3):
+                x = keep(B.gta_layer_prefill(x, t["w_qkc"], t["w_p"], t["w_g"], t["w_o"], k, c, n_q=4, workspace=lws))
+            for _ in range(3):
+                x_t = keep(B.gta_layer_decode(x_t, t["w_qkc"], t["w_p"], t["w_g"], t["w_o"], k, c, lens, n_q=4, workspace=lws))
+            x, x_t = t["x"], t["x"][:, 0].contiguous()
+        return outs + [lens]
+
+    want = calls(True)
+    assert want[-1].tolist() == [218, 21]
+    for rep in range(6):
+        k.zero_(); c.zero_()
+        got = calls(False)
+        torch.cuda.synchronize()
+        for i, (a, b) in enumerate(zip(got, want)):
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), (rep, i)
+
+
 def test_layer_prefill_repeats_bit_for_bit(B):
     w = I.Workload("layer", "prefill", "bf16", 2, 640, 512, 8, 4, 4, 1, 128, 512, seed=6)
     t = I.layer_inputs(w, device="cuda")
