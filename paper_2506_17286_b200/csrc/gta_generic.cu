@@ -1,6 +1,7 @@
 // Plain-ALU (fp32 FMA) prefill kernels: any supported shape, fp32 or bf16 storage.
 // They carry small fp32 calls (larger ones run on the tensor cores in bf16 pieces, f32_plan below) and every shape
-// the tcgen05 kernels do not cover.  Two kernels:
+// the tcgen05 kernels do not cover.  Two kernels, and one (short_prefill_f32_kernel) that does the work of both for a short
+// fp32 prompt:
 //   generic_attention_kernel : shared attention map per query group, online softmax, latent
 //                              P·C  ->  normalised L[n_q, B, N, d_l] (fp32, workspace)
 //   generic_decoder_kernel   : out_i = (L_{q(i)} W_P,i) (.) sigmoid(X W_G,i)
@@ -772,10 +773,12 @@ static cudaError_t launch_decoder(const Dims& d, const float* o_lat, const T* x,
 // w512 192 / 235, tiny 28 / 28; behind 1000 503 / 533, 69 / 62), the longer the more elements a token has, whose pieces are made for so
 // few rows: all of these stay on the FMA pipe.  Decoder: 1B 200 tokens (80 tiles of 64 x 64) 32.7 / 42.7, 333
 // (120) 54.4 / 42.6; tiny 700 (44) 28.4 / 30.3, 2048 (128) 45.3 / 38.7: from 100 tiles on; in blocks of 128 columns while those of
-// 256 are few (1B, 1000 tokens, 20 blocks of 256: 54.3 / 47.1 with 128; 1500, 30: 66.2 / 73.6).
+// 256 are few (us, 128 / 256: 1B, 1000 tokens, 20 blocks of 256, 44.1 / 56.7; 1100, 25, 46.5 / 56.6; 1200, 25, 60.5 / 56.9; 1400, 30,
+// 65.7 / 58.3; 16 heads of 128, 4 maps, 700, 24, 162 / 174; 1000, 32, 251 / 244).  The line of 100 tiles, plain / 128: 1B 80 33.8 / 42.8, 100
+// 44.1 / 42.9; 16 heads of 128, 64 77.8 / 78.6, 128 88.7 / 70.1; w512 96 61.1 / 50.1, 112 64.4 / 62.3; one map of 8 heads 88 38.9 / 30.4.
 //
-// CTAs that share the keys of a row tile: a key tile takes 1.25 us, a CTA 6 us more and 1 for every one that it merges with, a stage
-// of the decoder 0.9 or 1.05 us.  The decoder's gates run beside the attention kernel where both fit the chip at once (1B, 1000
+// CTAs that share the keys of a row tile (a model fitted to the tiny and the 1B layer, with 148 places for clusters too): a key tile
+// takes 1.25 us, a CTA 6 us more and 1 for every one that it merges with, a stage of the decoder 0.9 or 1.05 us.  The decoder's gates run beside the attention kernel where both fit the chip at once (1B, 1000
 // tokens: 47.1 with one, 54.6 with two; tiny, 2048: 75.5 / 48.8 / 38.7 with one / two / four); a plain decoder wants the SMs that a
 // split takes (1B, 200 tokens: 32.7 / 43.3; tiny, 333: 26.0 / 23.3).
 //
