@@ -1,8 +1,8 @@
 // fp32 attention on the tensor cores (head width 64): L = Softmax(scale Q K^T) C per attention map.
 //
 // Operands are sums of three bf16 pieces, exactly from 2^-110 on, and six of the nine products of pieces are taken (what is left
-// out is below 2^-24 of a product, 2^-26.5 rms); see gta_sm100_f32_decoder.cu.  A sum stays in tensor memory for 64 elements of its contraction
-// (the head width; the keys of a tile), small products first, and is added up in registers (rounded) from there.
+// out is below 2^-24 of a product, 2^-26.5 rms); see gta_sm100_f32_decoder.cu.  A sum stays in tensor memory for 64 elements of
+// its contraction (the head width; the keys of a tile), small products first, and is added up in registers (rounded) from there.
 //   split_rows_kernel        writes the pieces of K and C once ([piece][row], bf16, workspace), and per tile of 64
 //                            rows the first that holds an element without pieces: every map and row tile reads them.
 //   sm100_attention_f32_kernel  a CTA (or a cluster of two or four that take the key tiles in turn and merge at the end through

@@ -4,8 +4,8 @@
 // Every fp32 operand is the sum of three bf16 pieces, exactly from 2^-110 on (8 significant bits each, rounded to nearest, the
 // rest handed on); six of the nine products of pieces are taken (what is left out, of which two can reach 2^-25 of a product
 // each, is below 2^-24 of it, 2^-26.5 rms), each exact in the tensor core, which adds them in fp32 but cuts where fp32
-// arithmetic rounds.  So a sum stays in tensor memory for 32 elements of the contraction only, small products first, and is added up in registers (rounded) from there: against 64
-// bits the result is closer than the FMA chain of the plain-ALU kernel.
+// arithmetic rounds.  So a sum stays in tensor memory for 32 elements of the contraction only, small products first, and is
+// added up in registers (rounded) from there: against 64 bits the result is closer than the FMA chain of the plain-ALU kernel.
 //
 // CTA pairs, one item of 256 token rows x NT output columns of one attention map per pair.
 //   warp 0       (leader CTA) issues the MMAs: twelve per stage, two accumulators in tensor memory in turn.
@@ -20,8 +20,7 @@
 //
 // An element that is infinite, not a number or rounds to infinity in bf16 makes its row or column of the item not a number
 // (0 x infinity); the splitting threads see it, and where it is an infinity or a large number those rows and columns are done again
-// with plain FMAs.  So are rows and
-// columns whose elements are all too small for pieces (kPiecesFloor).
+// with plain FMAs.  So are rows and columns whose elements are all too small for pieces (kPiecesFloor).
 #include "gta_sm100.cuh"
 
 #include <cuda.h>
